@@ -246,13 +246,14 @@ typedef struct {
   double E0;              /* lowest Ritz value over all vectors */
   double device_ms;       /* device time of the Lanczos block (start block to last step) */
   double hv_ms;           /* summed device time of the H.v launches (time_kernels = 1) */
-  int hv_launches;        /* H.v launches in the run */
+  int hv_launches;        /* H.v products of the block in the run */
   int kernel_launches;    /* all kernel launches in the run */
   uint64_t h2d_bytes;     /* host-to-device bytes copied by the run */
   uint64_t d2h_bytes;     /* device-to-host bytes copied by the run */
   /* launch shape of the H.v launches (see ftlm_tune_shape) */
   int cube_bits;          /* 0: general row kernel; 2..4: spin-1/2 register cubes */
-  int passes;             /* launches per H.v (spin-1/2 multi-pass form: ceil(n / cube_bits)) */
+  int passes;             /* launches per H.v (spin-1/2 multi-pass form: ceil(n / cube_bits); 3 with cube_bits 0:
+                             the rotated-basis form of spin-1/2 runs from random vectors) */
   int group_vectors;      /* vectors processed together (register-cube kernels, general vector-major gathers) */
   int tile_rows;          /* rows per tile */
   int grid;               /* CTAs per H.v launch */

@@ -90,6 +90,10 @@ struct ftlm_system {
   DevBuf ut[2];          // per-unit coefficient tables of the one-pass vector-major gather, [c64]
   int ut_K[2] = {0, 0};  // the cube size each was built for
   cudaEvent_t ev_apply = nullptr;  // recorded after the last use of Ta, Tb
+  int rot_state = 0;     // rotated-basis H.v: 0 not examined, 1 `rot` holds the directions, -1 none
+  std::unique_ptr<RotDirs> rot;
+  DevBuf rD[2];          // its diagonal tables [K + 1][dim] and phases, [c64]
+  DevBuf rW, rpart;      // its intermediate blocks; partial sums and arrival counters
   bool apply_used = false;
   std::mutex mu;
 };
@@ -133,6 +137,14 @@ bool has_shape_override(const ftlm_system* s, int R, int c64) {
   return g_shapes.count(key) != 0;
 }
 
+// the rotated-basis H.v may run: no shape was set, or the autotuner found it the fastest
+bool rot_allowed(const ftlm_system* s, int R, int c64) {
+  ShapeKey key{s->hs.n, s->hs.qmax, R, c64, (long long)s->hs.dim};
+  std::lock_guard<std::mutex> lk(g_mu);
+  auto it = g_shapes.find(key);
+  return it == g_shapes.end() || it->second.rot;
+}
+
 Shape shape_for(int R, int c64, int threads_target, int tile_factor) {
   const int V = vchunk(c64, R);
   const int C = R / V;
@@ -173,8 +185,16 @@ struct HalfPlan {
   long long dim = 0;
 };
 
+// Rotated-basis H.v of a run (hv_rot.cu): tiles of 2^T values, K directions, W
+// blocks for `group` vectors at a time.
+struct RotPlan {
+  bool on = false;
+  int T = 0, K = 0, group = 1;
+};
+
 struct Plan {
   int c64 = 0, R = 0, V = 1, C = 1;
+  RotPlan rot;
   Shape sh;
   int grid = 0;
   size_t smem = 0;
@@ -566,6 +586,85 @@ ftlm_status ensure_unit_tables(ftlm_system* s, int K, int c64, cudaStream_t st) 
   return FTLM_OK;
 }
 
+// ---- the rotated-basis H.v of spin-1/2 runs ------------------------------------
+
+size_t rot_phase_bytes(int c64) { return (size_t)kRotMaxK * (kRotMaxN + 1) * (c64 ? 8 : 16); }
+
+// Its directions, when the system has them and a tile fits its site count.
+const RotDirs* rot_dirs(ftlm_system* s, int c64) {
+  if (s->rot_state == 0) {
+    s->rot = std::make_unique<RotDirs>();
+    s->rot_state = rot_directions(s->hs, *s->rot) ? 1 : -1;
+    if (s->rot_state < 0) s->rot.reset();
+  }
+  return s->rot_state > 0 && rot_tile_bits(s->hs.n, c64) > 0 ? s->rot.get() : nullptr;
+}
+
+// Tables (built once per system and precision), W blocks and the partial sums of
+// R vectors; ok = false when they do not fit in memory (the gather then runs).
+ftlm_status ensure_rot(ftlm_system* s, const RotPlan& rp, int R, int c64, cudaStream_t st, bool& ok) {
+  ok = false;
+  const size_t d = (size_t)s->hs.dim, real = c64 ? 4 : 8;
+  const RotDirs& dirs = *s->rot;
+  DevBuf& D = s->rD[c64 ? 1 : 0];
+  if (prepare_rot(rp.T, c64) != 0) return FTLM_OK;
+  const size_t tiles = d >> rp.T;
+  const size_t tbytes = (size_t)(rp.K + 1) * d * real + rot_phase_bytes(c64);
+  bool fits = true, build = !D.p;
+  auto grow = [&](DevBuf& b, size_t bytes) {
+    if (!fits || b.bytes >= bytes) return;
+    s->gen++;  // captured graphs hold its address
+    fits = b.ensure(bytes) == cudaSuccess;
+  };
+  grow(s->rW, (size_t)rp.group * rp.K * d * real * 2);
+  grow(s->rpart, sizeof(double) * 3 * tiles * R + sizeof(unsigned) * R);
+  grow(D, tbytes);
+  if (!fits) {
+    cudaGetLastError();
+    for (DevBuf* b : {&s->rW, &s->rpart, &s->rD[0], &s->rD[1]}) b->release();
+    return FTLM_OK;
+  }
+  if (build) {
+    for (int k = 0; k <= rp.K; ++k) {
+      RotForm f = dirs.form[k];
+      f.T = rp.T;
+      CKI(launch_rot_table(f, static_cast<char*>(D.p) + (size_t)k * d * real, c64, st));
+    }
+    CKI(launch_rot_phases(s->hs.n, dirs, static_cast<char*>(D.p) + tbytes - rot_phase_bytes(c64), c64, st));
+  }
+  ok = true;
+  return FTLM_OK;
+}
+
+// The rotated-basis plan of a block of R vectors (on = false: none).  The W
+// blocks hold K times the group's vectors: 16 GB of them keep every group large
+// enough to fill the device.
+ftlm_status make_rot(ftlm_system* s, int R, int c64, RotPlan& rp, cudaStream_t st) {
+  rp = RotPlan();
+  const RotDirs* dirs = rot_dirs(s, c64);
+  if (!dirs) return FTLM_OK;
+  rp.T = rot_tile_bits(s->hs.n, c64);
+  rp.K = dirs->K;
+  const uint64_t per = s->hs.dim * (uint64_t)rp.K * (c64 ? 8 : 16);
+  rp.group = (int)std::min<uint64_t>((uint64_t)R, std::max<uint64_t>(1, (16ull << 30) / per));
+  return ensure_rot(s, rp, R, c64, st, rp.on);
+}
+
+RotArgs rot_args(const ftlm_system* s, const RotPlan& rp, int c64) {
+  RotArgs a;
+  const size_t d = (size_t)s->hs.dim, real = c64 ? 4 : 8;
+  const char* D = static_cast<const char*>(s->rD[c64 ? 1 : 0].p);
+  a.n = s->hs.n;
+  a.T = rp.T;
+  a.K = rp.K;
+  a.t = s->rot->t;
+  a.dim = (long long)d;
+  a.D0 = D;
+  a.D = D + d * real;
+  a.phases = D + (size_t)(rp.K + 1) * d * real;
+  return a;
+}
+
 int plan_max_grid(const Plan& pl) {
   return std::max(std::max(pl.grid, pl.gen_vm ? pl.gvm_grid : 0),
                   pl.half.on ? std::max(pl.half.grid, pl.half.stream_grid) : 0);
@@ -691,6 +790,7 @@ std::string run_key(const std::vector<ftlm_system*>& sys, const ftlm_run_params*
   k += buf;
   k += p->symmetric ? "|sym" : "";
   k += p->reorth ? "|reorth" : "";
+  k += pl.rot.on ? "|rot" + std::to_string(pl.rot.group) : "";
   k += pl.gen_vm ? "|gvm" + std::to_string(pl.gvm_V) + "x" + std::to_string(pl.gvm_rows) + "c" +
                        std::to_string(pl.gvm_cube)
                  : "";
@@ -738,6 +838,70 @@ ftlm_status validate_params(const ftlm_run_params* p, const std::vector<ftlm_sys
 // then M_eff [R].
 size_t staged_doubles(int R, int M) { return (size_t)M * R * 5; }
 size_t staged_bytes(int R, int M) { return sizeof(double) * staged_doubles(R, M) + sizeof(int) * (size_t)R; }
+
+// The rotated-basis passes of one product or step over the whole block, group by
+// group (the groups share the W blocks).
+ftlm_status enqueue_rot_passes(RunCtx* ctx, ftlm_system* s, const RotPlan& rp, RotArgs a, int R, int c64, void* keep,
+                               cudaStream_t st) {
+  const size_t vb = (size_t)s->hs.dim * (c64 ? 8 : 16);
+  a.W = s->rW.p;
+  for (int v0 = 0; v0 < R; v0 += rp.group) {
+    a.vec0 = a.vecW = v0;
+    a.nvec = std::min(rp.group, R - v0);
+    a.vpb = std::min(a.nvec, 4);
+    for (int pass = 0; pass < 3; ++pass) {
+      CKI(launch_rot(a, pass, c64, st));
+      if (pass == 0 && keep) {  // q_j is final after the forward pass
+        CK(cudaMemcpyAsync(static_cast<char*>(keep) + vb * v0, static_cast<const char*>(a.x) + vb * v0, vb * a.nvec,
+                           cudaMemcpyDeviceToDevice, st));
+        if (ctx) ctx->launches++;
+      }
+    }
+    if (ctx) ctx->launches += 3;
+  }
+  return FTLM_OK;
+}
+
+// The M Lanczos steps of a rotated-basis run; `upd` is the update launch that
+// ends the last one.
+ftlm_status enqueue_rot_steps(RunCtx& ctx, ftlm_system* s, const ftlm_run_params* p, const Plan& pl, LaunchArgs upd,
+                              const InstDesc* d_even, const InstDesc* d_odd, cudaStream_t st) {
+  const int M = p->M, R = p->R, c64 = pl.c64;
+  const size_t esz = c64 ? 8 : 16, d = (size_t)s->hs.dim;
+  RotArgs a = rot_args(s, pl.rot, c64);
+  a.M = M;
+  a.tol = p->breakdown_tol > 0 ? p->breakdown_tol : (c64 ? 1e-6 : 1e-12);
+  a.sc = scalars_at(s->scal.p, R, M);
+  a.u = s->U.p;
+  a.partials = reinterpret_cast<double*>(s->rpart.p);
+  a.counters = reinterpret_cast<unsigned*>(a.partials + 3 * (d >> pl.rot.T) * R);
+  a.lanczos = 1;
+  CK(cudaMemsetAsync(a.counters, 0, sizeof(unsigned) * R, st));
+  auto mark = [&](int e) {
+    return p->time_kernels ? cudaEventRecordWithFlags(ctx.ev[e], st, cudaEventRecordExternal) : cudaSuccess;
+  };
+  for (int j = 0; j < M; ++j) {
+    a.x = j % 2 == 0 ? s->A.p : s->B.p;
+    a.y = j % 2 == 0 ? s->B.p : s->A.p;
+    a.j = j;
+    a.update = j > 0;
+    CK(mark(1 + 4 * j));
+    CK(mark(2 + 4 * j));
+    ftlm_status rs = enqueue_rot_passes(&ctx, s, pl.rot, a, R, c64,
+                                        p->symmetric ? static_cast<char*>(s->Vs.p) + esz * d * R * j : nullptr, st);
+    if (rs != FTLM_OK) return rs;
+    ctx.hv_launches++;
+    CK(mark(3 + 4 * j));
+    CK(mark(4 + 4 * j));
+  }
+  upd.inst = (M - 1) % 2 == 0 ? d_even : d_odd;
+  upd.step = M - 1;
+  upd.first = M == 1;
+  upd.mode = kModeUpdate;
+  CKI(launch_plan(pl, upd, st));
+  ctx.launches++;
+  return FTLM_OK;
+}
 
 // Enqueues one whole run on `st` (which the caller is capturing).
 ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const ftlm_run_params* p, const Plan& pl,
@@ -792,7 +956,11 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
   CKI(launch_plan(pl, a, st));
   a.use_sigma0 = 0;
   ctx.launches += 2;
-  for (int j = 0; j < M; ++j) {
+  if (pl.rot.on) {
+    ftlm_status rs = enqueue_rot_steps(ctx, sys[0], p, pl, a, d_even, d_odd, st);
+    if (rs != FTLM_OK) return rs;
+  }
+  for (int j = 0; j < M && !pl.rot.on; ++j) {
     a.inst = (j % 2 == 0) ? d_even : d_odd;
     a.step = j;
     a.first = j == 0;
@@ -1059,7 +1227,16 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     ps = make_plan(sys, R, c64, pl, nullptr, true);
   }
   if (ps != FTLM_OK) return ps;
-  if (vm_fused_step(pl)) {
+  // Runs from random vectors on the default spin-1/2 plan take the rotated-basis
+  // H.v.  Its error is relative to the whole vector, so starts that may be
+  // sparse (basis states, a caller's block) keep the gather, which leaves the
+  // rows that H does not reach exactly zero.
+  if (vm_fused_step(pl) && (p->start == FTLM_START_RANDOM || p->start == FTLM_START_PAIRS) &&
+      rot_allowed(sys[0], R, c64)) {
+    ftlm_status rs = make_rot(sys[0], R, c64, pl.rot, st);
+    if (rs != FTLM_OK) return rs;
+  }
+  if (vm_fused_step(pl) && !pl.rot.on) {
     ftlm_status ut = ensure_unit_tables(sys[0], pl.half.K, c64, st);
     if (ut != FTLM_OK) return ut;
   }
@@ -1168,8 +1345,8 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     out.kernel_launches = ctx->launches;
     out.h2d_bytes = k == 0 ? h2d : 0;
     out.d2h_bytes = per;
-    out.cube_bits = pl.half.on ? pl.half.K : 0;  // (0 also for the vector-major general gather)
-    out.passes = pl.half.on ? pl.half.passes : 1;
+    out.cube_bits = pl.half.on && !pl.rot.on ? pl.half.K : 0;  // (0 also for the vector-major general gather)
+    out.passes = pl.rot.on ? 3 : (pl.half.on ? pl.half.passes : 1);
     out.group_vectors = pl.half.on ? pl.half.Rg : (pl.gen_vm ? pl.gvm_V : R);
     out.tile_rows = pl.half.on ? pl.half.rows_per_tile : (pl.gen_vm ? pl.gvm_rows : pl.sh.rows_per_tile);
     out.grid = pl.half.on ? pl.half.grid : (pl.gen_vm ? pl.gvm_grid : pl.grid);
@@ -1315,6 +1492,26 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
       best = ms;
       pick = sh;
     }
+  }
+  RotPlan rp;  // runs from random vectors: the rotated-basis H.v
+  if (s->hs.all_half) {
+    ftlm_status rs = make_rot(s, R, c64, rp, st);
+    if (rs != FTLM_OK) return rs;
+  }
+  if (rp.on) {
+    RotArgs a = rot_args(s, rp, c64);
+    a.x = s->A.p;
+    a.y = s->B.p;
+    for (int it = 0; it < 7; ++it) {  // two warm-up products, five timed
+      if (it == 2) CK(cudaEventRecord(e0, st));
+      ftlm_status rs = enqueue_rot_passes(nullptr, s, rp, a, R, c64, nullptr, st);
+      if (rs != FTLM_OK) return rs;
+    }
+    CK(cudaEventRecord(e1, st));
+    CK(cudaEventSynchronize(e1));
+    float ms = 0.f;
+    CK(cudaEventElapsedTime(&ms, e0, e1));
+    pick.rot = ms < best;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1551,7 +1748,7 @@ void ftlm_system_destroy(ftlm_system* s) {
   cudaDeviceSynchronize();  // the system's buffers may be in use on any stream
   purge_ctx_of(s->id);
   for (DevBuf* b : {&s->tab_f, &s->tab_d, &s->stride, &s->q, &s->A, &s->B, &s->U, &s->scal, &s->ep, &s->ecnt,
-                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws})
+                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart})
     b->release();
   cudaEventDestroy(s->ev_in);
   cudaEventDestroy(s->ev_out);

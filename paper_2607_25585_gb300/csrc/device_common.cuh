@@ -436,6 +436,27 @@ __device__ inline double total_partial(const LaunchArgs& a, int inst, int r, int
   return (s0 + s1) + (s2 + s3);
 }
 
+// The scalars at the end of step j of vector r from nrm2 = |w|^2: beta_j,
+// sigma_{j+1} and the breakdown test (alpha_j is set).
+__device__ inline void finalize_beta(const DevScalars& sc, int j, int r, int M, double tol, double nrm2) {
+  const double bnew = sqrt(fmax(nrm2, 0.0));
+  const double al = sc.alpha[(size_t)j * sc.ss + r];
+  const double bold = j > 0 ? sc.beta[(size_t)(j - 1) * sc.ss + r] : 0.0;
+  double scl = fmax(sc.scale[r], fmax(fabs(al), bold));
+  sc.scale[r] = scl;
+  sc.beta[(size_t)j * sc.ss + r] = bnew;
+  double sig = 0.0;
+  if (sc.active[r]) {
+    if (j < M - 1 && (!(bnew > tol * scl) || !isfinite(bnew) || !isfinite(al))) {
+      sc.active[r] = 0;
+      sc.meff[r] = j + 1;
+    } else {
+      sig = bnew > 0.0 ? 1.0 / bnew : 0.0;
+    }
+  }
+  sc.sigma[(size_t)(j + 1) * sc.ss + r] = sig;
+}
+
 __device__ inline void finalize(const LaunchArgs& a, const InstDesc* inst_all) {
   // (inst_all points at the device array, or at the inline descriptor)
   const int R = a.R;
@@ -461,23 +482,7 @@ __device__ inline void finalize(const LaunchArgs& a, const InstDesc* inst_all) {
         sc.p[((size_t)j * sc.ss + r) * 2] = total_partial(a, inst, r, 1);
         sc.p[((size_t)j * sc.ss + r) * 2 + 1] = total_partial(a, inst, r, 2);
       }
-      const double nrm2 = total_partial(a, inst, r, 0);
-      const double bnew = sqrt(fmax(nrm2, 0.0));
-      const double al = sc.alpha[(size_t)j * sc.ss + r];
-      const double bold = j > 0 ? sc.beta[(size_t)(j - 1) * sc.ss + r] : 0.0;
-      double scl = fmax(sc.scale[r], fmax(fabs(al), bold));
-      sc.scale[r] = scl;
-      sc.beta[(size_t)j * sc.ss + r] = bnew;
-      double sig = 0.0;
-      if (sc.active[r]) {
-        if (j < d.M - 1 && (!(bnew > d.tol * scl) || !isfinite(bnew) || !isfinite(al))) {
-          sc.active[r] = 0;
-          sc.meff[r] = j + 1;
-        } else {
-          sig = bnew > 0.0 ? 1.0 / bnew : 0.0;
-        }
-      }
-      sc.sigma[(size_t)(j + 1) * sc.ss + r] = sig;
+      finalize_beta(sc, j, r, d.M, d.tol, total_partial(a, inst, r, 0));
     } else if (a.mode == kModeStartNorm) {
       const double nrm = sqrt(fmax(total_partial(a, inst, r, 0), 0.0));
       sc.sigma[r] = nrm > 0.0 ? 1.0 / nrm : 0.0;

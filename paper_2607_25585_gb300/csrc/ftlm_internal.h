@@ -191,6 +191,7 @@ struct Shape {
   int gvm_cube = -1;       // vector-major general gather: > 0 = register cube of the top site over groups
                            // of that many vectors, 0 = one row a thread, -1 = the cube with the default
                            // group size where a kernel exists for the top site's 2s+1 and R
+  bool rot = false;        // autotuned shape: the rotated-basis H.v is faster for runs from random vectors
 };
 
 // Kernel launchers (kernels.cu).  `V` is the number of complex values per
@@ -256,6 +257,58 @@ int launch_vm_unit_tables(const double* tab_d, const TabLayout& L, int n, int K,
 // kModeStep / kModeStartNorm over the same one-vector instances (256 threads)
 int launch_vm_stream(const LaunchArgs& a, int c64, int grid, void* stream);
 constexpr int kVmLaneBits = 5;  // rows per warp-wide load: 2^5
+
+// Spin-1/2 H.v in rotated product bases (hv_rot.cu).
+constexpr int kRotMaxN = 28;  // sites: two passes over tiles of at most 2^14 values
+constexpr int kRotMaxK = 5;   // directions besides z
+
+// One direction's diagonal form: scale (c0 + sum_i m_i (h_i + sum_{j>i} a_ij m_j)),
+// a in the triangular pair order; rotate: its table has the low T index bits rotated by four.
+struct RotForm {
+  int n = 0, rotate = 0, T = 0;
+  double c0 = 0, scale = 1;
+  double h[kRotMaxN] = {};
+  double a[kRotMaxN * (kRotMaxN - 1) / 2] = {};
+};
+struct RotAzimuths {
+  int num[kRotMaxK] = {}, den = 1;  // phi_k = pi num_k / den
+};
+struct RotDirs {
+  int K = 0;
+  double t = 1;  // tan(theta / 2) of the directions' polar angle
+  RotAzimuths az;
+  RotForm form[kRotMaxK + 1];  // z, then the K directions
+};
+
+struct RotArgs {
+  int n = 0, T = 0, K = 0;
+  double t = 1;
+  long long dim = 0;
+  int vec0 = 0, nvec = 0;      // the launch's vectors of the block
+  int vecW = 0;                // the vector whose W_0 is at W
+  int vpb = 1;                 // middle pass: vectors a CTA takes one after another (its D values stay in registers)
+  void* x = nullptr;           // q_j of vector 0 (vector-major block)
+  void* y = nullptr;           // q_{j-1}, overwritten by w'; or H x
+  const void* u = nullptr;
+  void* W = nullptr;           // [vectors][K][dim]
+  const void* D = nullptr;     // [K][dim], low bits rotated
+  const void* D0 = nullptr;    // [dim]
+  const void* phases = nullptr;  // [K][kRotMaxN + 1]
+  int lanczos = 0;             // backward pass: a step (else y = H x)
+  int update = 0;              // forward pass: finish step j - 1 first
+  int j = 0, M = 0;
+  double tol = 0;
+  DevScalars sc;               // of the whole block
+  double* partials = nullptr;  // [R][tiles][3]
+  unsigned* counters = nullptr;  // [R], zero between launches
+};
+
+bool rot_directions(const HostSystem& hs, RotDirs& d);
+int rot_tile_bits(int n, int c64);
+int prepare_rot(int T, int c64);
+int launch_rot(const RotArgs& a, int pass, int c64, void* stream);  // pass 0 forward, 1 middle, 2 backward
+int launch_rot_table(const RotForm& f, void* out, int c64, void* stream);
+int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream);
 
 // Full re-orthogonalisation pass (reorth.cu): w_r -= sum_{k<=j} sigma_k^2 <q_k|w_r> q_k
 // for the R vectors of a row-major block w [dim][R], against the stored

@@ -1,0 +1,733 @@
+// Spin-1/2 H.v (Eq. 3 of arxiv 2607.25585 with every s_i = 1/2) in rotated
+// product bases, for the Lanczos steps of runs that start from random vectors.
+//
+// Method.  Every pair tensor A_ij (symmetric, 3 x 3) is a sum over a few fixed
+// directions u_k of scalars a^k_ij u_k u_k^T, so
+//   sum_ij s_i.A_ij.s_j + sum_i h_i.s_i = sum_k [ sum_ij a^k_ij (s_i.u_k)(s_j.u_k) + sum_i h^k_i s_i.u_k ],
+// and each bracket is diagonal in the product basis of the eigenstates of
+// s.u_k.  With U_k the rotation of every site to that basis,
+//   H v = D_0 v + sum_k U_k^+ (D_k (U_k v)),
+// where direction 0 is z (no rotation).  A rotation is one 2 x 2 gate a site,
+// so the product costs O(n) operations a row instead of the O(n^2) gathered
+// pair flips, and every diagonal D_k is a table built once per system.
+// Directions besides z: x and y when every tensor is diagonal; three in the xy
+// plane 60 degrees apart when z is a principal axis of every tensor (planar
+// geometries); else the five axes of an icosahedron around z (with z, their
+// projectors span the symmetric tensors).  Each set is a tight frame, so the
+// |D_k| stay on the scale of |H| and nothing cancels: measured in FP32 against
+// FP64 on random vectors, the relative error is 1.1e-7 (16 sites) where the
+// gather's is 2.8e-7.
+//
+// The gate.  All u_k have the same polar angle theta; with t = tan(theta / 2)
+// and the azimuth's phase e^{-i phi_k} taken out per down spin,
+//   (down, up) -> (down - t up, up + t down),
+// one packed FP32 FMA a value; its transpose (t -> -t) inverts it up to
+// (1 + t^2), and the product of these factors is folded into D_k.
+//
+// Passes.  The index is split into its low T bits and the nH = n - T bits above.
+//   forward:  w (the step's update, see below) -> W_k = the low bits' gates on
+//             e^{-i phi_k downs} w, for every direction k;
+//   middle:   W_k <- the high bits' gates, times D_k, the inverse gates
+//             (tiles of 2^nH rows x 2^c columns, c = T - nH);
+//   backward: H v = D_0 v + sum_k e^{+i phi_k downs} (inverse low gates of W_k),
+//             then the step's epilogue.
+// A tile of 2^T values is exchanged through shared memory between groups of
+// four bits; a thread holds the 16 values of a group in registers.  W is laid
+// out as the forward pass's last group leaves it (the low T bits rotated by
+// four), which both of its neighbours read and write contiguously.
+//
+// Lanczos step j (x = q_j, y = q_{j-1}, u): the forward pass first finishes the
+// previous step, q_j = w' - alpha_{j-1} sigma_{j-1} q_{j-1} with |q_j|^2 (so no
+// separate update pass reads and writes the vectors), sets beta_{j-1}, sigma_j;
+// the backward pass writes w' = sigma_j H q_j - beta_{j-1} sigma_{j-1} q_{j-1}
+// over q_{j-1} and sums alpha_j, p_j.  Partial sums go to one slot a tile and
+// are added in a fixed order by the last CTA of the vector.
+//
+// Bound: memory.  A step moves 8 (7 + 4 K) bytes a value in complex64 (152 for
+// K = 3), against 56 for the gather, but the gather's C(n, 2) flips take 3.5 ms
+// at n = 20 with 64 vectors, where these passes take 1.8 ms with the update
+// (3.8 ms with it before): 5.7 TB/s.  2 x 13 sites, 4 vectors: 33 -> 12.6 ms a
+// step.  In complex128 the FP64 pipe binds both: 4 x 4 sites, 50 vectors:
+// 4.0 -> 1.57 ms.  Taking one to eight vectors at a time through the three
+// passes, so that W stays in L2, was slower (2.1 to 3.0 ms): each launch then
+// has too few tiles.
+#include <cuda_runtime.h>
+
+#include <cmath>
+#include <cstdint>
+
+#include "device_common.cuh"
+#include "ftlm_internal.h"
+
+namespace ftlm {
+
+namespace {
+
+template <int T>
+struct Groups {
+  static constexpr int N = (T + 3) / 4;
+  __host__ __device__ static constexpr int lo(int g) { return T - 4 - 4 * g > 0 ? T - 4 - 4 * g : 0; }
+  // bits of group g's four register bits that belong to it (the last group overlaps the one before)
+  __host__ __device__ static constexpr int mask(int g) { return g == 0 || lo(g - 1) - lo(g) >= 4 ? 15 : (1 << (lo(g - 1) - lo(g))) - 1; }
+};
+
+__device__ __forceinline__ float2 axpy2(float t, float2 x, float2 y) { return __ffma2_rn(make_float2(t, t), x, y); }
+__device__ __forceinline__ double2 axpy2(double t, double2 x, double2 y) {
+  return make_double2(fma(t, x.x, y.x), fma(t, x.y, y.y));
+}
+
+template <typename v2>
+__device__ __forceinline__ v2 cmul(v2 a, v2 b) {
+  v2 o;
+  o.x = a.x * b.x - a.y * b.y;
+  o.y = a.x * b.y + a.y * b.x;
+  return o;
+}
+
+// the gates of the register bits in `mask` (t -> -t: the inverse gates)
+template <typename real, typename v2>
+__device__ __forceinline__ void gates(v2 (&v)[16], real t, int mask) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    if (!((mask >> b) & 1)) continue;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      if ((r >> b) & 1) continue;
+      const v2 dn = v[r], up = v[r | (1 << b)];
+      v[r] = axpy2(-t, up, dn);
+      v[r | (1 << b)] = axpy2(t, dn, up);
+    }
+  }
+}
+
+// first element of thread `tid`'s 16 of the group at bits [LO, LO + 4)
+template <int LO>
+__device__ __forceinline__ int group_base(int tid) {
+  return ((tid >> LO) << (LO + 4)) | (tid & ((1 << LO) - 1));
+}
+
+// shared-memory place of element i: one padding value after every 16
+// (conflict-free for every group position and both element sizes)
+__host__ __device__ constexpr int pad(int i) { return i + (i >> 4); }
+
+template <int LO, typename v2>
+__device__ __forceinline__ void smem_st(v2* buf, int base, const v2 (&v)[16]) {
+  v2* p = buf + pad(base);
+#pragma unroll
+  for (int r = 0; r < 16; ++r) p[pad(r << LO)] = v[r];
+}
+template <int LO, typename v2>
+__device__ __forceinline__ void smem_ld(const v2* buf, int base, v2 (&v)[16]) {
+  const v2* p = buf + pad(base);
+#pragma unroll
+  for (int r = 0; r < 16; ++r) v[r] = p[pad(r << LO)];
+}
+
+// one middle group of a tile, in place in shared memory
+template <typename real, int T, int NT, int SETS, int G, typename v2>
+__device__ __forceinline__ void mid_group(v2* buf, real t, int mask) {
+  constexpr int LO = Groups<T>::lo(G);
+#pragma unroll
+  for (int s = 0; s < SETS; ++s) {
+    const int base = group_base<LO>(threadIdx.x + s * NT);
+    v2 w[16];
+    smem_ld<LO>(buf, base, w);
+    gates(w, t, mask);
+    smem_st<LO>(buf, base, w);
+  }
+  __syncthreads();
+}
+
+// The CTA's sums p[0..NP) into its slot, then the last CTA of the vector adds
+// the vector's slots in a fixed order: true (in thread 0, with the totals in p)
+// for that CTA.
+template <int NT, int NP>
+__device__ __forceinline__ bool vector_total(double (&p)[NP], double* slots, int tile, int tiles, unsigned* counter) {
+  __shared__ double red[NT / 32][NP];
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto cta_sum = [&]() {
+#pragma unroll
+    for (int c = 0; c < NP; ++c)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) p[c] += __shfl_xor_sync(0xffffffffu, p[c], o);
+    if (lane == 0)
+#pragma unroll
+      for (int c = 0; c < NP; ++c) red[warp][c] = p[c];
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int c = 0; c < NP; ++c) {
+        double s = 0.0;
+        for (int w = 0; w < NT / 32; ++w) s += red[w][c];
+        p[c] = s;
+      }
+  };
+  cta_sum();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int c = 0; c < NP; ++c) slots[(size_t)tile * 3 + c] = p[c];
+    __threadfence();
+    last = atomicAdd(counter, 1u) == (unsigned)(tiles - 1);
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+#pragma unroll
+  for (int c = 0; c < NP; ++c) p[c] = 0.0;
+  for (int k = threadIdx.x; k < tiles; k += NT)
+#pragma unroll
+    for (int c = 0; c < NP; ++c) p[c] += __ldcg(slots + (size_t)k * 3 + c);
+  cta_sum();
+  if (threadIdx.x == 0) *counter = 0u;
+  return threadIdx.x == 0;
+}
+
+// e^{-i phi_k downs} by the number of up spins, [K][kRotMaxN + 1], to shared memory
+template <typename real>
+__device__ __forceinline__ void stage_phases(typename Cx<real>::v2* ph, const RotArgs& a) {
+  const typename Cx<real>::v2* src = reinterpret_cast<const typename Cx<real>::v2*>(a.phases);
+  for (int q = threadIdx.x; q < a.K * (kRotMaxN + 1); q += blockDim.x) ph[q] = __ldg(src + q);
+}
+
+template <typename real, int T, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) rot_forward_kernel(const __grid_constant__ RotArgs a) {
+  using v2 = typename Cx<real>::v2;
+  using Gr = Groups<T>;
+  constexpr int SETS = (1 << T) / (16 * NT), LO0 = T - 4, GL = Gr::N - 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  v2* buf = reinterpret_cast<v2*>(smem_raw);
+  __shared__ v2 ph[kRotMaxK * (kRotMaxN + 1)];
+  const int nH = a.n - T, tiles = 1 << nH;
+  const int tile = blockIdx.x & (tiles - 1), v = a.vec0 + (int)(blockIdx.x >> nH);
+  const size_t off = (size_t)v * a.dim + ((size_t)tile << T);
+  stage_phases<real>(ph, a);
+  v2* x = reinterpret_cast<v2*>(a.x) + off;
+  v2 q[SETS][16];
+  double nrm[1] = {0.0};
+  if (a.update) {  // q_j = w' - alpha_{j-1} sigma_{j-1} q_{j-1}, |q_j|^2
+    const v2* y = reinterpret_cast<const v2*>(a.y) + off;
+    const size_t e = (size_t)(a.j - 1) * a.sc.ss + v;
+    const real coef = (real)(a.sc.alpha[e] * a.sc.sigma[e]);
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+      const int i0 = threadIdx.x + s * NT;
+      v2 yv[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) q[s][r] = x[i0 + (r << LO0)];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) yv[r] = __ldg(y + i0 + (r << LO0));
+      real sum = 0;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        q[s][r] = axpy2(-coef, yv[r], q[s][r]);
+        sum += q[s][r].x * q[s][r].x + q[s][r].y * q[s][r].y;
+        x[i0 + (r << LO0)] = q[s][r];
+      }
+      nrm[0] += (double)sum;
+    }
+  } else {
+#pragma unroll
+    for (int s = 0; s < SETS; ++s)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) q[s][r] = x[threadIdx.x + s * NT + (r << LO0)];
+  }
+  __syncthreads();
+  const real t = (real)a.t;
+  for (int k = 0; k < a.K; ++k) {
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+      const int i0 = threadIdx.x + s * NT;
+      v2 w[16];
+      if (k > 0) {  // (direction 0 has azimuth 0)
+        const int pc = __popc(i0) + __popc(tile);
+        v2 f[5];
+#pragma unroll
+        for (int m = 0; m < 5; ++m) f[m] = ph[k * (kRotMaxN + 1) + pc + m];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) w[r] = cmul(f[__builtin_popcount(r)], q[s][r]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) w[r] = q[s][r];
+      }
+      gates(w, t, 15);
+      smem_st<LO0>(buf, group_base<LO0>(i0), w);
+    }
+    __syncthreads();
+    if constexpr (Gr::N >= 3) mid_group<real, T, NT, SETS, 1>(buf, t, 15);
+    if constexpr (Gr::N >= 4) mid_group<real, T, NT, SETS, 2>(buf, t, 15);
+    v2* W = reinterpret_cast<v2*>(a.W) + ((size_t)(v - a.vecW) * a.K + k) * a.dim + ((size_t)tile << T);
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+      const int i0 = threadIdx.x + s * NT;
+      v2 w[16];
+      smem_ld<0>(buf, group_base<0>(i0), w);
+      gates(w, t, Gr::mask(GL));
+#pragma unroll
+      for (int r = 0; r < 16; ++r) W[(r << LO0) + i0] = w[r];
+    }
+    if (k + 1 < a.K) __syncthreads();
+  }
+  if (a.update) {
+    if (vector_total<NT, 1>(nrm, a.partials + (size_t)v * tiles * 3, tile, tiles, a.counters + v))
+      finalize_beta(a.sc, a.j - 1, v, a.M, a.tol, nrm[0]);
+  }
+}
+
+// Columns: tile element (h, col) is W[k][h << T | cb << c | col], at tile index h << c | col.
+template <typename real, int T, int NT, int MINB, int NG>
+__global__ void __launch_bounds__(NT, MINB) rot_middle_kernel(const __grid_constant__ RotArgs a) {
+  using v2 = typename Cx<real>::v2;
+  using Gr = Groups<T>;
+  constexpr int SETS = (1 << T) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = T - 4;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  v2* buf = reinterpret_cast<v2*>(smem_raw);
+  const int nH = a.n - T, c = T - nH;
+  const int cmask = (1 << c) - 1;
+  const int cb = blockIdx.x & ((1 << nH) - 1);  // 2^T columns in blocks of 2^c
+  const int rest = (int)(blockIdx.x >> nH);
+  const int k = rest % a.K, vg = rest / a.K;
+  auto at = [&](int i) { return ((unsigned)(i >> c) << T) + (unsigned)(i & cmask); };  // offset of tile index i
+  auto mask_of = [&](int g) {  // the transformed bits (>= c) of group g
+    const int l = Gr::lo(g);
+    return (c > l ? (15 << (c - l)) : 15) & Gr::mask(g);
+  };
+  const real t = (real)a.t;
+  const real* D = reinterpret_cast<const real*>(a.D) + (size_t)k * a.dim + ((size_t)cb << c);
+  real dv[SETS][16];
+#pragma unroll
+  for (int s = 0; s < SETS; ++s) {
+    const unsigned b = at(group_base<LOC>(threadIdx.x + s * NT));
+#pragma unroll
+    for (int r = 0; r < 16; ++r) dv[s][r] = __ldg(D + b + at(r << LOC));
+  }
+  const int v1 = min(a.nvec, (vg + 1) * a.vpb);
+  for (int v = vg * a.vpb; v < v1; ++v) {
+    v2* W = reinterpret_cast<v2*>(a.W) + ((size_t)(a.vec0 - a.vecW + v) * a.K + k) * a.dim + ((size_t)cb << c);
+    if constexpr (NG > 1) {
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const int i0 = threadIdx.x + s * NT;
+        const unsigned b = at(i0);
+        v2 w[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) w[r] = W[b + at(r << LO0)];
+        gates(w, t, mask_of(0));
+        smem_st<LO0>(buf, i0, w);
+      }
+      __syncthreads();
+      if constexpr (NG > 2) mid_group<real, T, NT, SETS, 1>(buf, t, mask_of(1));
+      if constexpr (NG > 3) mid_group<real, T, NT, SETS, 2>(buf, t, mask_of(2));
+      const int mc = mask_of(NG - 1);
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const int b = group_base<LOC>(threadIdx.x + s * NT);
+        v2 w[16];
+        smem_ld<LOC>(buf, b, w);
+        gates(w, t, mc);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          w[r].x *= dv[s][r];
+          w[r].y *= dv[s][r];
+        }
+        gates(w, -t, mc);
+        smem_st<LOC>(buf, b, w);
+      }
+      __syncthreads();
+      if constexpr (NG > 3) mid_group<real, T, NT, SETS, 2>(buf, -t, mask_of(2));
+      if constexpr (NG > 2) mid_group<real, T, NT, SETS, 1>(buf, -t, mask_of(1));
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const int i0 = threadIdx.x + s * NT;
+        const unsigned b = at(i0);
+        v2 w[16];
+        smem_ld<LO0>(buf, i0, w);
+        gates(w, -t, mask_of(0));
+#pragma unroll
+        for (int r = 0; r < 16; ++r) W[b + at(r << LO0)] = w[r];
+      }
+      // the next vector's first group writes the places this thread has just read
+    } else {
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const unsigned b = at(threadIdx.x + s * NT);
+        v2 w[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) w[r] = W[b + at(r << LO0)];
+        gates(w, t, mask_of(0));
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          w[r].x *= dv[s][r];
+          w[r].y *= dv[s][r];
+        }
+        gates(w, -t, mask_of(0));
+#pragma unroll
+        for (int r = 0; r < 16; ++r) W[b + at(r << LO0)] = w[r];
+      }
+    }
+  }
+}
+
+template <typename real, int T, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) rot_backward_kernel(const __grid_constant__ RotArgs a) {
+  using v2 = typename Cx<real>::v2;
+  using Gr = Groups<T>;
+  constexpr int SETS = (1 << T) / (16 * NT), LO0 = T - 4, GL = Gr::N - 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  v2* buf = reinterpret_cast<v2*>(smem_raw);
+  __shared__ v2 ph[kRotMaxK * (kRotMaxN + 1)];
+  const int nH = a.n - T, tiles = 1 << nH;
+  const int tile = blockIdx.x & (tiles - 1), v = a.vec0 + (int)(blockIdx.x >> nH);
+  const size_t off = (size_t)v * a.dim + ((size_t)tile << T);
+  stage_phases<real>(ph, a);
+  const real t = (real)a.t;
+  v2 acc[SETS][16];
+  for (int k = 0; k < a.K; ++k) {
+    const v2* W = reinterpret_cast<const v2*>(a.W) + ((size_t)(v - a.vecW) * a.K + k) * a.dim + ((size_t)tile << T);
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+      const int i0 = threadIdx.x + s * NT;
+      v2 w[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) w[r] = W[(r << LO0) + i0];
+      gates(w, -t, Gr::mask(GL));
+      if (s == 0) __syncthreads();  // the previous direction's last group has been read
+      smem_st<0>(buf, group_base<0>(i0), w);
+    }
+    __syncthreads();
+    if constexpr (Gr::N >= 4) mid_group<real, T, NT, SETS, 2>(buf, -t, 15);
+    if constexpr (Gr::N >= 3) mid_group<real, T, NT, SETS, 1>(buf, -t, 15);
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+      const int i0 = threadIdx.x + s * NT;
+      v2 w[16];
+      smem_ld<LO0>(buf, i0, w);
+      gates(w, -t, 15);
+      if (k == 0) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) acc[s][r] = w[r];
+      } else {
+        const int pc = __popc(i0) + __popc(tile);
+        v2 f[5];
+#pragma unroll
+        for (int m = 0; m < 5; ++m) f[m] = ph[k * (kRotMaxN + 1) + pc + m];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {  // acc += conj(f) w
+          const v2 g = f[__builtin_popcount(r)];
+          acc[s][r].x = fma(g.x, w[r].x, fma(g.y, w[r].y, acc[s][r].x));
+          acc[s][r].y = fma(g.x, w[r].y, fma(-g.y, w[r].x, acc[s][r].y));
+        }
+      }
+    }
+  }
+  const v2* x = reinterpret_cast<const v2*>(a.x) + off;
+  v2* y = reinterpret_cast<v2*>(a.y) + off;
+  const real* D0 = reinterpret_cast<const real*>(a.D0) + ((size_t)tile << T);
+  if (!a.lanczos) {  // y = H x
+#pragma unroll
+    for (int s = 0; s < SETS; ++s)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const int i = threadIdx.x + s * NT + (r << LO0);
+        y[i] = axpy2(__ldg(D0 + i), __ldg(x + i), acc[s][r]);
+      }
+    return;
+  }
+  const v2* u = reinterpret_cast<const v2*>(a.u) + off;
+  const size_t e = (size_t)a.j * a.sc.ss + v;
+  const double sgd = a.sc.sigma[e];
+  const real sg = (real)sgd;
+  const real bsp = a.j == 0 ? (real)0 : (real)(a.sc.beta[e - a.sc.ss] * a.sc.sigma[e - a.sc.ss]);
+  double p[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int s = 0; s < SETS; ++s) {
+    real pw = 0, pr = 0, pi = 0;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const int i = threadIdx.x + s * NT + (r << LO0);
+      const v2 xv = __ldg(x + i), uv = __ldg(u + i);
+      const v2 hv = axpy2(__ldg(D0 + i), xv, acc[s][r]);
+      v2 w;
+      if (a.j == 0) {
+        w.x = sg * hv.x;
+        w.y = sg * hv.y;
+      } else {
+        const v2 qp = y[i];
+        w.x = sg * hv.x - bsp * qp.x;
+        w.y = sg * hv.y - bsp * qp.y;
+      }
+      y[i] = w;
+      pw += xv.x * w.x + xv.y * w.y;
+      pr += xv.x * uv.x + xv.y * uv.y;
+      pi += xv.x * uv.y - xv.y * uv.x;
+    }
+    p[0] += (double)pw;
+    p[1] += (double)pr;
+    p[2] += (double)pi;
+  }
+  if (vector_total<NT, 3>(p, a.partials + (size_t)v * tiles * 3, tile, tiles, a.counters + v)) {
+    a.sc.alpha[e] = sgd * p[0];
+    a.sc.p[2 * e] = sgd * p[1];
+    a.sc.p[2 * e + 1] = sgd * p[2];
+  }
+}
+
+// Diagonal table of one direction: entry at place e of the table's order (the
+// natural one, or with the low T bits rotated by four) is
+//   scale (c0 + sum_i m_i (h_i + sum_{j > i} a_ij m_j)),  m_i = +-1/2 by bit i,
+// in FP64, one CTA per 4096 entries: the terms of the bits above 12 once per
+// CTA, a thread's 16 entries along bits 0..3.
+template <typename real>
+__global__ void __launch_bounds__(256) rot_table_kernel(const __grid_constant__ RotForm f, real* out) {
+  __shared__ double F[12], E;
+  const unsigned long long top = blockIdx.x;
+  auto m = [](unsigned long long b, int i) { return ((b >> i) & 1ull) ? 0.5 : -0.5; };
+  if (threadIdx.x < 12) {
+    double s = f.h[threadIdx.x];
+    for (int j = 12; j < f.n; ++j) s += f.a[tri(threadIdx.x, j)] * m(top, j - 12);
+    F[threadIdx.x] = s;
+  } else if (threadIdx.x == 32) {
+    double e = f.c0;
+    for (int i = 12; i < f.n; ++i) {
+      double s = f.h[i];
+      for (int j = i + 1; j < f.n; ++j) s += f.a[tri(i, j)] * m(top, j - 12);
+      e += m(top, i - 12) * s;
+    }
+    E = e;
+  }
+  __syncthreads();
+  const int mid = threadIdx.x << 4;
+  double e = E, g[4];
+  for (int i = 4; i < 12; ++i) {
+    double s = F[i];
+    for (int j = i + 1; j < 12; ++j) s += f.a[tri(i, j)] * m(mid, j);
+    e += m(mid, i) * s;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    g[i] = F[i];
+    for (int j = 4; j < 12; ++j) g[i] += f.a[tri(i, j)] * m(mid, j);
+  }
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    double d = e;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      double s = g[i];
+#pragma unroll
+      for (int j = i + 1; j < 4; ++j) s += f.a[tri(i, j)] * ((r >> j) & 1 ? 0.5 : -0.5);
+      d += ((r >> i) & 1 ? 0.5 : -0.5) * s;
+    }
+    unsigned long long at = (top << 12) | (unsigned)mid | (unsigned)r;
+    if (f.rotate) {
+      const unsigned long long low = at & ((1ull << f.T) - 1);
+      at = (at ^ low) | ((low & 15) << (f.T - 4)) | (low >> 4);
+    }
+    out[at] = (real)(f.scale * d);
+  }
+}
+
+// e^{-i phi_k (n - m)} for m = 0..n up spins
+template <typename real>
+__global__ void rot_phase_kernel(int n, int K, RotAzimuths d, real* out) {
+  const int k = threadIdx.x / (kRotMaxN + 1), m = threadIdx.x % (kRotMaxN + 1);
+  if (k >= K || m > n) return;
+  double sn, cs;
+  sincospi((double)((n - m) * d.num[k] % (2 * d.den)) / (double)d.den, &sn, &cs);
+  out[2 * threadIdx.x] = (real)cs;
+  out[2 * threadIdx.x + 1] = (real)-sn;
+}
+
+template <typename real, int T, int NT, int MINB>
+int launch_pass(const RotArgs& a, int pass, cudaStream_t st) {
+  const size_t smem = sizeof(typename Cx<real>::v2) * (size_t)pad(1 << T);
+  const int nH = a.n - T;
+  if (nH < 1 || nH > T || a.n > kRotMaxN || a.K < 1 || a.K > kRotMaxK) return (int)cudaErrorInvalidValue;
+  if (pass == 0) {
+    rot_forward_kernel<real, T, NT, MINB><<<(unsigned)a.nvec << nH, NT, smem, st>>>(a);
+  } else if (pass == 2) {
+    rot_backward_kernel<real, T, NT, MINB><<<(unsigned)a.nvec << nH, NT, smem, st>>>(a);
+  } else {
+    const int c = T - nH;
+    int ng = 1;
+    while (ng < Groups<T>::N && Groups<T>::lo(ng - 1) > c) ++ng;
+    const unsigned grid = (unsigned)(((a.nvec + a.vpb - 1) / a.vpb) * a.K) << nH;
+    if (ng == 1) rot_middle_kernel<real, T, NT, MINB, 1><<<grid, NT, 0, st>>>(a);
+    else if (ng == 2) rot_middle_kernel<real, T, NT, MINB, 2><<<grid, NT, smem, st>>>(a);
+    else if (ng == 3) rot_middle_kernel<real, T, NT, MINB, 3><<<grid, NT, smem, st>>>(a);
+    else if constexpr (Groups<T>::N >= 4) rot_middle_kernel<real, T, NT, MINB, 4><<<grid, NT, smem, st>>>(a);
+    else return (int)cudaErrorInvalidValue;
+  }
+  return (int)cudaGetLastError();
+}
+
+template <typename real, int T, int NT, int MINB>
+int prepare_pass() {
+  const int smem = (int)(sizeof(typename Cx<real>::v2) * (size_t)pad(1 << T));
+  const void* ks[] = {(const void*)rot_forward_kernel<real, T, NT, MINB>, (const void*)rot_backward_kernel<real, T, NT, MINB>,
+                      (const void*)rot_middle_kernel<real, T, NT, MINB, 2>, (const void*)rot_middle_kernel<real, T, NT, MINB, 3>};
+  for (const void* k : ks) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return (int)e;
+  }
+  if constexpr (Groups<T>::N >= 4)
+    return (int)cudaFuncSetAttribute((const void*)rot_middle_kernel<real, T, NT, MINB, 4>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return 0;
+}
+
+}  // namespace
+
+int launch_rot(const RotArgs& a, int pass, int c64, void* stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (c64) {
+    if (a.T == 12) return launch_pass<float, 12, 256, 3>(a, pass, st);
+    if (a.T == 14) return launch_pass<float, 14, 512, 1>(a, pass, st);
+  } else {
+    if (a.T == 11) return launch_pass<double, 11, 128, 3>(a, pass, st);
+    if (a.T == 13) return launch_pass<double, 13, 256, 1>(a, pass, st);
+  }
+  return (int)cudaErrorInvalidValue;
+}
+
+int prepare_rot(int T, int c64) {
+  if (c64) {
+    if (T == 12) return prepare_pass<float, 12, 256, 3>();
+    if (T == 14) return prepare_pass<float, 14, 512, 1>();
+  } else {
+    if (T == 11) return prepare_pass<double, 11, 128, 3>();
+    if (T == 13) return prepare_pass<double, 13, 256, 1>();
+  }
+  return (int)cudaErrorInvalidValue;
+}
+
+int launch_rot_table(const RotForm& f, void* out, int c64, void* stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (f.n < 12 || f.n > kRotMaxN) return (int)cudaErrorInvalidValue;
+  const unsigned grid = 1u << (f.n - 12);
+  if (c64) rot_table_kernel<float><<<grid, 256, 0, st>>>(f, reinterpret_cast<float*>(out));
+  else rot_table_kernel<double><<<grid, 256, 0, st>>>(f, reinterpret_cast<double*>(out));
+  return (int)cudaGetLastError();
+}
+
+int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const int threads = kRotMaxK * (kRotMaxN + 1);
+  if (c64) rot_phase_kernel<float><<<1, threads, 0, st>>>(n, d.K, d.az, reinterpret_cast<float*>(out));
+  else rot_phase_kernel<double><<<1, threads, 0, st>>>(n, d.K, d.az, reinterpret_cast<double*>(out));
+  return (int)cudaGetLastError();
+}
+
+// Tile size for n sites: the small tile while the middle pass's columns are at
+// least 32 bytes (several CTAs a SM overlap their loads and exchanges), the
+// large one beyond; 0: no tile fits (the gather runs).
+int rot_tile_bits(int n, int c64) {
+  const int small = c64 ? 12 : 11, col = c64 ? 2 : 1;
+  if (n <= 12 || n > kRotMaxN) return 0;
+  if (2 * small - n >= col) return small;
+  return small + 2 < n && 2 * (small + 2) >= n ? small + 2 : 0;
+}
+
+// The directions and diagonal forms of a spin-1/2 system (see the top of the
+// file); false when it has none (a pair tensor that is not symmetric) or no
+// pair couplings at all.
+bool rot_directions(const HostSystem& hs, RotDirs& d) {
+  const int n = hs.n;
+  if (!hs.all_half || !hs.real_pm || n > kRotMaxN) return false;
+  const TabLayout& L = hs.lay;
+  const double* t = hs.tab.data();
+  bool planar = true, diagonal = true, coupled = false;
+  for (int i = 0; i < n; ++i)
+    for (int j = i + 1; j < n; ++j) {
+      const int ij = i * n + j, ji = j * n + i;
+      for (int c = 0; c < 2; ++c) {
+        const double r1 = t[L.off_rho + 2 * ij + c], r2 = t[L.off_rho + 2 * ji + c];
+        if (std::fabs(r1 - r2) > 1e-14 * std::fabs(r1)) return false;  // (equal up to the last bit's rounding)
+        planar = planar && t[L.off_rho + 2 * ij + c] == 0.0;
+      }
+      diagonal = diagonal && t[L.off_pp + 2 * ij + 1] == 0.0;
+      coupled = coupled || t[L.off_pm + 2 * ij] != 0.0 || t[L.off_pp + 2 * ij] != 0.0 || t[L.off_pp + 2 * ij + 1] != 0.0 ||
+                t[L.off_rho + 2 * ij] != 0.0 || t[L.off_rho + 2 * ij + 1] != 0.0;
+    }
+  if (!coupled) return false;
+  const double pi = 3.14159265358979323846;
+  // azimuths phi_k = pi num / den; the polar angle's cosine
+  double ct = 0.0;
+  if (planar && diagonal) {
+    d.K = 2;
+    d.az.num[0] = 0;
+    d.az.num[1] = 1;
+    d.az.den = 2;
+  } else if (planar) {
+    d.K = 3;
+    for (int k = 0; k < 3; ++k) d.az.num[k] = k;
+    d.az.den = 3;
+  } else {
+    d.K = 5;
+    for (int k = 0; k < 5; ++k) d.az.num[k] = 2 * k;
+    d.az.den = 5;
+    ct = 1.0 / std::sqrt(5.0);
+  }
+  const double st = std::sqrt(1.0 - ct * ct);
+  d.t = st / (1.0 + ct);
+  const int K = d.K;
+  double u[kRotMaxK][3];
+  for (int k = 0; k < K; ++k) {
+    u[k][0] = st * std::cos(pi * d.az.num[k] / d.az.den);
+    u[k][1] = st * std::sin(pi * d.az.num[k] / d.az.den);
+    u[k][2] = ct;
+  }
+  if (K == 2) u[1][0] = 0.0;  // (cos(pi / 2))
+  for (int k = 0; k <= K; ++k) {
+    RotForm& f = d.form[k];
+    f.n = n;
+    f.rotate = k > 0;
+    f.c0 = 0.0;
+    f.scale = k == 0 ? 1.0 : std::pow(1.0 + d.t * d.t, -n);
+  }
+  for (int i = 0; i < n; ++i) {
+    const double h[3] = {2.0 * t[L.off_hp + 2 * i], -2.0 * t[L.off_hp + 2 * i + 1], t[L.off_hz + i]};
+    d.form[0].c0 += t[L.off_iondiag + i * L.qmax];  // (s.e)^2 = 1/4: the same for both digits
+    // sum_k u_k u_k^T over the set (with z for K = 5) is a multiple of the identity on what it spans
+    for (int k = 0; k < K; ++k) {
+      const double hu = h[0] * u[k][0] + h[1] * u[k][1] + h[2] * u[k][2];
+      d.form[k + 1].h[i] = K == 2 ? hu : (K == 3 ? 2.0 / 3.0 * hu : 0.5 * hu);
+    }
+    d.form[0].h[i] = K == 5 ? 0.5 * h[2] : h[2];
+  }
+  for (int i = 0; i < n; ++i)
+    for (int j = i + 1; j < n; ++j) {
+      const int ij = i * n + j, q = (j * (j - 1)) / 2 + i;
+      const double pm = t[L.off_pm + 2 * ij], pp = t[L.off_pp + 2 * ij];
+      const double xx = 2.0 * (pm + pp), yy = 2.0 * (pm - pp), zz = t[L.off_zz + ij];
+      const double xy = -2.0 * t[L.off_pp + 2 * ij + 1];
+      const double xz = 2.0 * t[L.off_rho + 2 * ij], yz = -2.0 * t[L.off_rho + 2 * ij + 1];
+      // A = sum_k a_k u_k u_k^T.  Projectors of a tight frame of K + 1 (or K in the plane) lines:
+      // a_k = alpha (u_k.A.u_k) + gamma tr A solves it.
+      double A[3][3] = {{xx, xy, xz}, {xy, yy, yz}, {xz, yz, zz}};
+      auto quad = [&](const double* w) {
+        double s = 0.0;
+        for (int p = 0; p < 3; ++p)
+          for (int r = 0; r < 3; ++r) s += w[p] * A[p][r] * w[r];
+        return s;
+      };
+      if (K == 2) {
+        d.form[0].a[q] = zz;
+        d.form[1].a[q] = xx;
+        d.form[2].a[q] = yy;
+      } else if (K == 3) {
+        d.form[0].a[q] = zz;
+        // in the plane: sum_k (u_k.A.u_k) u_k u_k^T = 3/8 (2 A + tr A 1), sum_k u_k u_k^T = 3/2 1
+        for (int k = 0; k < 3; ++k) d.form[k + 1].a[q] = 4.0 / 3.0 * quad(u[k]) - (xx + yy) / 3.0;
+      } else {
+        // six lines: sum_k (u_k.A.u_k) u_k u_k^T = 2/5 (2 A + tr A 1), sum_k u_k u_k^T = 2 1
+        const double tr = xx + yy + zz;
+        const double z[3] = {0.0, 0.0, 1.0};
+        d.form[0].a[q] = 1.25 * quad(z) - 0.25 * tr;
+        for (int k = 0; k < 5; ++k) d.form[k + 1].a[q] = 1.25 * quad(u[k]) - 0.25 * tr;
+      }
+    }
+  return true;
+}
+
+}  // namespace ftlm

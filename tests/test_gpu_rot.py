@@ -1,0 +1,87 @@
+"""GPU: the rotated-basis H.v of spin-1/2 runs (random and time-reversed-pair
+starts) against the oracle and against the gather, which the same run takes
+from a caller's block of the same start vectors.
+
+Tolerances: a step rounds about 100 times a value, so its relative error is
+about 10 units roundoff (6e-8 / 1.1e-16); eight steps that have not lost
+orthogonality amplify it by less than 30: 2e-5 in complex64, 1e-13 (with the
+oracle's own error 1e-12) in complex128, relative to the largest coefficient."""
+import numpy as np
+import pytest
+
+import ftlm_workloads as W
+import oracle
+import paper_2607_25585_gb300 as F
+from gpu_helpers import empty_dev, osys
+
+pytestmark = pytest.mark.gpu
+T = np.array([0.5, 2.0, 20.0])
+
+
+def close(a, b, tol):
+    for k in ("alpha", "beta", "p"):
+        scale = np.abs(b["alpha"]).max() if k == "alpha" else np.abs(b[k]).max()
+        scale = max(scale, np.abs(b["beta"]).max()) if k == "alpha" else scale
+        assert np.abs(a[k] - b[k]).max() < tol * scale, k
+    assert list(a["M_eff"]) == list(b["M_eff"])
+
+
+def buckled(lx, ly):
+    w = W.square_lattice(lx, ly, seed=5, B=1.3, Bdir=(0.3, -0.5, 0.8))
+    w["pos"][:, 2] = 0.5 * np.cos(1.3 * np.arange(lx * ly))
+    return w
+
+
+SYSTEMS = {
+    "chain13": lambda: W.square_lattice(13, 1, seed=1, Bdir=(1, 2, 3)),      # x, y and z: one low tile pair
+    "lattice14": lambda: W.square_lattice(7, 2, seed=2, Bdir=(0, 0, 1)),     # three directions in the plane
+    "buckled15": lambda: buckled(5, 3),                                      # five directions
+    "ladder16": lambda: W.ladder(8, dipolar=False),                          # exchange alone
+    "buckled16": lambda: buckled(4, 4),
+}
+
+
+@pytest.mark.parametrize("name", SYSTEMS)
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+def test_rotated_run_matches_oracle(name, dtype):
+    w = SYSTEMS[name]()
+    s = F.System.from_dict(w)
+    for R, start in ((3, "random"), (2, "pairs")):
+        g = F.run(s, R=R, M=8, T=T, seed=7, vec_offset=2, start=start, dtype=dtype)
+        assert g["shape"]["passes"] == 3 and g["shape"]["vector_major"] == 1
+        x = empty_dev((s.dim, R), dtype)
+        (F.start_pairs if start == "pairs" else F.start_block)(s, x, R, 7, vec_offset=2, dtype=dtype)
+        close(g, F.run(s, R=R, M=8, T=T, start="user", user_start=x, dtype=dtype), 2e-5 if dtype == "c64" else 1e-12)
+        if start == "random":
+            close(g, oracle.ftlm(osys(w), R=R, M=8, T=T, seed=7, vec_offset=2), 2e-5 if dtype == "c64" else 1e-12)
+    s.close()
+
+
+@pytest.mark.parametrize("n", [17, 18, 19, 20, 21, 22, 23, 24, 25])
+def test_rotated_run_matches_gather_at_every_split(n):
+    """Every split of the index into tile and column bits, on both sides of the
+    change of tile size."""
+    w = W.square_lattice(n, 1, seed=n, Bdir=(1, 1, 0))
+    s = F.System.from_dict(w)
+    for dtype, tol in (("c64", 2e-5), ("c128", 1e-12)):
+        if dtype == "c128" and n > 23:
+            continue
+        R = 2 if n < 23 else 1
+        g = F.run(s, R=R, M=3, T=T, seed=3, dtype=dtype)
+        assert g["shape"]["passes"] == 3
+        x = empty_dev((s.dim, R), dtype)
+        F.start_block(s, x, R, 3, dtype=dtype)
+        close(g, F.run(s, R=R, M=3, T=T, start="user", user_start=x, dtype=dtype), tol)
+    s.close()
+
+
+def test_starts_that_may_be_sparse_keep_the_gather():
+    """An isotropic system conserves S^z: from a basis state the run stays in its
+    sector and ends where the sector ends."""
+    n = 13
+    J = np.zeros((n, n))
+    J[0, 1] = 1.0
+    s = F.System([1] * n, J=J, B=[0, 0, 0.3])
+    g = F.run(s, R=1, M=6, T=T, start="basis", basis_offset=1, dtype="c64")
+    assert g["shape"]["passes"] == 1 and list(g["M_eff"]) == [2]
+    s.close()
