@@ -21,6 +21,7 @@
 
 #include "device_common.cuh"
 #include "ftlm_internal.h"
+#include "gauss.cuh"
 #include "rows_common.cuh"
 
 namespace ftlm {
@@ -431,24 +432,66 @@ __device__ __forceinline__ double unit53(unsigned hi, unsigned lo) {
   return ((double)k + 1.0) * (1.0 / 9007199254740992.0);
 }
 
+// Random vector number rg of the stream at basis state nu: complex64 by the
+// two-float form (gauss.cuh), complex128 in FP64.
+template <typename real>
+__device__ __forceinline__ typename Cx<real>::v2 gaussian(unsigned long long nu, unsigned long long rg,
+                                                          unsigned long long seed) {
+  unsigned c[4] = {(unsigned)nu, (unsigned)(nu >> 32), (unsigned)rg, (unsigned)(rg >> 32)};
+  philox4x32_10(c, (unsigned)seed, (unsigned)(seed >> 32));
+  typename Cx<real>::v2 out;
+  if (sizeof(real) == 4) {
+    const unsigned long long k1 = (((unsigned long long)c[0] << 21) | (c[1] >> 11)) + 1;
+    const unsigned long long k2 = (((unsigned long long)c[2] << 21) | (c[3] >> 11)) + 1;
+    Two cs, sn;
+    const Two rho = box_muller_radius(k1);
+    box_muller_angle(k2, cs, sn);
+    out.x = (real)round_product(rho, cs);
+    out.y = (real)round_product(rho, sn);
+  } else {
+    const double rho = sqrt(-2.0 * log(unit53(c[0], c[1])));
+    double sn, cs;
+    sincospi(2.0 * unit53(c[2], c[3]), &sn, &cs);
+    out.x = (real)(rho * cs);
+    out.y = (real)(rho * sn);
+  }
+  return out;
+}
+
+// A grid-stride walk over a block's elements e as (slow, fast) = (e / nfast,
+// e % nfast), advanced by carries: one 64-bit division a thread instead of one
+// an element.
+struct BlockWalk {
+  long long e, slow, fast, total, step, step_slow, step_fast, nfast;
+  __device__ BlockWalk(long long nslow, long long nfast_) : nfast(nfast_) {
+    total = nslow * nfast;
+    e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    step = (long long)gridDim.x * blockDim.x;
+    slow = e / nfast;
+    fast = e - slow * nfast;
+    step_slow = step / nfast;
+    step_fast = step - step_slow * nfast;
+  }
+  __device__ bool more() const { return e < total; }
+  __device__ void next() {
+    e += step;
+    slow += step_slow;
+    fast += step_fast;
+    if (fast >= nfast) {
+      fast -= nfast;
+      ++slow;
+    }
+  }
+};
+
 // VMAJ: vector-major output (element e = k * dim + nu), else row-major (e = nu * R + k).
 template <typename real, bool VMAJ>
-__global__ void start_random_kernel(long long dim, int R, unsigned long long seed, unsigned long long vec_offset,
-                                    real* out) {
-  const long long total = dim * R;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long nu = VMAJ ? e % dim : e / R;
-    const unsigned long long rg = vec_offset + (unsigned long long)(VMAJ ? e / dim : e - nu * R);
-    unsigned c[4] = {(unsigned)nu, (unsigned)((unsigned long long)nu >> 32), (unsigned)rg, (unsigned)(rg >> 32)};
-    philox4x32_10(c, (unsigned)seed, (unsigned)(seed >> 32));
-    const double u1 = unit53(c[0], c[1]);
-    const double u2 = unit53(c[2], c[3]);
-    const double rho = sqrt(-2.0 * log(u1));
-    double sn, cs;
-    sincospi(2.0 * u2, &sn, &cs);
-    out[2 * e] = (real)(rho * cs);
-    out[2 * e + 1] = (real)(rho * sn);
+__global__ void __launch_bounds__(256) start_random_kernel(long long dim, int R, unsigned long long seed,
+                                                           unsigned long long vec_offset, real* out) {
+  typename Cx<real>::v2* o = reinterpret_cast<typename Cx<real>::v2*>(out);
+  for (BlockWalk w(VMAJ ? R : dim, VMAJ ? dim : R); w.more(); w.next()) {
+    const long long nu = VMAJ ? w.fast : w.slow, k = VMAJ ? w.slow : w.fast;
+    o[w.e] = gaussian<real>((unsigned long long)nu, vec_offset + (unsigned long long)k, seed);
   }
 }
 
@@ -469,10 +512,17 @@ __global__ void start_basis_kernel(long long dim, int R, unsigned long long basi
 __device__ __forceinline__ int digit_parity(long long nu, int n, const int* q, int all_half) {
   if (all_half) return __popcll((unsigned long long)nu) & 1;
   int sum = 0;
-  for (int i = 0; i < n; ++i) {
+  int i = 0;
+  for (; i < n && (nu >> 32); ++i) {
     const int qi = __ldg(q + i);
     sum += (int)(nu % qi);
     nu /= qi;
+  }
+  unsigned rest = (unsigned)nu;  // 32-bit division once the index fits
+  for (; i < n; ++i) {
+    const unsigned qi = (unsigned)__ldg(q + i), nx = rest / qi;
+    sum += (int)(rest - nx * qi);
+    rest = nx;
   }
   return sum & 1;
 }
@@ -484,33 +534,23 @@ __device__ __forceinline__ int digit_parity(long long nu, int n, const int* q, i
 // since Theta = exp(-i pi S^y) K maps every digit a_i to 2 s_i - a_i, i.e.
 // the index nu to d - 1 - nu.  Unnormalised, like start_random_kernel.
 template <typename real, bool VMAJ>
-__global__ void start_pairs_kernel(long long dim, int R, unsigned long long seed, unsigned long long vec_offset,
-                                   int n, const int* q, int all_half, real* out) {
-  const long long total = dim * R;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long nu = VMAJ ? e % dim : e / R;
-    const unsigned long long v = vec_offset + (unsigned long long)(VMAJ ? e / dim : e - nu * R);
+__global__ void __launch_bounds__(256) start_pairs_kernel(long long dim, int R, unsigned long long seed,
+                                                          unsigned long long vec_offset, int n, const int* q,
+                                                          int all_half, real* out) {
+  typename Cx<real>::v2* o = reinterpret_cast<typename Cx<real>::v2*>(out);
+  for (BlockWalk w(VMAJ ? R : dim, VMAJ ? dim : R); w.more(); w.next()) {
+    const long long nu = VMAJ ? w.fast : w.slow;
+    const unsigned long long v = vec_offset + (unsigned long long)(VMAJ ? w.slow : w.fast);
     const bool rev = (v & 1ull) != 0;
-    const long long src = rev ? dim - 1 - nu : nu;
-    const unsigned long long rg = v >> 1;
-    unsigned c[4] = {(unsigned)src, (unsigned)((unsigned long long)src >> 32), (unsigned)rg, (unsigned)(rg >> 32)};
-    philox4x32_10(c, (unsigned)seed, (unsigned)(seed >> 32));
-    const double u1 = unit53(c[0], c[1]);
-    const double u2 = unit53(c[2], c[3]);
-    const double rho = sqrt(-2.0 * log(u1));
-    double sn, cs;
-    sincospi(2.0 * u2, &sn, &cs);
-    double re = rho * cs, im = rho * sn;
+    typename Cx<real>::v2 z = gaussian<real>((unsigned long long)(rev ? dim - 1 - nu : nu), v >> 1, seed);
     if (rev) {
-      im = -im;
+      z.y = -z.y;
       if (digit_parity(nu, n, q, all_half)) {
-        re = -re;
-        im = -im;
+        z.x = -z.x;
+        z.y = -z.y;
       }
     }
-    out[2 * e] = (real)re;
-    out[2 * e + 1] = (real)im;
+    o[w.e] = z;
   }
 }
 
