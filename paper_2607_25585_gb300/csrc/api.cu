@@ -172,6 +172,20 @@ InstDesc base_desc(const ftlm_system* s, int c64) {
   return d;
 }
 
+SdirArgs sdir_args(const ftlm_system* s, int c64, int R, const void* x, void* y) {
+  SdirArgs a;
+  const InstDesc d = base_desc(s, c64);
+  a.tab = d.tab;
+  a.lay = d.lay;
+  a.q = d.q;
+  a.n = d.n;
+  a.dim = d.dim;
+  a.R = R;
+  a.x = x;
+  a.y = y;
+  return a;
+}
+
 struct HalfPlan {
   bool on = false;
   bool vm = false;  // vector-major kernel: R instances of one vector each (nvg = R, Rg = 1)
@@ -484,7 +498,7 @@ int launch_plan(const Plan& pl, LaunchArgs a, void* st) {
     return launch_rows_vm(a, pl.gvm_V, pl.c64, pl.gvm_grid, 256, pl.gvm_smem, st);
   }
   if (pl.half.on && pl.half.vm &&
-      (a.mode == kModeStep || a.mode == kModeStartNorm || a.mode == kModeUpdate || a.mode == kModeApplyS)) {
+      (a.mode == kModeStep || a.mode == kModeStartNorm || a.mode == kModeUpdate)) {
     a.rows_per_tile = pl.half.stream_rows;
     a.tiles_per_vg = pl.half.stream_tiles_per_vg;
     a.n_inst = pl.half.nvg;
@@ -951,11 +965,14 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
   a.inst = d_start;  // sigma_0 = 1/|q_0|, then U = sigma_0 (u.S) q_0
   a.mode = kModeStartNorm;
   CKI(launch_plan(pl, a, st));
-  a.mode = kModeApplyS;
-  a.use_sigma0 = 1;
-  CKI(launch_plan(pl, a, st));
-  a.use_sigma0 = 0;
-  ctx.launches += 2;
+  ctx.launches++;
+  for (auto* s : sys) {
+    SdirArgs u = sdir_args(s, c64, R, s->A.p, s->U.p);
+    observable_coefs(s->hs, p->obs_dir, u.obs);
+    u.sigma = scalars_at(s->scal.p, R, M).sigma;
+    CKI(launch_sdir(u, s->hs.q.data(), c64, vmaj != 0, st));
+    ctx.launches++;
+  }
   if (pl.rot.on) {
     ftlm_status rs = enqueue_rot_steps(ctx, sys[0], p, pl, a, d_even, d_odd, st);
     if (rs != FTLM_OK) return rs;
@@ -1144,9 +1161,8 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
 // ---- symmetric estimator: O_ij = <v_i|u.S|v_j> per vector ---------------------
 
 // After a symmetric run: G_r[i][j] = <q_i|u.S q_j> for the stored unnormalised
-// vectors q_0 .. q_{M-1} of every vector r, in one fused kernel (u.S q_j is
-// formed tile by tile in shared memory, never stored) plus a fixed-order
-// reduction of its per-range partials; then O_ij = sigma_i sigma_j G_ij on
+// vectors q_0 .. q_{M-1} of every vector r: u.S of all of them, the contraction
+// and a fixed-order reduction of its per-range partials; then O_ij = sigma_i sigma_j G_ij on
 // the host.  Omat [R][M][M] complex row-major; sigma [M][R].
 ftlm_status symmetric_matrices(ftlm_system* s, const ftlm_run_params* p, cudaStream_t st, const double* sigma,
                                std::vector<double>& Omat, double& ms) {
@@ -1171,13 +1187,15 @@ ftlm_status symmetric_matrices(ftlm_system* s, const ftlm_run_params* p, cudaStr
       return fail(FTLM_ERR_OUT_OF_MEMORY, "symmetric run: " + std::to_string(wbytes) + " bytes for u.S of the Lanczos vectors");
   }
   void* W = s->Ws.p;
-  InstDesc hd = base_desc(s, c64);
-  observable_coefs(s->hs, p->obs_dir, hd.obs);
+  SdirArgs u = sdir_args(s, c64, R * M, s->Vs.p, W);
+  observable_coefs(s->hs, p->obs_dir, u.obs);
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   CK(cudaEventRecord(e0, st));
-  CKI(launch_sym_omat(&hd, s->Vs.p, W, R, M, nranges, reinterpret_cast<double*>(s->Wc.p),
+  if ((long long)R * M > 65535) return fail(FTLM_ERR_UNSUPPORTED, "symmetric run: R * M must not exceed 65535");
+  CKI(launch_sdir(u, s->hs.q.data(), c64, true, st));
+  CKI(launch_sym_omat(d, s->Vs.p, W, R, M, nranges, reinterpret_cast<double*>(s->Wc.p),
                       reinterpret_cast<double*>(s->Od.p), c64, st));
   CK(cudaEventRecord(e1, st));
   std::vector<double> host((size_t)R * M * M * 2);
@@ -1546,20 +1564,26 @@ ftlm_status check_device(const ftlm_system* s) {
   return FTLM_OK;
 }
 
-ftlm_status rows_entry(const ftlm_system* cs, int mode, const double* u, const void* x, void* y, int nvec,
-                       ftlm_dtype dtype, void* stream) {
-  ftlm_status v = check_block_args(cs, x, y, nvec, dtype);
+// The checks that ftlm_apply_h and ftlm_apply_sdir share.
+ftlm_status check_product(const ftlm_system* s, const void* x, const void* y, int nvec, ftlm_dtype dtype) {
+  ftlm_status v = check_block_args(s, x, y, nvec, dtype);
   if (v != FTLM_OK) return v;
-  v = check_device(cs);
+  v = check_device(s);
+  if (v != FTLM_OK) return v;
+  const size_t bytes = (size_t)s->hs.dim * nvec * (dtype == FTLM_C64 ? 8 : 16);
+  const uintptr_t xa = reinterpret_cast<uintptr_t>(x), ya = reinterpret_cast<uintptr_t>(y);
+  if (xa < ya + bytes && ya < xa + bytes) return fail(FTLM_ERR_INVALID_ARG, "x and y overlap");
+  return FTLM_OK;
+}
+
+ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nvec, ftlm_dtype dtype, void* stream) {
+  ftlm_status v = check_product(cs, x, y, nvec, dtype);
   if (v != FTLM_OK) return v;
   const int c64 = dtype == FTLM_C64;
   ftlm_system* s = const_cast<ftlm_system*>(cs);
-  const size_t bytes = (size_t)s->hs.dim * nvec * (c64 ? 8 : 16);
-  const uintptr_t xa = reinterpret_cast<uintptr_t>(x), ya = reinterpret_cast<uintptr_t>(y);
-  if (xa < ya + bytes && ya < xa + bytes) return fail(FTLM_ERR_INVALID_ARG, "x and y overlap");
   Plan pl;
   std::vector<ftlm_system*> one{s};
-  if (mode == kModeApply && nvec > 1 && !has_shape_override(s, nvec, c64)) {
+  if (nvec > 1 && !has_shape_override(s, nvec, c64)) {
     // spin-1/2 blocks on the default plan: transpose to vector-major, the runs'
     // gather, transpose back
     Plan vp;
@@ -1600,7 +1624,7 @@ ftlm_status rows_entry(const ftlm_system* cs, int mode, const double* u, const v
   }
   // one vector: the row-major and the vector-major layouts coincide, so H.v may
   // use the vector-major gather
-  ftlm_status ps = make_plan(one, nvec, c64, pl, nullptr, mode == kModeApply && nvec == 1);
+  ftlm_status ps = make_plan(one, nvec, c64, pl, nullptr, nvec == 1);
   if (ps != FTLM_OK) return ps;
   if (pl.half.vm && pl.half.passes > 1) {  // the multi-pass form writes one block per pass: not for a caller's y
     ps = make_plan(one, nvec, c64, pl);
@@ -1611,8 +1635,7 @@ ftlm_status rows_entry(const ftlm_system* cs, int mode, const double* u, const v
   a.one = base_desc(s, c64);
   a.one.x = x;
   a.one.y = y;
-  a.mode = mode;
-  observable_coefs(s->hs, u, a.one.obs);
+  a.mode = kModeApply;
   CKI(launch_plan(pl, a, pick_stream(s, stream)));
   return FTLM_OK;
 }
@@ -1766,14 +1789,20 @@ uint64_t ftlm_system_table_bytes(const ftlm_system* s) {
 }
 
 ftlm_status ftlm_apply_h(const ftlm_system* s, const void* x, void* y, int nvec, ftlm_dtype dtype, void* stream) {
-  return rows_entry(s, kModeApply, nullptr, x, y, nvec, dtype, stream);
+  return apply_h_entry(s, x, y, nvec, dtype, stream);
 }
 
 ftlm_status ftlm_apply_sdir(const ftlm_system* s, const double* u, const void* x, void* y, int nvec,
                             ftlm_dtype dtype, void* stream) {
   if (u && !(std::isfinite(u[0]) && std::isfinite(u[1]) && std::isfinite(u[2])))
     return fail(FTLM_ERR_INVALID_ARG, "u must be finite");
-  return rows_entry(s, kModeApplyS, u, x, y, nvec, dtype, stream);
+  ftlm_status v = check_product(s, x, y, nvec, dtype);
+  if (v != FTLM_OK) return v;
+  const int c64 = dtype == FTLM_C64;
+  SdirArgs a = sdir_args(s, c64, nvec, x, y);
+  observable_coefs(s->hs, u, a.obs);
+  CKI(launch_sdir(a, s->hs.q.data(), c64, false, pick_stream(s, stream)));
+  return FTLM_OK;
 }
 
 }  // extern "C"

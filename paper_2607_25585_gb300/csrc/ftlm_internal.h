@@ -107,7 +107,6 @@ enum KernelMode : int {
   kModeLanczos = 1,   // w = sigma_j H q_j - beta_j sigma_{j-1} q_{j-1} (in place in y), partials alpha, p
   kModeUpdate = 2,    // w -= alpha_j sigma_j q_j (in place in y), partials |w|^2, then beta, sigma
   kModeStartNorm = 3, // partials |x|^2, then sigma_0 = 1/|x|
-  kModeApplyS = 4,    // y = scale * (u.S) x  (scale = sigma_0 when Lanczos)
   kModeScale = 5,     // y = sigma_0 x (elementwise; y may equal x)
   kModeEpilogue = 6,  // as kModeLanczos with H q_j read from `hq` instead of gathered (elementwise)
   kModeStep = 7,      // the whole step after a gather that produced alpha_j (gather_alpha):
@@ -132,7 +131,6 @@ struct LaunchArgs {
   unsigned* counter = nullptr;    // zeroed; reset by the last block
   int tab_reals = 0;    // max table size over instances
   int max_n = 0;        // max sites over instances
-  int use_sigma0 = 0;   // kModeApplyS: multiply by sigma_0
   // spin-1/2 kernel only: vectors are processed in groups of Rg (tile order
   // is group-major so the gathered slice stays in L2)
   int Rg = 0;           // vectors per group
@@ -310,6 +308,21 @@ int launch_rot(const RotArgs& a, int pass, int c64, void* stream);  // pass 0 fo
 int launch_rot_table(const RotForm& f, void* out, int c64, void* stream);
 int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream);
 
+// y = c (u.S) x (sdir.cu): R vectors, c = sigma[vector] (null: 1).
+struct SdirArgs {
+  const void* tab = nullptr;
+  TabLayout lay;
+  const int* q = nullptr;  // device
+  int n = 0, R = 0;
+  long long dim = 0;
+  const void* x = nullptr;
+  void* y = nullptr;
+  double obs[3] = {0, 0, 0};
+  const double* sigma = nullptr;
+  int T = 0, n_low = 0;    // set by the launcher: tile rows, sites within a tile
+};
+int launch_sdir(SdirArgs a, const int* q, int c64, bool vmaj, void* stream);
+
 // Full re-orthogonalisation pass (reorth.cu): w_r -= sum_{k<=j} sigma_k^2 <q_k|w_r> q_k
 // for the R vectors of a row-major block w [dim][R], against the stored
 // vector-major q_k (Vs [M][R][dim]); G is [R][M] complex FP64 scratch, sigma [M+1][R].
@@ -321,9 +334,8 @@ int launch_reorth_pass(const void* Vs, void* w, long long dim, int R, int j, int
 // FP64 [R][M][M]; Gp holds sym_partial_doubles(R, M, nranges) doubles.
 int sym_ranges(long long dim, int R, int M);
 size_t sym_partial_doubles(int R, int M, int nranges);
-// W: space for (u.S) q_k of every stored vector (the size of Vs), formed
-// first and then loaded by the contraction.
-int launch_sym_omat(const InstDesc* h, const void* Vs, void* W, int R, int M, int nranges, double* Gp, double* G,
+// W: (u.S) q_k of every stored vector (launch_sdir over the R M vectors).
+int launch_sym_omat(long long dim, const void* Vs, const void* W, int R, int M, int nranges, double* Gp, double* G,
                     int c64, void* stream);
 
 // Stored-matrix comparison path (csr.cu): count, scan, fill, multiply.

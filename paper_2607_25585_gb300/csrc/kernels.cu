@@ -4,8 +4,8 @@
 //    element evaluated on the fly (no stored matrix, no atomics);
 //  * the Lanczos step epilogue fused into the matvec (w = H v_j - beta_j
 //    v_{j-1}, in place over v_{j-1}, with the partial sums of
-//    alpha_j = Re<v_j|w> and p_j = <v_j|u>), the orthogonalisation update,
-//    the start-vector norm and the observable u.S;
+//    alpha_j = Re<v_j|w> and p_j = <v_j|u>), the orthogonalisation update
+//    and the start-vector norm;
 //  * deterministic two-stage reductions: per-CTA partials in FP64, then the
 //    last CTA to finish sums them in a fixed order and writes the Lanczos
 //    scalars (alpha, p, beta, the breakdown test and the vector scales).
@@ -33,49 +33,6 @@ __device__ __forceinline__ void h_row(const SmemView& s, const TabLayout& L, int
                                       real* xi_own) {
   GatherSink<real, V> g{x, mu, R, col, ar, ai, xr_own, xi_own};
   row_terms<real>(s, L, n, mu, idx32, g);
-}
-
-// one row of (u.S) x: u_z sum_i m_i x_mu + a_u <a|s+|a-1> x_{mu - s_i} + conj(a_u) <a|s-|a+1> x_{mu + s_i}
-template <typename real, int V>
-__device__ __forceinline__ void s_row(const SmemView& s, const TabLayout& L, int n, long long mu, bool idx32,
-                                      const void* __restrict__ x, int R, int col, real uz, real aur, real aui,
-                                      real* ar, real* ai) {
-  const real* t = reinterpret_cast<const real*>(s.tab);
-  const int qm = L.qmax;
-  real msum = 0;
-#pragma unroll
-  for (int v = 0; v < V; ++v) ar[v] = ai[v] = 0;
-  unsigned long long rem = (unsigned long long)mu;
-  unsigned rem32 = (unsigned)mu;
-  for (int i = 0; i < n; ++i) {
-    int a_i;
-    if (idx32) {
-      const unsigned nq = rem32 / (unsigned)s.q[i];
-      a_i = (int)(rem32 - nq * (unsigned)s.q[i]);
-      rem32 = nq;
-    } else {
-      const unsigned long long nq = rem / (unsigned long long)s.q[i];
-      a_i = (int)(rem - nq * (unsigned long long)s.q[i]);
-      rem = nq;
-    }
-    msum += t[L.off_m + i * qm + a_i];
-    if (a_i >= 1) {
-      const real e = t[L.off_up1 + i * qm + a_i];
-      gather_mac<real, V>(x, mu - s.stride[i], R, col, aur * e, aui * e, ar, ai);
-    }
-    if (a_i + 1 < s.q[i]) {
-      const real e = t[L.off_dn1 + i * qm + a_i];
-      gather_mac<real, V>(x, mu + s.stride[i], R, col, aur * e, -aui * e, ar, ai);
-    }
-  }
-  real xr[V], xi[V];
-  VecIO<real, V>::ldg(x, mu * R + col, xr, xi);
-  const real dz = uz * msum;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    ar[v] = fma(dz, xr[v], ar[v]);
-    ai[v] = fma(dz, xi[v], ai[v]);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -168,7 +125,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 1) rows_kernel(co
       __syncthreads();
       if (threadIdx.x == 0) d = insts[inst];
       __syncthreads();
-      if (MODE == kModeApply || MODE == kModeLanczos || MODE == kModeApplyS) stage_instance<real>(d, s);
+      if (MODE == kModeApply || MODE == kModeLanczos) stage_instance<real>(d, s);
       const int j = a.step;
 #pragma unroll
       for (int v = 0; v < V; ++v) {
@@ -182,8 +139,6 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 1) rows_kernel(co
         } else if (MODE == kModeUpdate) {
           coef[v] = a.update_no_alpha ? (real)0
                                       : (real)(d.sc.alpha[(size_t)j * d.sc.ss + k] * d.sc.sigma[(size_t)j * d.sc.ss + k]);
-        } else if (MODE == kModeApplyS) {
-          coef[v] = a.use_sigma0 ? (real)d.sc.sigma[k] : (real)1;
         } else if (MODE == kModeScale) {
           coef[v] = (real)d.sc.sigma[k];
         }
@@ -290,16 +245,6 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 1) rows_kernel(co
           xi[v] *= coef[v];
         }
         VecIO<real, V>::st(d.y, idx, xr, xi);
-      } else if (MODE == kModeApplyS) {
-        real ar[V], ai[V];
-        s_row<real, V>(s, d.lay, d.n, row, idx32, d.x, a.R, col, (real)d.obs[0], (real)d.obs[1], (real)d.obs[2],
-                       ar, ai);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          ar[v] *= coef[v];
-          ai[v] *= coef[v];
-        }
-        VecIO<real, V>::st(d.y, idx, ar, ai);
       }
     }
     }
@@ -622,7 +567,7 @@ template <typename real, int V>
 static int allow_smem(int bytes) {
   const void* ks[] = {(const void*)rows_kernel<real, V, kModeApply>, (const void*)rows_kernel<real, V, kModeLanczos>,
                       (const void*)rows_kernel<real, V, kModeUpdate>, (const void*)rows_kernel<real, V, kModeStartNorm>,
-                      (const void*)rows_kernel<real, V, kModeApplyS>, (const void*)rows_kernel<real, V, kModeScale>,
+                      (const void*)rows_kernel<real, V, kModeScale>,
                       (const void*)rows_kernel<real, V, kModeEpilogue>, (const void*)rows_kernel<real, V, kModeStep>};
   for (const void* k : ks) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -662,7 +607,6 @@ static int launch_mode(const LaunchArgs& a, int grid, int threads, size_t smem, 
     case kModeLanczos: return launch_one<real, V, kModeLanczos>(a, grid, threads, smem, st);
     case kModeUpdate: return launch_one<real, V, kModeUpdate>(a, grid, threads, smem, st);
     case kModeStartNorm: return launch_one<real, V, kModeStartNorm>(a, grid, threads, smem, st);
-    case kModeApplyS: return launch_one<real, V, kModeApplyS>(a, grid, threads, smem, st);
     case kModeScale: return launch_one<real, V, kModeScale>(a, grid, threads, smem, st);
     case kModeEpilogue: return launch_one<real, V, kModeEpilogue>(a, grid, threads, smem, st);
     case kModeStep: return launch_one<real, V, kModeStep>(a, grid, threads, smem, st);

@@ -7,8 +7,7 @@
 // conj(a) S^-, a = (u_x - i u_y)/2, is one-body, so (u.S) q_j at a row needs
 // q_j at the row itself and at its single-site neighbours mu -+ stride_k.
 //
-// W_k = (u.S) q_k is formed first for every stored vector, vector after
-// vector so that each vector's single-site neighbourhood stays in L2; then a
+// W_k = (u.S) q_k is formed first for every stored vector (sdir.cu); then a
 // contraction kernel in which a CTA owns one vector r, a 16T x 16T block of
 // (i, j) and a range of rows.  Per tile of 64 rows (32 in complex128) it
 // stages q_i (the i block) and W_j (the j block) in shared memory, and every
@@ -140,81 +139,6 @@ __global__ void __launch_bounds__(kSymThreads, sizeof(real) == 4 ? 2 : 1) sym_om
     }
 }
 
-// W_k = (u.S) q_k for every stored vector k (Vs order), V consecutive stored
-// vectors a thread (the row's digits and coefficients formed once for them),
-// row tiles of one group in consecutive CTAs (blockIdx.x fastest) so that the
-// group's single-site neighbourhood is read from HBM once and then served by L2.
-template <typename real, int V>
-__global__ void __launch_bounds__(256) sym_sdir_kernel(const InstDesc d, const real* __restrict__ Vs,
-                                                     real* __restrict__ Wv, int rows_per_cta) {
-  using v2 = typename Cx<real>::v2;
-  const real* t = reinterpret_cast<const real*>(d.tab);
-  const TabLayout& L = d.lay;
-  const int qm = L.qmax, n = d.n;
-  const real uz = (real)d.obs[0], aur = (real)d.obs[1], aui = (real)d.obs[2];
-  const long long dim = d.dim;
-  const v2* x = reinterpret_cast<const v2*>(Vs) + (size_t)blockIdx.y * V * (size_t)dim;
-  v2* w = reinterpret_cast<v2*>(Wv) + (size_t)blockIdx.y * V * (size_t)dim;
-  const long long lo = (long long)blockIdx.x * rows_per_cta;
-  const long long hi = min(dim, lo + rows_per_cta);
-  const bool idx32 = dim <= 0xffffffffll;  // 32-bit digit division when the rows allow it
-  for (long long mu = lo + threadIdx.x; mu < hi; mu += blockDim.x) {
-    unsigned long long rem = (unsigned long long)mu;
-    unsigned rem32 = (unsigned)mu;
-    real ar[V], ai[V], ms = 0;
-#pragma unroll
-    for (int v = 0; v < V; ++v) ar[v] = ai[v] = 0;
-    for (int k = 0; k < n; ++k) {
-      const int qk = __ldg(d.q + k);
-      int a;
-      if (idx32) {
-        const unsigned nq = rem32 / (unsigned)qk;
-        a = (int)(rem32 - nq * (unsigned)qk);
-        rem32 = nq;
-      } else {
-        const unsigned long long nq = rem / (unsigned long long)qk;
-        a = (int)(rem - nq * (unsigned long long)qk);
-        rem = nq;
-      }
-      ms += t[L.off_m + k * qm + a];
-      const long long st = __ldg(d.stride + k);
-      if (a >= 1) {  // a S^+ : from mu - stride
-        const real c = t[L.off_up1 + k * qm + a];
-        const real cr = c * aur, ci = c * aui;
-        v2 xv[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) xv[v] = __ldg(x + (size_t)v * dim + mu - st);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          ar[v] += cr * xv[v].x - ci * xv[v].y;
-          ai[v] += cr * xv[v].y + ci * xv[v].x;
-        }
-      }
-      if (a + 1 < qk) {  // conj(a) S^- : from mu + stride
-        const real c = t[L.off_dn1 + k * qm + a];
-        const real cr = c * aur, ci = c * aui;
-        v2 xv[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) xv[v] = __ldg(x + (size_t)v * dim + mu + st);
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          ar[v] += cr * xv[v].x + ci * xv[v].y;
-          ai[v] += cr * xv[v].y - ci * xv[v].x;
-        }
-      }
-    }
-    const real dz = uz * ms;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const v2 xv = __ldg(x + (size_t)v * dim + mu);
-      v2 o;
-      o.x = ar[v] + dz * xv.x;
-      o.y = ai[v] + dz * xv.y;
-      w[(size_t)v * dim + mu] = o;
-    }
-  }
-}
-
 // G[r][i][j] = sum over the row ranges of the partials, in range order.
 __global__ void sym_reduce_kernel(const double* __restrict__ Gp, int R, int M, int nranges, double* __restrict__ G) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -274,31 +198,12 @@ cudaError_t launch_omat_t(const void* Vs, const void* W, long long dim, int R, i
 
 }  // namespace
 
-int launch_sym_omat(const InstDesc* h, const void* Vs, void* W, int R, int M, int nranges, double* Gp, double* G,
+int launch_sym_omat(long long dim, const void* Vs, const void* W, int R, int M, int nranges, double* Gp, double* G,
                     int c64, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (!W || R < 1 || R > 65535 || M < 1 || nranges < 1 || h->n > kMaxSites) return (int)cudaErrorInvalidValue;
+  if (!W || R < 1 || R > 65535 || M < 1 || nranges < 1) return (int)cudaErrorInvalidValue;
   if ((long long)R * M > 65535) return (int)cudaErrorInvalidValue;
-  const long long dim = h->dim;
   cudaError_t e;
-  {  // (u.S) q_k of every stored vector, vector by vector
-    const int trows = 1024;
-    const int nv = R * M, V = nv % 8 == 0 ? 8 : (nv % 4 == 0 ? 4 : (nv % 2 == 0 ? 2 : 1));
-    const dim3 g1((unsigned)((dim + trows - 1) / trows), (unsigned)(nv / V));
-    if (c64) {
-      if (V == 8) sym_sdir_kernel<float, 8><<<g1, 256, 0, st>>>(*h, (const float*)Vs, (float*)W, trows);
-      else if (V == 4) sym_sdir_kernel<float, 4><<<g1, 256, 0, st>>>(*h, (const float*)Vs, (float*)W, trows);
-      else if (V == 2) sym_sdir_kernel<float, 2><<<g1, 256, 0, st>>>(*h, (const float*)Vs, (float*)W, trows);
-      else sym_sdir_kernel<float, 1><<<g1, 256, 0, st>>>(*h, (const float*)Vs, (float*)W, trows);
-    } else {
-      if (V == 8) sym_sdir_kernel<double, 8><<<g1, 256, 0, st>>>(*h, (const double*)Vs, (double*)W, trows);
-      else if (V == 4) sym_sdir_kernel<double, 4><<<g1, 256, 0, st>>>(*h, (const double*)Vs, (double*)W, trows);
-      else if (V == 2) sym_sdir_kernel<double, 2><<<g1, 256, 0, st>>>(*h, (const double*)Vs, (double*)W, trows);
-      else sym_sdir_kernel<double, 1><<<g1, 256, 0, st>>>(*h, (const double*)Vs, (double*)W, trows);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return (int)e;
-  }
   e = c64 ? launch_omat_t<float>(Vs, W, dim, R, M, nranges, Gp, st)
           : launch_omat_t<double>(Vs, W, dim, R, M, nranges, Gp, st);
   if (e != cudaSuccess) return (int)e;
