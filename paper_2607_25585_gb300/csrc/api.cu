@@ -621,7 +621,7 @@ ftlm_status ensure_rot(ftlm_system* s, const RotPlan& rp, int R, int c64, cudaSt
   const size_t d = (size_t)s->hs.dim, real = c64 ? 4 : 8;
   const RotDirs& dirs = *s->rot;
   DevBuf& D = s->rD[c64 ? 1 : 0];
-  if (prepare_rot(rp.T, c64) != 0) return FTLM_OK;
+  if (prepare_rot(s->hs.n, c64) != 0) return FTLM_OK;
   const size_t tiles = d >> rp.T;
   const size_t tbytes = (size_t)(rp.K + 1) * d * real + rot_phase_bytes(c64);
   bool fits = true, build = !D.p;
@@ -641,7 +641,8 @@ ftlm_status ensure_rot(ftlm_system* s, const RotPlan& rp, int R, int c64, cudaSt
   if (build) {
     for (int k = 0; k <= rp.K; ++k) {
       RotForm f = dirs.form[k];
-      f.T = rp.T;
+      f.T = k > 0 ? rp.T : 0;
+      f.b = rot_run_bits(s->hs.n, c64);
       CKI(launch_rot_table(f, static_cast<char*>(D.p) + (size_t)k * d * real, c64, st));
     }
     CKI(launch_rot_phases(s->hs.n, dirs, static_cast<char*>(D.p) + tbytes - rot_phase_bytes(c64), c64, st));
@@ -670,6 +671,7 @@ RotArgs rot_args(const ftlm_system* s, const RotPlan& rp, int c64) {
   const char* D = static_cast<const char*>(s->rD[c64 ? 1 : 0].p);
   a.n = s->hs.n;
   a.T = rp.T;
+  a.b = rot_run_bits(s->hs.n, c64);
   a.K = rp.K;
   a.t = s->rot->t;
   a.dim = (long long)d;

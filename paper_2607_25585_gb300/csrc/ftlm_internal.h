@@ -261,9 +261,10 @@ constexpr int kRotMaxN = 28;  // sites: two passes over tiles of at most 2^14 va
 constexpr int kRotMaxK = 5;   // directions besides z
 
 // One direction's diagonal form: scale (c0 + sum_i m_i (h_i + sum_{j>i} a_ij m_j)),
-// a in the triangular pair order; rotate: its table has the low T index bits rotated by four.
+// a in the triangular pair order; T > 0: its table is in the order of the
+// intermediate blocks with T low bits and runs of 2^b.
 struct RotForm {
-  int n = 0, rotate = 0, T = 0;
+  int n = 0, T = 0, b = 0;
   double c0 = 0, scale = 1;
   double h[kRotMaxN] = {};
   double a[kRotMaxN * (kRotMaxN - 1) / 2] = {};
@@ -279,7 +280,7 @@ struct RotDirs {
 };
 
 struct RotArgs {
-  int n = 0, T = 0, K = 0;
+  int n = 0, T = 0, b = 0, K = 0;
   double t = 1;
   long long dim = 0;
   int vec0 = 0, nvec = 0;      // the launch's vectors of the block
@@ -289,7 +290,7 @@ struct RotArgs {
   void* y = nullptr;           // q_{j-1}, overwritten by w'; or H x
   const void* u = nullptr;
   void* W = nullptr;           // [vectors][K][dim]
-  const void* D = nullptr;     // [K][dim], low bits rotated
+  const void* D = nullptr;     // [K][dim], in W's order
   const void* D0 = nullptr;    // [dim]
   const void* phases = nullptr;  // [K][kRotMaxN + 1]
   int lanczos = 0;             // backward pass: a step (else y = H x)
@@ -303,7 +304,8 @@ struct RotArgs {
 
 bool rot_directions(const HostSystem& hs, RotDirs& d);
 int rot_tile_bits(int n, int c64);
-int prepare_rot(int T, int c64);
+int rot_run_bits(int n, int c64);
+int prepare_rot(int n, int c64);
 int launch_rot(const RotArgs& a, int pass, int c64, void* stream);  // pass 0 forward, 1 middle, 2 backward
 int launch_rot_table(const RotForm& f, void* out, int c64, void* stream);
 int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream);

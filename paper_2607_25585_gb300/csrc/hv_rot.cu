@@ -28,13 +28,18 @@
 //   forward:  w (the step's update, see below) -> W_k = the low bits' gates on
 //             e^{-i phi_k downs} w, for every direction k;
 //   middle:   W_k <- the high bits' gates, times D_k, the inverse gates
-//             (tiles of 2^nH rows x 2^c columns, c = T - nH);
+//             (tiles of 2^nH rows x 2^c columns);
 //   backward: H v = D_0 v + sum_k e^{+i phi_k downs} (inverse low gates of W_k),
 //             then the step's epilogue.
 // A tile of 2^T values is exchanged through shared memory between groups of
-// four bits; a thread holds the 16 values of a group in registers.  W is laid
-// out as the forward pass's last group leaves it (the low T bits rotated by
-// four), which both of its neighbours read and write contiguously.
+// four bits; a thread holds the 16 values of a group in registers.  W's order
+// serves both sides: with l the low T bits rotated by four, as the forward
+// pass's last group leaves them, and h the high bits, value (l, h) is at
+// (l >> b, h, low b bits of l): the outer passes move runs of 2^b values, the
+// middle pass reads rows of 2^c values 2^b apart.  b = T (whole tiles contiguous)
+// while the middle's rows are long; b = 4 (128 bytes) where they are 32 bytes,
+// which otherwise lie 2^T values apart: 6.5 -> 5.3 ms for the middle pass over
+// 2^26 x 4 values, against 0.2 ms more for the outer ones.
 //
 // Lanczos step j (x = q_j, y = q_{j-1}, u): the forward pass first finishes the
 // previous step, q_j = w' - alpha_{j-1} sigma_{j-1} q_{j-1} with |q_j|^2 (so no
@@ -45,14 +50,15 @@
 //
 // Bound: memory.  A step moves 8 (7 + 4 K) bytes a value in complex64 (152 for
 // K = 3), against 56 for the gather, but the gather's C(n, 2) flips take 3.5 ms
-// at n = 20 with 64 vectors, where these passes take 1.8 ms with the update
-// (3.8 ms with it before): 5.7 TB/s.  2 x 13 sites, 4 vectors: 33 -> 12.6 ms a
+// at n = 20 with 64 vectors, where these passes take 1.71 ms with the update
+// (3.8 ms with it before): 6.0 TB/s.  2 x 13 sites, 4 vectors: 33 -> 11.7 ms a
 // step.  In complex128 the FP64 pipe binds both: 4 x 4 sites, 50 vectors:
 // 4.0 -> 1.57 ms.  Taking one to eight vectors at a time through the three
 // passes, so that W stays in L2, was slower (2.1 to 3.0 ms): each launch then
 // has too few tiles.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -104,6 +110,11 @@ __device__ __forceinline__ void gates(v2 (&v)[16], real t, int mask) {
 template <int LO>
 __device__ __forceinline__ int group_base(int tid) {
   return ((tid >> LO) << (LO + 4)) | (tid & ((1 << LO) - 1));
+}
+
+// place in W of low part l (rotated) and high part 0; linear in disjoint sets of bits
+__host__ __device__ __forceinline__ unsigned w_place(unsigned l, int b, int nH) {
+  return ((l >> b) << (b + nH)) | (l & ((1u << b) - 1u));
 }
 
 // shared-memory place of element i: one padding value after every 16
@@ -256,15 +267,16 @@ __global__ void __launch_bounds__(NT, MINB) rot_forward_kernel(const __grid_cons
     __syncthreads();
     if constexpr (Gr::N >= 3) mid_group<real, T, NT, SETS, 1>(buf, t, 15);
     if constexpr (Gr::N >= 4) mid_group<real, T, NT, SETS, 2>(buf, t, 15);
-    v2* W = reinterpret_cast<v2*>(a.W) + ((size_t)(v - a.vecW) * a.K + k) * a.dim + ((size_t)tile << T);
+    v2* W = reinterpret_cast<v2*>(a.W) + ((size_t)(v - a.vecW) * a.K + k) * a.dim + ((size_t)tile << a.b);
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
       const int i0 = threadIdx.x + s * NT;
       v2 w[16];
       smem_ld<0>(buf, group_base<0>(i0), w);
       gates(w, t, Gr::mask(GL));
+      v2* p = W + w_place(i0, a.b, nH);
 #pragma unroll
-      for (int r = 0; r < 16; ++r) W[(r << LO0) + i0] = w[r];
+      for (int r = 0; r < 16; ++r) p[w_place(r << LO0, a.b, nH)] = w[r];
     }
     if (k + 1 < a.K) __syncthreads();
   }
@@ -274,95 +286,97 @@ __global__ void __launch_bounds__(NT, MINB) rot_forward_kernel(const __grid_cons
   }
 }
 
-// Columns: tile element (h, col) is W[k][h << T | cb << c | col], at tile index h << c | col.
-template <typename real, int T, int NT, int MINB, int NG>
+// Tiles of 2^TB values: 2^nH rows (the high bits) of 2^c columns, c = TB - nH <= b;
+// tile element (h, col) has tile index h << c | col.
+// NG: groups that hold transformed bits (the last one is transformed, multiplied
+// by D and transformed back in registers).
+template <typename real, int TB, int NT, int MINB, int NG>
 __global__ void __launch_bounds__(NT, MINB) rot_middle_kernel(const __grid_constant__ RotArgs a) {
   using v2 = typename Cx<real>::v2;
-  using Gr = Groups<T>;
-  constexpr int SETS = (1 << T) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = T - 4;
+  using Gr = Groups<TB>;
+  constexpr int SETS = (1 << TB) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = TB - 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   v2* buf = reinterpret_cast<v2*>(smem_raw);
-  const int nH = a.n - T, c = T - nH;
+  const int T = a.T, nH = a.n - T, c = TB - nH;
   const int cmask = (1 << c) - 1;
-  const int cb = blockIdx.x & ((1 << nH) - 1);  // 2^T columns in blocks of 2^c
-  const int rest = (int)(blockIdx.x >> nH);
+  const int ncb = 1 << (T - c);  // 2^T columns in blocks of 2^c
+  const int cb = blockIdx.x & (ncb - 1);
+  const int rest = (int)(blockIdx.x >> (T - c));
   const int k = rest % a.K, vg = rest / a.K;
-  auto at = [&](int i) { return ((unsigned)(i >> c) << T) + (unsigned)(i & cmask); };  // offset of tile index i
+  auto at = [&](int i) { return ((unsigned)(i >> c) << a.b) + (unsigned)(i & cmask); };  // offset of tile index i
+  // offset of value r of group 0: with two or more groups all its bits are high ones
+  const unsigned stride0 = 1u << (LO0 - (NG > 1 ? c : 0) + a.b);
+  auto at0 = [&](int r) { return NG > 1 ? r * stride0 : at(r << LO0); };
+  const size_t first = (size_t)k * a.dim + w_place((unsigned)cb << c, a.b, nH);
   auto mask_of = [&](int g) {  // the transformed bits (>= c) of group g
     const int l = Gr::lo(g);
     return (c > l ? (15 << (c - l)) : 15) & Gr::mask(g);
   };
   const real t = (real)a.t;
-  const real* D = reinterpret_cast<const real*>(a.D) + (size_t)k * a.dim + ((size_t)cb << c);
-  real dv[SETS][16];
-#pragma unroll
-  for (int s = 0; s < SETS; ++s) {
-    const unsigned b = at(group_base<LOC>(threadIdx.x + s * NT));
-#pragma unroll
-    for (int r = 0; r < 16; ++r) dv[s][r] = __ldg(D + b + at(r << LOC));
-  }
+  const real* D = reinterpret_cast<const real*>(a.D) + first;
   const int v1 = min(a.nvec, (vg + 1) * a.vpb);
   for (int v = vg * a.vpb; v < v1; ++v) {
-    v2* W = reinterpret_cast<v2*>(a.W) + ((size_t)(a.vec0 - a.vecW + v) * a.K + k) * a.dim + ((size_t)cb << c);
+    v2* W = reinterpret_cast<v2*>(a.W) + (size_t)(a.vec0 - a.vecW + v) * a.K * a.dim + first;
+    // gates of the last group, D (after the first vector from L1) and the inverse gates
+    auto centre = [&](v2(&w)[16], int b) {
+      const real* d = D + at(b);
+      const int m = mask_of(NG - 1);
+      gates(w, t, m);
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const real dv = __ldg(d + at(r << LOC));
+        w[r].x *= dv;
+        w[r].y *= dv;
+      }
+      gates(w, -t, m);
+    };
     if constexpr (NG > 1) {
 #pragma unroll
       for (int s = 0; s < SETS; ++s) {
         const int i0 = threadIdx.x + s * NT;
-        const unsigned b = at(i0);
+        const v2* p = W + at(i0);
         v2 w[16];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) w[r] = W[b + at(r << LO0)];
-        gates(w, t, mask_of(0));
+        for (int r = 0; r < 16; ++r) w[r] = p[at0(r)];
+        gates(w, t, 15);
         smem_st<LO0>(buf, i0, w);
       }
       __syncthreads();
-      if constexpr (NG > 2) mid_group<real, T, NT, SETS, 1>(buf, t, mask_of(1));
-      if constexpr (NG > 3) mid_group<real, T, NT, SETS, 2>(buf, t, mask_of(2));
-      const int mc = mask_of(NG - 1);
+      if constexpr (NG > 2) mid_group<real, TB, NT, SETS, 1>(buf, t, 15);
+      if constexpr (NG > 3) mid_group<real, TB, NT, SETS, 2>(buf, t, 15);
 #pragma unroll
       for (int s = 0; s < SETS; ++s) {
         const int b = group_base<LOC>(threadIdx.x + s * NT);
         v2 w[16];
         smem_ld<LOC>(buf, b, w);
-        gates(w, t, mc);
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          w[r].x *= dv[s][r];
-          w[r].y *= dv[s][r];
-        }
-        gates(w, -t, mc);
+        centre(w, b);
         smem_st<LOC>(buf, b, w);
       }
       __syncthreads();
-      if constexpr (NG > 3) mid_group<real, T, NT, SETS, 2>(buf, -t, mask_of(2));
-      if constexpr (NG > 2) mid_group<real, T, NT, SETS, 1>(buf, -t, mask_of(1));
+      if constexpr (NG > 3) mid_group<real, TB, NT, SETS, 2>(buf, -t, 15);
+      if constexpr (NG > 2) mid_group<real, TB, NT, SETS, 1>(buf, -t, 15);
 #pragma unroll
       for (int s = 0; s < SETS; ++s) {
         const int i0 = threadIdx.x + s * NT;
-        const unsigned b = at(i0);
+        v2* p = W + at(i0);
         v2 w[16];
         smem_ld<LO0>(buf, i0, w);
-        gates(w, -t, mask_of(0));
+        gates(w, -t, 15);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) W[b + at(r << LO0)] = w[r];
+        for (int r = 0; r < 16; ++r) p[at0(r)] = w[r];
       }
-      // the next vector's first group writes the places this thread has just read
+      // (the next vector's first group writes the places this thread has just read)
     } else {
 #pragma unroll
       for (int s = 0; s < SETS; ++s) {
-        const unsigned b = at(threadIdx.x + s * NT);
+        const int i0 = threadIdx.x + s * NT;
+        v2* p = W + at(i0);
         v2 w[16];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) w[r] = W[b + at(r << LO0)];
-        gates(w, t, mask_of(0));
+        for (int r = 0; r < 16; ++r) w[r] = p[at0(r)];
+        centre(w, i0);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          w[r].x *= dv[s][r];
-          w[r].y *= dv[s][r];
-        }
-        gates(w, -t, mask_of(0));
-#pragma unroll
-        for (int r = 0; r < 16; ++r) W[b + at(r << LO0)] = w[r];
+        for (int r = 0; r < 16; ++r) p[at0(r)] = w[r];
       }
     }
   }
@@ -383,13 +397,14 @@ __global__ void __launch_bounds__(NT, MINB) rot_backward_kernel(const __grid_con
   const real t = (real)a.t;
   v2 acc[SETS][16];
   for (int k = 0; k < a.K; ++k) {
-    const v2* W = reinterpret_cast<const v2*>(a.W) + ((size_t)(v - a.vecW) * a.K + k) * a.dim + ((size_t)tile << T);
+    const v2* W = reinterpret_cast<const v2*>(a.W) + ((size_t)(v - a.vecW) * a.K + k) * a.dim + ((size_t)tile << a.b);
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
       const int i0 = threadIdx.x + s * NT;
+      const v2* p = W + w_place(i0, a.b, nH);
       v2 w[16];
 #pragma unroll
-      for (int r = 0; r < 16; ++r) w[r] = W[(r << LO0) + i0];
+      for (int r = 0; r < 16; ++r) w[r] = p[w_place(r << LO0, a.b, nH)];
       gates(w, -t, Gr::mask(GL));
       if (s == 0) __syncthreads();  // the previous direction's last group has been read
       smem_st<0>(buf, group_base<0>(i0), w);
@@ -472,8 +487,7 @@ __global__ void __launch_bounds__(NT, MINB) rot_backward_kernel(const __grid_con
   }
 }
 
-// Diagonal table of one direction: entry at place e of the table's order (the
-// natural one, or with the low T bits rotated by four) is
+// Diagonal table of one direction, in the natural order or (f.T > 0) in W's:
 //   scale (c0 + sum_i m_i (h_i + sum_{j > i} a_ij m_j)),  m_i = +-1/2 by bit i,
 // in FP64, one CTA per 4096 entries: the terms of the bits above 12 once per
 // CTA, a thread's 16 entries along bits 0..3.
@@ -519,9 +533,9 @@ __global__ void __launch_bounds__(256) rot_table_kernel(const __grid_constant__ 
       d += ((r >> i) & 1 ? 0.5 : -0.5) * s;
     }
     unsigned long long at = (top << 12) | (unsigned)mid | (unsigned)r;
-    if (f.rotate) {
-      const unsigned long long low = at & ((1ull << f.T) - 1);
-      at = (at ^ low) | ((low & 15) << (f.T - 4)) | (low >> 4);
+    if (f.T > 0) {
+      const unsigned low = (unsigned)at & ((1u << f.T) - 1u);
+      at = w_place(((low & 15u) << (f.T - 4)) | (low >> 4), f.b, f.n - f.T) + ((at >> f.T) << f.b);
     }
     out[at] = (real)(f.scale * d);
   }
@@ -538,67 +552,98 @@ __global__ void rot_phase_kernel(int n, int K, RotAzimuths d, real* out) {
   out[2 * threadIdx.x + 1] = (real)-sn;
 }
 
+template <typename real, int T>
+constexpr size_t tile_smem() {
+  return sizeof(typename Cx<real>::v2) * (size_t)pad(1 << T);
+}
+
+// the forward and backward passes over tiles of 2^T values
 template <typename real, int T, int NT, int MINB>
-int launch_pass(const RotArgs& a, int pass, cudaStream_t st) {
-  const size_t smem = sizeof(typename Cx<real>::v2) * (size_t)pad(1 << T);
-  const int nH = a.n - T;
-  if (nH < 1 || nH > T || a.n > kRotMaxN || a.K < 1 || a.K > kRotMaxK) return (int)cudaErrorInvalidValue;
-  if (pass == 0) {
-    rot_forward_kernel<real, T, NT, MINB><<<(unsigned)a.nvec << nH, NT, smem, st>>>(a);
-  } else if (pass == 2) {
-    rot_backward_kernel<real, T, NT, MINB><<<(unsigned)a.nvec << nH, NT, smem, st>>>(a);
-  } else {
-    const int c = T - nH;
-    int ng = 1;
-    while (ng < Groups<T>::N && Groups<T>::lo(ng - 1) > c) ++ng;
-    const unsigned grid = (unsigned)(((a.nvec + a.vpb - 1) / a.vpb) * a.K) << nH;
-    if (ng == 1) rot_middle_kernel<real, T, NT, MINB, 1><<<grid, NT, 0, st>>>(a);
-    else if (ng == 2) rot_middle_kernel<real, T, NT, MINB, 2><<<grid, NT, smem, st>>>(a);
-    else if (ng == 3) rot_middle_kernel<real, T, NT, MINB, 3><<<grid, NT, smem, st>>>(a);
-    else if constexpr (Groups<T>::N >= 4) rot_middle_kernel<real, T, NT, MINB, 4><<<grid, NT, smem, st>>>(a);
-    else return (int)cudaErrorInvalidValue;
-  }
+int launch_outer(const RotArgs& a, int pass, cudaStream_t st) {
+  const unsigned grid = (unsigned)a.nvec << (a.n - T);
+  if (pass == 0) rot_forward_kernel<real, T, NT, MINB><<<grid, NT, tile_smem<real, T>(), st>>>(a);
+  else rot_backward_kernel<real, T, NT, MINB><<<grid, NT, tile_smem<real, T>(), st>>>(a);
   return (int)cudaGetLastError();
 }
 
+// the middle pass over tiles of 2^TB values
+template <typename real, int TB, int NT, int MINB>
+int launch_middle(const RotArgs& a, cudaStream_t st) {
+  using Gr = Groups<TB>;
+  const int nH = a.n - a.T, c = TB - nH;
+  const size_t smem = tile_smem<real, TB>();
+  int ng = 1;
+  while (ng < Gr::N && Gr::lo(ng - 1) > c) ++ng;
+  const unsigned grid = (unsigned)(((a.nvec + a.vpb - 1) / a.vpb) * a.K) << (a.T - c);
+  if (ng == 1) rot_middle_kernel<real, TB, NT, MINB, 1><<<grid, NT, 0, st>>>(a);
+  else if (ng == 2) rot_middle_kernel<real, TB, NT, MINB, 2><<<grid, NT, smem, st>>>(a);
+  else if (ng == 3) rot_middle_kernel<real, TB, NT, MINB, 3><<<grid, NT, smem, st>>>(a);
+  else if constexpr (Gr::N >= 4) rot_middle_kernel<real, TB, NT, MINB, 4><<<grid, NT, smem, st>>>(a);
+  else return (int)cudaErrorInvalidValue;
+  return (int)cudaGetLastError();
+}
+
+int allow(const void* k, size_t smem) {
+  return (int)cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
 template <typename real, int T, int NT, int MINB>
-int prepare_pass() {
-  const int smem = (int)(sizeof(typename Cx<real>::v2) * (size_t)pad(1 << T));
-  const void* ks[] = {(const void*)rot_forward_kernel<real, T, NT, MINB>, (const void*)rot_backward_kernel<real, T, NT, MINB>,
-                      (const void*)rot_middle_kernel<real, T, NT, MINB, 2>, (const void*)rot_middle_kernel<real, T, NT, MINB, 3>};
-  for (const void* k : ks) {
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return (int)e;
-  }
-  if constexpr (Groups<T>::N >= 4)
-    return (int)cudaFuncSetAttribute((const void*)rot_middle_kernel<real, T, NT, MINB, 4>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return 0;
+int prepare_outer() {
+  const int e = allow((const void*)rot_forward_kernel<real, T, NT, MINB>, tile_smem<real, T>());
+  return e ? e : allow((const void*)rot_backward_kernel<real, T, NT, MINB>, tile_smem<real, T>());
+}
+template <typename real, int TB, int NT, int MINB>
+int prepare_middle() {
+  int e = allow((const void*)rot_middle_kernel<real, TB, NT, MINB, 2>, tile_smem<real, TB>());
+  if (!e) e = allow((const void*)rot_middle_kernel<real, TB, NT, MINB, 3>, tile_smem<real, TB>());
+  if constexpr (Groups<TB>::N >= 4)
+    if (!e) e = allow((const void*)rot_middle_kernel<real, TB, NT, MINB, 4>, tile_smem<real, TB>());
+  return e;
+}
+
+// The middle pass's tile for nH high bits: the small one, of which an SM runs
+// four (three in complex128), while its rows are at least 32 bytes; else the
+// large one.  (2^13-value tiles with 16-byte rows, three an SM: 9.8 ms instead of
+// 6.5 for 2^26 x 4 values; L2 moves whole 32-byte sectors.)
+int middle_bits(int nH, int c64) {
+  if (c64) return nH <= 10 ? 12 : 14;
+  return nH <= 10 ? 11 : (nH <= 12 ? 12 : 13);
 }
 
 }  // namespace
 
-int launch_rot(const RotArgs& a, int pass, int c64, void* stream) {
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (c64) {
-    if (a.T == 12) return launch_pass<float, 12, 256, 3>(a, pass, st);
-    if (a.T == 14) return launch_pass<float, 14, 512, 1>(a, pass, st);
-  } else {
-    if (a.T == 11) return launch_pass<double, 11, 128, 3>(a, pass, st);
-    if (a.T == 13) return launch_pass<double, 13, 256, 1>(a, pass, st);
-  }
-  return (int)cudaErrorInvalidValue;
+// b of W's order for n sites (see the top of the file)
+int rot_run_bits(int n, int c64) {
+  const int T = rot_tile_bits(n, c64), nH = n - T;
+  return nH <= 10 ? T : std::max(middle_bits(nH, c64) - nH, c64 ? 4 : 3);
 }
 
-int prepare_rot(int T, int c64) {
-  if (c64) {
-    if (T == 12) return prepare_pass<float, 12, 256, 3>();
-    if (T == 14) return prepare_pass<float, 14, 512, 1>();
-  } else {
-    if (T == 11) return prepare_pass<double, 11, 128, 3>();
-    if (T == 13) return prepare_pass<double, 13, 256, 1>();
+int launch_rot(const RotArgs& a, int pass, int c64, void* stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (a.T != rot_tile_bits(a.n, c64) || a.T == 0 || a.K < 1 || a.K > kRotMaxK || a.vpb < 1) return (int)cudaErrorInvalidValue;
+  if (pass != 1) {
+    if (c64) return a.T == 12 ? launch_outer<float, 12, 256, 3>(a, pass, st) : launch_outer<float, 14, 512, 1>(a, pass, st);
+    return a.T == 11 ? launch_outer<double, 11, 128, 3>(a, pass, st) : launch_outer<double, 13, 256, 1>(a, pass, st);
   }
-  return (int)cudaErrorInvalidValue;
+  switch (middle_bits(a.n - a.T, c64)) {
+    case 11: return launch_middle<double, 11, 128, 3>(a, st);
+    case 12: return c64 ? launch_middle<float, 12, 256, 4>(a, st) : launch_middle<double, 12, 128, 3>(a, st);
+    case 13: return launch_middle<double, 13, 256, 1>(a, st);
+    default: return launch_middle<float, 14, 1024, 1>(a, st);
+  }
+}
+
+int prepare_rot(int n, int c64) {
+  int e;
+  const int T = rot_tile_bits(n, c64);
+  if (c64) e = T == 12 ? prepare_outer<float, 12, 256, 3>() : prepare_outer<float, 14, 512, 1>();
+  else e = T == 11 ? prepare_outer<double, 11, 128, 3>() : prepare_outer<double, 13, 256, 1>();
+  if (e) return e;
+  switch (middle_bits(n - T, c64)) {
+    case 11: return prepare_middle<double, 11, 128, 3>();
+    case 12: return c64 ? prepare_middle<float, 12, 256, 4>() : prepare_middle<double, 12, 128, 3>();
+    case 13: return prepare_middle<double, 13, 256, 1>();
+    default: return prepare_middle<float, 14, 1024, 1>();
+  }
 }
 
 int launch_rot_table(const RotForm& f, void* out, int c64, void* stream) {
@@ -618,14 +663,13 @@ int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream)
   return (int)cudaGetLastError();
 }
 
-// Tile size for n sites: the small tile while the middle pass's columns are at
-// least 32 bytes (several CTAs a SM overlap their loads and exchanges), the
-// large one beyond; 0: no tile fits (the gather runs).
+// Low tile bits for n sites (0: none, the gather runs): the small tile, of which
+// an SM runs three, while a middle tile has room for the other bits; then the
+// large one, one CTA an SM.
 int rot_tile_bits(int n, int c64) {
-  const int small = c64 ? 12 : 11, col = c64 ? 2 : 1;
-  if (n <= 12 || n > kRotMaxN) return 0;
-  if (2 * small - n >= col) return small;
-  return small + 2 < n && 2 * (small + 2) >= n ? small + 2 : 0;
+  if (n < 13) return 0;
+  if (c64) return n <= 24 ? 12 : (n <= 28 ? 14 : 0);
+  return n <= 23 ? 11 : (n <= 26 ? 13 : 0);
 }
 
 // The directions and diagonal forms of a spin-1/2 system (see the top of the
@@ -681,7 +725,6 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
   for (int k = 0; k <= K; ++k) {
     RotForm& f = d.form[k];
     f.n = n;
-    f.rotate = k > 0;
     f.c0 = 0.0;
     f.scale = k == 0 ? 1.0 : std::pow(1.0 + d.t * d.t, -n);
   }
