@@ -94,6 +94,10 @@ struct ftlm_system {
   std::unique_ptr<RotDirs> rot;
   DevBuf rD[2];          // its diagonal tables [K + 1][dim] and phases, [c64]
   DevBuf rW, rpart;      // its intermediate blocks; partial sums and arrival counters
+  DevBuf rows[2];        // stored rows of a small system, [c64]: values, columns, counts
+  cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written (on own_stream)
+  bool rows_done[2] = {false, false};           // that event has been seen complete
+  std::mutex rows_mu;
   bool apply_used = false;
   std::mutex mu;
 };
@@ -215,6 +219,7 @@ struct Plan {
   LaunchArgs base;
   std::vector<int> tile_start;
   HalfPlan half;  // spin-1/2 kernel for the H.v modes, when applicable
+  int storedV = 0;  // > 0: H.v of vector-major runs from stored rows, that many vectors a group
   int wideV = 0;  // general kernel: H.v with 4 or 8 complex64 vectors per thread (0 = off)
   // vector-major general plan (any spins, several systems): every vector of a
   // run contiguous; the streaming modes see one instance per (system, vector),
@@ -497,8 +502,7 @@ int launch_plan(const Plan& pl, LaunchArgs a, void* st) {
     if (pl.gvm_cube) return launch_cube(a, pl.gvm_cube, pl.gvm_V, pl.c64, pl.gvm_grid, 256, pl.gvm_smem, st);
     return launch_rows_vm(a, pl.gvm_V, pl.c64, pl.gvm_grid, 256, pl.gvm_smem, st);
   }
-  if (pl.half.on && pl.half.vm &&
-      (a.mode == kModeStep || a.mode == kModeStartNorm || a.mode == kModeUpdate)) {
+  if (pl.half.on && pl.half.vm && a.mode == kModeStep) {
     a.rows_per_tile = pl.half.stream_rows;
     a.tiles_per_vg = pl.half.stream_tiles_per_vg;
     a.n_inst = pl.half.nvg;
@@ -681,6 +685,58 @@ RotArgs rot_args(const ftlm_system* s, const RotPlan& rp, int c64) {
   return a;
 }
 
+// ---- stored rows of small systems -----------------------------------------------
+
+// Rows are stored up to a quarter of L2, where every product reads them from
+// there.  (Larger systems have rows enough to fill the chip with the gathers.)
+constexpr size_t kStoredBytes = 32u << 20;
+
+// The system's stored rows for work on stream st: written on the first call (on
+// the system's own stream; st waits for them).  ok = false: none (too large, or
+// not there yet while st is being captured; the gathers then run).
+ftlm_status ensure_stored(ftlm_system* s, int c64, cudaStream_t st, StoredRows& r, bool& ok) {
+  ok = false;
+  const int k = c64 ? 1 : 0;
+  const size_t d = (size_t)s->hs.dim, esz = c64 ? 8 : 16;
+  const size_t S = (size_t)stored_row_bound(s->hs);
+  if (S == 0 || d > kStoredBytes || d * S * (esz + 4) + d * 4 > kStoredBytes) return FTLM_OK;
+  std::lock_guard<std::mutex> lk(s->rows_mu);
+  DevBuf& b = s->rows[k];
+  if (!s->rows_done[k]) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+      return cudaGetLastError(), FTLM_OK;
+    if (!b.p) {
+      if (!s->ev_rows[k]) CK(cudaEventCreateWithFlags(&s->ev_rows[k], cudaEventDisableTiming));
+      if (b.ensure(d * S * (esz + 4) + d * 4) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
+      char* p = static_cast<char*>(b.p);
+      CKI(launch_stored_build(c64 ? s->tab_f.p : s->tab_d.p, s->hs.lay,
+                              reinterpret_cast<const long long*>(s->stride.p), reinterpret_cast<const int*>(s->q.p),
+                              s->hs.n, (int)d, (int)S, reinterpret_cast<int*>(p + d * S * esz), p,
+                              reinterpret_cast<int*>(p + d * S * (esz + 4)), c64, s->own_stream));
+      CK(cudaEventRecord(s->ev_rows[k], s->own_stream));
+    }
+    if (cudaEventQuery(s->ev_rows[k]) == cudaSuccess) s->rows_done[k] = true;
+    else CK(cudaStreamWaitEvent(st, s->ev_rows[k], 0));
+    cudaGetLastError();  // (not ready is no error)
+  }
+  const char* p = static_cast<const char*>(b.p);
+  r.val = p;
+  r.col = reinterpret_cast<const int*>(p + d * S * esz);
+  r.cnt = reinterpret_cast<const int*>(p + d * S * (esz + 4));
+  r.S = (long long)S;
+  ok = true;
+  return FTLM_OK;
+}
+
+// Vectors a CTA of the stored-row kernels takes: as many as leave the chip enough
+// threads (eight a row and group) to hide L2 latency; `divide`: a divisor of R.
+int stored_group(uint64_t rows, int R, bool divide) {
+  int V = 4;
+  while (V > 1 && (V > R || (divide && R % V != 0) || rows * 8 * (uint64_t)((R + V - 1) / V) < 200000)) V /= 2;
+  return V;
+}
+
 int plan_max_grid(const Plan& pl) {
   return std::max(std::max(pl.grid, pl.gen_vm ? pl.gvm_grid : 0),
                   pl.half.on ? std::max(pl.half.grid, pl.half.stream_grid) : 0);
@@ -761,6 +817,9 @@ struct RunCtx {
   cudaGraph_t g = nullptr;
   cudaGraphExec_t ex = nullptr;
   DevBuf desc, tiles, partials, counter;
+  DevBuf vslots;  // vector-major runs: arrival counters, then partial sums by (vector, tile)
+  int stream_grid = 0, stream_tiles = 0, stored_grid = 0, stored_tiles = 0, stream_at = 0, stored_at = 0;
+  bool even = false;  // every vector's length is even
   std::vector<cudaEvent_t> ev;  // [2M + 2] when kernel timing is on
   int launches = 0, hv_launches = 0;
   char* pinned = nullptr;
@@ -772,6 +831,7 @@ struct RunCtx {
     tiles.release();
     partials.release();
     counter.release();
+    vslots.release();
     for (auto e : ev) cudaEventDestroy(e);
     if (pinned) cudaFreeHost(pinned);
   }
@@ -806,6 +866,7 @@ std::string run_key(const std::vector<ftlm_system*>& sys, const ftlm_run_params*
   k += buf;
   k += p->symmetric ? "|sym" : "";
   k += p->reorth ? "|reorth" : "";
+  k += pl.storedV ? "|rows" + std::to_string(pl.storedV) : "";
   k += pl.rot.on ? "|rot" + std::to_string(pl.rot.group) : "";
   k += pl.gen_vm ? "|gvm" + std::to_string(pl.gvm_V) + "x" + std::to_string(pl.gvm_rows) + "c" +
                        std::to_string(pl.gvm_cube)
@@ -880,7 +941,7 @@ ftlm_status enqueue_rot_passes(RunCtx* ctx, ftlm_system* s, const RotPlan& rp, R
 
 // The M Lanczos steps of a rotated-basis run; `upd` is the update launch that
 // ends the last one.
-ftlm_status enqueue_rot_steps(RunCtx& ctx, ftlm_system* s, const ftlm_run_params* p, const Plan& pl, LaunchArgs upd,
+ftlm_status enqueue_rot_steps(RunCtx& ctx, ftlm_system* s, const ftlm_run_params* p, const Plan& pl, StreamArgs upd,
                               const InstDesc* d_even, const InstDesc* d_odd, cudaStream_t st) {
   const int M = p->M, R = p->R, c64 = pl.c64;
   const size_t esz = c64 ? 8 : 16, d = (size_t)s->hs.dim;
@@ -911,10 +972,8 @@ ftlm_status enqueue_rot_steps(RunCtx& ctx, ftlm_system* s, const ftlm_run_params
     CK(mark(4 + 4 * j));
   }
   upd.inst = (M - 1) % 2 == 0 ? d_even : d_odd;
-  upd.step = M - 1;
-  upd.first = M == 1;
-  upd.mode = kModeUpdate;
-  CKI(launch_plan(pl, upd, st));
+  upd.j = M - 1;
+  CKI(launch_stream_vectors(upd, kModeUpdate, c64, ctx.even, ctx.stream_grid, st));
   ctx.launches++;
   return FTLM_OK;
 }
@@ -964,9 +1023,24 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
       CKI(launch_copy_block(p->user_start, sys[k]->A.p, (size_t)dim * R * (c64 ? 8 : 16), st));
     ctx.launches++;
   }
+  // vector-major runs: streaming passes by vector
+  StreamArgs sa;
+  if (vmaj) {
+    sa.tile_start = reinterpret_cast<const int*>(ctx.tiles.p) + ctx.stream_at;
+    sa.vectors = nd;
+    sa.max_tiles = ctx.stream_tiles;
+    sa.counters = reinterpret_cast<unsigned*>(ctx.vslots.p);
+    sa.slots = reinterpret_cast<double*>(static_cast<char*>(ctx.vslots.p) + (((size_t)nd * 4 + 255) & ~size_t(255)));
+  }
+  auto stream = [&](int mode, const InstDesc* inst, int j) {
+    sa.inst = inst;
+    sa.j = j;
+    return launch_stream_vectors(sa, mode, c64, ctx.even, ctx.stream_grid, st);
+  };
   a.inst = d_start;  // sigma_0 = 1/|q_0|, then U = sigma_0 (u.S) q_0
   a.mode = kModeStartNorm;
-  CKI(launch_plan(pl, a, st));
+  if (vmaj) CKI(stream(kModeStartNorm, d_start, 0));
+  else CKI(launch_plan(pl, a, st));
   ctx.launches++;
   for (auto* s : sys) {
     SdirArgs u = sdir_args(s, c64, R, s->A.p, s->U.p);
@@ -976,7 +1050,7 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
     ctx.launches++;
   }
   if (pl.rot.on) {
-    ftlm_status rs = enqueue_rot_steps(ctx, sys[0], p, pl, a, d_even, d_odd, st);
+    ftlm_status rs = enqueue_rot_steps(ctx, sys[0], p, pl, sa, d_even, d_odd, st);
     if (rs != FTLM_OK) return rs;
   }
   for (int j = 0; j < M && !pl.rot.on; ++j) {
@@ -1001,29 +1075,27 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
       else CKI(launch_to_vector_major(q, dst, (long long)s0->hs.dim, R, c64, st));
       ctx.launches++;
     }
-    if (fused_step) {
-      LaunchArgs g = a;  // x = q_j, y = q_{j-1} (w' in place), u
+    if (pl.storedV) {  // stored rows: w' over q_{j-1}, alpha_j, p_j
+      StoredArgs g;
+      g.inst = a.inst;
+      g.tile_start = reinterpret_cast<const int*>(ctx.tiles.p) + ctx.stored_at;
+      g.groups = nd / pl.storedV;
+      g.max_tiles = ctx.stored_tiles;
+      g.j = j;
+      g.slots = sa.slots;
+      g.counters = sa.counters;
+      if (tk) CK(cudaEventRecordWithFlags(ctx.ev[evi++], st, cudaEventRecordExternal));
+      CKI(launch_stored_step(g, pl.storedV, c64, ctx.stored_grid, st));
+    } else if (fused_step || (pl.gen_vm && pl.gvm_cube)) {  // these gathers write w' over q_{j-1} and set alpha_j, p_j
+      LaunchArgs g = a;                                     // x = q_j, y = q_{j-1}, u
       g.mode = kModeApply;
       g.fused_step = 1;
       if (tk) CK(cudaEventRecordWithFlags(ctx.ev[evi++], st, cudaEventRecordExternal));
       CKI(launch_plan(pl, g, st));
-      if (tk) CK(cudaEventRecordWithFlags(ctx.ev[evi++], st, cudaEventRecordExternal));
-      a.mode = kModeUpdate;
-      CKI(launch_plan(pl, a, st));
-      ctx.launches += 2;
-      ctx.hv_launches++;
-      if (tk) CK(cudaEventRecordWithFlags(ctx.ev[4 + 4 * j], st, cudaEventRecordExternal));
-      continue;
     }
-    if (pl.gen_vm && pl.gvm_cube) {  // the cube gather writes w' over q_{j-1} and sets alpha_j, p_j
-      LaunchArgs g = a;  // x = q_j, y = q_{j-1}, u
-      g.mode = kModeApply;
-      g.fused_step = 1;
+    if (pl.storedV || fused_step || (pl.gen_vm && pl.gvm_cube)) {
       if (tk) CK(cudaEventRecordWithFlags(ctx.ev[evi++], st, cudaEventRecordExternal));
-      CKI(launch_plan(pl, g, st));
-      if (tk) CK(cudaEventRecordWithFlags(ctx.ev[evi++], st, cudaEventRecordExternal));
-      a.mode = kModeUpdate;
-      CKI(launch_plan(pl, a, st));
+      CKI(stream(kModeUpdate, a.inst, j));
       ctx.launches += 2;
       ctx.hv_launches++;
       if (tk) CK(cudaEventRecordWithFlags(ctx.ev[4 + 4 * j], st, cudaEventRecordExternal));
@@ -1058,7 +1130,8 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
       if (tk) CK(cudaEventRecordWithFlags(ctx.ev[evi++], st, cudaEventRecordExternal));
     }
     a.mode = kModeUpdate;
-    CKI(launch_plan(pl, a, st));
+    if (vmaj) CKI(stream(kModeUpdate, a.inst, j));
+    else CKI(launch_plan(pl, a, st));
     ctx.launches += 2;
     ctx.hv_launches++;
     if (p->reorth) {  // two Gram-Schmidt passes against q_0..q_j, then the norm of what is left
@@ -1120,6 +1193,13 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
     t.x = A;
     t.y = U;
     e.hq = o.hq = Hq;
+    if (pl.storedV) {
+      bool ok = false;  // (built by run_impl before the capture)
+      ftlm_status rs = ensure_stored(s, c64, st, e.stored, ok);
+      if (rs != FTLM_OK) return rs;
+      if (!ok) return fail(FTLM_ERR_CUDA, "stored rows are missing");
+      o.stored = e.stored;
+    }
     InstDesc ge = d, go = d;
     ge.x = A;
     ge.y = Hq;
@@ -1135,6 +1215,28 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
   CK(cudaMemcpy(c.desc.p, h.data(), sizeof(InstDesc) * h.size(), cudaMemcpyHostToDevice));
   std::vector<int> tiles = pl.tile_start;  // the instances' tile list, then the H.v groups' (vector-major general)
   tiles.insert(tiles.end(), pl.tile_start_g.begin(), pl.tile_start_g.end());
+  if (vmaj) {  // then the streaming passes' list by vector and the stored-row groups' list
+    c.even = true;
+    auto list = [&](int step, long long rows, int& at, int& most, int& grid) -> bool {
+      at = (int)tiles.size();
+      tiles.push_back(0);
+      for (int k = 0; k < nd; k += step) {
+        const long long t = ((long long)sys[k / R]->hs.dim + rows - 1) / rows;
+        if (tiles.back() + t > (1ll << 30)) return false;
+        tiles.push_back(tiles.back() + (int)t);
+        most = std::max(most, (int)t);
+        c.even = c.even && sys[k / R]->hs.dim % 2 == 0;
+      }
+      grid = tiles.back();
+      return true;
+    };
+    if (!list(1, kStreamChunk, c.stream_at, c.stream_tiles, c.stream_grid) ||
+        (pl.storedV && !list(pl.storedV, 32, c.stored_at, c.stored_tiles, c.stored_grid)))
+      return fail(FTLM_ERR_UNSUPPORTED, "too many tiles");
+    const size_t cnt = ((size_t)nd * 4 + 255) & ~size_t(255);
+    CK(c.vslots.ensure(cnt + sizeof(double) * 3 * (size_t)nd * std::max(c.stream_tiles, c.stored_tiles)));
+    CK(cudaMemset(c.vslots.p, 0, cnt));
+  }
   CK(c.tiles.ensure(sizeof(int) * tiles.size()));
   CK(cudaMemcpy(c.tiles.p, tiles.data(), sizeof(int) * tiles.size(), cudaMemcpyHostToDevice));
   CK(c.partials.ensure(sizeof(double) * (size_t)n * plan_max_grid(pl) * R * kNumPartials));  // n_inst x R = R x 1 when vector-major
@@ -1256,11 +1358,28 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     ftlm_status rs = make_rot(sys[0], R, c64, pl.rot, st);
     if (rs != FTLM_OK) return rs;
   }
-  if (vm_fused_step(pl) && !pl.rot.on) {
+  bool forced = false;
+  for (auto* s : sys) forced = forced || has_shape_override(s, R, c64);
+  if (plan_vmaj(pl) && !pl.rot.on && !forced) {  // small systems: stored rows in the gathers' place
+    bool all = true;
+    uint64_t rows = 0;
+    for (auto* s : sys) {
+      StoredRows r;
+      bool ok = false;
+      ftlm_status rs = ensure_stored(s, c64, st, r, ok);
+      if (rs != FTLM_OK) return rs;
+      all = all && ok;
+      rows += s->hs.dim;
+    }
+    if (all) pl.storedV = stored_group(rows, R, true);
+  }
+  if (vm_fused_step(pl) && !pl.rot.on && !pl.storedV) {
     ftlm_status ut = ensure_unit_tables(sys[0], pl.half.K, c64, st);
     if (ut != FTLM_OK) return ut;
   }
-  if (pl.half.on && !vm_fused_step(pl)) {  // (the fused vector-major step keeps no H q block)
+  if (pl.storedV) {
+    // (no H q block)
+  } else if (pl.half.on && !vm_fused_step(pl)) {  // (the fused vector-major step keeps no H q block)
     ftlm_status hs_ = ensure_hq(sys[0], R, c64, (pl.half.vm && !pl.half.hybrid) ? pl.half.passes : 1);
     if (hs_ != FTLM_OK) return hs_;
   } else if (pl.wideV || (pl.gen_vm && !pl.gvm_cube)) {  // (the cube gather keeps no H q block)
@@ -1400,6 +1519,12 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
   {
     std::lock_guard<std::mutex> lk(g_mu);
     if (g_shapes.count(key)) return FTLM_OK;
+  }
+  {  // stored rows have no shape to choose, and every gather is slower on systems that small
+    StoredRows r;
+    bool ok = false;
+    ftlm_status rs = ensure_stored(s, c64, st, r, ok);
+    if (rs != FTLM_OK || ok) return rs;
   }
   std::vector<Shape> cands;
   if (s->hs.all_half && s->hs.n >= 4) {
@@ -1583,6 +1708,21 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   if (v != FTLM_OK) return v;
   const int c64 = dtype == FTLM_C64;
   ftlm_system* s = const_cast<ftlm_system*>(cs);
+  if (!has_shape_override(s, nvec, c64)) {  // small systems: stored rows
+    StoredArgs a;
+    bool ok = false;
+    ftlm_status rs = ensure_stored(s, c64, pick_stream(s, stream), a.rows, ok);
+    if (rs != FTLM_OK) return rs;
+    if (ok) {
+      a.x = x;
+      a.y = y;
+      a.dim = (long long)s->hs.dim;
+      a.rs = a.R = nvec;
+      a.vs = 1;
+      CKI(launch_stored_product(a, stored_group(s->hs.dim, nvec, false), c64, pick_stream(s, stream)));
+      return FTLM_OK;
+    }
+  }
   Plan pl;
   std::vector<ftlm_system*> one{s};
   if (nvec > 1 && !has_shape_override(s, nvec, c64)) {
@@ -1773,11 +1913,13 @@ void ftlm_system_destroy(ftlm_system* s) {
   cudaDeviceSynchronize();  // the system's buffers may be in use on any stream
   purge_ctx_of(s->id);
   for (DevBuf* b : {&s->tab_f, &s->tab_d, &s->stride, &s->q, &s->A, &s->B, &s->U, &s->scal, &s->ep, &s->ecnt,
-                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart})
+                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart, &s->rows[0], &s->rows[1]})
     b->release();
   cudaEventDestroy(s->ev_in);
   cudaEventDestroy(s->ev_out);
   cudaEventDestroy(s->ev_apply);
+  for (cudaEvent_t e : s->ev_rows)
+    if (e) cudaEventDestroy(e);
   cudaStreamDestroy(s->own_stream);
   delete s;
 }

@@ -457,6 +457,60 @@ __device__ inline void finalize_beta(const DevScalars& sc, int j, int r, int M, 
   sc.sigma[(size_t)(j + 1) * sc.ss + r] = sig;
 }
 
+// The scalars of a start vector from nrm2 = |q_0|^2.
+__device__ inline void finalize_start(const DevScalars& sc, int r, int M, double nrm2) {
+  const double nrm = sqrt(fmax(nrm2, 0.0));
+  sc.sigma[r] = nrm > 0.0 ? 1.0 / nrm : 0.0;
+  sc.scale[r] = 0.0;
+  sc.active[r] = nrm > 0.0 ? 1 : 0;
+  sc.meff[r] = nrm > 0.0 ? M : 0;
+}
+
+// The CTA's sums p[0..NP) into its slot, then the last CTA of the vector adds
+// the vector's slots in a fixed order: true (in thread 0, with the totals in p)
+// for that CTA.
+template <int NT, int NP>
+__device__ __forceinline__ bool vector_total(double (&p)[NP], double* slots, int tile, int tiles, unsigned* counter) {
+  __shared__ double red[NT / 32][NP];
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto cta_sum = [&]() {
+#pragma unroll
+    for (int c = 0; c < NP; ++c)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) p[c] += __shfl_xor_sync(0xffffffffu, p[c], o);
+    if (lane == 0)
+#pragma unroll
+      for (int c = 0; c < NP; ++c) red[warp][c] = p[c];
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int c = 0; c < NP; ++c) {
+        double s = 0.0;
+        for (int w = 0; w < NT / 32; ++w) s += red[w][c];
+        p[c] = s;
+      }
+  };
+  cta_sum();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int c = 0; c < NP; ++c) slots[(size_t)tile * 3 + c] = p[c];
+    __threadfence();
+    last = atomicAdd(counter, 1u) == (unsigned)(tiles - 1);
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+#pragma unroll
+  for (int c = 0; c < NP; ++c) p[c] = 0.0;
+  for (int k = threadIdx.x; k < tiles; k += NT)
+#pragma unroll
+    for (int c = 0; c < NP; ++c) p[c] += __ldcg(slots + (size_t)k * 3 + c);
+  cta_sum();
+  if (threadIdx.x == 0) *counter = 0u;
+  return threadIdx.x == 0;
+}
+
 __device__ inline void finalize(const LaunchArgs& a, const InstDesc* inst_all) {
   // (inst_all points at the device array, or at the inline descriptor)
   const int R = a.R;
@@ -484,11 +538,7 @@ __device__ inline void finalize(const LaunchArgs& a, const InstDesc* inst_all) {
       }
       finalize_beta(sc, j, r, d.M, d.tol, total_partial(a, inst, r, 0));
     } else if (a.mode == kModeStartNorm) {
-      const double nrm = sqrt(fmax(total_partial(a, inst, r, 0), 0.0));
-      sc.sigma[r] = nrm > 0.0 ? 1.0 / nrm : 0.0;
-      sc.scale[r] = 0.0;
-      sc.active[r] = nrm > 0.0 ? 1 : 0;
-      sc.meff[r] = nrm > 0.0 ? d.M : 0;
+      finalize_start(sc, r, d.M, total_partial(a, inst, r, 0));
     }
   }
 }

@@ -83,6 +83,14 @@ struct DevScalars {
   int* meff = nullptr;       // [R]
 };
 
+// The stored rows of a small system (hv_stored.cu): row mu's entries at mu * S.
+struct StoredRows {
+  const int* col = nullptr;
+  const void* val = nullptr;  // complex
+  const int* cnt = nullptr;   // entries of each row
+  long long S = 0;
+};
+
 struct InstDesc {
   const void* tab = nullptr;       // table scalars (float or double)
   const long long* stride = nullptr;  // [n]
@@ -100,6 +108,7 @@ struct InstDesc {
   double tol = 0.0;          // breakdown tolerance
   int M = 0;
   double obs[3] = {0, 0, 0}; // observable u.S: u_z, Re a_u, Im a_u with a_u = (u_x - i u_y)/2
+  StoredRows stored;         // when the run's systems have them
 };
 
 enum KernelMode : int {
@@ -252,7 +261,7 @@ int vm_max_ctas_per_sm(int K, int min_blocks, int c64, int threads, size_t smem,
 int vm_unit_table_stride(int n, int K);
 int launch_vm_unit_tables(const double* tab_d, const TabLayout& L, int n, int K, long long nunits, void* out, int c64,
                           void* stream);
-// kModeStep / kModeStartNorm over the same one-vector instances (256 threads)
+// kModeStep over the same one-vector instances (256 threads)
 int launch_vm_stream(const LaunchArgs& a, int c64, int grid, void* stream);
 constexpr int kVmLaneBits = 5;  // rows per warp-wide load: 2^5
 
@@ -309,6 +318,40 @@ int prepare_rot(int n, int c64);
 int launch_rot(const RotArgs& a, int pass, int c64, void* stream);  // pass 0 forward, 1 middle, 2 backward
 int launch_rot_table(const RotForm& f, void* out, int c64, void* stream);
 int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream);
+
+// Stored rows and streaming passes (hv_stored.cu).
+constexpr int kStoredMaxSites = 32;
+constexpr int kStreamChunk = 4096;  // elements of a streaming pass's CTA
+
+struct StoredArgs {
+  // a Lanczos step: groups of V one-vector instances, CTAs by the groups' tile list
+  const InstDesc* inst = nullptr;
+  const int* tile_start = nullptr;  // [groups + 1], tiles of 32 rows
+  int groups = 0, max_tiles = 0;
+  int j = 0;
+  double* slots = nullptr;          // [vectors][max_tiles][3]
+  unsigned* counters = nullptr;     // [groups], zero between launches
+  // a product y = H x: element (row, v) at row * rs + v * vs
+  StoredRows rows;
+  const void* x = nullptr;
+  void* y = nullptr;
+  long long dim = 0, rs = 1, vs = 0;
+  int R = 0;
+};
+struct StreamArgs {
+  const InstDesc* inst = nullptr;   // one a vector
+  const int* tile_start = nullptr;  // [vectors + 1], tiles of kStreamChunk elements
+  int vectors = 0, max_tiles = 0;
+  int j = 0;
+  double* slots = nullptr;          // [vectors][max_tiles][3]
+  unsigned* counters = nullptr;     // [vectors], zero between launches
+};
+int stored_row_bound(const HostSystem& hs);
+int launch_stored_build(const void* tab, const TabLayout& L, const long long* stride, const int* q, int n, int dim,
+                        int S, int* col, void* val, int* cnt, int c64, void* stream);
+int launch_stored_step(const StoredArgs& a, int V, int c64, int grid, void* stream);
+int launch_stored_product(const StoredArgs& a, int V, int c64, void* stream);
+int launch_stream_vectors(const StreamArgs& a, int mode, int c64, bool even, int grid, void* stream);
 
 // y = c (u.S) x (sdir.cu): R vectors, c = sigma[vector] (null: 1).
 struct SdirArgs {

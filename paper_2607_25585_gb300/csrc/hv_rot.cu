@@ -149,51 +149,6 @@ __device__ __forceinline__ void mid_group(v2* buf, real t, int mask) {
   __syncthreads();
 }
 
-// The CTA's sums p[0..NP) into its slot, then the last CTA of the vector adds
-// the vector's slots in a fixed order: true (in thread 0, with the totals in p)
-// for that CTA.
-template <int NT, int NP>
-__device__ __forceinline__ bool vector_total(double (&p)[NP], double* slots, int tile, int tiles, unsigned* counter) {
-  __shared__ double red[NT / 32][NP];
-  __shared__ int last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto cta_sum = [&]() {
-#pragma unroll
-    for (int c = 0; c < NP; ++c)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) p[c] += __shfl_xor_sync(0xffffffffu, p[c], o);
-    if (lane == 0)
-#pragma unroll
-      for (int c = 0; c < NP; ++c) red[warp][c] = p[c];
-    __syncthreads();
-    if (threadIdx.x == 0)
-#pragma unroll
-      for (int c = 0; c < NP; ++c) {
-        double s = 0.0;
-        for (int w = 0; w < NT / 32; ++w) s += red[w][c];
-        p[c] = s;
-      }
-  };
-  cta_sum();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int c = 0; c < NP; ++c) slots[(size_t)tile * 3 + c] = p[c];
-    __threadfence();
-    last = atomicAdd(counter, 1u) == (unsigned)(tiles - 1);
-  }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-#pragma unroll
-  for (int c = 0; c < NP; ++c) p[c] = 0.0;
-  for (int k = threadIdx.x; k < tiles; k += NT)
-#pragma unroll
-    for (int c = 0; c < NP; ++c) p[c] += __ldcg(slots + (size_t)k * 3 + c);
-  cta_sum();
-  if (threadIdx.x == 0) *counter = 0u;
-  return threadIdx.x == 0;
-}
-
 // e^{-i phi_k downs} by the number of up spins, [K][kRotMaxN + 1], to shared memory
 template <typename real>
 __device__ __forceinline__ void stage_phases(typename Cx<real>::v2* ph, const RotArgs& a) {

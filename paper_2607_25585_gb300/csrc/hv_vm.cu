@@ -658,11 +658,11 @@ __global__ void __launch_bounds__(MINB == 1 ? 512 : 256, MINB) vm_kernel(const _
   if (threadIdx.x == 0) *a.counter = 0u;
 }
 
-// Streaming modes (kModeStep, kModeStartNorm) on the vector-major block: R
+// kModeStep on the vector-major block (after the multi-pass gathers): R
 // one-vector instances, tiles of a.rows_per_tile consecutive elements of one
 // vector (a.tiles_per_vg per vector); a thread moves 16 bytes per array and
 // item (two complex64 or one complex128 value).
-template <typename real, int MODE>
+template <typename real>
 __global__ void __launch_bounds__(256) vm_stream_kernel(const __grid_constant__ LaunchArgs a) {
   constexpr int V = sizeof(real) == 4 ? 2 : 1;
   __shared__ InstDesc d;
@@ -704,14 +704,10 @@ __global__ void __launch_bounds__(256) vm_stream_kernel(const __grid_constant__ 
       }
       __syncthreads();
       const int j = a.step;
-      real sg = 0, bs = 0, cf = 0;
-      if (MODE == kModeStep) {
-        sg = (real)d.sc.sigma[(size_t)j * d.sc.ss];
-        if (!a.first) bs = (real)(d.sc.beta[(size_t)(j - 1) * d.sc.ss] * d.sc.sigma[(size_t)(j - 1) * d.sc.ss]);
-        cf = (real)(d.sc.alpha[(size_t)j * d.sc.ss] * d.sc.sigma[(size_t)j * d.sc.ss]);
-      } else if (MODE == kModeUpdate) {  // the tail of the fused step: w = w' - alpha_j sigma_j q_j
-        cf = (real)(d.sc.alpha[(size_t)j * d.sc.ss] * d.sc.sigma[(size_t)j * d.sc.ss]);
-      }
+      const real sg = (real)d.sc.sigma[(size_t)j * d.sc.ss];
+      const real bs = a.first ? (real)0
+                              : (real)(d.sc.beta[(size_t)(j - 1) * d.sc.ss] * d.sc.sigma[(size_t)(j - 1) * d.sc.ss]);
+      const real cf = (real)(d.sc.alpha[(size_t)j * d.sc.ss] * d.sc.sigma[(size_t)j * d.sc.ss]);
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         sig[v] = sg;
@@ -727,17 +723,7 @@ __global__ void __launch_bounds__(256) vm_stream_kernel(const __grid_constant__ 
     for (int k = 0; k < V * kNumPartials; ++k) pacc[k] = 0;
     const long long step = (long long)bd * V;
     long long e = e0 + (long long)threadIdx.x * V;
-    if (MODE == kModeStep) {
-      step_stream<real, V, 4>(d, a, e, e_end, step, sig, bsp, coef, pacc);
-    } else if (MODE == kModeUpdate) {
-      update_stream<real, V, 4>(d, e, e_end, step, coef, pacc);
-    } else {
-      for (; e + step < e_end; e += 2 * step) {
-        elementwise_item<real, V, MODE>(d, a, e, sig, bsp, coef, pacc);
-        elementwise_item<real, V, MODE>(d, a, e + step, sig, bsp, coef, pacc);
-      }
-      if (e < e_end) elementwise_item<real, V, MODE>(d, a, e, sig, bsp, coef, pacc);
-    }
+    step_stream<real, V, 4>(d, a, e, e_end, step, sig, bsp, coef, pacc);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       real t = 0;
@@ -818,19 +804,9 @@ int launch_vm_unit_tables(const double* tab_d, const TabLayout& L, int n, int K,
 
 int launch_vm_stream(const LaunchArgs& a, int c64, int grid, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (a.inline_one || (a.rows_per_tile & 1)) return (int)cudaErrorInvalidValue;
-  if (a.mode == kModeStep) {
-    if (c64) vm_stream_kernel<float, kModeStep><<<grid, 256, 0, st>>>(a);
-    else vm_stream_kernel<double, kModeStep><<<grid, 256, 0, st>>>(a);
-  } else if (a.mode == kModeUpdate) {
-    if (c64) vm_stream_kernel<float, kModeUpdate><<<grid, 256, 0, st>>>(a);
-    else vm_stream_kernel<double, kModeUpdate><<<grid, 256, 0, st>>>(a);
-  } else if (a.mode == kModeStartNorm) {
-    if (c64) vm_stream_kernel<float, kModeStartNorm><<<grid, 256, 0, st>>>(a);
-    else vm_stream_kernel<double, kModeStartNorm><<<grid, 256, 0, st>>>(a);
-  } else {
-    return (int)cudaErrorInvalidValue;
-  }
+  if (a.inline_one || (a.rows_per_tile & 1) || a.mode != kModeStep) return (int)cudaErrorInvalidValue;
+  if (c64) vm_stream_kernel<float><<<grid, 256, 0, st>>>(a);
+  else vm_stream_kernel<double><<<grid, 256, 0, st>>>(a);
   return (int)cudaGetLastError();
 }
 

@@ -1,0 +1,94 @@
+"""GPU: products and steps of small systems from stored rows, against the oracle
+and the forced gathers: group sizes and remainders, rows that are no multiple of
+a CTA's 32, exact zeros, calls inside a stream capture.
+
+Tolerances: a row adds at most 200 products in two levels, so its relative
+error is below 30 units roundoff of the sum of magnitudes; the norms used here
+give 2e-6 in complex64 and 4e-15 in complex128 (1e-12 with the oracle's)."""
+import numpy as np
+import pytest
+from conftest import random_system
+
+import ftlm_workloads as W
+import oracle
+import paper_2607_25585_gb300 as F
+from gpu_helpers import empty_dev, osys, rel_l2, to_dev, torch_cuda
+
+pytestmark = pytest.mark.gpu
+TOL = {"c64": 2e-6, "c128": 1e-12}
+SYSTEMS = {
+    "one site": [4],
+    "two halves": [1, 1],
+    "mixed": [1, 2, 3, 5, 1, 2],
+    "halves": [1] * 11,
+    "ones": [2] * 6,
+    "large spins": [15, 7, 3],
+}
+
+
+@pytest.mark.parametrize("name", SYSTEMS)
+@pytest.mark.parametrize("R", [1, 2, 3, 4, 7, 8])
+def test_stored_product_matches_oracle(name, R, rng):
+    w = random_system(np.random.default_rng(5), SYSTEMS[name])
+    s = F.System.from_dict(w)
+    x = rng.normal(size=(s.dim, R)) + 1j * rng.normal(size=(s.dim, R))
+    for dtype in ("c64", "c128"):
+        xd = to_dev(x, dtype)
+        ref = oracle.apply_h(osys(w), xd.cpu().numpy().astype(np.complex128))
+        for _ in range(2):          # the call that writes the rows, and one that finds them
+            y = empty_dev((s.dim, R), dtype)
+            F.apply_h(s, xd, y, R, dtype)
+            assert rel_l2(y.cpu().numpy(), ref) < TOL[dtype]
+    s.close()
+
+
+def test_rows_that_are_not_connected_stay_zero():
+    J = np.zeros((10, 10))
+    J[0, 1] = J[1, 2] = 0.7
+    s = F.System([1] * 10, J=J, B=(0, 0, 0.4))
+    x = np.zeros((s.dim, 1))
+    x[1] = 1.0                      # one spin up: H keeps their number
+    y = empty_dev((s.dim, 1), "c64")
+    F.apply_h(s, to_dev(x, "c64"), y, 1, "c64")
+    got = y.cpu().numpy()[:, 0]
+    assert set(np.flatnonzero(got)) <= {1, 2} and got[2] != 0
+    s.close()
+
+
+@pytest.mark.parametrize("R", [1, 6, 8])
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+def test_stored_run_matches_forced_gather(R, dtype):
+    T = np.array([0.5, 5.0])
+    w = W.chain(7, Bdir=(0.3, -0.2, 0.9))           # d = 2187
+    s = F.System.from_dict(w)
+    a = F.run(s, R=R, M=10, T=T, seed=3, dtype=dtype)
+    F.tune_shape(s, R, dtype, 0, 0, 1, 1)           # the one-row vector-major gather
+    try:
+        b = F.run(s, R=R, M=10, T=T, seed=3, dtype=dtype)
+    finally:
+        F.tune_shape(s, R, dtype, -1)
+    for k in ("alpha", "beta", "p"):                # ten steps amplify rounding by less than 30
+        assert np.abs(a[k] - b[k]).max() < 30 * TOL[dtype] * max(np.abs(b[k]).max(), np.abs(b["beta"]).max() * (k == "alpha"))
+    s.close()
+
+
+def test_product_inside_a_capture():
+    torch = torch_cuda()
+    w = W.ring(N=5, two_s=2)
+    x = torch.randn(243, 4, dtype=torch.complex128, device="cuda")
+    ref = oracle.apply_h(osys(w), x.cpu().numpy())
+    for warm in (False, True):      # rows not written before the capture (the gather is captured), and written
+        s = F.System.from_dict(w)
+        y = torch.empty_like(x)
+        if warm:
+            F.apply_h(s, x, y, 4, "c128")
+            torch.cuda.synchronize()
+            F.apply_h(s, x, y, 4, "c128")
+            y.zero_()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            F.apply_h(s, x, y, 4, "c128")
+        g.replay()
+        torch.cuda.synchronize()
+        assert rel_l2(y.cpu().numpy(), ref) < 1e-12
+        s.close()
