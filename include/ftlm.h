@@ -308,8 +308,8 @@ ftlm_status ftlm_run_batch(int n, const ftlm_system* const* systems, const ftlm_
  * processes: gather alpha, beta, p, M_eff from all of them and call this
  * once.  Host-only: needs no GPU.  The R tridiagonal eigenproblems and the
  * temperatures are spread over up to min(R, hardware threads, 32) host
- * threads created and joined inside the call; the result does not depend on
- * their number (each sum runs in a fixed order).  ftlm_run, ftlm_run_batch
+ * threads created and joined inside the call (as many as the work pays for);
+ * the result does not depend on their number (each sum runs in a fixed order).  ftlm_run, ftlm_run_batch
  * and ftlm_sums_sym do the same for their host part.
  *  dim  Hilbert-space dimension d; g  g factor.
  */

@@ -1451,28 +1451,46 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     dev_ms = ms;
   }
   const size_t per = staged_bytes(R, M);
-  for (int k = 0; k < n; ++k) {  // host: eigensolve + sums per instance
+  struct HostPart {
+    std::vector<double> al, be, pp;  // [R][M], [R][M], [R][M][2]
+    std::vector<int> me;
+    ftlm_status status = FTLM_OK;
+    std::string msg;
+  };
+  std::vector<HostPart> host(n);
+  const bool hosted = parallel_for(n, n > 1 ? n * host_sums_ns(R, M, p->nT) : 0.0, [&](int k) {  // eigensolves and sums
+    HostPart& h = host[k];
     const char* src = ctx->pinned + per * k;
     const double* alpha_d = reinterpret_cast<const double*>(src);  // [M][R]
     const double* beta_d = alpha_d + (size_t)M * R;
     const double* p_d = beta_d + (size_t)M * R;                     // [M][R][2]
     const int* meff = reinterpret_cast<const int*>(src + sizeof(double) * staged_doubles(R, M));
-    std::vector<double> al((size_t)R * M), be((size_t)R * M), pp((size_t)R * M * 2);
+    h.al.resize((size_t)R * M);
+    h.be.resize((size_t)R * M);
+    h.pp.resize((size_t)R * M * 2);
     for (int r = 0; r < R; ++r)
       for (int j = 0; j < M; ++j) {
-        al[(size_t)r * M + j] = alpha_d[(size_t)j * R + r];
-        be[(size_t)r * M + j] = beta_d[(size_t)j * R + r];
-        pp[((size_t)r * M + j) * 2] = p_d[((size_t)j * R + r) * 2];
-        pp[((size_t)r * M + j) * 2 + 1] = p_d[((size_t)j * R + r) * 2 + 1];
+        h.al[(size_t)r * M + j] = alpha_d[(size_t)j * R + r];
+        h.be[(size_t)r * M + j] = beta_d[(size_t)j * R + r];
+        h.pp[((size_t)r * M + j) * 2] = p_d[((size_t)j * R + r) * 2];
+        h.pp[((size_t)r * M + j) * 2 + 1] = p_d[((size_t)j * R + r) * 2 + 1];
       }
-    std::vector<int> me(meff, meff + R);
+    h.me.assign(meff, meff + R);
     for (int r = 0; r < R; ++r)
-      if (me[r] < 1 || me[r] > M) return fail(FTLM_ERR_NUMERICAL, "start vector of zero norm");
+      if (h.me[r] < 1 || h.me[r] > M) {
+        h.status = FTLM_ERR_NUMERICAL;
+        h.msg = "start vector of zero norm";
+        return;
+      }
+    h.status = host_sums(R, M, h.me.data(), h.al.data(), h.be.data(), h.pp.data(), (double)sys[k]->hs.dim,
+                         sys[k]->hs.g, p->T, p->nT, &res[k], h.msg, n == 1);
+  });
+  if (!hosted) return fail(FTLM_ERR_OUT_OF_MEMORY, "out of host memory");
+  for (int k = 0; k < n; ++k) {
+    const std::vector<double>&al = host[k].al, &be = host[k].be, &pp = host[k].pp;
+    const std::vector<int>& me = host[k].me;
     ftlm_result& out = res[k];
-    std::string msg;
-    ftlm_status ss = host_sums(R, M, me.data(), al.data(), be.data(), pp.data(), (double)sys[k]->hs.dim,
-                               sys[k]->hs.g, p->T, p->nT, &out, msg);
-    if (ss != FTLM_OK) return fail(ss, msg);
+    if (host[k].status != FTLM_OK) return fail(host[k].status, host[k].msg);
     if (out.alpha) std::memcpy(out.alpha, al.data(), sizeof(double) * al.size());
     if (out.beta) std::memcpy(out.beta, be.data(), sizeof(double) * be.size());
     if (out.p) std::memcpy(out.p, pp.data(), sizeof(double) * pp.size());
@@ -1494,7 +1512,7 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     out.site_cube = pl.gen_vm ? pl.gvm_cube : 0;
     out.sym_ms = 0.0;
     if (p->symmetric) {  // Eqs. (E-2-G), (E-2-H)
-      const double* sigma_d = p_d + (size_t)M * R * 2;  // [M][R]
+      const double* sigma_d = reinterpret_cast<const double*>(ctx->pinned + per * k) + (size_t)M * R * 4;  // [M][R]
       std::vector<double> Omat;
       double sms = 0.0;
       ftlm_status os = symmetric_matrices(sys[k], p, st, sigma_d, Omat, sms);

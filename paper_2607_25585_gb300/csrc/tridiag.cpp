@@ -11,6 +11,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <limits>
 #include <thread>
 #include <vector>
@@ -29,27 +30,10 @@ inline double norm2(double a, double b) {
   return std::hypot(a, b);
 }
 
-// fn(i) for i in [0, n) on up to hardware_concurrency host threads (the
-// caller's thread works too); each i runs exactly once
-template <typename Fn>
-void parallel_for(int n, Fn&& fn) {
-  const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
-  const int nth = std::min(std::min(n, hw), 32);
-  std::atomic<int> next{0};
-  auto work = [&]() {
-    for (int i; (i = next.fetch_add(1)) < n;) fn(i);
-  };
-  std::vector<std::thread> pool;
-  for (int k = 1; k < nth; ++k) {
-    try {
-      pool.emplace_back(work);
-    } catch (...) {
-      break;  // fewer threads: the others take the remaining items
-    }
-  }
-  work();
-  for (auto& t : pool) t.join();
-}
+// Estimated cost of one run's eigenproblem with `rows` rotated rows, and of one
+// (temperature, Ritz value) term of the sums, in nanoseconds.
+double ql_ns(int m, int rows) { return 1.7 * m * m * (20.0 + 2.0 * rows); }
+constexpr double kTermNs = 12.0;
 
 // Eigenvalues of tridiag(d, e) (d[0..m-1], e[0..m-2] off-diagonal) with the
 // rotations applied to the rows z[k][0..m-1], k < nz.  Returns false if the
@@ -109,8 +93,38 @@ bool ql_implicit(int m, double* d, double* e_in, int nz, double** z) {
 
 }  // namespace
 
+// fn(i) for i in [0, n), each exactly once, on the caller's thread and as many
+// others as the work pays for: starting and joining a thread costs some 20 us,
+// so each gets at least 50 us of `total_ns` (with one thread an item, ten
+// eigenproblems of 24 rows, 0.2 ms in all, took 1.5 ms).
+// false: an item threw (out of memory).
+bool parallel_for(int n, double total_ns, const std::function<void(int)>& fn) {
+  const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
+  const int nth = std::min({n, hw, 32, 1 + (int)std::min(1e6, total_ns / 50e3)});
+  std::atomic<int> next{0};
+  std::atomic<bool> ok{true};
+  auto work = [&]() {
+    try {
+      for (int i; (i = next.fetch_add(1)) < n;) fn(i);
+    } catch (...) {
+      ok = false;
+    }
+  };
+  std::vector<std::thread> pool;
+  try {
+    for (int k = 1; k < nth; ++k) pool.emplace_back(work);
+  } catch (...) {  // fewer threads: the others take the remaining items
+  }
+  work();
+  for (auto& t : pool) t.join();
+  return ok;
+}
+
+double host_sums_ns(int R, int M, int nT) { return R * (ql_ns(M, 3) + kTermNs * M * nT); }
+
 ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const double* beta, const double* p,
-                      double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg) {
+                      double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg, bool threads) {
+  const char* memory = "out of host memory";
   if (R < 1 || M < 1 || !M_eff || !alpha || !beta || !p || !T || nT < 1 || !res || !(dim > 0)) {
     msg = "ftlm_sums: invalid arguments";
     return FTLM_ERR_INVALID_ARG;
@@ -131,7 +145,7 @@ ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const
     }
   // the runs' eigenproblems are independent: one per host thread
   std::vector<int> bad(R, 0);  // 1: non-finite coefficient, 2: no convergence
-  parallel_for(R, [&](int r) {
+  const bool solved = parallel_for(R, threads ? R * ql_ns(M, 3) : 0.0, [&](int r) {
     const int m = M_eff[r];
     Run& run = runs[r];
     run.eps.assign(alpha + (size_t)r * M, alpha + (size_t)r * M + m);
@@ -153,6 +167,7 @@ ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const
     double* rows[3] = {run.w0.data(), run.qr.data(), run.qi.data()};
     if (!ql_implicit(m, run.eps.data(), e.data(), 3, rows)) bad[r] = 2;
   });
+  if (!solved) return msg = memory, FTLM_ERR_OUT_OF_MEMORY;
   double E0 = std::numeric_limits<double>::infinity();
   for (int r = 0; r < R; ++r) {
     if (bad[r] == 1) {
@@ -167,13 +182,16 @@ ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const
   }
   res->E0 = E0;
   // the temperatures are independent too (each sums the runs in order)
-  parallel_for(nT, [&](int t) {
+  const bool summed = parallel_for(nT, threads ? kTermNs * nT * R * M : 0.0, [&](int t) {
     const double b = 1.0 / T[t];
     double z = 0.0, e1 = 0.0, orr = 0.0, oi = 0.0;
+    std::vector<double> ws;  // the weights, for the variance
+    ws.reserve((size_t)R * M);
     for (const Run& run : runs)
       for (size_t n = 0; n < run.eps.size(); ++n) {
         const double boltz = std::exp(-b * (run.eps[n] - E0));
         const double w = run.w0[n] * run.w0[n] * boltz;
+        ws.push_back(w);
         z += w;
         e1 += w * run.eps[n];
         orr += boltz * run.w0[n] * run.qr[n];
@@ -181,17 +199,16 @@ ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const
       }
     const double Em = e1 / z;
     double var = 0.0;
+    const double* w = ws.data();
     for (const Run& run : runs)
-      for (size_t n = 0; n < run.eps.size(); ++n) {
-        const double w = run.w0[n] * run.w0[n] * std::exp(-b * (run.eps[n] - E0));
-        var += w * (run.eps[n] - Em) * (run.eps[n] - Em);
-      }
+      for (size_t n = 0; n < run.eps.size(); ++n) var += *w++ * (run.eps[n] - Em) * (run.eps[n] - Em);
     if (res->lnZ) res->lnZ[t] = std::log(dim / R * z) - b * E0;
     if (res->E) res->E[t] = Em;
     if (res->C) res->C[t] = b * b * var / z;
     if (res->M_B) res->M_B[t] = -g * orr / z;
     if (res->M_B_imag) res->M_B_imag[t] = -g * oi / z;
   });
+  if (!summed) return msg = memory, FTLM_ERR_OUT_OF_MEMORY;
   return FTLM_OK;
 }
 
@@ -220,7 +237,7 @@ ftlm_status host_sums_sym(int R, int M, const int* M_eff, const double* alpha, c
       return FTLM_ERR_INVALID_ARG;
     }
   std::vector<int> bad(R, 0);
-  parallel_for(R, [&](int r) {
+  const bool solved = parallel_for(R, R * ql_ns(M, M), [&](int r) {
     Run& run = runs[r];
     const int m = run.m = M_eff[r];
     run.eps.assign(alpha + (size_t)r * M, alpha + (size_t)r * M + m);
@@ -234,6 +251,7 @@ ftlm_status host_sums_sym(int R, int M, const int* M_eff, const double* alpha, c
     }
     if (!ql_implicit(m, run.eps.data(), e.data(), m, rows.data())) bad[r] = 1;
   });
+  if (!solved) return msg = "out of host memory", FTLM_ERR_OUT_OF_MEMORY;
   double E0 = std::numeric_limits<double>::infinity();
   for (int r = 0; r < R; ++r) {
     if (bad[r]) {
@@ -242,7 +260,7 @@ ftlm_status host_sums_sym(int R, int M, const int* M_eff, const double* alpha, c
     }
     for (double v : runs[r].eps) E0 = std::min(E0, v);
   }
-  parallel_for(nT, [&](int t) {
+  const bool summed = parallel_for(nT, 3.0 * nT * R * M * M, [&](int t) {
     const double b = 1.0 / T[t];
     double den = 0.0, nre = 0.0, nim = 0.0;
     for (int r = 0; r < R; ++r) {
@@ -270,6 +288,7 @@ ftlm_status host_sums_sym(int R, int M, const int* M_eff, const double* alpha, c
     MB_sym[t] = -g * nre / den;
     if (MB_sym_imag) MB_sym_imag[t] = -g * nim / den;
   });
+  if (!summed) return msg = "out of host memory", FTLM_ERR_OUT_OF_MEMORY;
   return FTLM_OK;
 }
 
