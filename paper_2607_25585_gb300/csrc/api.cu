@@ -87,11 +87,11 @@ struct ftlm_system {
   DevBuf Ws;             // symmetric runs: u.S of the stored vectors (when it fits)
   DevBuf Gre;            // re-orthogonalised runs: <q_k|w_r> coefficients [R][M] complex
   DevBuf Ta, Tb;         // ftlm_apply_h on spin-1/2 blocks: x and H x in the vector-major layout
+  DevBuf Tw, Ts;         // its rotated-basis blocks and the vectors' statistics
   DevBuf ut[2];          // per-unit coefficient tables of the one-pass vector-major gather, [c64]
   int ut_K[2] = {0, 0};  // the cube size each was built for
   cudaEvent_t ev_apply = nullptr;  // recorded after the last use of Ta, Tb
-  int rot_state = 0;     // rotated-basis H.v: 0 not examined, 1 `rot` holds the directions, -1 none
-  std::unique_ptr<RotDirs> rot;
+  std::unique_ptr<RotDirs> rot;  // the rotated-basis H.v's directions, if the system has any
   DevBuf rD[2];          // its diagonal tables [K + 1][dim] and phases, [c64]
   DevBuf rW, rpart;      // its intermediate blocks; partial sums and arrival counters
   DevBuf rows[2];        // stored rows of a small system, [c64]: values, columns, counts
@@ -99,6 +99,7 @@ struct ftlm_system {
   bool rows_done[2] = {false, false};           // that event has been seen complete
   std::mutex rows_mu;
   bool apply_used = false;
+  std::mutex apply_mu;   // the blocks, event and tables that products use; a run holds it only to look at them
   std::mutex mu;
 };
 
@@ -608,65 +609,68 @@ ftlm_status ensure_unit_tables(ftlm_system* s, int K, int c64, cudaStream_t st) 
 
 size_t rot_phase_bytes(int c64) { return (size_t)kRotMaxK * (kRotMaxN + 1) * (c64 ? 8 : 16); }
 
-// Its directions, when the system has them and a tile fits its site count.
-const RotDirs* rot_dirs(ftlm_system* s, int c64) {
-  if (s->rot_state == 0) {
-    s->rot = std::make_unique<RotDirs>();
-    s->rot_state = rot_directions(s->hs, *s->rot) ? 1 : -1;
-    if (s->rot_state < 0) s->rot.reset();
-  }
-  return s->rot_state > 0 && rot_tile_bits(s->hs.n, c64) > 0 ? s->rot.get() : nullptr;
-}
-
-// Tables (built once per system and precision), W blocks and the partial sums of
-// R vectors; ok = false when they do not fit in memory (the gather then runs).
-ftlm_status ensure_rot(ftlm_system* s, const RotPlan& rp, int R, int c64, cudaStream_t st, bool& ok) {
+// Its tables, built once per system and precision on stream st; ok = false when
+// they do not fit in memory (the gather then runs).
+ftlm_status ensure_rot_tables(ftlm_system* s, const RotPlan& rp, int c64, cudaStream_t st, bool& ok) {
   ok = false;
   const size_t d = (size_t)s->hs.dim, real = c64 ? 4 : 8;
-  const RotDirs& dirs = *s->rot;
   DevBuf& D = s->rD[c64 ? 1 : 0];
   if (prepare_rot(s->hs.n, c64) != 0) return FTLM_OK;
-  const size_t tiles = d >> rp.T;
-  const size_t tbytes = (size_t)(rp.K + 1) * d * real + rot_phase_bytes(c64);
-  bool fits = true, build = !D.p;
-  auto grow = [&](DevBuf& b, size_t bytes) {
-    if (!fits || b.bytes >= bytes) return;
-    s->gen++;  // captured graphs hold its address
-    fits = b.ensure(bytes) == cudaSuccess;
-  };
-  grow(s->rW, (size_t)rp.group * rp.K * d * real * 2);
-  grow(s->rpart, sizeof(double) * 3 * tiles * R + sizeof(unsigned) * R);
-  grow(D, tbytes);
-  if (!fits) {
-    cudaGetLastError();
-    for (DevBuf* b : {&s->rW, &s->rpart, &s->rD[0], &s->rD[1]}) b->release();
-    return FTLM_OK;
-  }
-  if (build) {
+  if (!D.p) {
+    const size_t bytes = (size_t)(rp.K + 1) * d * real + rot_phase_bytes(c64);
+    if (D.ensure(bytes) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
     for (int k = 0; k <= rp.K; ++k) {
-      RotForm f = dirs.form[k];
+      RotForm f = s->rot->form[k];
       f.T = k > 0 ? rp.T : 0;
       f.b = rot_run_bits(s->hs.n, c64);
       CKI(launch_rot_table(f, static_cast<char*>(D.p) + (size_t)k * d * real, c64, st));
     }
-    CKI(launch_rot_phases(s->hs.n, dirs, static_cast<char*>(D.p) + tbytes - rot_phase_bytes(c64), c64, st));
+    CKI(launch_rot_phases(s->hs.n, *s->rot, static_cast<char*>(D.p) + bytes - rot_phase_bytes(c64), c64, st));
   }
   ok = true;
   return FTLM_OK;
 }
 
-// The rotated-basis plan of a block of R vectors (on = false: none).  The W
-// blocks hold K times the group's vectors: 16 GB of them keep every group large
-// enough to fill the device.
-ftlm_status make_rot(ftlm_system* s, int R, int c64, RotPlan& rp, cudaStream_t st) {
+// The tables, W blocks and partial sums of a run over R vectors.
+ftlm_status ensure_rot(ftlm_system* s, const RotPlan& rp, int R, int c64, cudaStream_t st, bool& ok) {
+  ok = false;
+  const size_t d = (size_t)s->hs.dim;
+  bool fits = true;
+  auto grow = [&](DevBuf& b, size_t bytes) {
+    if (!fits || b.bytes >= bytes) return;
+    s->gen++;  // captured graphs hold its address
+    fits = b.ensure(bytes) == cudaSuccess;
+  };
+  grow(s->rW, (size_t)rp.group * rp.K * d * (c64 ? 8 : 16));
+  grow(s->rpart, sizeof(double) * 3 * (d >> rp.T) * R + sizeof(unsigned) * R);
+  if (fits) {
+    std::lock_guard<std::mutex> lk(s->apply_mu);
+    ftlm_status ts = ensure_rot_tables(s, rp, c64, st, ok);
+    if (ts != FTLM_OK) return ts;
+  }
+  if (!ok) {
+    cudaGetLastError();
+    s->rW.release();
+    s->rpart.release();
+  }
+  return FTLM_OK;
+}
+
+// The rotated-basis plan of a block of R vectors (false: the system has none).
+// The W blocks hold K times the group's vectors: 16 GB of them keep every group
+// large enough to fill the device.
+bool rot_shape(ftlm_system* s, int R, int c64, RotPlan& rp) {
   rp = RotPlan();
-  const RotDirs* dirs = rot_dirs(s, c64);
-  if (!dirs) return FTLM_OK;
   rp.T = rot_tile_bits(s->hs.n, c64);
-  rp.K = dirs->K;
+  if (!s->rot || !rp.T) return false;
+  rp.K = s->rot->K;
   const uint64_t per = s->hs.dim * (uint64_t)rp.K * (c64 ? 8 : 16);
   rp.group = (int)std::min<uint64_t>((uint64_t)R, std::max<uint64_t>(1, (16ull << 30) / per));
-  return ensure_rot(s, rp, R, c64, st, rp.on);
+  return true;
+}
+
+ftlm_status make_rot(ftlm_system* s, int R, int c64, RotPlan& rp, cudaStream_t st) {
+  return rot_shape(s, R, c64, rp) ? ensure_rot(s, rp, R, c64, st, rp.on) : FTLM_OK;
 }
 
 RotArgs rot_args(const ftlm_system* s, const RotPlan& rp, int c64) {
@@ -683,6 +687,14 @@ RotArgs rot_args(const ftlm_system* s, const RotPlan& rp, int c64) {
   a.D = D + d * real;
   a.phases = D + (size_t)(rp.K + 1) * d * real;
   return a;
+}
+
+// Work enqueued on the stream is being captured (or may not be asked now).
+bool stream_captures(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool yes = cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return yes;
 }
 
 // ---- stored rows of small systems -----------------------------------------------
@@ -703,9 +715,7 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, cudaStream_t st, StoredRows& 
   std::lock_guard<std::mutex> lk(s->rows_mu);
   DevBuf& b = s->rows[k];
   if (!s->rows_done[k]) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
-      return cudaGetLastError(), FTLM_OK;
+    if (stream_captures(st)) return FTLM_OK;
     if (!b.p) {
       if (!s->ev_rows[k]) CK(cudaEventCreateWithFlags(&s->ev_rows[k], cudaEventDisableTiming));
       if (b.ensure(d * S * (esz + 4) + d * 4) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
@@ -921,7 +931,6 @@ size_t staged_bytes(int R, int M) { return sizeof(double) * staged_doubles(R, M)
 ftlm_status enqueue_rot_passes(RunCtx* ctx, ftlm_system* s, const RotPlan& rp, RotArgs a, int R, int c64, void* keep,
                                cudaStream_t st) {
   const size_t vb = (size_t)s->hs.dim * (c64 ? 8 : 16);
-  a.W = s->rW.p;
   for (int v0 = 0; v0 < R; v0 += rp.group) {
     a.vec0 = a.vecW = v0;
     a.nvec = std::min(rp.group, R - v0);
@@ -950,6 +959,7 @@ ftlm_status enqueue_rot_steps(RunCtx& ctx, ftlm_system* s, const ftlm_run_params
   a.tol = p->breakdown_tol > 0 ? p->breakdown_tol : (c64 ? 1e-6 : 1e-12);
   a.sc = scalars_at(s->scal.p, R, M);
   a.u = s->U.p;
+  a.W = s->rW.p;
   a.partials = reinterpret_cast<double*>(s->rpart.p);
   a.counters = reinterpret_cast<unsigned*>(a.partials + 3 * (d >> pl.rot.T) * R);
   a.lanczos = 1;
@@ -1428,6 +1438,10 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     if (g_ctx.size() > 8) g_ctx.erase(g_ctx.begin());
   }
   const auto t0 = std::chrono::steady_clock::now();
+  for (auto* s : sys) {  // after products of the systems still in flight (they may be writing the tables)
+    std::lock_guard<std::mutex> lk(s->apply_mu);
+    if (s->apply_used) CK(cudaStreamWaitEvent(st, s->ev_apply, 0));
+  }
   CK(cudaEventRecord(sys[0]->ev_in, caller));  // after the caller's prior work (e.g. a user start block)
   CK(cudaStreamWaitEvent(st, sys[0]->ev_in, 0));
   CK(cudaGraphLaunch(ctx->ex, st));
@@ -1665,6 +1679,7 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
     RotArgs a = rot_args(s, rp, c64);
     a.x = s->A.p;
     a.y = s->B.p;
+    a.W = s->rW.p;
     for (int it = 0; it < 7; ++it) {  // two warm-up products, five timed
       if (it == 2) CK(cudaEventRecord(e0, st));
       ftlm_status rs = enqueue_rot_passes(nullptr, s, rp, a, R, c64, nullptr, st);
@@ -1743,43 +1758,73 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   }
   Plan pl;
   std::vector<ftlm_system*> one{s};
-  if (nvec > 1 && !has_shape_override(s, nvec, c64)) {
-    // spin-1/2 blocks on the default plan: transpose to vector-major, the runs'
-    // gather, transpose back
+  const cudaStream_t st = pick_stream(s, stream);
+  if (!has_shape_override(s, nvec, c64) && (nvec > 1 || !stream_captures(st))) {
+    // spin-1/2 blocks on the default plan: transpose to vector-major (one vector
+    // is), the rotated-basis passes and, when these find the block not to be
+    // dense, the runs' gather; transpose back
     Plan vp;
     ftlm_status ps = make_plan(one, nvec, c64, vp, nullptr, true);
-    if (ps == FTLM_OK && vp.half.on && vp.half.vm && vp.half.passes == 1 && !vp.half.hybrid) {
-      // the system's two transposed blocks are shared by its calls: a call waits
-      // for the previous one's kernels (on whatever stream it ran) before reusing them
-      std::lock_guard<std::mutex> lk(s->mu);
+    RotPlan rp;
+    const bool vm = ps == FTLM_OK && vp.half.on && vp.half.vm && vp.half.passes == 1 && !vp.half.hybrid;
+    bool rot = vm && !stream_captures(st) && rot_shape(s, nvec, c64, rp);
+    if (vm && (nvec > 1 || rot)) {
+      // the system's blocks are shared by its calls: a call waits for the
+      // previous one's kernels (on whatever stream it ran) before reusing them
+      std::unique_lock<std::mutex> run_lk(s->mu, std::defer_lock);
+      if (nvec > 1) run_lk.lock();  // (the unit tables belong to runs too)
+      std::lock_guard<std::mutex> lk(s->apply_mu);
       const size_t block = (size_t)s->hs.dim * nvec * (c64 ? 8 : 16);
-      if (s->Ta.bytes < block || s->Tb.bytes < block) {
-        if (s->apply_used) CK(cudaEventSynchronize(s->ev_apply));
-        s->Ta.release();
-        s->Tb.release();
-        CK(s->Ta.ensure(block));
-        CK(s->Tb.ensure(block));
-        s->apply_used = false;
+      auto grow = [&](DevBuf& b, size_t bytes) {
+        if (b.bytes >= bytes) return cudaSuccess;
+        if (s->apply_used) cudaEventSynchronize(s->ev_apply);
+        return b.ensure(bytes);
+      };
+      if (nvec > 1) {
+        CK(grow(s->Ta, block));
+        CK(grow(s->Tb, block));
       }
-      cudaStream_t st = pick_stream(s, stream);
-      if (s->apply_used) CK(cudaStreamWaitEvent(st, s->ev_apply, 0));
-      ftlm_status ut = ensure_unit_tables(s, vp.half.K, c64, st);
-      if (ut != FTLM_OK) return ut;
-      CKI(launch_to_vector_major(x, s->Ta.p, (long long)s->hs.dim, nvec, c64, st));
-      LaunchArgs a = vp.base;
-      a.unit_tab = s->ut[c64 ? 1 : 0].p;
-      a.inline_one = 1;
-      a.one = base_desc(s, c64);
-      a.one.x = s->Ta.p;
-      a.one.y = s->Tb.p;
-      a.vm_stride = (long long)s->hs.dim * (c64 ? 8 : 16);
-      a.mode = kModeApply;
-      a.gather_alpha = 0;
-      CKI(launch_plan(vp, a, st));
-      CKI(launch_from_vector_major(s->Tb.p, y, (long long)s->hs.dim, nvec, c64, st));
-      CK(cudaEventRecord(s->ev_apply, st));
-      s->apply_used = true;
-      return FTLM_OK;
+      const size_t sbytes = sizeof(RotDensity) * nvec + 16;
+      if (rot) rot = grow(s->Tw, block / nvec * rp.group * rp.K) == cudaSuccess && grow(s->Ts, sbytes) == cudaSuccess;
+      cudaGetLastError();
+      if (nvec > 1 || rot) {
+        if (s->apply_used) CK(cudaStreamWaitEvent(st, s->ev_apply, 0));
+        ftlm_status ut = nvec > 1 ? ensure_unit_tables(s, vp.half.K, c64, st) : FTLM_OK;
+        if (ut != FTLM_OK) return ut;
+        if (rot) {
+          ut = ensure_rot_tables(s, rp, c64, st, rot);
+          if (ut != FTLM_OK) return ut;
+        }
+        const void* xv = nvec > 1 ? s->Ta.p : x;
+        void* yv = nvec > 1 ? s->Tb.p : y;
+        if (nvec > 1) CKI(launch_to_vector_major(x, s->Ta.p, (long long)s->hs.dim, nvec, c64, st));
+        LaunchArgs a = vp.base;
+        if (rot) {
+          CK(cudaMemsetAsync(s->Ts.p, 0, sbytes, st));
+          RotArgs r = rot_args(s, rp, c64);
+          r.x = const_cast<void*>(xv);
+          r.y = yv;
+          r.W = s->Tw.p;
+          r.density = reinterpret_cast<RotDensity*>(s->Ts.p);
+          r.sparse = reinterpret_cast<int*>(r.density + nvec);
+          ut = enqueue_rot_passes(nullptr, s, rp, r, nvec, c64, nullptr, st);
+          if (ut != FTLM_OK) return ut;
+          a.only_if = r.sparse;
+        }
+        a.unit_tab = nvec > 1 ? s->ut[c64 ? 1 : 0].p : nullptr;
+        a.inline_one = 1;
+        a.one = base_desc(s, c64);
+        a.one.x = xv;
+        a.one.y = yv;
+        a.vm_stride = (long long)s->hs.dim * (c64 ? 8 : 16);
+        a.mode = kModeApply;
+        a.gather_alpha = 0;
+        CKI(launch_plan(vp, a, st));
+        if (nvec > 1) CKI(launch_from_vector_major(s->Tb.p, y, (long long)s->hs.dim, nvec, c64, st));
+        CK(cudaEventRecord(s->ev_apply, st));
+        s->apply_used = true;
+        return FTLM_OK;
+      }
     }
   }
   // one vector: the row-major and the vector-major layouts coincide, so H.v may
@@ -1796,7 +1841,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   a.one.x = x;
   a.one.y = y;
   a.mode = kModeApply;
-  CKI(launch_plan(pl, a, pick_stream(s, stream)));
+  CKI(launch_plan(pl, a, st));
   return FTLM_OK;
 }
 
@@ -1899,6 +1944,8 @@ ftlm_status ftlm_system_create(int n_sites, const int* two_s, const double* J, c
     s->id = g_next_id++;
   }
   const HostSystem& hs = s->hs;
+  s->rot = std::make_unique<RotDirs>();
+  if (!rot_directions(hs, *s->rot)) s->rot.reset();
   std::vector<float> tf(hs.tab.begin(), hs.tab.end());
   std::vector<long long> stv(hs.stride.begin(), hs.stride.end());
   cudaError_t e = s->tab_d.ensure(hs.tab.size() * sizeof(double));
@@ -1931,7 +1978,7 @@ void ftlm_system_destroy(ftlm_system* s) {
   cudaDeviceSynchronize();  // the system's buffers may be in use on any stream
   purge_ctx_of(s->id);
   for (DevBuf* b : {&s->tab_f, &s->tab_d, &s->stride, &s->q, &s->A, &s->B, &s->U, &s->scal, &s->ep, &s->ecnt,
-                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart, &s->rows[0], &s->rows[1]})
+                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart, &s->rows[0], &s->rows[1], &s->Tw, &s->Ts})
     b->release();
   cudaEventDestroy(s->ev_in);
   cudaEventDestroy(s->ev_out);

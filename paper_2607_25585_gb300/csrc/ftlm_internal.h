@@ -176,6 +176,8 @@ struct LaunchArgs {
   // Re<q_j|w'> and <q_j|u>; its last CTA sets alpha_j and p_j.  The rest of
   // the step, w = w' - alpha_j sigma_j q_j with |w|^2, is kModeUpdate.
   int fused_step = 0;
+  // vector-major one-pass gather: run only when this flag is set (null: always)
+  const int* only_if = nullptr;
   // vector-major one-pass gather: the system's per-unit coefficient tables
   // (launch_vm_unit_tables), or nullptr to build them in the kernel
   const void* unit_tab = nullptr;
@@ -289,6 +291,13 @@ struct RotDirs {
   RotForm form[kRotMaxK + 1];  // z, then the K directions
 };
 
+// statistics of one vector: biased binary exponents of |x|^2
+struct RotDensity {
+  int largest;
+  unsigned zeros, arrived, pad;
+  unsigned long long sum;
+};
+
 struct RotArgs {
   int n = 0, T = 0, b = 0, K = 0;
   double t = 1;
@@ -310,6 +319,8 @@ struct RotArgs {
   DevScalars sc;               // of the whole block
   double* partials = nullptr;  // [R][tiles][3]
   unsigned* counters = nullptr;  // [R], zero between launches
+  RotDensity* density = nullptr;  // [R], zeroed: a product on a caller's block takes its statistics
+  int* sparse = nullptr;          // set by them: the later passes return
 };
 
 bool rot_directions(const HostSystem& hs, RotDirs& d);

@@ -1,5 +1,6 @@
 // Spin-1/2 H.v (Eq. 3 of arxiv 2607.25585 with every s_i = 1/2) in rotated
-// product bases, for the Lanczos steps of runs that start from random vectors.
+// product bases: the Lanczos steps of runs that start from random vectors, and
+// ftlm_apply_h on dense blocks.
 //
 // Method.  Every pair tensor A_ij (symmetric, 3 x 3) is a sum over a few fixed
 // directions u_k of scalars a^k_ij u_k u_k^T, so
@@ -47,6 +48,12 @@
 // the backward pass writes w' = sigma_j H q_j - beta_{j-1} sigma_{j-1} q_{j-1}
 // over q_{j-1} and sums alpha_j, p_j.  Partial sums go to one slot a tile and
 // are added in a fixed order by the last CTA of the vector.
+//
+// Its error is relative to the whole vector, where a gathered row's is relative
+// to that row's terms, and a value that is not finite reaches every row.  So
+// ftlm_apply_h takes these passes only for blocks that are dense and far from
+// overflow: the forward pass takes the vectors' statistics as it reads them, and
+// the other passes return, and the gather after them runs, when one is not.
 //
 // Bound: memory.  A step moves 8 (7 + 4 K) bytes a value in complex64 (152 for
 // K = 3), against 56 for the gather, but the gather's C(n, 2) flips take 3.5 ms
@@ -156,6 +163,51 @@ __device__ __forceinline__ void stage_phases(typename Cx<real>::v2* ph, const Ro
   for (int q = threadIdx.x; q < a.K * (kRotMaxN + 1); q += blockDim.x) ph[q] = __ldg(src + q);
 }
 
+// binary exponent (biased) of a sum of squares; 0 for zero and denormals
+__device__ __forceinline__ int exponent_of(float s) { return (__float_as_int(s) >> 23) & 0xff; }
+__device__ __forceinline__ int exponent_of(double s) { return (__double2hiint(s) >> 20) & 0x7ff; }
+
+// Adds the exponents of |x|^2 of the CTA's values to the vector's statistics; the
+// vector's last CTA raises a.sparse[0] unless the vector is dense: at most one
+// zero in 1024, the largest |x|^2 within 2^12 of the (geometric) mean -- a
+// Gaussian vector stays within 2^6 at 2^28 values -- and far from overflow.
+// Integer sums: the decision does not depend on the order of the CTAs.
+template <typename real, int NT>
+__device__ __forceinline__ void vector_density(const RotArgs& a, int v, int tiles, int largest, int sum, int zeros) {
+  __shared__ int red[NT / 32][3];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  largest = __reduce_max_sync(0xffffffffu, largest);
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  zeros = __reduce_add_sync(0xffffffffu, zeros);
+  if (lane == 0) {
+    red[warp][0] = largest;
+    red[warp][1] = sum;
+    red[warp][2] = zeros;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < NT / 32; ++w) {
+      largest = max(largest, red[w][0]);
+      sum += red[w][1];
+      zeros += red[w][2];
+    }
+    RotDensity* d = a.density + v;
+    atomicMax(&d->largest, largest);
+    atomicAdd(&d->sum, (unsigned long long)sum);
+    atomicAdd(&d->zeros, (unsigned)zeros);
+    __threadfence();
+    if (atomicAdd(&d->arrived, 1u) == (unsigned)(tiles - 1)) {
+      __threadfence();
+      constexpr int bias = sizeof(real) == 4 ? 127 : 1023, range = sizeof(real) == 4 ? 60 : 400;
+      const int top = atomicMax(&d->largest, 0);
+      const long long total = (long long)atomicAdd(&d->sum, 0ull), z = (long long)atomicAdd(&d->zeros, 0u);
+      const bool dense = z * 1024 <= a.dim && (long long)top * (a.dim - z) - total <= 12 * (a.dim - z) &&
+                         top >= bias - range && top <= bias + range;
+      if (!dense) atomicExch(a.sparse, 1);
+    }
+  }
+}
+
 template <typename real, int T, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) rot_forward_kernel(const __grid_constant__ RotArgs a) {
   using v2 = typename Cx<real>::v2;
@@ -197,6 +249,19 @@ __global__ void __launch_bounds__(NT, MINB) rot_forward_kernel(const __grid_cons
     for (int s = 0; s < SETS; ++s)
 #pragma unroll
       for (int r = 0; r < 16; ++r) q[s][r] = x[threadIdx.x + s * NT + (r << LO0)];
+    if (a.density) {
+      int largest = 0, sum = 0, zeros = 0;
+#pragma unroll
+      for (int s = 0; s < SETS; ++s)
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          const int e = exponent_of(q[s][r].x * q[s][r].x + q[s][r].y * q[s][r].y);
+          largest = max(largest, e);
+          sum += e;
+          zeros += e == 0;
+        }
+      vector_density<real, NT>(a, v, tiles, largest, sum, zeros);
+    }
   }
   __syncthreads();
   const real t = (real)a.t;
@@ -250,6 +315,7 @@ __global__ void __launch_bounds__(NT, MINB) rot_middle_kernel(const __grid_const
   using v2 = typename Cx<real>::v2;
   using Gr = Groups<TB>;
   constexpr int SETS = (1 << TB) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = TB - 4;
+  if (a.sparse && *a.sparse) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   v2* buf = reinterpret_cast<v2*>(smem_raw);
   const int T = a.T, nH = a.n - T, c = TB - nH;
@@ -342,6 +408,7 @@ __global__ void __launch_bounds__(NT, MINB) rot_backward_kernel(const __grid_con
   using v2 = typename Cx<real>::v2;
   using Gr = Groups<T>;
   constexpr int SETS = (1 << T) / (16 * NT), LO0 = T - 4, GL = Gr::N - 1;
+  if (a.sparse && *a.sparse) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   v2* buf = reinterpret_cast<v2*>(smem_raw);
   __shared__ v2 ph[kRotMaxK * (kRotMaxN + 1)];

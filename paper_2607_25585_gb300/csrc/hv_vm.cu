@@ -184,6 +184,7 @@ __device__ __forceinline__ int vm_pass_lo(int p, int K, int n) { return min(kLan
 // thread as 2; one copy of the tables per SM leaves more of it to L1).
 template <typename real, int K, bool MP, int MINB>
 __global__ void __launch_bounds__(MINB == 1 ? 512 : 256, MINB) vm_kernel(const __grid_constant__ LaunchArgs a) {
+  if (a.only_if && !*a.only_if) return;
   using v2 = typename Cx<real>::v2;
   constexpr int NR = 1 << K;
   constexpr int CB = kLaneBits;  // lane bits [0, CB)

@@ -12,7 +12,7 @@ import pytest
 import ftlm_workloads as W
 import oracle
 import paper_2607_25585_gb300 as F
-from gpu_helpers import empty_dev, osys
+from gpu_helpers import empty_dev, osys, to_dev
 
 pytestmark = pytest.mark.gpu
 T = np.array([0.5, 2.0, 20.0])
@@ -84,4 +84,71 @@ def test_starts_that_may_be_sparse_keep_the_gather():
     s = F.System([1] * n, J=J, B=[0, 0, 0.3])
     g = F.run(s, R=1, M=6, T=T, start="basis", basis_offset=1, dtype="c64")
     assert g["shape"]["passes"] == 1 and list(g["M_eff"]) == [2]
+    s.close()
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("R", [1, 3, 4])
+def test_product_on_dense_and_other_blocks(R, dtype, rng):
+    """ftlm_apply_h: a dense block (rotated passes), and blocks with one vector
+    that is not (the gather): a basis state, whose product is exactly zero where H
+    has no element; a value that is not finite, which reaches only its
+    neighbours; values near the ends of the range.  Tolerance of a product:
+    about 200 roundings, 15 units roundoff, relative to the norm."""
+    w = buckled(4, 4)
+    s = F.System.from_dict(w)
+    tol = 1e-6 if dtype == "c64" else 4e-15 + 1e-13
+    x = rng.normal(size=(s.dim, R)) + 1j * rng.normal(size=(s.dim, R))
+
+    def product(x):
+        y = empty_dev((s.dim, R), dtype)
+        xd = to_dev(x, dtype)
+        F.apply_h(s, xd, y, R, dtype)
+        return xd.cpu().numpy().astype(np.complex128), y.cpu().numpy()
+
+    def check(x, y, cols):
+        ref = oracle.apply_h(osys(w), np.ascontiguousarray(x[:, cols]))
+        for k, c in enumerate(cols):
+            top = np.abs(ref[:, k]).max()     # (a norm's squares may leave the range)
+            assert np.linalg.norm((y[:, c] - ref[:, k]) / top) < tol * np.linalg.norm(ref[:, k] / top)
+        return ref
+
+    check(*product(x), range(R))
+    e = x.copy()
+    e[:, R - 1] = 0
+    e[777, R - 1] = 1
+    xe, y = product(e)
+    ref = check(xe, y, range(R))
+    assert np.all(y[ref[:, -1] == 0, R - 1] == 0)
+    for scale in ((1e-30, 1e28) if dtype == "c64" else (1e-200, 1e200)):
+        check(*product(x * scale), range(R))
+    bad = x.copy()
+    bad[777, R - 1] = np.nan
+    y = product(bad)[1]
+    assert np.array_equal(np.isnan(y[:, R - 1].real), np.abs(ref[:, -1]) > 0)
+    s.close()
+
+
+def test_products_on_two_streams():
+    """Two products of one system on different streams share its blocks in order."""
+    torch = pytest.importorskip("torch")
+    w = W.square_lattice(4, 4, seed=3)
+    s = F.System.from_dict(w)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    xs = [torch.view_as_complex(torch.randn(s.dim, R, 2, device="cuda", generator=g)) for R in (8, 5, 1, 8)]
+    want = []
+    for x in xs:
+        y = torch.empty_like(x)
+        F.apply_h(s, x, y, x.shape[1], "c64")
+        torch.cuda.synchronize()
+        want.append(y)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    got = [torch.empty_like(x) for x in xs]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for k, x in enumerate(xs):
+            F.apply_h(s, x, got[k], x.shape[1], "c64", stream=(a, b)[k % 2])
+    torch.cuda.synchronize()
+    for p, q in zip(got, want):
+        assert torch.equal(p, q)
     s.close()
