@@ -229,6 +229,7 @@ struct Plan {
   int gvm_V = 1, gvm_groups = 0, gvm_ntiles = 0, gvm_rows = 0, gvm_grid = 0;
   int gvm_cube = 0;  // > 0: cube_gather_kernel with the top site's 2s+1 rows per thread
   size_t gvm_smem = 0;
+  TilePlan tile;  // V > 0: that H.v over tiles of low sites (hv_tile.cu; gvm_cube is its Q)
   std::vector<int> tile_start_g;  // prefix sum of H.v tiles over the groups
 };
 
@@ -367,6 +368,26 @@ ftlm_status make_general(const std::vector<ftlm_system*>& sys, int R, int c64, P
   return FTLM_OK;
 }
 
+// The tile plan of the systems (all with top radix Q), complex64: the tile's
+// low sites have to have the same radices in every system.
+bool plan_tile(const std::vector<ftlm_system*>& sys, int R, int Q, TilePlan& p) {
+  if (R < 2) return false;
+  int common = sys[0]->hs.n - 1, tab = 0;
+  for (auto* s : sys) {
+    if (s->hs.dim < (1u << 15) || s->hs.dim >= (1ull << 31)) return false;
+    common = std::min(common, s->hs.n - 1);
+    tab = std::max(tab, s->hs.lay.total);
+    for (int i = 0; i < common; ++i)
+      if (s->hs.q[i] != sys[0]->hs.q[i]) common = i;
+  }
+  p = TilePlan();
+  p.Q = Q;
+  p.V = Q >= 5 || R < 4 ? 2 : 4;  // 2 x 5 or 4 x 3 values a thread fill its registers
+  p.L = 1;
+  while (p.nl < common && p.L * sys[0]->hs.q[p.nl] <= 256) p.L *= sys[0]->hs.q[p.nl++];
+  return p.L >= 32 && make_tile(p, tab);
+}
+
 // allow_vm: the caller keeps its Lanczos block vector-major (ftlm_run); for
 // row-major blocks a vector-major shape falls back to the row-major cube kernel.
 ftlm_status make_plan(const std::vector<ftlm_system*>& sys, int R, int c64, Plan& pl, const Shape* force = nullptr,
@@ -429,8 +450,11 @@ ftlm_status make_plan(const std::vector<ftlm_system*>& sys, int R, int c64, Plan
     return 0;
   };
   const int Vdef = cube_group(0);
+  TilePlan tile;
+  const bool tiled = c64 && allow_vm && !force && pl.sh.general_vm < 0 && pl.sh.half_K == 0 && !pl.sh.explicit_general &&
+                     Qtop && plan_tile(sys, R, Qtop, tile);
   const bool gvm_fits = (long long)big->hs.dim * R * (c64 ? 8 : 16) <= device_l2_bytes();
-  const bool gvm_default = gvm_fits || Vdef > 0;
+  const bool gvm_default = gvm_fits || Vdef > 0 || tiled;
   const bool want_gvm = pl.sh.general_vm == 1 || (pl.sh.general_vm < 0 && !force && gvm_default);
   if (allow_vm && want_gvm && pl.sh.half_K == 0 && !pl.sh.explicit_general) {
     int V = 1;
@@ -443,8 +467,9 @@ ftlm_status make_plan(const std::vector<ftlm_system*>& sys, int R, int c64, Plan
     // spin and a kernel exists for it and for a group size dividing R
     const int Q = Qtop;
     const int Vc = (Q && pl.sh.gvm_cube != 0) ? cube_group(std::max(0, pl.sh.gvm_cube)) : 0;
-    const bool cube = Vc > 0;
-    if (cube) V = Vc;
+    const bool cube = Vc > 0 || tiled;
+    if (tiled) V = tile.V;
+    else if (cube) V = Vc;
     std::vector<ftlm_system*> vecs;  // one instance per (system, vector), system-major
     for (auto* s : sys)
       for (int k = 0; k < R; ++k) vecs.push_back(s);
@@ -459,9 +484,13 @@ ftlm_status make_plan(const std::vector<ftlm_system*>& sys, int R, int c64, Plan
     // 1024 rows: four a thread of a 256-thread CTA; with the cube, 256 bases
     // (one a thread: the CTAs then share the neighbourhoods they gather in L2)
     pl.gvm_rows = keep.gvm_rows > 0 && keep.general_vm == 1 ? keep.gvm_rows : (cube ? 256 : 1024);
+    if (tiled) {
+      pl.tile = tile;
+      pl.gvm_rows = tile.L;
+    }
     pl.tile_start_g.assign(1, 0);
     for (auto* s : sys)
-      for (int g = 0; g < R / V; ++g) {
+      for (int g = 0; g < (R + V - 1) / V; ++g) {
         const long long rows = cube ? (long long)s->hs.dim / Q : (long long)s->hs.dim;  // bases, or rows
         const long long tiles = (rows + pl.gvm_rows - 1) / pl.gvm_rows;
         if (pl.tile_start_g.back() + tiles > (1ll << 30)) return fail(FTLM_ERR_UNSUPPORTED, "too many tiles");
@@ -470,7 +499,9 @@ ftlm_status make_plan(const std::vector<ftlm_system*>& sys, int R, int c64, Plan
     pl.gvm_groups = (int)pl.tile_start_g.size() - 1;
     pl.gvm_ntiles = pl.tile_start_g.back();
     int per_sm = 1;
-    if (cube) {
+    if (tiled) {
+      per_sm = tile.per_sm;
+    } else if (cube) {
       pl.gvm_smem = gather_smem_bytes(pl.base, c64, 256);  // tables and per-thread columns, no reduction space
       CKI(prepare_cube(Q, V, c64, std::max<size_t>(pl.gvm_smem, 48 * 1024)));
       per_sm = cube_ctas_per_sm(Q, V, c64, 256, pl.gvm_smem);
@@ -500,6 +531,7 @@ int launch_plan(const Plan& pl, LaunchArgs a, void* st) {
     a.ntiles = pl.gvm_ntiles;
     a.rows_per_tile = pl.gvm_rows;
     if (!a.inline_one) a.tile_start += pl.base.n_inst + 1;
+    if (pl.tile.V) return launch_tile(a, pl.tile, pl.R, pl.gvm_grid, st);
     if (pl.gvm_cube) return launch_cube(a, pl.gvm_cube, pl.gvm_V, pl.c64, pl.gvm_grid, 256, pl.gvm_smem, st);
     return launch_rows_vm(a, pl.gvm_V, pl.c64, pl.gvm_grid, 256, pl.gvm_smem, st);
   }
@@ -879,7 +911,7 @@ std::string run_key(const std::vector<ftlm_system*>& sys, const ftlm_run_params*
   k += pl.storedV ? "|rows" + std::to_string(pl.storedV) : "";
   k += pl.rot.on ? "|rot" + std::to_string(pl.rot.group) : "";
   k += pl.gen_vm ? "|gvm" + std::to_string(pl.gvm_V) + "x" + std::to_string(pl.gvm_rows) + "c" +
-                       std::to_string(pl.gvm_cube)
+                       std::to_string(pl.gvm_cube) + "L" + std::to_string(pl.tile.L)
                  : "";
   snprintf(buf, sizeof buf, "|half%d vm%d hy%d K%d Rg%d rpt%d g%d P%d mb%d", pl.half.on ? 1 : 0, pl.half.vm ? 1 : 0,
            pl.half.hybrid ? 1 : 0,
@@ -1521,7 +1553,7 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     out.group_vectors = pl.half.on ? pl.half.Rg : (pl.gen_vm ? pl.gvm_V : R);
     out.tile_rows = pl.half.on ? pl.half.rows_per_tile : (pl.gen_vm ? pl.gvm_rows : pl.sh.rows_per_tile);
     out.grid = pl.half.on ? pl.half.grid : (pl.gen_vm ? pl.gvm_grid : pl.grid);
-    out.threads = pl.half.on ? pl.half.threads : (pl.gen_vm ? 256 : pl.sh.threads);
+    out.threads = pl.half.on ? pl.half.threads : (pl.tile.V ? pl.tile.threads : (pl.gen_vm ? 256 : pl.sh.threads));
     out.vector_major = plan_vmaj(pl) ? 1 : 0;
     out.site_cube = pl.gen_vm ? pl.gvm_cube : 0;
     out.sym_ms = 0.0;
@@ -1821,6 +1853,38 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
         a.gather_alpha = 0;
         CKI(launch_plan(vp, a, st));
         if (nvec > 1) CKI(launch_from_vector_major(s->Tb.p, y, (long long)s->hs.dim, nvec, c64, st));
+        CK(cudaEventRecord(s->ev_apply, st));
+        s->apply_used = true;
+        return FTLM_OK;
+      }
+    }
+  }
+  if (c64 && nvec > 1 && !has_shape_override(s, nvec, c64) && !stream_captures(st)) {
+    // other spins, complex64 blocks: transposed to the tile gather's layout and back
+    Plan tp;
+    ftlm_status ps = make_plan(one, nvec, c64, tp, nullptr, true);
+    if (ps == FTLM_OK && tp.gen_vm && tp.tile.V) {
+      std::lock_guard<std::mutex> lk(s->apply_mu);
+      const size_t block = (size_t)s->hs.dim * nvec * 8;
+      bool fits = true;
+      for (DevBuf* b : {&s->Ta, &s->Tb}) {
+        if (b->bytes < block && s->apply_used) CK(cudaEventSynchronize(s->ev_apply));
+        fits = fits && b->ensure(block) == cudaSuccess;
+      }
+      cudaGetLastError();
+      if (fits) {
+        if (s->apply_used) CK(cudaStreamWaitEvent(st, s->ev_apply, 0));
+        CKI(launch_to_vector_major(x, s->Ta.p, (long long)s->hs.dim, nvec, c64, st));
+        LaunchArgs a = tp.base;
+        a.inline_one = 1;
+        a.one = base_desc(s, c64);
+        a.one.x = s->Ta.p;
+        a.one.y = s->Tb.p;
+        a.vm_stride = (long long)s->hs.dim * 8;
+        a.tiles_per_vg = tp.gvm_ntiles / tp.gvm_groups;
+        a.mode = kModeApply;
+        CKI(launch_plan(tp, a, st));
+        CKI(launch_from_vector_major(s->Tb.p, y, (long long)s->hs.dim, nvec, c64, st));
         CK(cudaEventRecord(s->ev_apply, st));
         s->apply_used = true;
         return FTLM_OK;

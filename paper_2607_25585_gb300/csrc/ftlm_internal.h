@@ -331,6 +331,16 @@ int launch_rot(const RotArgs& a, int pass, int c64, void* stream);  // pass 0 fo
 int launch_rot_table(const RotForm& f, void* out, int c64, void* stream);
 int launch_rot_phases(int n, const RotDirs& d, void* out, int c64, void* stream);
 
+// The vector-major general H.v over tiles of low sites (hv_tile.cu, complex64):
+// L bases a tile (the nl low sites' digits), Q rows of the top site, V vectors.
+struct TilePlan {
+  int Q = 0, V = 0, L = 0, nl = 0;
+  int threads = 0, per_sm = 0;  // set by make_tile
+  size_t smem = 0;
+};
+int make_tile(TilePlan& p, int tab_reals);  // 0: no kernel for it
+int launch_tile(const LaunchArgs& a, const TilePlan& p, int R, int grid, void* stream);
+
 // Stored rows and streaming passes (hv_stored.cu).
 constexpr int kStoredMaxSites = 32;
 constexpr int kStreamChunk = 4096;  // elements of a streaming pass's CTA
