@@ -386,7 +386,7 @@ struct SdirArgs {
   void* y = nullptr;
   double obs[3] = {0, 0, 0};
   const double* sigma = nullptr;
-  int T = 0, n_low = 0;    // set by the launcher: tile rows, sites within a tile
+  int T = 0, n_low = 0, cols = 0;  // set by the launcher: tile rows, sites within a tile, packs of a row a CTA takes
 };
 int launch_sdir(SdirArgs a, const int* q, int c64, bool vmaj, void* stream);
 

@@ -30,8 +30,8 @@ constexpr int kThreads = 256;
 constexpr int kTileBytes = 48 * 1024;
 constexpr int kMaxSmem = kTileBytes + 4 * kMaxSites * kMaxQ * 8;  // the tile and every site's coefficients
 
-template <typename real, int V, bool VMAJ>
-__global__ void __launch_bounds__(kThreads) sdir_kernel(const __grid_constant__ SdirArgs a) {
+template <typename real, int V>
+__global__ void __launch_bounds__(kThreads) sdir_vectors_kernel(const __grid_constant__ SdirArgs a) {
   using v2 = typename Cx<real>::v2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   real* site = reinterpret_cast<real*>(smem_raw);                   // [n][qmax][4]: up, down, m, -
@@ -47,19 +47,11 @@ __global__ void __launch_bounds__(kThreads) sdir_kernel(const __grid_constant__ 
   const long long row0 = (long long)blockIdx.x * T;
   const v2* x = reinterpret_cast<const v2*>(a.x);
   v2* y = reinterpret_cast<v2*>(a.y);
-  // vector v of row mu
-  auto at = [&](long long mu, int v) { return VMAJ ? (long long)(v0 + v) * a.dim + mu : mu * a.R + v0 + v; };
-  if (VMAJ) {
+  auto at = [&](long long mu, int v) { return (long long)(v0 + v) * a.dim + mu; };  // vector v of row mu
 #pragma unroll
-    for (int v = 0; v < V; ++v)
-      if (v < nv)
-        for (int e = threadIdx.x; e < T; e += kThreads) tile[v * T + e] = __ldg(x + at(row0 + e, v));
-  } else {
-    for (int k = threadIdx.x; k < T * nv; k += kThreads) {
-      const int e = k / nv, v = k - e * nv;
-      tile[v * T + e] = __ldg(x + at(row0 + e, v));
-    }
-  }
+  for (int v = 0; v < V; ++v)
+    if (v < nv)
+      for (int e = threadIdx.x; e < T; e += kThreads) tile[v * T + e] = __ldg(x + at(row0 + e, v));
   __syncthreads();
   const real uz = (real)a.obs[0], aur = (real)a.obs[1], aui = (real)a.obs[2];
   real c[V];
@@ -94,7 +86,6 @@ __global__ void __launch_bounds__(kThreads) sdir_kernel(const __grid_constant__ 
     unsigned long long high = blockIdx.x;
     long long far = T;
     const v2* own = x + at(row0 + e, 0);
-    const long long vs = VMAJ ? a.dim : 1, rs = VMAJ ? 1 : a.R;
     for (int i = a.n_low; i < a.n; ++i) {  // the high sites: the same digits for the whole CTA
       const unsigned q = (unsigned)__ldg(a.q + i);
       const unsigned long long nx = (high >> 32) ? high / q : (unsigned)high / q;
@@ -102,8 +93,8 @@ __global__ void __launch_bounds__(kThreads) sdir_kernel(const __grid_constant__ 
       high = nx;
       const real* s = site + 4 * (i * qm + d);
       msum += s[2];
-      if (d > 0) mac(up, s[0], own - far * rs, vs);
-      if (d + 1 < (int)q) mac(dn, s[1], own + far * rs, vs);
+      if (d > 0) mac(up, s[0], own - far, a.dim);
+      if (d + 1 < (int)q) mac(dn, s[1], own + far, a.dim);
       far *= q;
     }
     const real dz = uz * msum;
@@ -119,13 +110,99 @@ __global__ void __launch_bounds__(kThreads) sdir_kernel(const __grid_constant__ 
   }
 }
 
-template <typename real, int V>
-int launch_v(const SdirArgs& a, bool vmaj, dim3 grid, size_t smem, cudaStream_t st) {
-  const void* k = vmaj ? (const void*)sdir_kernel<real, V, true> : (const void*)sdir_kernel<real, V, false>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-  if (e != cudaSuccess) return (int)e;
-  void* args[] = {const_cast<SdirArgs*>(&a)};
-  return (int)cudaLaunchKernel(k, grid, dim3(kThreads), args, smem, st);
+// The row-major form: neighbouring lanes take neighbouring vectors of one row (W a
+// lane, 16 bytes where that is aligned), so every access is a run of the row's
+// vectors; with lanes along rows, 32 bytes a lane, the loads of the high sites
+// touched a sector each (1.53 ms for 2^20 x 32 complex64 values, 0.65 ms so).
+template <typename real, int W>
+__global__ void __launch_bounds__(kThreads) sdir_rows_kernel(const __grid_constant__ SdirArgs a) {
+  using v2 = typename Cx<real>::v2;
+  struct __align__(sizeof(v2) * W) Pack {
+    v2 z[W];
+  };
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  real* site = reinterpret_cast<real*>(smem_raw);                   // [n][qmax][4]: up, down, m, -
+  Pack* tile = reinterpret_cast<Pack*>(site + 4 * a.n * a.lay.qmax);  // [T][C]
+  const real* t = reinterpret_cast<const real*>(a.tab);
+  const int qm = a.lay.qmax, T = a.T, C = a.cols;
+  for (int k = threadIdx.x; k < a.n * qm; k += kThreads) {
+    site[4 * k] = t[a.lay.off_up1 + k];
+    site[4 * k + 1] = t[a.lay.off_dn1 + k];
+    site[4 * k + 2] = t[a.lay.off_m + k];
+  }
+  auto ld = [](const Pack* p) {
+    if constexpr (W == 2) {
+      const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+      Pack o;
+      o.z[0].x = f.x;
+      o.z[0].y = f.y;
+      o.z[1].x = f.z;
+      o.z[1].y = f.w;
+      return o;
+    } else {
+      Pack o;
+      o.z[0] = __ldg(reinterpret_cast<const v2*>(p));
+      return o;
+    }
+  };
+  const int RW = a.R / W;                                  // packs of a row
+  const int c0 = blockIdx.y * C, nc = min(C, RW - c0);
+  const long long row0 = (long long)blockIdx.x * T;
+  const Pack* x = reinterpret_cast<const Pack*>(a.x);
+  Pack* y = reinterpret_cast<Pack*>(a.y);
+  for (int k = threadIdx.x; k < T * nc; k += kThreads) tile[k] = ld(x + (row0 + k / nc) * RW + c0 + k % nc);
+  __syncthreads();
+  const real uz = (real)a.obs[0], aur = (real)a.obs[1], aui = (real)a.obs[2];
+  for (int k = threadIdx.x; k < T * nc; k += kThreads) {
+    const int e = k / nc, c = k - e * nc;
+    Pack up, dn;
+#pragma unroll
+    for (int w = 0; w < W; ++w) up.z[w].x = up.z[w].y = dn.z[w].x = dn.z[w].y = 0;
+    real msum = 0;
+    auto mac = [&](Pack& s, real f, const Pack& p) {
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        s.z[w].x = fma(f, p.z[w].x, s.z[w].x);
+        s.z[w].y = fma(f, p.z[w].y, s.z[w].y);
+      }
+    };
+    unsigned rem = (unsigned)e;
+    int stride = nc;
+    for (int i = 0; i < a.n_low; ++i) {
+      const unsigned q = (unsigned)__ldg(a.q + i), nx = rem / q;
+      const int d = (int)(rem - nx * q);
+      rem = nx;
+      const real* s = site + 4 * (i * qm + d);
+      msum += s[2];
+      if (d > 0) mac(up, s[0], tile[k - stride]);
+      if (d + 1 < (int)q) mac(dn, s[1], tile[k + stride]);
+      stride *= (int)q;
+    }
+    unsigned long long high = blockIdx.x;
+    const Pack* own = x + (row0 + e) * RW + c0 + c;
+    long long far = (long long)T * RW;
+    for (int i = a.n_low; i < a.n; ++i) {
+      const unsigned q = (unsigned)__ldg(a.q + i);
+      const unsigned long long nx = (high >> 32) ? high / q : (unsigned)high / q;
+      const int d = (int)(high - nx * q);
+      high = nx;
+      const real* s = site + 4 * (i * qm + d);
+      msum += s[2];
+      if (d > 0) mac(up, s[0], ld(own - far));
+      if (d + 1 < (int)q) mac(dn, s[1], ld(own + far));
+      far *= q;
+    }
+    const real dz = uz * msum;
+    Pack o;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const v2 z = tile[k].z[w], p = up.z[w], m = dn.z[w];
+      const real f = a.sigma ? (real)a.sigma[(c0 + c) * W + w] : (real)1;
+      o.z[w].x = f * fma(dz, z.x, fma(aur, p.x + m.x, -aui * (p.y - m.y)));
+      o.z[w].y = f * fma(dz, z.y, fma(aur, p.y + m.y, aui * (p.x - m.x)));
+    }
+    y[(row0 + e) * RW + c0 + c] = o;
+  }
 }
 
 }  // namespace
@@ -135,21 +212,32 @@ int launch_v(const SdirArgs& a, bool vmaj, dim3 grid, size_t smem, cudaStream_t 
 int launch_sdir(SdirArgs a, const int* q, int c64, bool vmaj, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int esz = c64 ? 8 : 16;
-  // four complex64 or two complex128 vectors a CTA: wider groups leave the tile fewer low sites
+  // vector-major: four complex64 or two complex128 vectors a CTA (wider groups
+  // leave the tile fewer low sites); row-major: up to 128 bytes of a row
   const int V = std::min(a.R, c64 ? 4 : 2) == 3 ? 4 : std::min(a.R, c64 ? 4 : 2);
+  const int W = c64 && a.R % 2 == 0 ? 2 : 1;
+  a.cols = std::min(a.R / W, 128 / (W * esz));
+  const int width = vmaj ? V : a.cols * W;
   a.T = 1;
   a.n_low = 0;
-  while (a.n_low < a.n && (a.n_low == 0 || (long long)a.T * q[a.n_low] * V * esz <= kTileBytes)) a.T *= q[a.n_low++];
-  const size_t smem = (size_t)4 * a.n * a.lay.qmax * (esz / 2) + (size_t)a.T * V * esz;
-  const dim3 grid((unsigned)(a.dim / a.T), (unsigned)((a.R + V - 1) / V));
+  while (a.n_low < a.n && (a.n_low == 0 || (long long)a.T * q[a.n_low] * width * esz <= kTileBytes)) a.T *= q[a.n_low++];
+  const size_t smem = (size_t)4 * a.n * a.lay.qmax * (esz / 2) + (size_t)a.T * width * esz;
+  const dim3 grid((unsigned)(a.dim / a.T), (unsigned)((a.R + width - 1) / width));
   if (a.R < 1 || a.dim / a.T > 0x7fffffffll || grid.y > 65535) return (int)cudaErrorInvalidValue;
-  if (c64) {
-    if (V == 4) return launch_v<float, 4>(a, vmaj, grid, smem, st);
-    if (V == 2) return launch_v<float, 2>(a, vmaj, grid, smem, st);
-    return launch_v<float, 1>(a, vmaj, grid, smem, st);
+  const void* k;
+  if (!vmaj) {
+    k = W == 2 ? (const void*)sdir_rows_kernel<float, 2>
+               : (c64 ? (const void*)sdir_rows_kernel<float, 1> : (const void*)sdir_rows_kernel<double, 1>);
+  } else if (c64) {
+    k = V == 4 ? (const void*)sdir_vectors_kernel<float, 4>
+               : (V == 2 ? (const void*)sdir_vectors_kernel<float, 2> : (const void*)sdir_vectors_kernel<float, 1>);
+  } else {
+    k = V == 2 ? (const void*)sdir_vectors_kernel<double, 2> : (const void*)sdir_vectors_kernel<double, 1>;
   }
-  if (V == 2) return launch_v<double, 2>(a, vmaj, grid, smem, st);
-  return launch_v<double, 1>(a, vmaj, grid, smem, st);
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (e != cudaSuccess) return (int)e;
+  void* args[] = {&a};
+  return (int)cudaLaunchKernel(k, grid, dim3(kThreads), args, smem, st);
 }
 
 }  // namespace ftlm
