@@ -221,6 +221,7 @@ struct Plan {
   std::vector<int> tile_start;
   HalfPlan half;  // spin-1/2 kernel for the H.v modes, when applicable
   int storedV = 0;  // > 0: H.v of vector-major runs from stored rows, that many vectors a group
+  int small = 0;    // > 0: the whole run in one launch, clusters of that many CTAs
   int wideV = 0;  // general kernel: H.v with 4 or 8 complex64 vectors per thread (0 = off)
   // vector-major general plan (any spins, several systems): every vector of a
   // run contiguous; the streaming modes see one instance per (system, vector),
@@ -908,7 +909,7 @@ std::string run_key(const std::vector<ftlm_system*>& sys, const ftlm_run_params*
   k += buf;
   k += p->symmetric ? "|sym" : "";
   k += p->reorth ? "|reorth" : "";
-  k += pl.storedV ? "|rows" + std::to_string(pl.storedV) : "";
+  k += pl.storedV ? "|rows" + std::to_string(pl.storedV) + "s" + std::to_string(pl.small) : "";
   k += pl.rot.on ? "|rot" + std::to_string(pl.rot.group) : "";
   k += pl.gen_vm ? "|gvm" + std::to_string(pl.gvm_V) + "x" + std::to_string(pl.gvm_rows) + "c" +
                        std::to_string(pl.gvm_cube) + "L" + std::to_string(pl.tile.L)
@@ -1095,7 +1096,18 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
     ftlm_status rs = enqueue_rot_steps(ctx, sys[0], p, pl, sa, d_even, d_odd, st);
     if (rs != FTLM_OK) return rs;
   }
-  for (int j = 0; j < M && !pl.rot.on; ++j) {
+  if (pl.small) {
+    SmallRunArgs g;
+    g.inst = d_even;
+    g.keep = p->symmetric ? sys[0]->Vs.p : nullptr;
+    g.R = R;
+    long long most = 0;
+    for (auto* s : sys) most = std::max(most, (long long)s->hs.dim);
+    CKI(launch_small_run(g, nd, pl.small, most, c64, st));
+    ctx.launches++;
+    ctx.hv_launches = M;
+  }
+  for (int j = 0; j < M && !pl.rot.on && !pl.small; ++j) {
     a.inst = (j % 2 == 0) ? d_even : d_odd;
     a.step = j;
     a.first = j == 0;
@@ -1414,6 +1426,15 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
       rows += s->hs.dim;
     }
     if (all) pl.storedV = stored_group(rows, R, true);
+    // one launch for all steps while every cluster is resident at once (two CTAs an
+    // SM at most): more vectors or rows have work enough to fill the chip step by step
+    long long most = 0;
+    for (auto* s : sys) most = std::max(most, (long long)s->hs.dim);
+    for (int c = 8; c >= 1 && all && !p->time_kernels && !pl.small; c /= 2) {
+      const size_t smem = small_run_smem(most, c, c64);
+      const int fit = smem <= kSmallRunBytes ? std::min<int>(2, (int)(200 * 1024 / (smem + 4096))) * std::max(1, device_sm_count()) : 0;
+      if ((long long)n * R * c <= fit) pl.small = c;
+    }
   }
   if (vm_fused_step(pl) && !pl.rot.on && !pl.storedV) {
     ftlm_status ut = ensure_unit_tables(sys[0], pl.half.K, c64, st);

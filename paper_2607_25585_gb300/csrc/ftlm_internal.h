@@ -368,6 +368,15 @@ struct StreamArgs {
   double* slots = nullptr;          // [vectors][max_tiles][3]
   unsigned* counters = nullptr;     // [vectors], zero between launches
 };
+// Whole Lanczos runs of small systems, a cluster per vector (run_small.cu).
+constexpr size_t kSmallRunBytes = 96 * 1024;  // shared memory of a CTA at most: two an SM
+struct SmallRunArgs {
+  const InstDesc* inst = nullptr;  // one a vector: x = q_0, u, scalars, stored rows
+  void* keep = nullptr;            // symmetric runs: the Lanczos vectors [M][R][dim]
+  int R = 0;
+};
+size_t small_run_smem(long long dim, int ctas, int c64);
+int launch_small_run(const SmallRunArgs& a, int vectors, int ctas, long long max_dim, int c64, void* stream);
 int stored_row_bound(const HostSystem& hs);
 int launch_stored_build(const void* tab, const TabLayout& L, const long long* stride, const int* q, int n, int dim,
                         int S, int* col, void* val, int* cnt, int c64, void* stream);

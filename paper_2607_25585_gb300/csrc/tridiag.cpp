@@ -31,9 +31,10 @@ inline double norm2(double a, double b) {
 }
 
 // Estimated cost of one run's eigenproblem with `rows` rotated rows, and of one
-// (temperature, Ritz value) term of the sums, in nanoseconds.
-double ql_ns(int m, int rows) { return 1.7 * m * m * (20.0 + 2.0 * rows); }
-constexpr double kTermNs = 12.0;
+// (temperature, Ritz value) term of the sums, in nanoseconds (measured on the
+// Grace cores: 16 us for 24 rows, 190 us for 100; 4 ns a term).
+double ql_ns(int m, int rows) { return 1.7 * m * m * (8.0 + 1.2 * rows); }
+constexpr double kTermNs = 4.0;
 
 // Eigenvalues of tridiag(d, e) (d[0..m-1], e[0..m-2] off-diagonal) with the
 // rotations applied to the rows z[k][0..m-1], k < nz.  Returns false if the
@@ -94,13 +95,13 @@ bool ql_implicit(int m, double* d, double* e_in, int nz, double** z) {
 }  // namespace
 
 // fn(i) for i in [0, n), each exactly once, on the caller's thread and as many
-// others as the work pays for: starting and joining a thread costs some 20 us,
-// so each gets at least 50 us of `total_ns` (with one thread an item, ten
-// eigenproblems of 24 rows, 0.2 ms in all, took 1.5 ms).
+// others as the work pays for: starting and joining a thread costs some 60 us,
+// so each gets at least 200 us of `total_ns` (ten eigenproblems of 24 rows and
+// their sums, 0.2 ms on one thread, took 0.4 ms on six and 1.5 ms on ten and more).
 // false: an item threw (out of memory).
 bool parallel_for(int n, double total_ns, const std::function<void(int)>& fn) {
   const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
-  const int nth = std::min({n, hw, 32, 1 + (int)std::min(1e6, total_ns / 50e3)});
+  const int nth = std::min({n, hw, 32, 1 + (int)std::min(1e6, total_ns / 200e3)});
   std::atomic<int> next{0};
   std::atomic<bool> ok{true};
   auto work = [&]() {

@@ -92,3 +92,26 @@ def test_product_inside_a_capture():
         torch.cuda.synchronize()
         assert rel_l2(y.cpu().numpy(), ref) < 1e-12
         s.close()
+
+
+@pytest.mark.parametrize("R", [1, 5, 16, 40, 80, 200])
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+def test_whole_run_in_one_launch_matches_steps(R, dtype):
+    """Clusters of 8, 4, 2 and 1 CTAs a vector (by the number of vectors) against the
+    same run step by step (kernel timing asks for it), for rows that the CTAs do
+    not share evenly, a symmetric run's stored vectors, and a breakdown."""
+    T = np.array([0.5, 5.0])
+    for ts in ([2] * 5, [4], [1, 2, 1]):
+        w = random_system(np.random.default_rng(8), ts)
+        s = F.System.from_dict(w)
+        M = min(10, s.dim + 2)
+        kw = dict(R=R, M=M, T=T, seed=3, dtype=dtype, symmetric=len(ts) == 5)
+        a, b = F.run(s, **kw), F.run(s, time_kernels=True, **kw)
+        assert list(a["M_eff"]) == list(b["M_eff"])
+        m = min(M, max(1, s.dim // 3))              # the steps well before the Krylov space is exhausted
+        for k in ("alpha", "beta", "p"):
+            scale = max(np.abs(b[k][:, :m]).max(), np.abs(b["beta"]).max() * (k == "alpha"))
+            assert np.abs(a[k][:, :m] - b[k][:, :m]).max() < 30 * TOL[dtype] * scale, (ts, k)
+        if len(ts) == 5:
+            assert np.abs(a["O"] - b["O"]).max() < 30 * TOL[dtype] * np.abs(b["O"]).max()
+        s.close()
