@@ -733,31 +733,44 @@ bool stream_captures(cudaStream_t st) {
 // ---- stored rows of small systems -----------------------------------------------
 
 // Rows are stored up to a quarter of L2, where every product reads them from
-// there.  (Larger systems have rows enough to fill the chip with the gathers.)
-constexpr size_t kStoredBytes = 32u << 20;
+// there; larger systems have rows enough to fill the chip with the gathers.  But
+// where these form coefficients for one or two vectors at a time in FP64, that
+// costs more than reading them from HBM: complex128, up to 2 GB for the
+// call's n systems then (a product of nine spins 3/2 and 2, 327,680 states, in
+// complex128: 1.22 -> 0.29 ms for one vector, 12.6 -> 2.1 ms for eight).  Spin-1/2
+// systems have the rotated-basis passes.
+constexpr size_t kStoredL2 = 32u << 20;
+size_t stored_limit(const ftlm_system* s, int c64, int n = 1) {
+  return !s->hs.all_half && !c64 ? std::max(kStoredL2, ((size_t)2 << 30) / n) : kStoredL2;
+}
 
 // The system's stored rows for work on stream st: written on the first call (on
-// the system's own stream; st waits for them).  ok = false: none (too large, or
-// not there yet while st is being captured; the gathers then run).
-ftlm_status ensure_stored(ftlm_system* s, int c64, cudaStream_t st, StoredRows& r, bool& ok) {
+// the system's own stream; st waits for them).  ok = false: the gathers run -- the
+// rows are too large, or beyond L2 for a call of fewer than four products of a
+// vector (writing them costs about two), or st is being captured.  The choice
+// depends on the call alone, so a repeated call gives the same bits.
+ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long products, cudaStream_t st, StoredRows& r,
+                          bool& ok) {
   ok = false;
   const int k = c64 ? 1 : 0;
   const size_t d = (size_t)s->hs.dim, esz = c64 ? 8 : 16;
   const size_t S = (size_t)stored_row_bound(s->hs);
-  if (S == 0 || d > kStoredBytes || d * S * (esz + 4) + d * 4 > kStoredBytes) return FTLM_OK;
+  if (S == 0 || d > limit || d * S * (esz + 4) + d * 4 > (products < 4 ? kStoredL2 : limit)) return FTLM_OK;
+  if (stream_captures(st)) return FTLM_OK;
   std::lock_guard<std::mutex> lk(s->rows_mu);
   DevBuf& b = s->rows[k];
   if (!s->rows_done[k]) {
-    if (stream_captures(st)) return FTLM_OK;
     if (!b.p) {
       if (!s->ev_rows[k]) CK(cudaEventCreateWithFlags(&s->ev_rows[k], cudaEventDisableTiming));
       if (b.ensure(d * S * (esz + 4) + d * 4) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
       char* p = static_cast<char*>(b.p);
-      CKI(launch_stored_build(c64 ? s->tab_f.p : s->tab_d.p, s->hs.lay,
-                              reinterpret_cast<const long long*>(s->stride.p), reinterpret_cast<const int*>(s->q.p),
-                              s->hs.n, (int)d, (int)S, reinterpret_cast<int*>(p + d * S * esz), p,
-                              reinterpret_cast<int*>(p + d * S * (esz + 4)), c64, s->own_stream));
-      CK(cudaEventRecord(s->ev_rows[k], s->own_stream));
+      int e = launch_stored_build(c64 ? s->tab_f.p : s->tab_d.p, s->hs.lay,
+                                  reinterpret_cast<const long long*>(s->stride.p), reinterpret_cast<const int*>(s->q.p),
+                                  s->hs.n, (int)d, (int)S, reinterpret_cast<int*>(p + d * S * esz), p,
+                                  reinterpret_cast<int*>(p + d * S * (esz + 4)), c64, s->own_stream);
+      if (!e) e = (int)cudaEventRecord(s->ev_rows[k], s->own_stream);
+      if (e) b.release();
+      CKI(e);
     }
     if (cudaEventQuery(s->ev_rows[k]) == cudaSuccess) s->rows_done[k] = true;
     else CK(cudaStreamWaitEvent(st, s->ev_rows[k], 0));
@@ -773,10 +786,10 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, cudaStream_t st, StoredRows& 
 }
 
 // Vectors a CTA of the stored-row kernels takes: as many as leave the chip enough
-// threads (eight a row and group) to hide L2 latency; `divide`: a divisor of R.
-int stored_group(uint64_t rows, int R, bool divide) {
+// threads (eight a row and group) to hide L2 latency.
+int stored_group(uint64_t rows, int R) {
   int V = 4;
-  while (V > 1 && (V > R || (divide && R % V != 0) || rows * 8 * (uint64_t)((R + V - 1) / V) < 200000)) V /= 2;
+  while (V > 1 && (V / 2 >= R || rows * 8 * (uint64_t)((R + V - 1) / V) < 200000)) V /= 2;
   return V;
 }
 
@@ -1133,7 +1146,8 @@ ftlm_status enqueue_run(RunCtx& ctx, const std::vector<ftlm_system*>& sys, const
       StoredArgs g;
       g.inst = a.inst;
       g.tile_start = reinterpret_cast<const int*>(ctx.tiles.p) + ctx.stored_at;
-      g.groups = nd / pl.storedV;
+      g.groups = n * ((R + pl.storedV - 1) / pl.storedV);
+      g.R = R;
       g.max_tiles = ctx.stored_tiles;
       g.j = j;
       g.slots = sa.slots;
@@ -1249,7 +1263,7 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
     e.hq = o.hq = Hq;
     if (pl.storedV) {
       bool ok = false;  // (built by run_impl before the capture)
-      ftlm_status rs = ensure_stored(s, c64, st, e.stored, ok);
+      ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64, n), (long long)R * M, st, e.stored, ok);
       if (rs != FTLM_OK) return rs;
       if (!ok) return fail(FTLM_ERR_CUDA, "stored rows are missing");
       o.stored = e.stored;
@@ -1274,13 +1288,14 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
     auto list = [&](int step, long long rows, int& at, int& most, int& grid) -> bool {
       at = (int)tiles.size();
       tiles.push_back(0);
-      for (int k = 0; k < nd; k += step) {
-        const long long t = ((long long)sys[k / R]->hs.dim + rows - 1) / rows;
-        if (tiles.back() + t > (1ll << 30)) return false;
-        tiles.push_back(tiles.back() + (int)t);
-        most = std::max(most, (int)t);
-        c.even = c.even && sys[k / R]->hs.dim % 2 == 0;
-      }
+      for (int k = 0; k < n; ++k)
+        for (int v = 0; v < R; v += step) {
+          const long long t = ((long long)sys[k]->hs.dim + rows - 1) / rows;
+          if (tiles.back() + t > (1ll << 30)) return false;
+          tiles.push_back(tiles.back() + (int)t);
+          most = std::max(most, (int)t);
+          c.even = c.even && sys[k]->hs.dim % 2 == 0;
+        }
       grid = tiles.back();
       return true;
     };
@@ -1420,12 +1435,12 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     for (auto* s : sys) {
       StoredRows r;
       bool ok = false;
-      ftlm_status rs = ensure_stored(s, c64, st, r, ok);
+      ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64, n), (long long)R * M, st, r, ok);
       if (rs != FTLM_OK) return rs;
       all = all && ok;
       rows += s->hs.dim;
     }
-    if (all) pl.storedV = stored_group(rows, R, true);
+    if (all) pl.storedV = stored_group(rows, R);
     // one launch for all steps while every cluster is resident at once (two CTAs an
     // SM at most): more vectors or rows have work enough to fill the chip step by step
     long long most = 0;
@@ -1608,7 +1623,7 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
   {  // stored rows have no shape to choose, and every gather is slower on systems that small
     StoredRows r;
     bool ok = false;
-    ftlm_status rs = ensure_stored(s, c64, st, r, ok);
+    ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), R, st, r, ok);
     if (rs != FTLM_OK || ok) return rs;
   }
   std::vector<Shape> cands;
@@ -1797,7 +1812,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   if (!has_shape_override(s, nvec, c64)) {  // small systems: stored rows
     StoredArgs a;
     bool ok = false;
-    ftlm_status rs = ensure_stored(s, c64, pick_stream(s, stream), a.rows, ok);
+    ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), nvec, pick_stream(s, stream), a.rows, ok);
     if (rs != FTLM_OK) return rs;
     if (ok) {
       a.x = x;
@@ -1805,7 +1820,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
       a.dim = (long long)s->hs.dim;
       a.rs = a.R = nvec;
       a.vs = 1;
-      CKI(launch_stored_product(a, stored_group(s->hs.dim, nvec, false), c64, pick_stream(s, stream)));
+      CKI(launch_stored_product(a, stored_group(s->hs.dim, nvec), c64, pick_stream(s, stream)));
       return FTLM_OK;
     }
   }

@@ -346,7 +346,7 @@ constexpr int kStoredMaxSites = 32;
 constexpr int kStreamChunk = 4096;  // elements of a streaming pass's CTA
 
 struct StoredArgs {
-  // a Lanczos step: groups of V one-vector instances, CTAs by the groups' tile list
+  // a Lanczos step: groups of V one-vector instances (R a system), CTAs by the groups' tile list
   const InstDesc* inst = nullptr;
   const int* tile_start = nullptr;  // [groups + 1], tiles of 32 rows
   int groups = 0, max_tiles = 0;

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256) stored_rows_kernel(const __grid_constant_
   __shared__ double red[8][V * 3];
   __shared__ int last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane & (kLanes - 1);
-  int g = 0, tile = blockIdx.x, tiles = 0, nv = V;
+  int g = 0, tile = blockIdx.x, tiles = 0, nv = V, vec0 = 0;
   const InstDesc* in = nullptr;
   StoredRows H;
   const v2* x;
@@ -137,7 +137,10 @@ __global__ void __launch_bounds__(256) stored_rows_kernel(const __grid_constant_
     const int t0 = __ldg(a.tile_start + g);
     tiles = __ldg(a.tile_start + g + 1) - t0;
     tile -= t0;
-    in = a.inst + (size_t)g * V;
+    const int per_system = (a.R + V - 1) / V, first = g % per_system * V;  // (a system's last group may be smaller)
+    vec0 = g / per_system * a.R + first;
+    nv = min(V, a.R - first);
+    in = a.inst + vec0;
     H = in->stored;
     dim = in->dim;
     x = reinterpret_cast<const v2*>(in->x);
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(256) stored_rows_kernel(const __grid_constant_
       const v2* p = x + (long long)__ldg(col + e) * rs;
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        if (!STEP && v >= nv) break;
+        if (v >= nv) break;
         const v2 z = __ldg(p + v * vs);
         ar[v] = fma(h.x, z.x, fma(-h.y, z.y, ar[v]));
         ai[v] = fma(h.x, z.y, fma(h.y, z.x, ai[v]));
@@ -225,8 +228,8 @@ __global__ void __launch_bounds__(256) stored_rows_kernel(const __grid_constant_
 #pragma unroll
     for (int c = 0; c < 3; ++c) red[warp][lane * 3 + c] = p[c];
   __syncthreads();
-  double* slots = a.slots + (size_t)g * V * a.max_tiles * 3;  // [vector][tile][3]
-  if (threadIdx.x < V * 3) {
+  double* slots = a.slots + (size_t)vec0 * a.max_tiles * 3;  // [vector][tile][3]
+  if ((int)threadIdx.x < nv * 3) {
     double s = 0.0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(256) stored_rows_kernel(const __grid_constant_
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int k = warp; k < V * 3; k += 8) {
+  for (int k = warp; k < nv * 3; k += 8) {
     const int v = k / 3, c = k % 3;
     double s = 0.0;
     for (int i = lane; i < tiles; i += 32) s += __ldcg(slots + ((size_t)v * a.max_tiles + i) * 3 + c);

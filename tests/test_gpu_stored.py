@@ -77,7 +77,7 @@ def test_product_inside_a_capture():
     w = W.ring(N=5, two_s=2)
     x = torch.randn(243, 4, dtype=torch.complex128, device="cuda")
     ref = oracle.apply_h(osys(w), x.cpu().numpy())
-    for warm in (False, True):      # rows not written before the capture (the gather is captured), and written
+    for warm in (False, True):      # the gather is captured, whether the rows have been written or not
         s = F.System.from_dict(w)
         y = torch.empty_like(x)
         if warm:
@@ -115,3 +115,31 @@ def test_whole_run_in_one_launch_matches_steps(R, dtype):
         if len(ts) == 5:
             assert np.abs(a["O"] - b["O"]).max() < 30 * TOL[dtype] * np.abs(b["O"]).max()
         s.close()
+
+
+@pytest.mark.parametrize("dtype,R", [("c128", 1), ("c128", 3), ("c128", 8)])
+def test_rows_beyond_l2(dtype, R):
+    """Complex128 systems keep their rows up to 2 GB: products and
+    runs against the forced row-major gather (d = 59,049)."""
+    T = np.array([0.5, 5.0])
+    w = W.chain(10, Bdir=(0.3, -0.2, 0.9))
+    s = F.System.from_dict(w)
+    g = np.random.default_rng(4)
+    x = to_dev(g.normal(size=(s.dim, R)) + 1j * g.normal(size=(s.dim, R)), dtype)
+    y, z = empty_dev((s.dim, R), dtype), empty_dev((s.dim, R), dtype)
+    F.apply_h(s, x, y, R, dtype)    # (one and three vectors: the gather)
+    first = y.clone()
+    a = F.run(s, R=R, M=6, T=T, seed=3, dtype=dtype)
+    F.tune_shape(s, R, dtype, 0, 1, 1, 0)
+    try:
+        F.apply_h(s, x, z, R, dtype)
+        b = F.run(s, R=R, M=6, T=T, seed=3, dtype=dtype)
+    finally:
+        F.tune_shape(s, R, dtype, -1)
+    assert rel_l2(y.cpu().numpy(), z.cpu().numpy()) < TOL[dtype]
+    F.apply_h(s, x, y, R, dtype)    # after a run has written the rows: the same bits
+    assert bool((y == first).all())
+    for k in ("alpha", "beta", "p"):
+        scale = max(np.abs(b[k]).max(), np.abs(b["beta"]).max() * (k == "alpha"))
+        assert np.abs(a[k] - b[k]).max() < 10 * TOL[dtype] * scale
+    s.close()
