@@ -707,8 +707,7 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
     for (int j = i + 1; j < n; ++j) {
       const int ij = i * n + j, ji = j * n + i;
       for (int c = 0; c < 2; ++c) {
-        const double r1 = t[L.off_rho + 2 * ij + c], r2 = t[L.off_rho + 2 * ji + c];
-        if (std::fabs(r1 - r2) > 1e-14 * std::fabs(r1)) return false;  // (equal up to the last bit's rounding)
+        if (t[L.off_rho + 2 * ij + c] != t[L.off_rho + 2 * ji + c]) return false;
         planar = planar && t[L.off_rho + 2 * ij + c] == 0.0;
       }
       diagonal = diagonal && t[L.off_pp + 2 * ij + 1] == 0.0;

@@ -152,7 +152,10 @@ ftlm_status build_host_system(int n, const int* two_s, const double* J, const do
         }
         const double pref = C_dip * g * g / (r2 * std::sqrt(r2));
         for (int x = 0; x < 3; ++x)
-          for (int y = 0; y < 3; ++y) a[3 * x + y] += pref * ((x == y ? 1.0 : 0.0) - 3.0 * r[x] * r[y] / r2);
+          for (int y = x; y < 3; ++y) {  // (formed once: 3 r_x r_y and 3 r_y r_x may round differently)
+            a[3 * x + y] += pref * ((x == y ? 1.0 : 0.0) - 3.0 * r[x] * r[y] / r2);
+            a[3 * y + x] = a[3 * x + y];
+          }
       }
     }
 

@@ -38,6 +38,8 @@ SYSTEMS = {
     "buckled15": lambda: buckled(5, 3),                                      # five directions
     "ladder16": lambda: W.ladder(8, dipolar=False),                          # exchange alone
     "buckled16": lambda: buckled(4, 4),
+    "ring13": lambda: W.ring(13, two_s=1, radius=5.0, Bdir=(1, 2, 2)),       # bonds at every angle of the plane
+    "ring15": lambda: W.ring(15, two_s=1, radius=6.0),
 }
 
 
