@@ -58,7 +58,7 @@
 // Bound: memory.  A step moves 8 (7 + 4 K) bytes a value in complex64 (152 for
 // K = 3), against 56 for the gather, but the gather's C(n, 2) flips take 3.5 ms
 // at n = 20 with 64 vectors, where these passes take 1.71 ms with the update
-// (3.8 ms with it before): 6.0 TB/s.  2 x 13 sites, 4 vectors: 33 -> 11.7 ms a
+// (3.8 ms with it before): 6.0 TB/s.  2 x 13 sites, 4 vectors: 33 -> 11.0 ms a
 // step.  In complex128 the FP64 pipe binds both: 4 x 4 sites, 50 vectors:
 // 4.0 -> 1.57 ms.  Taking one to eight vectors at a time through the three
 // passes, so that W stays in L2, was slower (2.1 to 3.0 ms): each launch then
@@ -403,6 +403,109 @@ __global__ void __launch_bounds__(NT, MINB) rot_middle_kernel(const __grid_const
   }
 }
 
+// The same for the large tile (NG >= 3): one CTA an SM takes tiles one after another and loads the next into
+// registers while this one is exchanged: the large tile alone fills an SM's shared
+// memory, and without it loads, exchanges and stores took turns (5.3 -> 4.6 ms for
+// 2^26 x 4 complex64 values).
+template <typename real, int TB, int NT, int NG>
+__global__ void __launch_bounds__(NT, 1) rot_middle_ahead_kernel(const __grid_constant__ RotArgs a) {
+  using v2 = typename Cx<real>::v2;
+  using Gr = Groups<TB>;
+  constexpr int SETS = (1 << TB) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = TB - 4;
+  if (a.sparse && *a.sparse) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  v2* buf = reinterpret_cast<v2*>(smem_raw);
+  const int T = a.T, nH = a.n - T, c = TB - nH;
+  const int cmask = (1 << c) - 1;
+  const int ncb = 1 << (T - c);  // 2^T columns in blocks of 2^c
+  auto at = [&](int i) { return ((unsigned)(i >> c) << a.b) + (unsigned)(i & cmask); };  // offset of tile index i
+  // offset of value r of group 0 (all its bits are high ones)
+  const unsigned stride0 = 1u << (LO0 - c + a.b);
+  auto at0 = [&](int r) { return r * stride0; };
+  auto mask_of = [&](int g) {  // the transformed bits (>= c) of group g
+    const int l = Gr::lo(g);
+    return (c > l ? (15 << (c - l)) : 15) & Gr::mask(g);
+  };
+  const real t = (real)a.t;
+  // column block q of all directions and vector groups; its first value and its vectors
+  const int blocks = ncb * a.K * ((a.nvec + a.vpb - 1) / a.vpb);
+  auto first_of = [&](int q) { return (size_t)((q >> (T - c)) % a.K) * a.dim + w_place((unsigned)(q & (ncb - 1)) << c, a.b, nH); };
+  auto vec_of = [&](int q) { return ((q >> (T - c)) / a.K) * a.vpb; };
+  auto tile_of = [&](int q, int v) { return reinterpret_cast<v2*>(a.W) + (size_t)(a.vec0 - a.vecW + v) * a.K * a.dim + first_of(q); };
+  v2 nx[SETS][16];
+  {
+    const v2* W = tile_of(blockIdx.x, vec_of(blockIdx.x));
+#pragma unroll
+    for (int s = 0; s < SETS; ++s)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) nx[s][r] = W[at(threadIdx.x + s * NT) + at0(r)];
+  }
+  for (int q = blockIdx.x; q < blocks; q += (int)gridDim.x) {
+    const real* D = reinterpret_cast<const real*>(a.D) + first_of(q);
+    const int v0 = vec_of(q), v1 = min(a.nvec, v0 + a.vpb);
+    for (int v = v0; v < v1; ++v) {
+      v2* W = tile_of(q, v);
+      // gates of the last group, D (after the first vector from L1) and the inverse gates
+      auto centre = [&](v2(&w)[16], int b) {
+        const real* d = D + at(b);
+        const int m = mask_of(NG - 1);
+        gates(w, t, m);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          const real dv = __ldg(d + at(r << LOC));
+          w[r].x *= dv;
+          w[r].y *= dv;
+        }
+        gates(w, -t, m);
+      };
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const int i0 = threadIdx.x + s * NT;
+        v2 w[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) w[r] = nx[s][r];
+        gates(w, t, 15);
+        smem_st<LO0>(buf, i0, w);
+      }
+      {
+        const int qn = v + 1 < v1 ? q : q + (int)gridDim.x;
+        if (qn < blocks) {
+          const v2* N = tile_of(qn, v + 1 < v1 ? v + 1 : vec_of(qn));
+#pragma unroll
+          for (int s = 0; s < SETS; ++s)
+#pragma unroll
+            for (int r = 0; r < 16; ++r) nx[s][r] = N[at(threadIdx.x + s * NT) + at0(r)];
+        }
+      }
+      __syncthreads();
+      if constexpr (NG > 2) mid_group<real, TB, NT, SETS, 1>(buf, t, 15);
+      if constexpr (NG > 3) mid_group<real, TB, NT, SETS, 2>(buf, t, 15);
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const int b = group_base<LOC>(threadIdx.x + s * NT);
+        v2 w[16];
+        smem_ld<LOC>(buf, b, w);
+        centre(w, b);
+        smem_st<LOC>(buf, b, w);
+      }
+      __syncthreads();
+      if constexpr (NG > 3) mid_group<real, TB, NT, SETS, 2>(buf, -t, 15);
+      if constexpr (NG > 2) mid_group<real, TB, NT, SETS, 1>(buf, -t, 15);
+#pragma unroll
+      for (int s = 0; s < SETS; ++s) {
+        const int i0 = threadIdx.x + s * NT;
+        v2* p = W + at(i0);
+        v2 w[16];
+        smem_ld<LO0>(buf, i0, w);
+        gates(w, -t, 15);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) p[at0(r)] = w[r];
+      }
+      // (the next tile's first group writes the places this thread has just read)
+    }
+  }
+}
+
 template <typename real, int T, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) rot_backward_kernel(const __grid_constant__ RotArgs a) {
   using v2 = typename Cx<real>::v2;
@@ -588,19 +691,38 @@ int launch_outer(const RotArgs& a, int pass, cudaStream_t st) {
   return (int)cudaGetLastError();
 }
 
+// groups that hold high bits of the middle pass's tile
+template <int TB>
+int middle_groups(const RotArgs& a) {
+  const int c = TB - (a.n - a.T);
+  int ng = 1;
+  while (ng < Groups<TB>::N && Groups<TB>::lo(ng - 1) > c) ++ng;
+  return ng;
+}
+
 // the middle pass over tiles of 2^TB values
 template <typename real, int TB, int NT, int MINB>
 int launch_middle(const RotArgs& a, cudaStream_t st) {
-  using Gr = Groups<TB>;
-  const int nH = a.n - a.T, c = TB - nH;
+  const int ng = middle_groups<TB>(a);
   const size_t smem = tile_smem<real, TB>();
-  int ng = 1;
-  while (ng < Gr::N && Gr::lo(ng - 1) > c) ++ng;
-  const unsigned grid = (unsigned)(((a.nvec + a.vpb - 1) / a.vpb) * a.K) << (a.T - c);
+  const unsigned grid = (unsigned)(((a.nvec + a.vpb - 1) / a.vpb) * a.K) << (a.n - TB);
   if (ng == 1) rot_middle_kernel<real, TB, NT, MINB, 1><<<grid, NT, 0, st>>>(a);
   else if (ng == 2) rot_middle_kernel<real, TB, NT, MINB, 2><<<grid, NT, smem, st>>>(a);
   else if (ng == 3) rot_middle_kernel<real, TB, NT, MINB, 3><<<grid, NT, smem, st>>>(a);
-  else if constexpr (Gr::N >= 4) rot_middle_kernel<real, TB, NT, MINB, 4><<<grid, NT, smem, st>>>(a);
+  else if constexpr (Groups<TB>::N >= 4) rot_middle_kernel<real, TB, NT, MINB, 4><<<grid, NT, smem, st>>>(a);
+  else return (int)cudaErrorInvalidValue;
+  return (int)cudaGetLastError();
+}
+
+// the same, one CTA an SM and the next tile loaded ahead
+template <typename real, int TB, int NT>
+int launch_middle_ahead(const RotArgs& a, cudaStream_t st) {
+  const int ng = middle_groups<TB>(a);
+  const size_t smem = tile_smem<real, TB>();
+  const unsigned grid = std::min((unsigned)(((a.nvec + a.vpb - 1) / a.vpb) * a.K) << (a.n - TB),
+                                 (unsigned)std::max(1, device_sm_count()));
+  if (ng == 3) rot_middle_ahead_kernel<real, TB, NT, 3><<<grid, NT, smem, st>>>(a);
+  else if (ng == 4) rot_middle_ahead_kernel<real, TB, NT, 4><<<grid, NT, smem, st>>>(a);
   else return (int)cudaErrorInvalidValue;
   return (int)cudaGetLastError();
 }
@@ -620,6 +742,11 @@ int prepare_middle() {
   if constexpr (Groups<TB>::N >= 4)
     if (!e) e = allow((const void*)rot_middle_kernel<real, TB, NT, MINB, 4>, tile_smem<real, TB>());
   return e;
+}
+template <typename real, int TB, int NT>
+int prepare_middle_ahead() {
+  const int e = allow((const void*)rot_middle_ahead_kernel<real, TB, NT, 3>, tile_smem<real, TB>());
+  return e ? e : allow((const void*)rot_middle_ahead_kernel<real, TB, NT, 4>, tile_smem<real, TB>());
 }
 
 // The middle pass's tile for nH high bits: the small one, of which an SM runs
@@ -650,7 +777,7 @@ int launch_rot(const RotArgs& a, int pass, int c64, void* stream) {
     case 11: return launch_middle<double, 11, 128, 3>(a, st);
     case 12: return c64 ? launch_middle<float, 12, 256, 4>(a, st) : launch_middle<double, 12, 128, 3>(a, st);
     case 13: return launch_middle<double, 13, 256, 1>(a, st);
-    default: return launch_middle<float, 14, 1024, 1>(a, st);
+    default: return launch_middle_ahead<float, 14, 512>(a, st);
   }
 }
 
@@ -664,7 +791,7 @@ int prepare_rot(int n, int c64) {
     case 11: return prepare_middle<double, 11, 128, 3>();
     case 12: return c64 ? prepare_middle<float, 12, 256, 4>() : prepare_middle<double, 12, 128, 3>();
     case 13: return prepare_middle<double, 13, 256, 1>();
-    default: return prepare_middle<float, 14, 1024, 1>();
+    default: return prepare_middle_ahead<float, 14, 512>();
   }
 }
 

@@ -77,6 +77,20 @@ def test_rotated_run_matches_gather_at_every_split(n):
     s.close()
 
 
+@pytest.mark.parametrize("n,R", [(24, 3), (26, 2), (27, 1)])
+def test_large_middle_tiles(n, R):
+    """The middle pass over its large tile: a CTA takes several tiles in turn, of one
+    vector or more, and with few enough columns every group of the index has high bits."""
+    w = W.square_lattice(n, 1, seed=n, Bdir=(1, 1, 0))
+    s = F.System.from_dict(w)
+    g = F.run(s, R=R, M=3, T=T, seed=3, dtype="c64")
+    assert g["shape"]["passes"] == 3
+    x = empty_dev((s.dim, R), "c64")
+    F.start_block(s, x, R, 3, dtype="c64")
+    close(g, F.run(s, R=R, M=3, T=T, start="user", user_start=x, dtype="c64"), 2e-5)
+    s.close()
+
+
 def test_starts_that_may_be_sparse_keep_the_gather():
     """An isotropic system conserves S^z: from a basis state the run stays in its
     sector and ends where the sector ends."""
