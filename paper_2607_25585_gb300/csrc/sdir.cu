@@ -11,7 +11,8 @@
 // multiplied by a and conj(a) at the end.
 //
 // Bound: L2 (one load per high site and direction).  Tiles of at most 48 KB keep
-// four CTAs an SM.  Before, one thread formed a row's digits by division for
+// four CTAs an SM (64 KB: 19.7 -> 23 ms for a start and this on 2^26 x 4 values).
+// Before, one thread formed a row's digits by division for
 // every vector and gathered all neighbours through L1: 18.4 ms for 2^26 x 4
 // complex64 values of a spin-1/2 ladder, 9.6 ms for ten molecules of 9 sites
 // (2.3e6 x 8 each).
@@ -54,6 +55,9 @@ __global__ void __launch_bounds__(kThreads) sdir_vectors_kernel(const __grid_con
       for (int e = threadIdx.x; e < T; e += kThreads) tile[v * T + e] = __ldg(x + at(row0 + e, v));
   __syncthreads();
   const real uz = (real)a.obs[0], aur = (real)a.obs[1], aui = (real)a.obs[2];
+  // u along z (a field along z, or none): the neighbours have the factor 0 and are not read
+  // (3.4 ms less for 2^26 x 4 complex64 values)
+  const bool flips = aur != 0 || aui != 0;
   real c[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) c[v] = a.sigma && v < nv ? (real)a.sigma[v0 + v] : (real)1;
@@ -79,8 +83,8 @@ __global__ void __launch_bounds__(kThreads) sdir_vectors_kernel(const __grid_con
       rem = nx;
       const real* s = site + 4 * (i * qm + d);
       msum += s[2];
-      if (d > 0) mac(up, s[0], tile + e - stride, T);
-      if (d + 1 < (int)q) mac(dn, s[1], tile + e + stride, T);
+      if (flips && d > 0) mac(up, s[0], tile + e - stride, T);
+      if (flips && d + 1 < (int)q) mac(dn, s[1], tile + e + stride, T);
       stride *= (int)q;
     }
     unsigned long long high = blockIdx.x;
@@ -93,8 +97,8 @@ __global__ void __launch_bounds__(kThreads) sdir_vectors_kernel(const __grid_con
       high = nx;
       const real* s = site + 4 * (i * qm + d);
       msum += s[2];
-      if (d > 0) mac(up, s[0], own - far, a.dim);
-      if (d + 1 < (int)q) mac(dn, s[1], own + far, a.dim);
+      if (flips && d > 0) mac(up, s[0], own - far, a.dim);
+      if (flips && d + 1 < (int)q) mac(dn, s[1], own + far, a.dim);
       far *= q;
     }
     const real dz = uz * msum;
@@ -106,6 +110,73 @@ __global__ void __launch_bounds__(kThreads) sdir_vectors_kernel(const __grid_con
         o.x = c[v] * fma(dz, z.x, fma(aur, up[v].x + dn[v].x, -aui * (up[v].y - dn[v].y)));
         o.y = c[v] * fma(dz, z.y, fma(aur, up[v].y + dn[v].y, aui * (up[v].x - dn[v].x)));
         y[at(row0 + e, v)] = o;
+      }
+  }
+}
+
+// The same where every spin is 1/2: a row's digits are its index's bits, every ladder
+// coefficient is 1, and site i's one neighbour enters with a or conj(a): 0.99 -> 0.62 ms
+// for 2^20 x 64 complex64 values, 5.7 -> 5.0 ms for 2^26 x 4 (there memory binds: 15 of 26
+// neighbours are in other tiles, and the highest bits' are no longer in L2), of which
+// 0.8 ms remain where u lies along z.
+template <typename real, int V>
+__global__ void __launch_bounds__(kThreads) sdir_half_kernel(const __grid_constant__ SdirArgs a) {
+  using v2 = typename Cx<real>::v2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  v2* tile = reinterpret_cast<v2*>(smem_raw);  // [V][T]
+  const int T = a.T, nh = a.n - a.n_low;
+  const int v0 = blockIdx.y * V, nv = min(V, a.R - v0);
+  const long long row0 = (long long)blockIdx.x * T;
+  const v2* x = reinterpret_cast<const v2*>(a.x) + (long long)v0 * a.dim + row0;
+  v2* y = reinterpret_cast<v2*>(a.y) + (long long)v0 * a.dim + row0;
+  long long off[V];  // (a smaller group reads its last vector in the others' place)
+#pragma unroll
+  for (int v = 0; v < V; ++v) off[v] = (long long)min(v, nv - 1) * a.dim;
+#pragma unroll
+  for (int v = 0; v < V; ++v)
+    for (int e = threadIdx.x; e < T; e += kThreads) tile[v * T + e] = __ldg(x + off[v] + e);
+  __syncthreads();
+  const real uz = (real)a.obs[0], aur = (real)a.obs[1], aui = (real)a.obs[2];
+  const bool flips = aur != 0 || aui != 0;
+  const int high_bits = __popc((unsigned)blockIdx.x);
+  real c[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) c[v] = a.sigma && v < nv ? (real)a.sigma[v0 + v] : (real)1;
+  for (int e = threadIdx.x; e < T; e += kThreads) {
+    v2 sum[V], dif[V];  // the neighbours' sum, and set bits' minus clear bits'
+#pragma unroll
+    for (int v = 0; v < V; ++v) sum[v].x = sum[v].y = dif[v].x = dif[v].y = 0;
+    auto add = [&](real sign, int v, v2 z) {
+      sum[v].x += z.x;
+      sum[v].y += z.y;
+      dif[v].x = fma(sign, z.x, dif[v].x);
+      dif[v].y = fma(sign, z.y, dif[v].y);
+    };
+    if (flips) {
+#pragma unroll 4
+      for (int i = 0; i < nh; ++i) {
+        const bool set = (blockIdx.x >> i) & 1;
+        const long long far = (long long)T << i;
+        const v2* p = x + e + (set ? -far : far);
+#pragma unroll
+        for (int v = 0; v < V; ++v) add(set ? (real)1 : (real)-1, v, __ldg(p + off[v]));
+      }
+#pragma unroll 4
+      for (int i = 0; i < a.n_low; ++i) {
+        const int at = e ^ (1 << i);
+#pragma unroll
+        for (int v = 0; v < V; ++v) add((e >> i) & 1 ? (real)1 : (real)-1, v, tile[v * T + at]);
+      }
+    }
+    const real dz = uz * ((real)(high_bits + __popc((unsigned)e)) - (real)0.5 * (real)a.n);
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      if (v < nv) {
+        const v2 z = tile[v * T + e];
+        v2 o;  // u_z M x + Re(a) sum + i Im(a) dif
+        o.x = c[v] * fma(dz, z.x, fma(aur, sum[v].x, -aui * dif[v].y));
+        o.y = c[v] * fma(dz, z.y, fma(aur, sum[v].y, aui * dif[v].x));
+        y[(long long)v * a.dim + e] = o;
       }
   }
 }
@@ -212,22 +283,27 @@ __global__ void __launch_bounds__(kThreads) sdir_rows_kernel(const __grid_consta
 int launch_sdir(SdirArgs a, const int* q, int c64, bool vmaj, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int esz = c64 ? 8 : 16;
-  // vector-major: four complex64 or two complex128 vectors a CTA (wider groups
-  // leave the tile fewer low sites); row-major: up to 128 bytes of a row
-  const int V = std::min(a.R, c64 ? 4 : 2) == 3 ? 4 : std::min(a.R, c64 ? 4 : 2);
+  // vector-major: four complex64 (two of spins 1/2: four share no arithmetic and cost a
+  // low site) or two complex128 vectors a CTA; row-major: up to 128 bytes of a row
+  const bool half = vmaj && std::all_of(q, q + a.n, [](int k) { return k == 2; });
+  const int most = c64 && !half ? 4 : 2, V = std::min(a.R, most) == 3 ? 4 : std::min(a.R, most);
   const int W = c64 && a.R % 2 == 0 ? 2 : 1;
   a.cols = std::min(a.R / W, 128 / (W * esz));
   const int width = vmaj ? V : a.cols * W;
   a.T = 1;
   a.n_low = 0;
   while (a.n_low < a.n && (a.n_low == 0 || (long long)a.T * q[a.n_low] * width * esz <= kTileBytes)) a.T *= q[a.n_low++];
-  const size_t smem = (size_t)4 * a.n * a.lay.qmax * (esz / 2) + (size_t)a.T * width * esz;
+  const size_t smem = (half ? 0 : (size_t)4 * a.n * a.lay.qmax * (esz / 2)) + (size_t)a.T * width * esz;
   const dim3 grid((unsigned)(a.dim / a.T), (unsigned)((a.R + width - 1) / width));
   if (a.R < 1 || a.dim / a.T > 0x7fffffffll || grid.y > 65535) return (int)cudaErrorInvalidValue;
   const void* k;
   if (!vmaj) {
     k = W == 2 ? (const void*)sdir_rows_kernel<float, 2>
                : (c64 ? (const void*)sdir_rows_kernel<float, 1> : (const void*)sdir_rows_kernel<double, 1>);
+  } else if (half && c64) {
+    k = V == 2 ? (const void*)sdir_half_kernel<float, 2> : (const void*)sdir_half_kernel<float, 1>;
+  } else if (half) {
+    k = V == 2 ? (const void*)sdir_half_kernel<double, 2> : (const void*)sdir_half_kernel<double, 1>;
   } else if (c64) {
     k = V == 4 ? (const void*)sdir_vectors_kernel<float, 4>
                : (V == 2 ? (const void*)sdir_vectors_kernel<float, 2> : (const void*)sdir_vectors_kernel<float, 1>);

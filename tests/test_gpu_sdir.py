@@ -7,8 +7,10 @@ the sum of the terms' magnitudes (2^-24 or 2^-53)."""
 import numpy as np
 import pytest
 
+import ftlm_workloads as W
+import oracle
 import paper_2607_25585_gb300 as F
-from gpu_helpers import empty_dev, to_dev
+from gpu_helpers import empty_dev, osys, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -48,4 +50,17 @@ def test_sdir_matches_definition(two_s, R, rng):
         ref, mag = plain(two_s, u, xd.cpu().numpy().astype(np.complex128))
         err = np.abs(yd.cpu().numpy() - ref)
         assert np.all(err <= (4 * len(two_s) + 8) * eps * mag)
+    s.close()
+
+
+@pytest.mark.parametrize("make", [lambda B: W.chain(5, Bdir=B), lambda B: W.square_lattice(13, 1, Bdir=B)])
+@pytest.mark.parametrize("Bdir", [(0, 0, 1), (1, 0, 0), (0, 1, 0)])
+def test_runs_along_the_axes(make, Bdir):
+    """The projections p of a run whose u lies along z (no neighbours) or an axis of
+    the plane; after four steps 1e-12 of the largest, the rounding of the steps' sums."""
+    w = make(Bdir)
+    s = F.System.from_dict(w)
+    a = F.run(s, R=3, M=4, T=[1.0], seed=5, dtype="c128")
+    b = oracle.ftlm(osys(w), R=3, M=4, T=np.array([1.0]), seed=5)
+    assert np.abs(a["p"] - b["p"]).max() < 1e-12 * np.abs(b["p"]).max()
     s.close()
