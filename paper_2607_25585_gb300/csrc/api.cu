@@ -139,7 +139,8 @@ std::map<ShapeKey, Shape> g_shapes;
 bool has_shape_override(const ftlm_system* s, int R, int c64) {
   ShapeKey key{s->hs.n, s->hs.qmax, R, c64, (long long)s->hs.dim};
   std::lock_guard<std::mutex> lk(g_mu);
-  return g_shapes.count(key) != 0;
+  auto it = g_shapes.find(key);
+  return it != g_shapes.end() && !it->second.plain;
 }
 
 // the rotated-basis H.v may run: no shape was set, or the autotuner found it the fastest
@@ -1676,6 +1677,9 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
         sh.gvm_cube = cube;
         cands.push_back(sh);
       }
+    Shape sh = default_shape(R, c64);  // and the default plan where it is the tile gather
+    sh.plain = true;
+    cands.push_back(sh);
   }
   ftlm_status w = ensure_workspace(s, R, 1, c64);
   if (w != FTLM_OK) return w;
@@ -1703,7 +1707,9 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
   std::vector<ftlm_system*> one{s};
   for (const Shape& sh : cands) {
     Plan pl;
-    if (make_plan(one, R, c64, pl, &sh, sh.half_vm != 0 || sh.general_vm == 1) != FTLM_OK) continue;
+    if (make_plan(one, R, c64, pl, sh.plain ? nullptr : &sh, sh.half_vm != 0 || sh.general_vm == 1 || sh.plain) != FTLM_OK)
+      continue;
+    if (sh.plain && !pl.tile.V) continue;
     if (sh.half_K > 0 && (!pl.half.on || pl.half.vm != (sh.half_vm != 0))) continue;
     if (sh.general_vm == 1 && (!pl.gen_vm || (sh.gvm_cube > 0 && (!pl.gvm_cube || pl.gvm_V != sh.gvm_cube)))) continue;
     LaunchArgs a = pl.base;

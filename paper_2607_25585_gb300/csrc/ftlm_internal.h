@@ -202,6 +202,7 @@ struct Shape {
                            // of that many vectors, 0 = one row a thread, -1 = the cube with the default
                            // group size where a kernel exists for the top site's 2s+1 and R
   bool rot = false;        // autotuned shape: the rotated-basis H.v is faster for runs from random vectors
+  bool plain = false;      // autotuned shape: the default plan was the fastest (the tile gather)
 };
 
 // Kernel launchers (kernels.cu).  `V` is the number of complex values per

@@ -60,3 +60,22 @@ def test_tile_batch_matches_single_runs():
         for k in ("alpha", "beta", "p"):
             assert np.abs(r[k] - one[k]).max() < 2e-6 * max(np.abs(one[k]).max(), np.abs(one["beta"]).max() * (k == "alpha"))
         s.close()
+
+
+@pytest.mark.parametrize("name", ["ones", "cube"])
+def test_autotuned_runs(name):
+    """The autotuner times the tile gather with the other shapes: whichever it keeps,
+    the run's results are the default plan's, and a later product is right."""
+    s = F.System.from_dict(random_system(np.random.default_rng(12), SYSTEMS[name]))
+    kw = dict(R=4, M=6, T=T, seed=2, dtype="c64")
+    a, b = F.run(s, **kw), F.run(s, autotune=True, **kw)
+    x, y, z = (empty_dev((s.dim, 4), "c64") for _ in range(3))
+    F.start_block(s, x, 4, 2, dtype="c64")
+    F.apply_h(s, x, y, 4, "c64")
+    F.tune_shape(s, 4, "c64", -1)
+    F.apply_h(s, x, z, 4, "c64")
+    assert rel_l2(y.cpu().numpy(), z.cpu().numpy()) < 2e-6
+    scale = max(np.abs(b["beta"]).max(), np.abs(b["alpha"]).max())
+    for k in ("alpha", "beta"):
+        assert np.abs(a[k] - b[k]).max() < 2e-5 * scale
+    s.close()
