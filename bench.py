@@ -66,8 +66,29 @@ def algorithmic_flops_per_sv(two_s, epilogue=True):
     return float(flops)
 
 
+ROT_DIRECTIONS = 3  # rotated bases besides z that a planar geometry's tensors take
+
+
+def rotated(shp):
+    """A launch shape of the rotated-basis passes (spin-1/2 runs from random vectors)."""
+    return bool(shp.get("vector_major")) and shp.get("passes") == 3 and shp.get("cube_bits", 0) == 0
+
+
+def rotated_bytes_per_sv(directions=ROT_DIRECTIONS, esz=8):
+    """Bytes the three rotated-basis passes of one Lanczos step move per state x
+    vector: forward reads w', q_{j-1} and writes q_j and a block per direction,
+    middle reads and writes the direction blocks, backward reads them, q_j,
+    q_{j-1}, u and writes w'."""
+    return esz * (7 + 4 * directions)
+
+
 def gather_kernel_name(shp):
     """The H.v kernel a launch shape names."""
+    if rotated(shp):
+        return "rot_forward/middle/backward_kernel<float> (rotated-basis passes with the step's update)"
+    if shp.get("vector_major") and shp.get("site_cube", 0) > 0 and shp.get("tile_rows", 256) % 256:
+        return (f"tile_gather_kernel<{shp['site_cube']},{shp['group_vectors']}> (vector-major general gather over "
+                f"shared-memory tiles of {shp['tile_rows']} low-site bases, the step's w' in its epilogue)")
     if shp.get("vector_major") and shp.get("cube_bits", 0) > 0:
         return f"vm_kernel<float,{shp['cube_bits']}> (vector-major spin-1/2 gather)"
     if shp.get("vector_major") and shp.get("site_cube", 0) > 0:
@@ -221,14 +242,16 @@ def run_ours(args):
     hbm = peaks.get("hbm_gbs", 6778.0)
     line = None
     if rank == 0:
-        # dominant kernel: the fused H.v + Lanczos epilogue
+        # dominant kernel: the fused H.v + Lanczos step
         hv_per_launch_ms = hv_ms / max(1, hv_launches)
         flops_sv = algorithmic_flops_per_sv(w["two_s"])
         achieved = flops_sv * d * R / (hv_per_launch_ms / 1e3) / 1e12
         sm_max = clocks.get("sm_max_mhz") or peaks.get("sm_max_mhz", 2070.0)
         fp32_peak = SM_COUNT * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
         shp = results["shape"]
-        if shp.get("vector_major"):
+        if rotated(shp):
+            kname = gather_kernel_name(shp)
+        elif shp.get("vector_major"):
             kname = (f"vm_kernel<float,{shp['cube_bits']},{'multi' if shp['passes'] > 1 else 'single'}> "
                      f"(vector-major spin-1/2 gather{', %d passes' % shp['passes'] if shp['passes'] > 1 else ''})")
         elif shp["cube_bits"] > 0:
@@ -236,6 +259,14 @@ def run_ours(args):
                      f"{'multi' if shp['passes'] > 1 else 'single'}> (spin-1/2 register-cube gather)")
         else:
             kname = "rows_kernel<float,2,Lanczos> (general gather with the fused step)"
+        if rotated(shp):  # a launch: the three passes of one step
+            step_bytes = rotated_bytes_per_sv() * d * R
+            bound = {"bound": "hbm", "achieved": step_bytes / (hv_per_launch_ms / 1e3) / 1e9, "peak": hbm,
+                     "unit": "GB/s", "bytes_per_launch": step_bytes,
+                     "peak_note": "MEASURED_PEAKS.json hbm_gbs (measured copy bandwidth)"}
+        else:
+            bound = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
+                     "peak_note": "FP32 FMA peak = 152 SMs x 128 lanes x 2 flop x max SM clock (derived)"}
         traffic = measured_traffic(shp)
         precision = None if args.no_precision else precision_legs(F, T, stream, args, s, spec, results)
         plain = None if args.no_plain else plain_fp64(F, s, T, spec, stream, args)
@@ -247,14 +278,14 @@ def run_ours(args):
             "config": {"workload": f"open 4x5 s=1/2 lattice, all-pairs dipolar, d={d}, R={R} vectors, M={M} "
                                    "Lanczos steps, complex64 vectors, FP32 matvec, FP64 scalars/eigensolve/sums",
                        "d": d, "R": R, "M": M, "global_batch_vectors": R * ws, "parallelism": f"replicas x{ws}",
-                       "l2": "inputs larger than L2 (four 512 MB vector blocks: q_j, q_{j-1}, H q_j, u)"},
+                       "l2": "inputs larger than L2 (three 512 MB vector blocks, q_j, q_{j-1} and u, and three "
+                             "of the rotated bases)"},
             "hbm_roof_frac": value / ws * 32 / (hbm * 1e9),
-            "roofline": {"bound": "alu", "kernel": kname,
-                         "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s", "frac": achieved / fp32_peak,
+            "roofline": {**bound, "kernel": kname, "frac": bound["achieved"] / bound["peak"],
                          "traffic": traffic, "algorithmic_flops_per_sv": flops_sv,
                          "hv_ms_per_launch": hv_per_launch_ms, "launch_shape": results["shape"],
                          "launch_gap_ms_per_step": results["gap_ms"] / max(1, M - 1),
-                         "peak_note": "FP32 FMA peak = 152 SMs x 128 lanes x 2 flop x max SM clock (derived)"},
+                         },
             "hbm": {"bytes_per_sv": 32, "peak_gbs": hbm, "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)",
                     "frac": value / ws * 32 / (hbm * 1e9)},
             "plain_fp64": plain,
@@ -696,8 +727,8 @@ def run_profile_batch(args):
 
 def run_hv_only(args):
     """ftlm_apply_h alone: args.hv_only launches of H.v on the workload's
-    row-major [d][R] complex64 block (the row-major kernels, as a caller of
-    ftlm_apply_h gets them), timed with CUDA events."""
+    row-major [d][R] complex64 block (the kernels that a caller of
+    ftlm_apply_h gets), timed with CUDA events."""
     import torch
 
     import paper_2607_25585_gb300 as F
