@@ -117,7 +117,13 @@ uint64_t ftlm_system_table_bytes(const ftlm_system* sys);
  * matrix-vector product that Sec. II.C calls the heart of every Lanczos
  * procedure), evaluated row by row on the GPU from coupling tables: each
  * output row gathers its own terms, so there are no atomics and the result
- * is bitwise reproducible.
+ * is bitwise reproducible.  Which kernels run depends on the system and on this
+ * call alone: stored rows where they take at most 32 MB (complex128 on spins
+ * other than 1/2 and nvec >= 4: 2 GB), built on the first such call; for spin-1/2
+ * blocks the rotated-basis passes where every vector is dense and far from the
+ * ends of the dtype's range (found out on the device; else the gather); for
+ * other spins in complex64 the tile gather.  A call on a stream that is being
+ * captured takes the gathers that need nothing of the host.
  *  x, y   device blocks [dim][nvec] of dtype; must not overlap.
  *  nvec   1..512 (c64) or 1..256 (c128).
  *  stream cudaStream_t or NULL.
@@ -250,7 +256,8 @@ typedef struct {
   int kernel_launches;    /* all kernel launches in the run */
   uint64_t h2d_bytes;     /* host-to-device bytes copied by the run */
   uint64_t d2h_bytes;     /* device-to-host bytes copied by the run */
-  /* launch shape of the H.v launches (see ftlm_tune_shape) */
+  /* launch shape of the H.v launches (see ftlm_tune_shape); of the gather's plan where stored
+     rows or the one launch of a small run take its place */
   int cube_bits;          /* 0: general row kernel; 2..4: spin-1/2 register cubes */
   int passes;             /* launches per H.v (spin-1/2 multi-pass form: ceil(n / cube_bits); 3 with cube_bits 0:
                              the rotated-basis form of spin-1/2 runs from random vectors) */
