@@ -22,6 +22,9 @@
 // vectors: 16.1 -> 13.7 ms.  Coefficients with no imaginary part (all s+ s- ones, and s+
 // s+ ones of chains along an axis) take one packed FMA a value instead of two.
 // Tiles of 81 bases (9.3 ms) or 729 (8.4 ms, one CTA an SM) were slower.
+// Copying all the high sites' rows ahead through shared memory (8.1 ms on the chains,
+// 13.0 to 13.7 on the molecules) or the shifted tiles alone (7.2 and 13.3) did not pay:
+// the copies take the issue slots that the waits left.
 #include <cuda_runtime.h>
 
 #include <algorithm>
