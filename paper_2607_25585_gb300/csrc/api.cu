@@ -61,7 +61,7 @@ struct DevBuf {
     release();
     cudaError_t e = cudaMalloc(&p, b);
     if (e == cudaSuccess) bytes = b;
-    else p = nullptr;
+    else p = nullptr, cudaGetLastError();  // (reported here: the caller's next CUDA call must not find it)
     return e;
   }
 };
