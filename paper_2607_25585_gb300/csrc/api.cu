@@ -93,6 +93,7 @@ struct ftlm_system {
   cudaEvent_t ev_apply = nullptr;  // recorded after the last use of Ta, Tb
   std::unique_ptr<RotDirs> rot;  // the rotated-basis H.v's directions, if the system has any
   DevBuf rD[2];          // its diagonal tables [K + 1][dim] and phases, [c64]
+  cudaEvent_t ev_rot[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
   DevBuf rW, rpart;      // its intermediate blocks; partial sums and arrival counters
   DevBuf rows[2];        // stored rows of a small system, [c64]: values, columns, counts
   cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written (on own_stream)
@@ -643,24 +644,34 @@ ftlm_status ensure_unit_tables(ftlm_system* s, int K, int c64, cudaStream_t st) 
 
 size_t rot_phase_bytes(int c64) { return (size_t)kRotMaxK * (kRotMaxN + 1) * (c64 ? 8 : 16); }
 
-// Its tables, built once per system and precision on stream st; ok = false when
-// they do not fit in memory (the gather then runs).
+// Its tables, written once per system and precision (the caller holds apply_mu).
+// The stream that wrote them may be another call's -- a run's own stream, which a
+// product of one vector does not wait for, nor one after a run that failed before
+// its end -- so st waits for the event recorded behind the launches that write.
+// ok = false when they do not fit in memory (the gather then runs).
 ftlm_status ensure_rot_tables(ftlm_system* s, const RotPlan& rp, int c64, cudaStream_t st, bool& ok) {
   ok = false;
   const size_t d = (size_t)s->hs.dim, real = c64 ? 4 : 8;
   DevBuf& D = s->rD[c64 ? 1 : 0];
+  cudaEvent_t& ev = s->ev_rot[c64 ? 1 : 0];
   if (prepare_rot(s->hs.n, c64) != 0) return FTLM_OK;
+  if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
   if (!D.p) {
     const size_t bytes = (size_t)(rp.K + 1) * d * real + rot_phase_bytes(c64);
     if (D.ensure(bytes) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
-    for (int k = 0; k <= rp.K; ++k) {
+    int e = 0;
+    for (int k = 0; k <= rp.K && !e; ++k) {
       RotForm f = s->rot->form[k];
       f.T = k > 0 ? rp.T : 0;
       f.b = rot_run_bits(s->hs.n, c64);
-      CKI(launch_rot_table(f, static_cast<char*>(D.p) + (size_t)k * d * real, c64, st));
+      e = launch_rot_table(f, static_cast<char*>(D.p) + (size_t)k * d * real, c64, st);
     }
-    CKI(launch_rot_phases(s->hs.n, *s->rot, static_cast<char*>(D.p) + bytes - rot_phase_bytes(c64), c64, st));
+    if (!e) e = launch_rot_phases(s->hs.n, *s->rot, static_cast<char*>(D.p) + bytes - rot_phase_bytes(c64), c64, st);
+    if (!e) e = (int)cudaEventRecord(ev, st);
+    if (e) D.release();
+    CKI(e);
   }
+  CK(cudaStreamWaitEvent(st, ev, 0));
   ok = true;
   return FTLM_OK;
 }
@@ -2089,7 +2100,7 @@ void ftlm_system_destroy(ftlm_system* s) {
   cudaEventDestroy(s->ev_in);
   cudaEventDestroy(s->ev_out);
   cudaEventDestroy(s->ev_apply);
-  for (cudaEvent_t e : s->ev_rows)
+  for (cudaEvent_t e : {s->ev_rows[0], s->ev_rows[1], s->ev_rot[0], s->ev_rot[1]})
     if (e) cudaEventDestroy(e);
   cudaStreamDestroy(s->own_stream);
   delete s;
