@@ -14,10 +14,12 @@
 // Directions besides z: x and y when every tensor is diagonal; three in the xy
 // plane 60 degrees apart when z is a principal axis of every tensor (planar
 // geometries); else the five axes of an icosahedron around z (with z, their
-// projectors span the symmetric tensors).  Each set is a tight frame, so the
-// |D_k| stay on the scale of |H| and nothing cancels: measured in FP32 against
-// FP64 on random vectors, the relative error is 1.1e-7 (16 sites) where the
-// gather's is 2.8e-7.
+// projectors span the symmetric tensors).  The sets are tight frames (the six
+// lines within 3e-8), so the |D_k| stay on the scale of |H| and nothing cancels.
+// Complex64 runs of five steps against complex128, 14 to 27 sites in and out of
+// the plane, five to eight seeds each, root mean square of the relative error:
+// alpha 4e-8 to 9e-8 (16e-8 at 14 sites) where the gather's is 4e-8 to 11e-8 (63e-8),
+// beta and p 3e-8 to 5e-8 in both.
 //
 // The gate.  All u_k have the same polar angle theta; with t = tan(theta / 2)
 // and the azimuth's phase e^{-i phi_k} taken out per down spin,
@@ -821,6 +823,33 @@ int rot_tile_bits(int n, int c64) {
   return n <= 23 ? 11 : (n <= 26 ? 13 : 0);
 }
 
+// Row k: the a_k of A = a_0 z z^T + sum_k a_k u_k u_k^T as combinations of A's
+// elements xx, yy, zz, xy, xz, yz: the inverse of the 6 x 6 matrix whose columns
+// are those of the projectors (Gauss-Jordan; its condition number is 2.2).
+static void six_lines(const double (*u)[3], double (&inv)[6][6]) {
+  double m[6][12] = {};
+  for (int c = 0; c < 6; ++c) {
+    const double z[3] = {0.0, 0.0, 1.0}, *w = c == 0 ? z : u[c - 1];
+    const double e[6] = {w[0] * w[0], w[1] * w[1], w[2] * w[2], w[0] * w[1], w[0] * w[2], w[1] * w[2]};
+    for (int r = 0; r < 6; ++r) m[r][c] = e[r];
+    m[c][6 + c] = 1.0;
+  }
+  for (int c = 0; c < 6; ++c) {
+    int p = c;
+    for (int r = c + 1; r < 6; ++r)
+      if (std::fabs(m[r][c]) > std::fabs(m[p][c])) p = r;
+    for (int k = 0; k < 12; ++k) std::swap(m[c][k], m[p][k]);
+    const double d = 1.0 / m[c][c];
+    for (int k = 0; k < 12; ++k) m[c][k] *= d;
+    for (int r = 0; r < 6; ++r) {
+      const double f = r == c ? 0.0 : m[r][c];
+      for (int k = 0; k < 12; ++k) m[r][k] -= f * m[c][k];
+    }
+  }
+  for (int r = 0; r < 6; ++r)
+    for (int k = 0; k < 6; ++k) inv[r][k] = m[r][6 + k];
+}
+
 // The directions and diagonal forms of a spin-1/2 system (see the top of the
 // file); false when it has none (a pair tensor that is not symmetric) or no
 // pair couplings at all.
@@ -860,8 +889,14 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
     d.az.den = 5;
     ct = 1.0 / std::sqrt(5.0);
   }
-  const double st = std::sqrt(1.0 - ct * ct);
-  d.t = st / (1.0 + ct);
+  // The gates multiply by t in the product's precision and the tables undo
+  // (1 + t^2)^n: t has to be one number in both.  So the polar angle is the one
+  // whose t is an FP32 value (1 already is; 0.618... moves by 2.7e-8, and the six
+  // lines are then no longer exactly an icosahedron's).  With t rounded in the gates
+  // alone every product in complex64 was off by n x 1.5e-8 of itself (3e-7 at 20 sites).
+  d.t = (double)(float)(std::sqrt(1.0 - ct * ct) / (1.0 + ct));
+  ct = (1.0 - d.t * d.t) / (1.0 + d.t * d.t);
+  const double st = 2.0 * d.t / (1.0 + d.t * d.t);
   const int K = d.K;
   double u[kRotMaxK][3];
   for (int k = 0; k < K; ++k) {
@@ -870,6 +905,9 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
     u[k][2] = ct;
   }
   if (K == 2) u[1][0] = 0.0;  // (cos(pi / 2))
+  const double inv_plane = 1.0 / (2.5 * st * st), inv_z = 1.0 / (1.0 + 5.0 * ct * ct);  // (K = 5) of sum u u^T over the six lines
+  double six[6][6] = {};  // (K = 5) a_k of each element of A
+  if (K == 5) six_lines(u, six);
   for (int k = 0; k <= K; ++k) {
     RotForm& f = d.form[k];
     f.n = n;
@@ -879,12 +917,12 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
   for (int i = 0; i < n; ++i) {
     const double h[3] = {2.0 * t[L.off_hp + 2 * i], -2.0 * t[L.off_hp + 2 * i + 1], t[L.off_hz + i]};
     d.form[0].c0 += t[L.off_iondiag + i * L.qmax];  // (s.e)^2 = 1/4: the same for both digits
-    // sum_k u_k u_k^T over the set (with z for K = 5) is a multiple of the identity on what it spans
+    // h = sum_k (u_k . S^-1 h) u_k, S = sum_k u_k u_k^T over the set (with z for K = 5): diagonal
     for (int k = 0; k < K; ++k) {
-      const double hu = h[0] * u[k][0] + h[1] * u[k][1] + h[2] * u[k][2];
-      d.form[k + 1].h[i] = K == 2 ? hu : (K == 3 ? 2.0 / 3.0 * hu : 0.5 * hu);
+      const double hp = h[0] * u[k][0] + h[1] * u[k][1];
+      d.form[k + 1].h[i] = K == 2 ? hp : (K == 3 ? 2.0 / 3.0 * hp : inv_plane * hp + inv_z * h[2] * u[k][2]);
     }
-    d.form[0].h[i] = K == 5 ? 0.5 * h[2] : h[2];
+    d.form[0].h[i] = K == 5 ? inv_z * h[2] : h[2];
   }
   for (int i = 0; i < n; ++i)
     for (int j = i + 1; j < n; ++j) {
@@ -893,15 +931,8 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
       const double xx = 2.0 * (pm + pp), yy = 2.0 * (pm - pp), zz = t[L.off_zz + ij];
       const double xy = -2.0 * t[L.off_pp + 2 * ij + 1];
       const double xz = 2.0 * t[L.off_rho + 2 * ij], yz = -2.0 * t[L.off_rho + 2 * ij + 1];
-      // A = sum_k a_k u_k u_k^T.  Projectors of a tight frame of K + 1 (or K in the plane) lines:
+      // A = sum_k a_k u_k u_k^T.  In the plane, projectors of a tight frame:
       // a_k = alpha (u_k.A.u_k) + gamma tr A solves it.
-      double A[3][3] = {{xx, xy, xz}, {xy, yy, yz}, {xz, yz, zz}};
-      auto quad = [&](const double* w) {
-        double s = 0.0;
-        for (int p = 0; p < 3; ++p)
-          for (int r = 0; r < 3; ++r) s += w[p] * A[p][r] * w[r];
-        return s;
-      };
       if (K == 2) {
         d.form[0].a[q] = zz;
         d.form[1].a[q] = xx;
@@ -909,13 +940,17 @@ bool rot_directions(const HostSystem& hs, RotDirs& d) {
       } else if (K == 3) {
         d.form[0].a[q] = zz;
         // in the plane: sum_k (u_k.A.u_k) u_k u_k^T = 3/8 (2 A + tr A 1), sum_k u_k u_k^T = 3/2 1
-        for (int k = 0; k < 3; ++k) d.form[k + 1].a[q] = 4.0 / 3.0 * quad(u[k]) - (xx + yy) / 3.0;
+        for (int k = 0; k < 3; ++k) {
+          const double quad = xx * u[k][0] * u[k][0] + 2.0 * xy * u[k][0] * u[k][1] + yy * u[k][1] * u[k][1];
+          d.form[k + 1].a[q] = 4.0 / 3.0 * quad - (xx + yy) / 3.0;
+        }
       } else {
-        // six lines: sum_k (u_k.A.u_k) u_k u_k^T = 2/5 (2 A + tr A 1), sum_k u_k u_k^T = 2 1
-        const double tr = xx + yy + zz;
-        const double z[3] = {0.0, 0.0, 1.0};
-        d.form[0].a[q] = 1.25 * quad(z) - 0.25 * tr;
-        for (int k = 0; k < 5; ++k) d.form[k + 1].a[q] = 1.25 * quad(u[k]) - 0.25 * tr;
+        const double A[6] = {xx, yy, zz, xy, xz, yz};
+        for (int k = 0; k < 6; ++k) {
+          double a = 0.0;
+          for (int r = 0; r < 6; ++r) a += six[k][r] * A[r];
+          d.form[k].a[q] = a;
+        }
       }
     }
   return true;
