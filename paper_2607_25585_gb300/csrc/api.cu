@@ -96,7 +96,7 @@ struct ftlm_system {
   cudaEvent_t ev_rot[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
   DevBuf rW, rpart;      // its intermediate blocks; partial sums and arrival counters
   DevBuf rows[2];        // stored rows of a small system, [c64]: values, columns, counts
-  cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written (on own_stream)
+  cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
   bool rows_done[2] = {false, false};           // that event has been seen complete
   std::mutex rows_mu;
   bool apply_used = false;
@@ -756,8 +756,9 @@ size_t stored_limit(const ftlm_system* s, int c64, int n = 1) {
   return !s->hs.all_half && !c64 ? std::max(kStoredL2, ((size_t)2 << 30) / n) : kStoredL2;
 }
 
-// The system's stored rows for work on stream st: written on the first call (on
-// the system's own stream; st waits for them).  ok = false: the gathers run -- the
+// The system's stored rows for work on stream st: written by the first call, on
+// its st (not on the system's own stream, which another thread's run may be
+// capturing); other streams wait for them.  ok = false: the gathers run -- the
 // rows are too large, or beyond L2 for a call of fewer than four products of a
 // vector (writing them costs about two), or st is being captured.  The choice
 // depends on the call alone, so a repeated call gives the same bits.
@@ -779,8 +780,8 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long produ
       int e = launch_stored_build(c64 ? s->tab_f.p : s->tab_d.p, s->hs.lay,
                                   reinterpret_cast<const long long*>(s->stride.p), reinterpret_cast<const int*>(s->q.p),
                                   s->hs.n, (int)d, (int)S, reinterpret_cast<int*>(p + d * S * esz), p,
-                                  reinterpret_cast<int*>(p + d * S * (esz + 4)), c64, s->own_stream);
-      if (!e) e = (int)cudaEventRecord(s->ev_rows[k], s->own_stream);
+                                  reinterpret_cast<int*>(p + d * S * (esz + 4)), c64, st);
+      if (!e) e = (int)cudaEventRecord(s->ev_rows[k], st);
       if (e) b.release();
       CKI(e);
     }

@@ -1,6 +1,7 @@
 """GPU: what a system's calls share -- tables written by one call and read by
 another on a different stream or from another host thread."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -65,4 +66,38 @@ def test_product_after_a_run_that_failed_before_its_end():
         F.run(s, R=1, M=100000, T=T, seed=1, dtype="c64", symmetric=True)
     assert e.value.status == 2
     assert torch.equal(product(s, x, stream), ref)
+    s.close()
+
+
+def test_first_product_while_a_run_is_captured():
+    """The rows of a small system are written by the first call that wants them; a run
+    of another precision that another thread is capturing at that moment takes no
+    part in it."""
+    torch = torch_cuda()
+    w = W.ring(N=6, two_s=2)
+    kw = dict(R=2, M=150, T=T, seed=1, dtype="c64", reorth=True)     # (the row-major gather; a long capture)
+    want = want_run = None
+    for trial in range(12):
+        s = F.System.from_dict(w)
+        x = dense(s, 3, 11).to(torch.complex128)
+        y = torch.zeros_like(x)
+        stream = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        out = {}
+        run = threading.Thread(target=lambda: out.update(F.run(s, **kw)))
+        run.start()
+        time.sleep(0.002 * (trial % 6))
+        F.apply_h(s, x, y, 3, "c128", stream=stream)
+        stream.synchronize()
+        run.join()
+        want, want_run = (y, out) if want is None else (want, want_run)
+        assert torch.equal(y, want), trial
+        for k in ("alpha", "beta", "p", "lnZ"):
+            assert np.array_equal(out[k], want_run[k]), (trial, k)
+        s.close()
+    s = F.System.from_dict(w)
+    z = torch.zeros_like(want)
+    F.apply_h(s, dense(s, 3, 11).to(torch.complex128), z, 3, "c128")
+    torch.cuda.synchronize()
+    assert torch.equal(z, want)
     s.close()
