@@ -760,8 +760,8 @@ size_t stored_limit(const ftlm_system* s, int c64, int n = 1) {
 // its st (not on the system's own stream, which another thread's run may be
 // capturing); other streams wait for them.  ok = false: the gathers run -- the
 // rows are too large, or beyond L2 for a call of fewer than four products of a
-// vector (writing them costs about two), or st is being captured.  The choice
-// depends on the call alone, so a repeated call gives the same bits.
+// vector (writing them costs about two).  The choice depends on the call alone, so
+// a repeated call gives the same bits.  st must not be capturing.
 ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long products, cudaStream_t st, StoredRows& r,
                           bool& ok) {
   ok = false;
@@ -769,7 +769,6 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long produ
   const size_t d = (size_t)s->hs.dim, esz = c64 ? 8 : 16;
   const size_t S = (size_t)stored_row_bound(s->hs);
   if (S == 0 || d > limit || d * S * (esz + 4) + d * 4 > (products < 4 ? kStoredL2 : limit)) return FTLM_OK;
-  if (stream_captures(st)) return FTLM_OK;
   std::lock_guard<std::mutex> lk(s->rows_mu);
   DevBuf& b = s->rows[k];
   if (!s->rows_done[k]) {
@@ -1636,7 +1635,7 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
   {  // stored rows have no shape to choose, and every gather is slower on systems that small
     StoredRows r;
     bool ok = false;
-    ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), R, st, r, ok);
+    ftlm_status rs = stream_captures(st) ? FTLM_OK : ensure_stored(s, c64, stored_limit(s, c64), R, st, r, ok);
     if (rs != FTLM_OK || ok) return rs;
   }
   std::vector<Shape> cands;
@@ -1827,10 +1826,16 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   if (v != FTLM_OK) return v;
   const int c64 = dtype == FTLM_C64;
   ftlm_system* s = const_cast<ftlm_system*>(cs);
-  if (!has_shape_override(s, nvec, c64)) {  // small systems: stored rows
+  const cudaStream_t st = pick_stream(s, stream);
+  // Everything but the gathers on the caller's layout keeps blocks, tables or events
+  // of the system, which a captured call may neither allocate nor write (a table's
+  // writing would only happen when the graph runs) nor wait for: such a call takes
+  // those gathers.  So does one whose shape was set.
+  const bool plain = stream_captures(st) || has_shape_override(s, nvec, c64);
+  if (!plain) {  // small systems: stored rows
     StoredArgs a;
     bool ok = false;
-    ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), nvec, pick_stream(s, stream), a.rows, ok);
+    ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), nvec, st, a.rows, ok);
     if (rs != FTLM_OK) return rs;
     if (ok) {
       a.x = x;
@@ -1838,14 +1843,13 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
       a.dim = (long long)s->hs.dim;
       a.rs = a.R = nvec;
       a.vs = 1;
-      CKI(launch_stored_product(a, stored_group(s->hs.dim, nvec), c64, pick_stream(s, stream)));
+      CKI(launch_stored_product(a, stored_group(s->hs.dim, nvec), c64, st));
       return FTLM_OK;
     }
   }
   Plan pl;
   std::vector<ftlm_system*> one{s};
-  const cudaStream_t st = pick_stream(s, stream);
-  if (!has_shape_override(s, nvec, c64) && (nvec > 1 || !stream_captures(st))) {
+  if (!plain) {
     // spin-1/2 blocks on the default plan: transpose to vector-major (one vector
     // is), the rotated-basis passes and, when these find the block not to be
     // dense, the runs' gather; transpose back
@@ -1853,7 +1857,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
     ftlm_status ps = make_plan(one, nvec, c64, vp, nullptr, true);
     RotPlan rp;
     const bool vm = ps == FTLM_OK && vp.half.on && vp.half.vm && vp.half.passes == 1 && !vp.half.hybrid;
-    bool rot = vm && !stream_captures(st) && rot_shape(s, nvec, c64, rp);
+    bool rot = vm && rot_shape(s, nvec, c64, rp);
     if (vm && (nvec > 1 || rot)) {
       // the system's blocks are shared by its calls: a call waits for the
       // previous one's kernels (on whatever stream it ran) before reusing them
@@ -1913,7 +1917,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
       }
     }
   }
-  if (c64 && nvec > 1 && !has_shape_override(s, nvec, c64) && !stream_captures(st)) {
+  if (c64 && nvec > 1 && !plain) {
     // other spins, complex64 blocks: transposed to the tile gather's layout and back
     Plan tp;
     ftlm_status ps = make_plan(one, nvec, c64, tp, nullptr, true);

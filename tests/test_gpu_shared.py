@@ -7,8 +7,9 @@ import numpy as np
 import pytest
 
 import ftlm_workloads as W
+import oracle
 import paper_2607_25585_gb300 as F
-from gpu_helpers import empty_dev, torch_cuda
+from gpu_helpers import empty_dev, osys, rel_l2, torch_cuda
 
 pytestmark = pytest.mark.gpu
 T = np.array([0.5, 5.0])
@@ -100,4 +101,38 @@ def test_first_product_while_a_run_is_captured():
     F.apply_h(s, dense(s, 3, 11).to(torch.complex128), z, 3, "c128")
     torch.cuda.synchronize()
     assert torch.equal(z, want)
+    s.close()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+@pytest.mark.parametrize("nvec", [1, 4])
+@pytest.mark.parametrize("system", ["halves", "ones"])
+def test_captured_product_leaves_the_system_usable(system, nvec, warm):
+    """A product on a capturing stream takes nothing of the system's blocks, tables and
+    events, whether earlier calls have made them or not: it replays, and products
+    and runs after it work.  (200 roundings: 1e-6 of the norm.)"""
+    torch = torch_cuda()
+    w = W.square_lattice(4, 4, seed=3) if system == "halves" else W.chain(10, Bdir=(0.3, -0.2, 0.9))
+    s = F.System.from_dict(w)
+    x = dense(s, nvec, 5)
+    ref = oracle.apply_h(osys(w), x.cpu().numpy().astype(np.complex128))
+    y = torch.zeros_like(x)
+    torch.cuda.synchronize()
+    if warm:
+        F.apply_h(s, x, y, nvec, "c64")
+        F.run(s, R=nvec, M=3, T=T, seed=1, dtype="c64")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        F.apply_h(s, x, y, nvec, "c64")
+    y.zero_()
+    z = torch.zeros_like(x)
+    F.apply_h(s, x, z, nvec, "c64")           # before the graph has ever run
+    torch.cuda.synchronize()
+    assert rel_l2(z.cpu().numpy(), ref) < 1e-6
+    a = F.run(s, R=nvec, M=3, T=T, seed=1, dtype="c64")
+    g.replay()
+    torch.cuda.synchronize()
+    assert rel_l2(y.cpu().numpy(), ref) < 1e-6
+    b = F.run(s, R=nvec, M=3, T=T, seed=1, dtype="c64")
+    assert np.array_equal(a["alpha"], b["alpha"])
     s.close()
