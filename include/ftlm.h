@@ -115,15 +115,21 @@ uint64_t ftlm_system_table_bytes(const ftlm_system* sys);
 /*
  * ftlm_apply_h -- y = H x for a block of nvec vectors, matrix-free (the
  * matrix-vector product that Sec. II.C calls the heart of every Lanczos
- * procedure), evaluated row by row on the GPU from coupling tables: each
- * output row gathers its own terms, so there are no atomics and the result
- * is bitwise reproducible.  Which kernels run depends on the system and on this
- * call alone: stored rows where they take at most 32 MB (complex128 on spins
- * other than 1/2 and nvec >= 4: 2 GB), built on the first such call; for spin-1/2
- * blocks the rotated-basis passes where every vector is dense and far from the
- * ends of the dtype's range (found out on the device; else the gather); for
- * other spins in complex64 the tile gather.  A call on a stream that is being
- * captured takes the gathers that need nothing of the host.
+ * procedure), evaluated on the GPU from coupling tables, without atomics on
+ * values, so a repeated call gives the same bits.  Which kernels run depends on
+ * the system, on this call and, within a block, on each vector by itself: stored
+ * rows where they take at most 32 MB (complex128 on spins other than 1/2 and
+ * nvec >= 4: 2 GB), built on the first such call; for spin-1/2 blocks the
+ * rotated-basis passes; for other spins in complex64 the tile gather; else, and
+ * on a stream that is being captured, gathers that keep nothing.  Where the
+ * memory for one of them cannot be had, the gathers run.
+ * Rounding: a gathered row's error is relative to the sum of its terms'
+ * magnitudes, and rows that H does not reach are exactly zero.  The
+ * rotated-basis passes' is relative to the whole vector, so they take only the
+ * vectors whose values are spread like a complex Gaussian's (found out on the
+ * device): no zeros, at most 1 in 32 of |x|^2 2^-12 below the largest, 1 in 2^11
+ * 2^-18 below, 1 in 2^17 2^-24 below, and far from the ends of the dtype's range;
+ * the block's other vectors take the gather.
  *  x, y   device blocks [dim][nvec] of dtype; must not overlap.
  *  nvec   1..512 (c64) or 1..256 (c128).
  *  stream cudaStream_t or NULL.

@@ -1851,8 +1851,8 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   std::vector<ftlm_system*> one{s};
   if (!plain) {
     // spin-1/2 blocks on the default plan: transpose to vector-major (one vector
-    // is), the rotated-basis passes and, when these find the block not to be
-    // dense, the runs' gather; transpose back
+    // is), the rotated-basis passes, the runs' gather for the vectors that these
+    // found not to be dense; transpose back
     Plan vp;
     ftlm_status ps = make_plan(one, nvec, c64, vp, nullptr, true);
     RotPlan rp;
@@ -1874,7 +1874,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
         CK(grow(s->Ta, block));
         CK(grow(s->Tb, block));
       }
-      const size_t sbytes = sizeof(RotDensity) * nvec + 16;
+      const size_t sbytes = (sizeof(RotDensity) + sizeof(int)) * nvec;
       if (rot) rot = grow(s->Tw, block / nvec * rp.group * rp.K) == cudaSuccess && grow(s->Ts, sbytes) == cudaSuccess;
       cudaGetLastError();
       if (nvec > 1 || rot) {

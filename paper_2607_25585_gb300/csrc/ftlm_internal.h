@@ -176,7 +176,7 @@ struct LaunchArgs {
   // Re<q_j|w'> and <q_j|u>; its last CTA sets alpha_j and p_j.  The rest of
   // the step, w = w' - alpha_j sigma_j q_j with |w|^2, is kModeUpdate.
   int fused_step = 0;
-  // vector-major one-pass gather: run only when this flag is set (null: always)
+  // vector-major one-pass gather: only the vectors whose flag is set (null: all)
   const int* only_if = nullptr;
   // vector-major one-pass gather: the system's per-unit coefficient tables
   // (launch_vm_unit_tables), or nullptr to build them in the kernel
@@ -292,11 +292,14 @@ struct RotDirs {
   RotForm form[kRotMaxK + 1];  // z, then the K directions
 };
 
-// statistics of one vector: biased binary exponents of |x|^2
+// Statistics of one vector, from its tiles: biased binary exponents of |x|^2 (the
+// largest of a tile; kRotBottom minus the smallest such) and how many values lie
+// 2^-12, 2^-18 and 2^-24 below their tile's largest.
+constexpr int kRotBottom = 1 << 12;
 struct RotDensity {
-  int largest;
-  unsigned zeros, arrived, pad;
-  unsigned long long sum;
+  int top, bottom;
+  int c12, c18, c24;
+  unsigned arrived;
 };
 
 struct RotArgs {
@@ -305,7 +308,7 @@ struct RotArgs {
   long long dim = 0;
   int vec0 = 0, nvec = 0;      // the launch's vectors of the block
   int vecW = 0;                // the vector whose W_0 is at W
-  int vpb = 1;                 // middle pass: vectors a CTA takes one after another (its D values stay in registers)
+  int vpb = 1;                 // middle pass: vectors a CTA takes one after another (D then comes from L1)
   void* x = nullptr;           // q_j of vector 0 (vector-major block)
   void* y = nullptr;           // q_{j-1}, overwritten by w'; or H x
   const void* u = nullptr;
@@ -321,7 +324,7 @@ struct RotArgs {
   double* partials = nullptr;  // [R][tiles][3]
   unsigned* counters = nullptr;  // [R], zero between launches
   RotDensity* density = nullptr;  // [R], zeroed: a product on a caller's block takes its statistics
-  int* sparse = nullptr;          // set by them: the later passes return
+  int* sparse = nullptr;          // [R], zeroed: set by them for the vectors the passes leave to the gather
 };
 
 bool rot_directions(const HostSystem& hs, RotDirs& d);

@@ -53,9 +53,11 @@
 //
 // Its error is relative to the whole vector, where a gathered row's is relative
 // to that row's terms, and a value that is not finite reaches every row.  So
-// ftlm_apply_h takes these passes only for blocks that are dense and far from
-// overflow: the forward pass takes the vectors' statistics as it reads them, and
-// the other passes return, and the gather after them runs, when one is not.
+// ftlm_apply_h takes these passes only for vectors whose values are spread like a
+// Gaussian's (vector_density): no row is then much smaller than the vector but
+// those few that a Gaussian vector has too.  The forward pass takes each vector's
+// statistics as it reads it; for one that fails, the passes return and the gather
+// after them runs.
 //
 // Bound: memory.  A step moves 8 (7 + 4 K) bytes a value in complex64 (152 for
 // K = 3), against 56 for the gather, but the gather's C(n, 2) flips take 3.5 ms
@@ -169,45 +171,107 @@ __device__ __forceinline__ void stage_phases(typename Cx<real>::v2* ph, const Ro
 __device__ __forceinline__ int exponent_of(float s) { return (__float_as_int(s) >> 23) & 0xff; }
 __device__ __forceinline__ int exponent_of(double s) { return (__double2hiint(s) >> 20) & 0x7ff; }
 
-// Adds the exponents of |x|^2 of the CTA's values to the vector's statistics; the
-// vector's last CTA raises a.sparse[0] unless the vector is dense: at most one
-// zero in 1024, the largest |x|^2 within 2^12 of the (geometric) mean -- a
-// Gaussian vector stays within 2^6 at 2^28 values -- and far from overflow.
-// Integer sums: the decision does not depend on the order of the CTAs.
-template <typename real, int NT>
-__device__ __forceinline__ void vector_density(const RotArgs& a, int v, int tiles, int largest, int sum, int zeros) {
-  __shared__ int red[NT / 32][3];
+// Values a dense vector may have below its largest |x|^2: of n values 8 + n / 2^5
+// at 2^-12, 8 + n / 2^11 at 2^-18 and 8 + n / 2^17 at 2^-24.  A complex Gaussian
+// vector has an eighth to half of the fractions there (its largest of 2^11 to 2^28
+// values is 2^3 to 2^5 times the mean, and the fraction below s times the mean is
+// s); 8 is its Poisson tail where less than one value is expected.
+struct FewBelow {
+  int c12, c18, c24;
+  __device__ bool in(long long n) const { return c12 <= 8 + (n >> 5) && c18 <= 8 + (n >> 11) && c24 <= 8 + (n >> 17); }
+};
+
+// Whether the CTA's values let the vector be dense: spread like those of a complex
+// Gaussian -- no zero, few far below the largest (FewBelow, over each CTA's values
+// and over the vector's), the CTAs' largest within 2^4 of each other -- and far
+// from the ends of the range.  A CTA that says no raises a.sparse[v] and the
+// vector's other CTAs return as they start; the sums over all CTAs are the last
+// one's to judge.  Integers throughout: the outcome does not depend on the order of
+// the CTAs, nor on the other vectors of the block.  A vector that is not dense costs
+// the gather and a little: 64 basis states of 20 sites 3.73 -> 3.85 ms, one vector of
+// them 0.139 -> 0.155 ms (the passes' launches), at most the forward pass (4.06 ms)
+// where only the sums tell; with one flag for the block, raised by its last CTA, one
+// such vector among 64 cost 4.12 ms, and 1.92 now.
+template <typename real, int NT, int SETS, typename v2>
+__device__ __forceinline__ bool vector_density(const RotArgs& a, int v, int tiles, const v2 (&q)[SETS][16]) {
+  constexpr int W = NT / 32, N = SETS * 16 * NT;
+  constexpr int bias = sizeof(real) == 4 ? 127 : 1023, range = sizeof(real) == 4 ? 60 : 400;
+  __shared__ int red[W][2];
+  __shared__ int raised;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  largest = __reduce_max_sync(0xffffffffu, largest);
-  sum = __reduce_add_sync(0xffffffffu, sum);
-  zeros = __reduce_add_sync(0xffffffffu, zeros);
+  if (threadIdx.x == 0) raised = __ldcg(a.sparse + v);
+  auto each = [&](auto&& fn) {
+#pragma unroll
+    for (int s = 0; s < SETS; ++s)
+#pragma unroll
+      for (int r = 0; r < 16; ++r) fn(exponent_of(q[s][r].x * q[s][r].x + q[s][r].y * q[s][r].y));
+  };
+  int top = 0, low = 0x7fffffff;
+  each([&](int e) {
+    top = max(top, e);
+    low = min(low, e);
+  });
+  top = __reduce_max_sync(0xffffffffu, top);
+  low = __reduce_min_sync(0xffffffffu, low);
   if (lane == 0) {
-    red[warp][0] = largest;
-    red[warp][1] = sum;
-    red[warp][2] = zeros;
+    red[warp][0] = top;
+    red[warp][1] = low;
   }
   __syncthreads();
+  if (raised) return false;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    top = max(top, red[w][0]);
+    low = min(low, red[w][1]);
+  }
+  __syncthreads();
+  FewBelow f = {0, 0, 0};
+  each([&](int e) {
+    f.c12 += e <= top - 12;
+    f.c18 += e <= top - 18;
+    f.c24 += e <= top - 24;
+  });
+  const int lo = __reduce_add_sync(0xffffffffu, f.c12 | f.c18 << 16), hi = __reduce_add_sync(0xffffffffu, f.c24);
+  if (lane == 0) {
+    red[warp][0] = lo;
+    red[warp][1] = hi;
+  }
+  __syncthreads();
+  f = {0, 0, 0};
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    f.c12 += red[w][0] & 0xffff;
+    f.c18 += red[w][0] >> 16;
+    f.c24 += red[w][1];
+  }
+  const bool dense = low > 0 && top >= bias - range && top <= bias + range && f.in(N);
   if (threadIdx.x == 0) {
-    for (int w = 1; w < NT / 32; ++w) {
-      largest = max(largest, red[w][0]);
-      sum += red[w][1];
-      zeros += red[w][2];
-    }
-    RotDensity* d = a.density + v;
-    atomicMax(&d->largest, largest);
-    atomicAdd(&d->sum, (unsigned long long)sum);
-    atomicAdd(&d->zeros, (unsigned)zeros);
-    __threadfence();
-    if (atomicAdd(&d->arrived, 1u) == (unsigned)(tiles - 1)) {
+    if (!dense) {
+      atomicExch(a.sparse + v, 1);
+    } else {
+      RotDensity* d = a.density + v;
+      const int spread = max(atomicMax(&d->top, top), top) + max(atomicMax(&d->bottom, kRotBottom - top), kRotBottom - top);
+      if (spread > kRotBottom + 4) atomicExch(a.sparse + v, 1);
+      atomicAdd(&d->c12, f.c12);
+      atomicAdd(&d->c18, f.c18);
+      atomicAdd(&d->c24, f.c24);
       __threadfence();
-      constexpr int bias = sizeof(real) == 4 ? 127 : 1023, range = sizeof(real) == 4 ? 60 : 400;
-      const int top = atomicMax(&d->largest, 0);
-      const long long total = (long long)atomicAdd(&d->sum, 0ull), z = (long long)atomicAdd(&d->zeros, 0u);
-      const bool dense = z * 1024 <= a.dim && (long long)top * (a.dim - z) - total <= 12 * (a.dim - z) &&
-                         top >= bias - range && top <= bias + range;
-      if (!dense) atomicExch(a.sparse, 1);
+      if (atomicAdd(&d->arrived, 1u) == (unsigned)(tiles - 1)) {
+        __threadfence();
+        const FewBelow all = {atomicAdd(&d->c12, 0), atomicAdd(&d->c18, 0), atomicAdd(&d->c24, 0)};
+        if (!all.in(a.dim)) atomicExch(a.sparse + v, 1);
+      }
     }
   }
+  return dense;
+}
+
+// every vector of the launch has been found not to be dense
+__device__ __forceinline__ bool all_sparse(const RotArgs& a) {
+  if (!a.sparse) return false;
+  bool dense = false;
+  for (int v = threadIdx.x; v < a.nvec; v += blockDim.x) dense = dense || !a.sparse[a.vec0 + v];
+  return !__syncthreads_or(dense);
 }
 
 template <typename real, int T, int NT, int MINB>
@@ -251,19 +315,7 @@ __global__ void __launch_bounds__(NT, MINB) rot_forward_kernel(const __grid_cons
     for (int s = 0; s < SETS; ++s)
 #pragma unroll
       for (int r = 0; r < 16; ++r) q[s][r] = x[threadIdx.x + s * NT + (r << LO0)];
-    if (a.density) {
-      int largest = 0, sum = 0, zeros = 0;
-#pragma unroll
-      for (int s = 0; s < SETS; ++s)
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          const int e = exponent_of(q[s][r].x * q[s][r].x + q[s][r].y * q[s][r].y);
-          largest = max(largest, e);
-          sum += e;
-          zeros += e == 0;
-        }
-      vector_density<real, NT>(a, v, tiles, largest, sum, zeros);
-    }
+    if (a.density && !vector_density<real, NT, SETS>(a, v, tiles, q)) return;
   }
   __syncthreads();
   const real t = (real)a.t;
@@ -317,7 +369,7 @@ __global__ void __launch_bounds__(NT, MINB) rot_middle_kernel(const __grid_const
   using v2 = typename Cx<real>::v2;
   using Gr = Groups<TB>;
   constexpr int SETS = (1 << TB) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = TB - 4;
-  if (a.sparse && *a.sparse) return;
+  if (all_sparse(a)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   v2* buf = reinterpret_cast<v2*>(smem_raw);
   const int T = a.T, nH = a.n - T, c = TB - nH;
@@ -339,6 +391,7 @@ __global__ void __launch_bounds__(NT, MINB) rot_middle_kernel(const __grid_const
   const real* D = reinterpret_cast<const real*>(a.D) + first;
   const int v1 = min(a.nvec, (vg + 1) * a.vpb);
   for (int v = vg * a.vpb; v < v1; ++v) {
+    if (a.sparse && a.sparse[a.vec0 + v]) continue;
     v2* W = reinterpret_cast<v2*>(a.W) + (size_t)(a.vec0 - a.vecW + v) * a.K * a.dim + first;
     // gates of the last group, D (after the first vector from L1) and the inverse gates
     auto centre = [&](v2(&w)[16], int b) {
@@ -414,7 +467,7 @@ __global__ void __launch_bounds__(NT, 1) rot_middle_ahead_kernel(const __grid_co
   using v2 = typename Cx<real>::v2;
   using Gr = Groups<TB>;
   constexpr int SETS = (1 << TB) / (16 * NT), LOC = Gr::lo(NG - 1), LO0 = TB - 4;
-  if (a.sparse && *a.sparse) return;
+  if (all_sparse(a)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   v2* buf = reinterpret_cast<v2*>(smem_raw);
   const int T = a.T, nH = a.n - T, c = TB - nH;
@@ -513,12 +566,12 @@ __global__ void __launch_bounds__(NT, MINB) rot_backward_kernel(const __grid_con
   using v2 = typename Cx<real>::v2;
   using Gr = Groups<T>;
   constexpr int SETS = (1 << T) / (16 * NT), LO0 = T - 4, GL = Gr::N - 1;
-  if (a.sparse && *a.sparse) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   v2* buf = reinterpret_cast<v2*>(smem_raw);
   __shared__ v2 ph[kRotMaxK * (kRotMaxN + 1)];
   const int nH = a.n - T, tiles = 1 << nH;
   const int tile = blockIdx.x & (tiles - 1), v = a.vec0 + (int)(blockIdx.x >> nH);
+  if (a.sparse && a.sparse[v]) return;
   const size_t off = (size_t)v * a.dim + ((size_t)tile << T);
   stage_phases<real>(ph, a);
   const real t = (real)a.t;

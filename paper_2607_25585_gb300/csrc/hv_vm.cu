@@ -184,7 +184,11 @@ __device__ __forceinline__ int vm_pass_lo(int p, int K, int n) { return min(kLan
 // thread as 2; one copy of the tables per SM leaves more of it to L1).
 template <typename real, int K, bool MP, int MINB>
 __global__ void __launch_bounds__(MINB == 1 ? 512 : 256, MINB) vm_kernel(const __grid_constant__ LaunchArgs a) {
-  if (a.only_if && !*a.only_if) return;
+  if (a.only_if) {
+    bool any = false;
+    for (int k = threadIdx.x; k < a.n_inst; k += blockDim.x) any = any || a.only_if[k];
+    if (!__syncthreads_or(any)) return;
+  }
   using v2 = typename Cx<real>::v2;
   constexpr int NR = 1 << K;
   constexpr int CB = kLaneBits;  // lane bits [0, CB)
@@ -339,6 +343,7 @@ __global__ void __launch_bounds__(MINB == 1 ? 512 : 256, MINB) vm_kernel(const _
   for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
     // tiles: [vector][pass][tile of the pass]
     const int inst = tile / (P * a.tiles_per_vg);
+    if (a.only_if && !a.only_if[inst]) continue;
     const int pass = MP ? (tile / a.tiles_per_vg) % P : 0;
     const int ptile = tile % a.tiles_per_vg;
     if (inst != cur) {  // per-vector pointers (the tables are shared)

@@ -191,3 +191,70 @@ def test_product_has_no_systematic_error(name):
         along = torch.vdot(ref[:, k], y[:, k] - ref[:, k]).real / torch.vdot(ref[:, k], ref[:, k]).real
         assert abs(float(along)) < 2.0 ** -24
     s.close()
+
+
+def sectors(n):
+    mu = np.arange(1 << n)
+    return np.array([bin(m).count("1") for m in mu])
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("R", [1, 3])
+def test_sectors_without_weight_stay_without_weight(dtype, R, rng):
+    """A Hamiltonian that conserves S^z and a block whose outer sectors are exactly
+    zero -- two rows of them, or a few hundred -- in its last vector: so is the product."""
+    w = W.ladder(8, dipolar=False)
+    s = F.System.from_dict(w)
+    up = sectors(16)
+    for keep in (1, 3):
+        x = rng.normal(size=(s.dim, R)) + 1j * rng.normal(size=(s.dim, R))
+        out = (up < keep) | (up > 16 - keep)
+        x[out, -1] = 0
+        y = empty_dev((s.dim, R), dtype)
+        F.apply_h(s, to_dev(x, dtype), y, R, dtype)
+        y = y.cpu().numpy()
+        assert np.all(y[out, -1] == 0) and np.all(y[~out, -1] != 0), keep
+    s.close()
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("amplitude", [2.0 ** -46, 2.0 ** -20, 2.0 ** -12, 2.0 ** -8])
+def test_small_sectors_keep_their_digits(dtype, amplitude, rng):
+    """The same with one sector of 1820 rows (1 in 36) at a small amplitude: its rows of
+    the product have the error of their own terms (200 roundings, 15 units roundoff
+    of the sector's norm), not of the vector's."""
+    w = W.ladder(8, dipolar=False)
+    s = F.System.from_dict(w)
+    x = rng.normal(size=(s.dim, 2)) + 1j * rng.normal(size=(s.dim, 2))
+    small = sectors(16) == 4
+    x[small, 1] *= amplitude
+    xd = to_dev(x, dtype)
+    y = empty_dev((s.dim, 2), dtype)
+    F.apply_h(s, xd, y, 2, dtype)
+    ref = oracle.apply_h(osys(w), xd.cpu().numpy().astype(np.complex128))
+    tol = 1e-6 if dtype == "c64" else 4e-15 + 1e-13
+    e = y.cpu().numpy() - ref
+    for rows in (small, ~small):
+        for k in range(2):
+            assert np.linalg.norm(e[rows, k]) < tol * np.linalg.norm(ref[rows, k])
+    s.close()
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
+def test_vectors_of_a_block_do_not_choose_for_each_other(dtype, rng):
+    """A vector's product has the same bits whichever vectors share its block."""
+    w = buckled(4, 4)
+    s = F.System.from_dict(w)
+    R = 5
+    x = rng.normal(size=(s.dim, R)) + 1j * rng.normal(size=(s.dim, R))
+    y = [empty_dev((s.dim, R), dtype) for _ in range(3)]
+    F.apply_h(s, to_dev(x, dtype), y[0], R, dtype)
+    x[:, 1] = 0
+    x[4321, 1] = 1
+    F.apply_h(s, to_dev(x, dtype), y[1], R, dtype)
+    x[:, [0, 2, 3, 4]] = x[:, [1, 1, 1, 1]]
+    F.apply_h(s, to_dev(x, dtype), y[2], R, dtype)
+    a, b, c = (t.cpu().numpy() for t in y)
+    for k in (0, 2, 3, 4):
+        assert np.array_equal(a[:, k], b[:, k]) and np.array_equal(c[:, k], b[:, 1])
+    s.close()
