@@ -377,30 +377,42 @@ __device__ __forceinline__ double unit53(unsigned hi, unsigned lo) {
   return ((double)k + 1.0) * (1.0 / 9007199254740992.0);
 }
 
-// Random vector number rg of the stream at basis state nu: complex64 by the
-// two-float form (gauss.cuh), complex128 in FP64.
+template <typename real>
+__device__ __forceinline__ typename Cx<real>::v2 box_muller(const unsigned (&c)[4]) {
+  const double rho = sqrt(-2.0 * log(unit53(c[0], c[1])));
+  double sn, cs;
+  sincospi(2.0 * unit53(c[2], c[3]), &sn, &cs);
+  typename Cx<real>::v2 out;
+  out.x = (real)(rho * cs);
+  out.y = (real)(rho * sn);
+  return out;
+}
+// (out of line: rarely needed, and its registers are not the kernel's)
+__device__ __noinline__ float2 box_muller_rounded(unsigned c0, unsigned c1, unsigned c2, unsigned c3) {
+  const unsigned c[4] = {c0, c1, c2, c3};
+  return box_muller<float>(c);
+}
+
+// Random vector number rg of the stream at basis state nu, by Box-Muller in FP64,
+// rounded to the dtype: in complex64 by the two-float form wherever that rounds
+// to the same number (gauss.cuh).
 template <typename real>
 __device__ __forceinline__ typename Cx<real>::v2 gaussian(unsigned long long nu, unsigned long long rg,
                                                           unsigned long long seed) {
   unsigned c[4] = {(unsigned)nu, (unsigned)(nu >> 32), (unsigned)rg, (unsigned)(rg >> 32)};
   philox4x32_10(c, (unsigned)seed, (unsigned)(seed >> 32));
-  typename Cx<real>::v2 out;
-  if (sizeof(real) == 4) {
+  if constexpr (sizeof(real) == 4) {
     const unsigned long long k1 = (((unsigned long long)c[0] << 21) | (c[1] >> 11)) + 1;
     const unsigned long long k2 = (((unsigned long long)c[2] << 21) | (c[3] >> 11)) + 1;
     Two cs, sn;
     const Two rho = box_muller_radius(k1);
     box_muller_angle(k2, cs, sn);
-    out.x = (real)round_product(rho, cs);
-    out.y = (real)round_product(rho, sn);
+    float2 out;
+    const bool sure = rounded(rho, cs, out.x) & rounded(rho, sn, out.y);
+    return sure ? out : box_muller_rounded(c[0], c[1], c[2], c[3]);
   } else {
-    const double rho = sqrt(-2.0 * log(unit53(c[0], c[1])));
-    double sn, cs;
-    sincospi(2.0 * unit53(c[2], c[3]), &sn, &cs);
-    out.x = (real)(rho * cs);
-    out.y = (real)(rho * sn);
+    return box_muller<real>(c);
   }
-  return out;
 }
 
 // A grid-stride walk over a block's elements e as (slow, fast) = (e / nfast,
