@@ -1548,11 +1548,10 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
   struct HostPart {
     std::vector<double> al, be, pp;  // [R][M], [R][M], [R][M][2]
     std::vector<int> me;
-    ftlm_status status = FTLM_OK;
-    std::string msg;
   };
   std::vector<HostPart> host(n);
-  const bool hosted = parallel_for(n, n > 1 ? n * host_sums_ns(R, M, p->nT) : 0.0, [&](int k) {  // eigensolves and sums
+  std::vector<HostSums> sums(n);
+  for (int k = 0; k < n; ++k) {
     HostPart& h = host[k];
     const char* src = ctx->pinned + per * k;
     const double* alpha_d = reinterpret_cast<const double*>(src);  // [M][R]
@@ -1571,20 +1570,16 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
       }
     h.me.assign(meff, meff + R);
     for (int r = 0; r < R; ++r)
-      if (h.me[r] < 1 || h.me[r] > M) {
-        h.status = FTLM_ERR_NUMERICAL;
-        h.msg = "start vector of zero norm";
-        return;
-      }
-    h.status = host_sums(R, M, h.me.data(), h.al.data(), h.be.data(), h.pp.data(), (double)sys[k]->hs.dim,
-                         sys[k]->hs.g, p->T, p->nT, &res[k], h.msg, n == 1);
-  });
-  if (!hosted) return fail(FTLM_ERR_OUT_OF_MEMORY, "out of host memory");
+      if (h.me[r] < 1 || h.me[r] > M) return fail(FTLM_ERR_NUMERICAL, "start vector of zero norm");
+    sums[k] = {R, M, h.me.data(), h.al.data(), h.be.data(), h.pp.data(), (double)sys[k]->hs.dim, sys[k]->hs.g,
+               p->T, p->nT, &res[k]};
+  }
+  host_sums_many(sums);  // eigensolves and sums of all systems
   for (int k = 0; k < n; ++k) {
     const std::vector<double>&al = host[k].al, &be = host[k].be, &pp = host[k].pp;
     const std::vector<int>& me = host[k].me;
     ftlm_result& out = res[k];
-    if (host[k].status != FTLM_OK) return fail(host[k].status, host[k].msg);
+    if (sums[k].status != FTLM_OK) return fail(sums[k].status, sums[k].msg);
     if (out.alpha) std::memcpy(out.alpha, al.data(), sizeof(double) * al.size());
     if (out.beta) std::memcpy(out.beta, be.data(), sizeof(double) * be.size());
     if (out.p) std::memcpy(out.p, pp.data(), sizeof(double) * pp.size());

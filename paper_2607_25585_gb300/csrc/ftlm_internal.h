@@ -2,7 +2,6 @@
 #pragma once
 
 #include <cstdint>
-#include <functional>
 #include <string>
 #include <vector>
 
@@ -428,14 +427,22 @@ int csr_scan(const int* counts, long long* rp, long long dim, void* stream);
 int launch_csr_spmm(long long dim, int R, const long long* rp, const int* col, const void* val, const void* x,
                     void* y, int c64, void* stream);
 
-// fn(0) .. fn(n - 1) on host threads, as many as total_ns of work pays for (tridiag.cpp)
-bool parallel_for(int n, double total_ns, const std::function<void(int)>& fn);
-double host_sums_ns(int R, int M, int nT);  // estimated cost of host_sums
-// Host tridiagonal eigensolver + sums (tridiag.cpp); host_sums_sym: the
-// symmetric estimator of M_B from the matrices O_ij = <v_i|u.S|v_j>.
+// Host tridiagonal eigensolver + sums (tridiag.cpp), of one system or of a batch's;
+// host_sums_sym: the symmetric estimator of M_B from the matrices O_ij = <v_i|u.S|v_j>.
+struct HostSums {
+  int R = 0, M = 0;
+  const int* M_eff = nullptr;
+  const double *alpha = nullptr, *beta = nullptr, *p = nullptr;
+  double dim = 0, g = 0;
+  const double* T = nullptr;
+  int nT = 0;
+  ftlm_result* res = nullptr;
+  ftlm_status status = FTLM_OK;  // set by host_sums_many, with msg
+  std::string msg;
+};
+void host_sums_many(std::vector<HostSums>& sums);
 ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const double* beta, const double* p,
-                      double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg,
-                      bool threads = true);
+                      double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg);
 ftlm_status host_sums_sym(int R, int M, const int* M_eff, const double* alpha, const double* beta,
                           const double* Omat, double g, const double* T, int nT, double* MB_sym, double* MB_sym_imag,
                           std::string& msg);

@@ -13,7 +13,9 @@
 #include <cstring>
 #include <functional>
 #include <limits>
+#include <string>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include "ftlm_internal.h"
@@ -92,8 +94,6 @@ bool ql_implicit(int m, double* d, double* e_in, int nz, double** z) {
   return true;
 }
 
-}  // namespace
-
 // fn(i) for i in [0, n), each exactly once, on the caller's thread and as many
 // others as the work pays for: starting and joining a thread costs some 60 us,
 // so each gets at least 200 us of `total_ns` (ten eigenproblems of 24 rows and
@@ -121,96 +121,151 @@ bool parallel_for(int n, double total_ns, const std::function<void(int)>& fn) {
   return ok;
 }
 
-double host_sums_ns(int R, int M, int nT) { return R * (ql_ns(M, 3) + kTermNs * M * nT); }
+// One run's eigenproblem: its Ritz values, the weights' row U_0n and the rows Re, Im
+// of sum_j conj(p_j) U_jn.
+struct Ritz {
+  std::vector<double> eps, w0, qr, qi;
+};
+
+// null, or what is wrong with run r
+const char* solve_run(const HostSums& s, int r, Ritz& run) {
+  const int m = s.M_eff[r], M = s.M;
+  run.eps.assign(s.alpha + (size_t)r * M, s.alpha + (size_t)r * M + m);
+  std::vector<double> e(m > 1 ? m - 1 : 1, 0.0);
+  for (int j = 0; j + 1 < m; ++j) e[j] = s.beta[(size_t)r * M + j];
+  run.w0.assign(m, 0.0);
+  run.w0[0] = 1.0;
+  run.qr.resize(m);
+  run.qi.resize(m);
+  for (int j = 0; j < m; ++j) {  // conj(p_j)
+    run.qr[j] = s.p[((size_t)r * M + j) * 2];
+    run.qi[j] = -s.p[((size_t)r * M + j) * 2 + 1];
+  }
+  for (int j = 0; j < m; ++j)
+    if (!std::isfinite(run.eps[j]) || (j + 1 < m && !std::isfinite(e[j]))) return "non-finite Lanczos coefficient in run ";
+  double* rows[3] = {run.w0.data(), run.qr.data(), run.qi.data()};
+  return ql_implicit(m, run.eps.data(), e.data(), 3, rows) ? nullptr : "tridiagonal eigensolver did not converge (run ";
+}
+
+// the results at temperature t, from the solved runs in order
+void sum_runs(const HostSums& s, const std::vector<Ritz>& runs, double E0, int t) {
+  const double b = 1.0 / s.T[t];
+  double z = 0.0, e1 = 0.0, orr = 0.0, oi = 0.0;
+  std::vector<double> ws;  // the weights, for the variance
+  ws.reserve((size_t)s.R * s.M);
+  for (const Ritz& run : runs)
+    for (size_t n = 0; n < run.eps.size(); ++n) {
+      const double boltz = std::exp(-b * (run.eps[n] - E0));
+      const double w = run.w0[n] * run.w0[n] * boltz;
+      ws.push_back(w);
+      z += w;
+      e1 += w * run.eps[n];
+      orr += boltz * run.w0[n] * run.qr[n];
+      oi += boltz * run.w0[n] * run.qi[n];
+    }
+  const double Em = e1 / z;
+  double var = 0.0;
+  const double* w = ws.data();
+  for (const Ritz& run : runs)
+    for (size_t n = 0; n < run.eps.size(); ++n) var += *w++ * (run.eps[n] - Em) * (run.eps[n] - Em);
+  ftlm_result* res = s.res;
+  if (res->lnZ) res->lnZ[t] = std::log(s.dim / s.R * z) - b * E0;
+  if (res->E) res->E[t] = Em;
+  if (res->C) res->C[t] = b * b * var / z;
+  if (res->M_B) res->M_B[t] = -s.g * orr / z;
+  if (res->M_B_imag) res->M_B_imag[t] = -s.g * oi / z;
+}
+}  // namespace
+
+// All systems' eigenproblems, then all their temperatures, as one list of items: a
+// batch of two long runs keeps as many threads busy as a batch of many short ones
+// (2 x 64 vectors of 200 steps: a thread a system took 52 ms).  A temperature's item
+// comes after every eigenproblem's, so the one it may have to wait for is being
+// solved on another thread.
+void host_sums_many(std::vector<HostSums>& sums) {
+  struct Work {
+    std::vector<Ritz> runs;
+    std::vector<const char*> bad;
+    std::atomic<int> left{0};
+    std::atomic<bool> memory{false};
+    double E0 = std::numeric_limits<double>::infinity();
+  };
+  const int n = (int)sums.size();
+  std::vector<Work> work(n);
+  std::vector<std::pair<int, int>> solve, sum;  // (system, run), (system, temperature)
+  double ns = 0.0;
+  for (int k = 0; k < n; ++k) {
+    HostSums& s = sums[k];
+    s.status = FTLM_ERR_INVALID_ARG;
+    if (s.R < 1 || s.M < 1 || !s.M_eff || !s.alpha || !s.beta || !s.p || !s.T || s.nT < 1 || !s.res || !(s.dim > 0)) {
+      s.msg = "ftlm_sums: invalid arguments";
+      continue;
+    }
+    s.msg.clear();
+    for (int t = 0; t < s.nT; ++t)
+      if (!(s.T[t] > 0.0) || !std::isfinite(s.T[t])) s.msg = "temperatures must be positive and finite";
+    for (int r = 0; r < s.R && s.msg.empty(); ++r)
+      if (s.M_eff[r] < 1 || s.M_eff[r] > s.M) s.msg = "M_eff out of range";
+    if (!s.msg.empty()) continue;
+    s.status = FTLM_OK;
+    work[k].runs.resize(s.R);
+    work[k].bad.assign(s.R, nullptr);
+    work[k].left = s.R;
+    for (int r = 0; r < s.R; ++r) solve.emplace_back(k, r);
+    for (int t = 0; t < s.nT; ++t) sum.emplace_back(k, t);
+    ns += s.R * (ql_ns(s.M, 3) + kTermNs * s.M * s.nT);
+  }
+  parallel_for((int)(solve.size() + sum.size()), ns, [&](int i) {
+    if (i < (int)solve.size()) {
+      const int k = solve[i].first, r = solve[i].second;
+      Work& w = work[k];
+      try {
+        w.bad[r] = solve_run(sums[k], r, w.runs[r]);
+      } catch (...) {
+        w.memory = true;
+      }
+      if (w.left.fetch_sub(1) == 1) {  // the system's last: its lowest Ritz value
+        for (const Ritz& run : w.runs)
+          for (double e : run.eps) w.E0 = std::min(w.E0, e);
+        w.left.store(-1);
+      }
+      return;
+    }
+    const auto [k, t] = sum[i - solve.size()];
+    Work& w = work[k];
+    while (w.left.load() >= 0) std::this_thread::yield();
+    for (const char* b : w.bad)
+      if (b || w.memory) return;
+    try {
+      sum_runs(sums[k], w.runs, w.E0, t);
+    } catch (...) {
+      w.memory = true;
+    }
+  });
+  for (int k = 0; k < n; ++k) {
+    HostSums& s = sums[k];
+    if (s.status != FTLM_OK) continue;
+    if (work[k].memory) {
+      s.status = FTLM_ERR_OUT_OF_MEMORY;
+      s.msg = "out of host memory";
+      continue;
+    }
+    for (int r = 0; r < s.R && s.status == FTLM_OK; ++r)
+      if (const char* b = work[k].bad[r]) {
+        s.status = FTLM_ERR_NUMERICAL;
+        s.msg = b + std::to_string(r) + (std::strchr(b, '(') ? ")" : "");
+      }
+    if (s.status == FTLM_OK) s.res->E0 = work[k].E0;
+  }
+}
 
 ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const double* beta, const double* p,
-                      double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg, bool threads) {
-  const char* memory = "out of host memory";
-  if (R < 1 || M < 1 || !M_eff || !alpha || !beta || !p || !T || nT < 1 || !res || !(dim > 0)) {
-    msg = "ftlm_sums: invalid arguments";
-    return FTLM_ERR_INVALID_ARG;
-  }
-  for (int t = 0; t < nT; ++t)
-    if (!(T[t] > 0.0) || !std::isfinite(T[t])) {
-      msg = "temperatures must be positive and finite";
-      return FTLM_ERR_INVALID_ARG;
-    }
-  struct Run {
-    std::vector<double> eps, w0, qr, qi;  // Ritz values, U_0n, Re/Im of sum_j conj(p_j) U_jn
-  };
-  std::vector<Run> runs(R);
-  for (int r = 0; r < R; ++r)
-    if (M_eff[r] < 1 || M_eff[r] > M) {
-      msg = "M_eff out of range";
-      return FTLM_ERR_INVALID_ARG;
-    }
-  // the runs' eigenproblems are independent: one per host thread
-  std::vector<int> bad(R, 0);  // 1: non-finite coefficient, 2: no convergence
-  const bool solved = parallel_for(R, threads ? R * ql_ns(M, 3) : 0.0, [&](int r) {
-    const int m = M_eff[r];
-    Run& run = runs[r];
-    run.eps.assign(alpha + (size_t)r * M, alpha + (size_t)r * M + m);
-    std::vector<double> e(m > 1 ? m - 1 : 1, 0.0);
-    for (int j = 0; j + 1 < m; ++j) e[j] = beta[(size_t)r * M + j];
-    run.w0.assign(m, 0.0);
-    run.w0[0] = 1.0;
-    run.qr.resize(m);
-    run.qi.resize(m);
-    for (int j = 0; j < m; ++j) {  // conj(p_j)
-      run.qr[j] = p[((size_t)r * M + j) * 2];
-      run.qi[j] = -p[((size_t)r * M + j) * 2 + 1];
-    }
-    for (int j = 0; j < m; ++j)
-      if (!std::isfinite(run.eps[j]) || (j + 1 < m && !std::isfinite(e[j]))) {
-        bad[r] = 1;
-        return;
-      }
-    double* rows[3] = {run.w0.data(), run.qr.data(), run.qi.data()};
-    if (!ql_implicit(m, run.eps.data(), e.data(), 3, rows)) bad[r] = 2;
-  });
-  if (!solved) return msg = memory, FTLM_ERR_OUT_OF_MEMORY;
-  double E0 = std::numeric_limits<double>::infinity();
-  for (int r = 0; r < R; ++r) {
-    if (bad[r] == 1) {
-      msg = "non-finite Lanczos coefficient in run " + std::to_string(r);
-      return FTLM_ERR_NUMERICAL;
-    }
-    if (bad[r] == 2) {
-      msg = "tridiagonal eigensolver did not converge (run " + std::to_string(r) + ")";
-      return FTLM_ERR_NUMERICAL;
-    }
-    for (double v : runs[r].eps) E0 = std::min(E0, v);
-  }
-  res->E0 = E0;
-  // the temperatures are independent too (each sums the runs in order)
-  const bool summed = parallel_for(nT, threads ? kTermNs * nT * R * M : 0.0, [&](int t) {
-    const double b = 1.0 / T[t];
-    double z = 0.0, e1 = 0.0, orr = 0.0, oi = 0.0;
-    std::vector<double> ws;  // the weights, for the variance
-    ws.reserve((size_t)R * M);
-    for (const Run& run : runs)
-      for (size_t n = 0; n < run.eps.size(); ++n) {
-        const double boltz = std::exp(-b * (run.eps[n] - E0));
-        const double w = run.w0[n] * run.w0[n] * boltz;
-        ws.push_back(w);
-        z += w;
-        e1 += w * run.eps[n];
-        orr += boltz * run.w0[n] * run.qr[n];
-        oi += boltz * run.w0[n] * run.qi[n];
-      }
-    const double Em = e1 / z;
-    double var = 0.0;
-    const double* w = ws.data();
-    for (const Run& run : runs)
-      for (size_t n = 0; n < run.eps.size(); ++n) var += *w++ * (run.eps[n] - Em) * (run.eps[n] - Em);
-    if (res->lnZ) res->lnZ[t] = std::log(dim / R * z) - b * E0;
-    if (res->E) res->E[t] = Em;
-    if (res->C) res->C[t] = b * b * var / z;
-    if (res->M_B) res->M_B[t] = -g * orr / z;
-    if (res->M_B_imag) res->M_B_imag[t] = -g * oi / z;
-  });
-  if (!summed) return msg = memory, FTLM_ERR_OUT_OF_MEMORY;
-  return FTLM_OK;
+                      double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg) {
+  std::vector<HostSums> one(1);
+  one[0] = {R, M, M_eff, alpha, beta, p, dim, g, T, nT, res};
+  host_sums_many(one);
+  msg = one[0].msg;
+  return one[0].status;
 }
 
 // Symmetric FTLM for O = u.S, Eqs. (E-2-G), (E-2-H): per run,
