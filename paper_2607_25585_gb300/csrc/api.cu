@@ -756,6 +756,18 @@ size_t stored_limit(const ftlm_system* s, int c64, int n = 1) {
   return !s->hs.all_half && !c64 ? std::max(kStoredL2, ((size_t)2 << 30) / n) : kStoredL2;
 }
 
+// bytes of the system's stored rows; 0: too many sites for their builder
+size_t stored_bytes(const ftlm_system* s, int c64) {
+  const size_t S = (size_t)stored_row_bound(s->hs);
+  return S == 0 || s->hs.dim > ((size_t)2 << 30) ? 0 : (size_t)s->hs.dim * (S * (c64 ? 12 : 20) + 4);
+}
+
+// Whether a call with `products` products of a vector wants them.
+bool stored_fits(const ftlm_system* s, int c64, size_t limit, long long products) {
+  const size_t b = stored_bytes(s, c64);
+  return b != 0 && b <= (products < 4 ? kStoredL2 : limit);
+}
+
 // The system's stored rows for work on stream st: written by the first call, on
 // its st (not on the system's own stream, which another thread's run may be
 // capturing); other streams wait for them.  ok = false: the gathers run -- the
@@ -767,14 +779,14 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long produ
   ok = false;
   const int k = c64 ? 1 : 0;
   const size_t d = (size_t)s->hs.dim, esz = c64 ? 8 : 16;
+  if (!stored_fits(s, c64, limit, products)) return FTLM_OK;
   const size_t S = (size_t)stored_row_bound(s->hs);
-  if (S == 0 || d > limit || d * S * (esz + 4) + d * 4 > (products < 4 ? kStoredL2 : limit)) return FTLM_OK;
   std::lock_guard<std::mutex> lk(s->rows_mu);
   DevBuf& b = s->rows[k];
   if (!s->rows_done[k]) {
     if (!b.p) {
       if (!s->ev_rows[k]) CK(cudaEventCreateWithFlags(&s->ev_rows[k], cudaEventDisableTiming));
-      if (b.ensure(d * S * (esz + 4) + d * 4) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
+      if (b.ensure(stored_bytes(s, c64)) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
       char* p = static_cast<char*>(b.p);
       int e = launch_stored_build(c64 ? s->tab_f.p : s->tab_d.p, s->hs.lay,
                                   reinterpret_cast<const long long*>(s->stride.p), reinterpret_cast<const int*>(s->q.p),
@@ -1442,14 +1454,15 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
   bool forced = false;
   for (auto* s : sys) forced = forced || has_shape_override(s, R, c64);
   if (plan_vmaj(pl) && !pl.rot.on && !forced) {  // small systems: stored rows in the gathers' place
-    bool all = true;
+    bool all = true;  // (every system's or none's: nothing is written for a batch that one system keeps on the gathers)
     uint64_t rows = 0;
+    for (auto* s : sys) all = all && stored_fits(s, c64, stored_limit(s, c64, n), (long long)R * M);
     for (auto* s : sys) {
       StoredRows r;
-      bool ok = false;
-      ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64, n), (long long)R * M, st, r, ok);
-      if (rs != FTLM_OK) return rs;
-      all = all && ok;
+      if (all) {
+        ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64, n), (long long)R * M, st, r, all);
+        if (rs != FTLM_OK) return rs;
+      }
       rows += s->hs.dim;
     }
     if (all) pl.storedV = stored_group(rows, R);

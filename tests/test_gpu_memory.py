@@ -22,3 +22,21 @@ def test_a_failed_allocation_leaves_no_error_behind():
     x += 1
     assert float(x.sum()) == 1 << 20
     s.close()
+
+
+def used():
+    torch = torch_cuda()
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+def test_a_batch_on_the_gathers_writes_no_rows():
+    """Rows are written for every system of a batch or for none: 0.9 GB of the smaller
+    one's would be of no use beside a sibling whose rows are too large."""
+    small, large = F.System.from_dict(W.chain(11, Bdir=(1, 0, 1))), F.System.from_dict(W.chain(12, Bdir=(1, 0, 1)))
+    before = used()
+    F.run_batch([small, large], R=2, M=4, T=T, seed=1, dtype="c128")
+    assert used() - before < 400 << 20          # workspaces: four blocks of 2 x 708,588 values, 0.1 GB
+    small.close()
+    large.close()
