@@ -87,14 +87,14 @@ struct ftlm_system {
   DevBuf Ws;             // symmetric runs: u.S of the stored vectors (when it fits)
   DevBuf Gre;            // re-orthogonalised runs: <q_k|w_r> coefficients [R][M] complex
   DevBuf Ta, Tb;         // ftlm_apply_h on spin-1/2 blocks: x and H x in the vector-major layout
-  DevBuf Tw, Ts;         // its rotated-basis blocks and the vectors' statistics
+  DevBuf Tw, Ts;         // its rotated-basis blocks for one vector (more: rW) and the vectors' statistics
   DevBuf ut[2];          // per-unit coefficient tables of the one-pass vector-major gather, [c64]
   int ut_K[2] = {0, 0};  // the cube size each was built for
   cudaEvent_t ev_apply = nullptr;  // recorded after the last use of Ta, Tb
   std::unique_ptr<RotDirs> rot;  // the rotated-basis H.v's directions, if the system has any
   DevBuf rD[2];          // its diagonal tables [K + 1][dim] and phases, [c64]
   cudaEvent_t ev_rot[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
-  DevBuf rW, rpart;      // its intermediate blocks; partial sums and arrival counters
+  DevBuf rW, rpart;      // its intermediate blocks (also of products of several vectors); partial sums and counters
   DevBuf rows[2];        // stored rows of a small system, [c64]: values, columns, counts
   cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
   bool rows_done[2] = {false, false};           // that event has been seen complete
@@ -676,41 +676,44 @@ ftlm_status ensure_rot_tables(ftlm_system* s, const RotPlan& rp, int c64, cudaSt
   return FTLM_OK;
 }
 
+// The intermediate blocks' buffer rW, for holders of the system's mu and apply_mu.
+// Products still in flight may read the old one; captured graphs hold its address.
+bool grow_rot_blocks(ftlm_system* s, size_t bytes) {
+  if (s->rW.bytes >= bytes) return true;
+  if (s->apply_used) cudaEventSynchronize(s->ev_apply);
+  s->gen++;
+  return s->rW.ensure(bytes) == cudaSuccess;
+}
+
+size_t rot_block_bytes(const ftlm_system* s, const RotPlan& rp, int c64) {
+  return (size_t)rp.group * rp.K * (size_t)s->hs.dim * (c64 ? 8 : 16);
+}
+
 // The tables, W blocks and partial sums of a run over R vectors.
 ftlm_status ensure_rot(ftlm_system* s, const RotPlan& rp, int R, int c64, cudaStream_t st, bool& ok) {
   ok = false;
-  const size_t d = (size_t)s->hs.dim;
-  bool fits = true;
-  auto grow = [&](DevBuf& b, size_t bytes) {
-    if (!fits || b.bytes >= bytes) return;
-    s->gen++;  // captured graphs hold its address
-    fits = b.ensure(bytes) == cudaSuccess;
-  };
-  grow(s->rW, (size_t)rp.group * rp.K * d * (c64 ? 8 : 16));
-  grow(s->rpart, sizeof(double) * 3 * (d >> rp.T) * R + sizeof(unsigned) * R);
-  if (fits) {
-    std::lock_guard<std::mutex> lk(s->apply_mu);
-    ftlm_status ts = ensure_rot_tables(s, rp, c64, st, ok);
-    if (ts != FTLM_OK) return ts;
+  const size_t pbytes = sizeof(double) * 3 * ((size_t)s->hs.dim >> rp.T) * R + sizeof(unsigned) * R;
+  std::lock_guard<std::mutex> lk(s->apply_mu);
+  bool fits = grow_rot_blocks(s, rot_block_bytes(s, rp, c64));
+  if (fits && s->rpart.bytes < pbytes) {
+    s->gen++;
+    fits = s->rpart.ensure(pbytes) == cudaSuccess;
   }
-  if (!ok) {
-    cudaGetLastError();
-    s->rW.release();
-    s->rpart.release();
-  }
-  return FTLM_OK;
+  return fits ? ensure_rot_tables(s, rp, c64, st, ok) : FTLM_OK;
 }
 
 // The rotated-basis plan of a block of R vectors (false: the system has none).
-// The W blocks hold K times the group's vectors: 16 GB of them keep every group
-// large enough to fill the device.
+// The W blocks hold K times the group's vectors; a system keeps at most kRotBlocks
+// of them, or one vector's: four vectors of 26 sites in one group take 11.0 ms a
+// step, in groups of two (4 GB) 11.1, one at a time (2 GB) 11.5.
+constexpr size_t kRotBlocks = (size_t)8 << 30;
 bool rot_shape(ftlm_system* s, int R, int c64, RotPlan& rp) {
   rp = RotPlan();
   rp.T = rot_tile_bits(s->hs.n, c64);
   if (!s->rot || !rp.T) return false;
   rp.K = s->rot->K;
   const uint64_t per = s->hs.dim * (uint64_t)rp.K * (c64 ? 8 : 16);
-  rp.group = (int)std::min<uint64_t>((uint64_t)R, std::max<uint64_t>(1, (16ull << 30) / per));
+  rp.group = (int)std::min<uint64_t>((uint64_t)R, std::max<uint64_t>(1, kRotBlocks / per));
   return true;
 }
 
@@ -1773,6 +1776,10 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
     a.x = s->A.p;
     a.y = s->B.p;
     a.W = s->rW.p;
+    {  // after products still in flight, which use these blocks too
+      std::lock_guard<std::mutex> lk(s->apply_mu);
+      if (s->apply_used) CK(cudaStreamWaitEvent(st, s->ev_apply, 0));
+    }
     for (int it = 0; it < 7; ++it) {  // two warm-up products, five timed
       if (it == 2) CK(cudaEventRecord(e0, st));
       ftlm_status rs = enqueue_rot_passes(nullptr, s, rp, a, R, c64, nullptr, st);
@@ -1870,7 +1877,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
       // the system's blocks are shared by its calls: a call waits for the
       // previous one's kernels (on whatever stream it ran) before reusing them
       std::unique_lock<std::mutex> run_lk(s->mu, std::defer_lock);
-      if (nvec > 1) run_lk.lock();  // (the unit tables belong to runs too)
+      if (nvec > 1) run_lk.lock();  // (the unit tables and W blocks belong to runs too)
       std::lock_guard<std::mutex> lk(s->apply_mu);
       const size_t block = (size_t)s->hs.dim * nvec * (c64 ? 8 : 16);
       auto grow = [&](DevBuf& b, size_t bytes) {
@@ -1883,7 +1890,9 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
         CK(grow(s->Tb, block));
       }
       const size_t sbytes = (sizeof(RotDensity) + sizeof(int)) * nvec;
-      if (rot) rot = grow(s->Tw, block / nvec * rp.group * rp.K) == cudaSuccess && grow(s->Ts, sbytes) == cudaSuccess;
+      if (rot && nvec > 1) rot = grow_rot_blocks(s, rot_block_bytes(s, rp, c64));  // (a run waits for ev_apply)
+      else if (rot) rot = grow(s->Tw, rot_block_bytes(s, rp, c64)) == cudaSuccess;
+      if (rot) rot = grow(s->Ts, sbytes) == cudaSuccess;
       cudaGetLastError();
       if (nvec > 1 || rot) {
         if (s->apply_used) CK(cudaStreamWaitEvent(st, s->ev_apply, 0));
@@ -1902,7 +1911,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
           RotArgs r = rot_args(s, rp, c64);
           r.x = const_cast<void*>(xv);
           r.y = yv;
-          r.W = s->Tw.p;
+          r.W = nvec > 1 ? s->rW.p : s->Tw.p;
           r.density = reinterpret_cast<RotDensity*>(s->Ts.p);
           r.sparse = reinterpret_cast<int*>(r.density + nvec);
           ut = enqueue_rot_passes(nullptr, s, rp, r, nvec, c64, nullptr, st);

@@ -40,3 +40,57 @@ def test_a_batch_on_the_gathers_writes_no_rows():
     assert used() - before < 400 << 20          # workspaces: four blocks of 2 x 708,588 values, 0.1 GB
     small.close()
     large.close()
+
+
+def test_rotated_blocks_are_bounded_and_shared():
+    """Runs and products of one system use the same intermediate blocks, of at most 8 GB:
+    22 sites, 64 vectors, three directions would be 6.4 GB for each."""
+    torch = torch_cuda()
+    s = F.System.from_dict(W.square_lattice(11, 2, seed=2))
+    R = 64
+    x = torch.view_as_complex(torch.randn(s.dim, R, 2, device="cuda"))
+    y = torch.empty_like(x)
+    block = s.dim * R * 8
+    before = used()
+    F.apply_h(s, x, y, R, "c64")                                  # two transposed blocks and the W blocks, 3 of them
+    F.run(s, R=R, M=2, T=T, seed=1, dtype="c64")                  # three blocks of its own
+    assert used() - before < (2 + 3 + 3) * block + (1 << 30)
+    s.close()
+    s = F.System.from_dict(W.square_lattice(12, 2, seed=2))       # W of 64 vectors: 25.8 GB
+    before = used()
+    a = F.run(s, R=R, M=3, T=T, seed=1, dtype="c64")
+    assert a["shape"]["passes"] == 3 and used() - before < 3 * s.dim * R * 8 + (10 << 30)
+    b = F.run(s, R=4, M=3, T=T, seed=1, vec_offset=38, dtype="c64")   # the same vectors, in one group: the same bits
+    for k in ("alpha", "beta", "p"):
+        assert np.array_equal(a[k][38:42], b[k])
+    s.close()
+
+
+def test_runs_and_products_share_their_blocks_in_order():
+    """Products on two streams between runs of the same system: the same bits as alone."""
+    torch = torch_cuda()
+    s = F.System.from_dict(W.square_lattice(4, 4, seed=3))
+    g = torch.Generator(device="cuda").manual_seed(1)
+    xs = [torch.view_as_complex(torch.randn(s.dim, R, 2, device="cuda", generator=g)) for R in (3, 9, 1, 40)]
+    kw = dict(R=5, M=6, T=T, seed=1, dtype="c64")
+    want = []
+    for x in xs:
+        y = torch.empty_like(x)
+        F.apply_h(s, x, y, x.shape[1], "c64")
+        torch.cuda.synchronize()
+        want.append(y)
+    run = F.run(s, **kw)
+    s.close()
+    s = F.System.from_dict(W.square_lattice(4, 4, seed=3))        # (the blocks grow while products are in flight)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    got = [torch.empty_like(x) for x in xs]
+    torch.cuda.synchronize()
+    for _ in range(4):
+        for k, x in enumerate(xs):
+            F.apply_h(s, x, got[k], x.shape[1], "c64", stream=streams[k % 2])
+        again = F.run(s, stream=streams[0], **kw)
+        assert np.array_equal(run["alpha"], again["alpha"])
+        torch.cuda.synchronize()
+        for p, q in zip(got, want):
+            assert torch.equal(p, q)
+    s.close()
