@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -98,6 +99,7 @@ struct ftlm_system {
   DevBuf rows[2];        // stored rows of a small system, [c64]: values, columns, counts
   cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
   bool rows_done[2] = {false, false};           // that event has been seen complete
+  bool rows_never[2] = {false, false};          // there was no room for them: the gathers run from then on
   std::mutex rows_mu;
   bool apply_used = false;
   std::mutex apply_mu;   // the blocks, event and tables that products use; a run holds it only to look at them
@@ -771,12 +773,30 @@ bool stored_fits(const ftlm_system* s, int c64, size_t limit, long long products
   return b != 0 && b <= (products < 4 ? kStoredL2 : limit);
 }
 
+// Rows of all live systems together, at most: a program may hold hundreds of systems
+// (fields, orientations), and the gathers need no memory.  A system that finds no room
+// stays with the gathers, so that its repeated calls give the same bits.
+constexpr size_t kStoredTotal = (size_t)16 << 30;
+std::atomic<size_t> g_stored_total{0};
+
+bool reserve_stored(size_t bytes) {
+  size_t t = g_stored_total.load();
+  while (t + bytes <= kStoredTotal)
+    if (g_stored_total.compare_exchange_weak(t, t + bytes)) return true;
+  return false;
+}
+
+void release_stored(DevBuf& b) {
+  g_stored_total -= b.bytes;
+  b.release();
+}
+
 // The system's stored rows for work on stream st: written by the first call, on
 // its st (not on the system's own stream, which another thread's run may be
 // capturing); other streams wait for them.  ok = false: the gathers run -- the
 // rows are too large, or beyond L2 for a call of fewer than four products of a
-// vector (writing them costs about two).  The choice depends on the call alone, so
-// a repeated call gives the same bits.  st must not be capturing.
+// vector (writing them costs about two), or there was no room for them.  A repeated
+// call gives the same bits.  st must not be capturing.
 ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long products, cudaStream_t st, StoredRows& r,
                           bool& ok) {
   ok = false;
@@ -786,17 +806,24 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long produ
   const size_t S = (size_t)stored_row_bound(s->hs);
   std::lock_guard<std::mutex> lk(s->rows_mu);
   DevBuf& b = s->rows[k];
+  if (s->rows_never[k]) return FTLM_OK;
   if (!s->rows_done[k]) {
     if (!b.p) {
       if (!s->ev_rows[k]) CK(cudaEventCreateWithFlags(&s->ev_rows[k], cudaEventDisableTiming));
-      if (b.ensure(stored_bytes(s, c64)) != cudaSuccess) return cudaGetLastError(), FTLM_OK;
+      const size_t bytes = stored_bytes(s, c64);
+      s->rows_never[k] = !reserve_stored(bytes);
+      if (!s->rows_never[k] && b.ensure(bytes) != cudaSuccess) {
+        g_stored_total -= bytes;
+        s->rows_never[k] = true;
+      }
+      if (s->rows_never[k]) return FTLM_OK;
       char* p = static_cast<char*>(b.p);
       int e = launch_stored_build(c64 ? s->tab_f.p : s->tab_d.p, s->hs.lay,
                                   reinterpret_cast<const long long*>(s->stride.p), reinterpret_cast<const int*>(s->q.p),
                                   s->hs.n, (int)d, (int)S, reinterpret_cast<int*>(p + d * S * esz), p,
                                   reinterpret_cast<int*>(p + d * S * (esz + 4)), c64, st);
       if (!e) e = (int)cudaEventRecord(s->ev_rows[k], st);
-      if (e) b.release();
+      if (e) release_stored(b);
       CKI(e);
     }
     if (cudaEventQuery(s->ev_rows[k]) == cudaSuccess) s->rows_done[k] = true;
@@ -2117,8 +2144,9 @@ void ftlm_system_destroy(ftlm_system* s) {
   cudaDeviceSynchronize();  // the system's buffers may be in use on any stream
   purge_ctx_of(s->id);
   for (DevBuf* b : {&s->tab_f, &s->tab_d, &s->stride, &s->q, &s->A, &s->B, &s->U, &s->scal, &s->ep, &s->ecnt,
-                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart, &s->rows[0], &s->rows[1], &s->Tw, &s->Ts})
+                    &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart, &s->Tw, &s->Ts})
     b->release();
+  for (DevBuf& b : s->rows) release_stored(b);
   cudaEventDestroy(s->ev_in);
   cudaEventDestroy(s->ev_out);
   cudaEventDestroy(s->ev_apply);

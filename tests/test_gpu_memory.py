@@ -94,3 +94,26 @@ def test_runs_and_products_share_their_blocks_in_order():
         for p, q in zip(got, want):
             assert torch.equal(p, q)
     s.close()
+
+
+def test_stored_rows_of_many_systems_are_bounded():
+    """Twenty systems whose rows take 0.9 GB each: 16 GB are kept, the others' runs take
+    the gathers, with the same numbers (30 x 1e-12: six steps)."""
+    systems = [F.System.from_dict(W.chain(11, Bdir=(0.3, -0.2, 0.9))) for _ in range(20)]
+    before = used()
+    out = [F.run(s, R=4, M=6, T=T, seed=1, dtype="c128") for s in systems]
+    assert used() - before < (17 << 30) + (1 << 29)               # and 20 workspaces of 45 MB
+    again = F.run(systems[-1], R=4, M=6, T=T, seed=1, dtype="c128")
+    assert np.array_equal(out[-1]["alpha"], again["alpha"])
+    for o in out[1:]:
+        for k in ("alpha", "beta", "p"):
+            scale = max(np.abs(out[0][k]).max(), np.abs(out[0]["beta"]).max() * (k == "alpha"))
+            assert np.abs(o[k] - out[0][k]).max() < 3e-11 * scale
+    for s in systems[:2]:
+        s.close()
+    s = F.System.from_dict(W.chain(11, Bdir=(0.3, -0.2, 0.9)))    # room again: the stored rows' bits
+    new = F.run(s, R=4, M=6, T=T, seed=1, dtype="c128")
+    assert np.array_equal(new["alpha"], out[0]["alpha"])
+    for t in systems[2:] + [s]:
+        t.close()
+    assert used() - before < 1 << 30
