@@ -2367,6 +2367,10 @@ struct ftlm_csr {
   long long dim = 0;
   uint64_t nnz = 0;
   DevBuf rp, col, val;
+  DevBuf counts;  // of the rows, while it is assembled
+  ~ftlm_csr() {
+    for (DevBuf* b : {&rp, &col, &val, &counts}) b->release();
+  }
 };
 
 extern "C" {
@@ -2395,15 +2399,14 @@ ftlm_status ftlm_csr_create(const ftlm_system* s, ftlm_dtype dtype, ftlm_csr** o
   if (smem > 227 * 1024) return fail(FTLM_ERR_UNSUPPORTED, "coupling tables do not fit in shared memory");
   CKI(csr_prepare(std::max<size_t>(smem, 48 * 1024)));
   cudaStream_t st = s->own_stream;
-  DevBuf counts;
-  if (counts.ensure(sizeof(int) * (size_t)dim) != cudaSuccess || m->rp.ensure(sizeof(long long) * (size_t)(dim + 1)) != cudaSuccess)
+  if (m->counts.ensure(sizeof(int) * (size_t)dim) != cudaSuccess || m->rp.ensure(sizeof(long long) * (size_t)(dim + 1)) != cudaSuccess)
     return fail(FTLM_ERR_OUT_OF_MEMORY, "row pointers");
-  CKI(launch_csr_count(a, c64, smem, reinterpret_cast<int*>(counts.p), st));
-  CKI(csr_scan(reinterpret_cast<const int*>(counts.p), reinterpret_cast<long long*>(m->rp.p), dim, st));
+  CKI(launch_csr_count(a, c64, smem, reinterpret_cast<int*>(m->counts.p), st));
+  CKI(csr_scan(reinterpret_cast<const int*>(m->counts.p), reinterpret_cast<long long*>(m->rp.p), dim, st));
   long long nnz = 0;
   CK(cudaMemcpyAsync(&nnz, reinterpret_cast<long long*>(m->rp.p) + dim, sizeof(long long), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  counts.release();
+  m->counts.release();
   m->nnz = (uint64_t)nnz;
   if (m->col.ensure(sizeof(int) * (size_t)nnz) != cudaSuccess || m->val.ensure((size_t)nnz * (c64 ? 8 : 16)) != cudaSuccess)
     return fail(FTLM_ERR_OUT_OF_MEMORY, "stored matrix of " + std::to_string(nnz) + " elements");

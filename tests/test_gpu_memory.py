@@ -117,3 +117,15 @@ def test_stored_rows_of_many_systems_are_bounded():
     for t in systems[2:] + [s]:
         t.close()
     assert used() - before < 1 << 30
+
+
+def test_a_stored_matrix_gives_its_memory_back():
+    s = F.System.from_dict(W.square_lattice(5, 3, seed=1))
+    F.CsrMatrix(s, "c64").close()
+    before = used()
+    for _ in range(3):
+        m = F.CsrMatrix(s, "c64")
+        assert used() - before > m.bytes // 2
+        m.close()
+        assert used() == before
+    s.close()
