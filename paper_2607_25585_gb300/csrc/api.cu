@@ -13,6 +13,8 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <new>
+#include <shared_mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -104,9 +106,13 @@ struct ftlm_system {
   bool apply_used = false;
   std::mutex apply_mu;   // the blocks, event and tables that products use; a run holds it only to look at them
   std::mutex mu;
+  std::shared_mutex use;  // shared: a call that uses the system's blocks; exclusive: giving optional ones back
 };
 
 namespace {
+
+std::mutex g_live_mu;
+std::vector<ftlm_system*> g_live;  // every system that has not been destroyed
 
 std::mutex g_mu;
 uint64_t g_next_id = 1;
@@ -791,6 +797,56 @@ void release_stored(DevBuf& b) {
   b.release();
 }
 
+// Gives back what the current device's systems keep for speed alone (the
+// rotated-basis blocks and tables, stored rows, transposed blocks) where no call is
+// using them; true if there was any.
+bool give_back() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaGetLastError(), false;
+  std::lock_guard<std::mutex> live(g_live_mu);
+  bool any = false;
+  for (ftlm_system* s : g_live) {
+    if (s->device != dev) continue;
+    std::unique_lock<std::shared_mutex> lk(s->use, std::try_to_lock);
+    if (!lk) continue;
+    for (DevBuf* b : {&s->rW, &s->Tw, &s->rD[0], &s->rD[1], &s->Ta, &s->Tb, &s->rows[0], &s->rows[1]}) {
+      if (!b->p) continue;
+      if (!any && cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), false;  // products may be in flight
+      any = true;
+      if (b == &s->rows[0] || b == &s->rows[1]) release_stored(*b);
+      else b->release();
+    }
+    s->rows_done[0] = s->rows_done[1] = false;
+    s->gen++;  // captured graphs hold their addresses
+  }
+  return any;
+}
+
+// Runs an entry point's body for the systems; where device memory does not suffice,
+// gives back what systems keep for speed alone and runs it once more, `lean`: without
+// taking such blocks again.  Nothing thrown crosses the C interface.
+template <typename Body>
+ftlm_status with_memory(const std::vector<ftlm_system*>& sys, Body&& body) {
+  try {
+    for (const bool lean : {false, true}) {
+      ftlm_status st;
+      {
+        std::vector<std::shared_lock<std::shared_mutex>> locks;
+        for (ftlm_system* s : sys) locks.emplace_back(s->use);
+        st = body(lean);
+      }
+      if (st != FTLM_ERR_OUT_OF_MEMORY || lean) return st;
+      const std::string what = g_err;
+      if (!give_back()) return fail(st, what);
+    }
+  } catch (const std::bad_alloc&) {
+    return fail(FTLM_ERR_OUT_OF_MEMORY, "out of host memory");
+  } catch (const std::exception& e) {
+    return fail(FTLM_ERR_CUDA, e.what());
+  }
+  return FTLM_ERR_OUT_OF_MEMORY;
+}
+
 // The system's stored rows for work on stream st: written by the first call, on
 // its st (not on the system's own stream, which another thread's run may be
 // capturing); other streams wait for them.  ok = false: the gathers run -- the
@@ -1387,6 +1443,20 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
 
 // ---- symmetric estimator: O_ij = <v_i|u.S|v_j> per vector ---------------------
 
+// A symmetric run's blocks besides its Lanczos vectors: partial sums of O, the O
+// matrices, and u.S q_k of all stored vectors (as large as these).
+ftlm_status ensure_symmetric(ftlm_system* s, int R, int M, int c64) {
+  const long long d = (long long)s->hs.dim;
+  if ((long long)R * M > 65535) return fail(FTLM_ERR_UNSUPPORTED, "symmetric run: R * M must not exceed 65535");
+  const size_t pbytes = sizeof(double) * sym_partial_doubles(R, M, sym_ranges(d, R, M));
+  const size_t obytes = sizeof(double) * 2 * (size_t)R * M * M, wbytes = (size_t)d * R * (c64 ? 8 : 16) * M;
+  if (s->Wc.ensure(pbytes) != cudaSuccess) return fail(FTLM_ERR_OUT_OF_MEMORY, "O matrix partial sums");
+  if (s->Od.ensure(obytes) != cudaSuccess) return fail(FTLM_ERR_OUT_OF_MEMORY, "O matrices");
+  if (s->Ws.ensure(wbytes) != cudaSuccess)
+    return fail(FTLM_ERR_OUT_OF_MEMORY, "symmetric run: " + std::to_string(wbytes) + " bytes for u.S of the Lanczos vectors");
+  return FTLM_OK;
+}
+
 // After a symmetric run: G_r[i][j] = <q_i|u.S q_j> for the stored unnormalised
 // vectors q_0 .. q_{M-1} of every vector r: u.S of all of them, the contraction
 // and a fixed-order reduction of its per-range partials; then O_ij = sigma_i sigma_j G_ij on
@@ -1396,23 +1466,7 @@ ftlm_status symmetric_matrices(ftlm_system* s, const ftlm_run_params* p, cudaStr
   const int R = p->R, M = p->M, c64 = p->dtype == FTLM_C64;
   const long long d = (long long)s->hs.dim;
   const int nranges = sym_ranges(d, R, M);
-  const size_t pbytes = sizeof(double) * sym_partial_doubles(R, M, nranges);
-  if (s->Wc.bytes < pbytes) {
-    s->Wc.release();
-    if (s->Wc.ensure(pbytes) != cudaSuccess) return fail(FTLM_ERR_OUT_OF_MEMORY, "O matrix partial sums");
-  }
   const size_t obytes = sizeof(double) * 2 * (size_t)R * M * M;
-  if (s->Od.bytes < obytes) {
-    s->Od.release();
-    if (s->Od.ensure(obytes) != cudaSuccess) return fail(FTLM_ERR_OUT_OF_MEMORY, "O matrices");
-  }
-  // u.S q_k of all stored vectors (as large as the stored vectors)
-  const size_t wbytes = (size_t)d * R * (c64 ? 8 : 16) * M;
-  if (s->Ws.bytes < wbytes) {
-    s->Ws.release();
-    if (s->Ws.ensure(wbytes) != cudaSuccess)
-      return fail(FTLM_ERR_OUT_OF_MEMORY, "symmetric run: " + std::to_string(wbytes) + " bytes for u.S of the Lanczos vectors");
-  }
   void* W = s->Ws.p;
   SdirArgs u = sdir_args(s, c64, R * M, s->Vs.p, W);
   observable_coefs(s->hs, p->obs_dir, u.obs);
@@ -1420,7 +1474,6 @@ ftlm_status symmetric_matrices(ftlm_system* s, const ftlm_run_params* p, cudaStr
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   CK(cudaEventRecord(e0, st));
-  if ((long long)R * M > 65535) return fail(FTLM_ERR_UNSUPPORTED, "symmetric run: R * M must not exceed 65535");
   CKI(launch_sdir(u, s->hs.q.data(), c64, true, st));
   CKI(launch_sym_omat(d, s->Vs.p, W, R, M, nranges, reinterpret_cast<double*>(s->Wc.p),
                       reinterpret_cast<double*>(s->Od.p), c64, st));
@@ -1445,7 +1498,8 @@ ftlm_status symmetric_matrices(ftlm_system* s, const ftlm_run_params* p, cudaStr
   return FTLM_OK;
 }
 
-ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ftlm_result* res) {
+// lean: without the blocks that a run keeps for speed alone
+ftlm_status run_impl(const std::vector<ftlm_system*>& sys, const ftlm_run_params* p, ftlm_result* res, bool lean) {
   ftlm_status vs = validate_params(p, sys);
   if (vs != FTLM_OK) return vs;
   if (!res) return fail(FTLM_ERR_INVALID_ARG, "result is NULL");
@@ -1472,16 +1526,41 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     ps = make_plan(sys, R, c64, pl, nullptr, true);
   }
   if (ps != FTLM_OK) return ps;
+  // (what a run cannot do without comes before what it takes for speed)
+  if (p->symmetric || p->reorth) {  // the M Lanczos vectors of every vector
+    ftlm_system* s0 = sys[0];
+    const size_t vb = (size_t)s0->hs.dim * R * (c64 ? 8 : 16) * M;
+    if (s0->Vs.bytes < vb) {
+      s0->Vs.release();
+      if (s0->Vs.ensure(vb) != cudaSuccess)
+        return fail(FTLM_ERR_OUT_OF_MEMORY, std::string(p->symmetric ? "symmetric" : "re-orthogonalised") +
+                                                " run: " + std::to_string(vb) + " bytes of Lanczos vectors");
+      s0->gen++;
+    }
+  }
+  if (p->symmetric) {
+    ftlm_status ss = ensure_symmetric(sys[0], R, M, c64);
+    if (ss != FTLM_OK) return ss;
+  }
+  if (p->reorth) {
+    ftlm_system* s0 = sys[0];
+    const size_t gb = sizeof(double) * 2 * (size_t)R * M;
+    if (s0->Gre.bytes < gb) {
+      s0->Gre.release();
+      CK(s0->Gre.ensure(gb));
+      s0->gen++;
+    }
+  }
   // Runs from random vectors on the default spin-1/2 plan take the rotated-basis
   // H.v.  Its error is relative to the whole vector, so starts that may be
   // sparse (basis states, a caller's block) keep the gather, which leaves the
   // rows that H does not reach exactly zero.
-  if (vm_fused_step(pl) && (p->start == FTLM_START_RANDOM || p->start == FTLM_START_PAIRS) &&
+  if (!lean && vm_fused_step(pl) && (p->start == FTLM_START_RANDOM || p->start == FTLM_START_PAIRS) &&
       rot_allowed(sys[0], R, c64)) {
     ftlm_status rs = make_rot(sys[0], R, c64, pl.rot, st);
     if (rs != FTLM_OK) return rs;
   }
-  bool forced = false;
+  bool forced = lean;
   for (auto* s : sys) forced = forced || has_shape_override(s, R, c64);
   if (plan_vmaj(pl) && !pl.rot.on && !forced) {  // small systems: stored rows in the gathers' place
     bool all = true;  // (every system's or none's: nothing is written for a batch that one system keeps on the gathers)
@@ -1519,26 +1598,6 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
     for (auto* s : sys) {
       ftlm_status hs_ = ensure_hq(s, R, c64, 1);
       if (hs_ != FTLM_OK) return hs_;
-    }
-  }
-  if (p->symmetric || p->reorth) {  // the M Lanczos vectors of every vector
-    ftlm_system* s0 = sys[0];
-    const size_t vb = (size_t)s0->hs.dim * R * (c64 ? 8 : 16) * M;
-    if (s0->Vs.bytes < vb) {
-      s0->Vs.release();
-      if (s0->Vs.ensure(vb) != cudaSuccess)
-        return fail(FTLM_ERR_OUT_OF_MEMORY, std::string(p->symmetric ? "symmetric" : "re-orthogonalised") +
-                                                " run: " + std::to_string(vb) + " bytes of Lanczos vectors");
-      s0->gen++;
-    }
-  }
-  if (p->reorth) {
-    ftlm_system* s0 = sys[0];
-    const size_t gb = sizeof(double) * 2 * (size_t)R * M;
-    if (s0->Gre.bytes < gb) {
-      s0->Gre.release();
-      CK(s0->Gre.ensure(gb));
-      s0->gen++;
     }
   }
   const std::string key = run_key(sys, p, pl);
@@ -1664,7 +1723,7 @@ ftlm_status run_impl(std::vector<ftlm_system*> sys, const ftlm_run_params* p, ft
 
 // Times candidate launch shapes of the H.v kernel on the system's workspace
 // and keeps the fastest for (n, 2s+1, R, dtype, d).
-ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
+ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st, bool lean) {
   ShapeKey key{s->hs.n, s->hs.qmax, R, c64, (long long)s->hs.dim};
   {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -1673,7 +1732,7 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
   {  // stored rows have no shape to choose, and every gather is slower on systems that small
     StoredRows r;
     bool ok = false;
-    ftlm_status rs = stream_captures(st) ? FTLM_OK : ensure_stored(s, c64, stored_limit(s, c64), R, st, r, ok);
+    ftlm_status rs = lean || stream_captures(st) ? FTLM_OK : ensure_stored(s, c64, stored_limit(s, c64), R, st, r, ok);
     if (rs != FTLM_OK || ok) return rs;
   }
   std::vector<Shape> cands;
@@ -1794,7 +1853,7 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st) {
     }
   }
   RotPlan rp;  // runs from random vectors: the rotated-basis H.v
-  if (s->hs.all_half) {
+  if (s->hs.all_half && !lean) {
     ftlm_status rs = make_rot(s, R, c64, rp, st);
     if (rs != FTLM_OK) return rs;
   }
@@ -1863,9 +1922,8 @@ ftlm_status check_product(const ftlm_system* s, const void* x, const void* y, in
   return FTLM_OK;
 }
 
-ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nvec, ftlm_dtype dtype, void* stream) {
-  ftlm_status v = check_product(cs, x, y, nvec, dtype);
-  if (v != FTLM_OK) return v;
+ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nvec, ftlm_dtype dtype, void* stream,
+                          bool lean) {
   const int c64 = dtype == FTLM_C64;
   ftlm_system* s = const_cast<ftlm_system*>(cs);
   const cudaStream_t st = pick_stream(s, stream);
@@ -1874,7 +1932,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   // writing would only happen when the graph runs) nor wait for: such a call takes
   // those gathers.  So does one whose shape was set.
   const bool plain = stream_captures(st) || has_shape_override(s, nvec, c64);
-  if (!plain) {  // small systems: stored rows
+  if (!plain && !lean) {  // small systems: stored rows
     StoredArgs a;
     bool ok = false;
     ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), nvec, st, a.rows, ok);
@@ -1899,7 +1957,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
     ftlm_status ps = make_plan(one, nvec, c64, vp, nullptr, true);
     RotPlan rp;
     const bool vm = ps == FTLM_OK && vp.half.on && vp.half.vm && vp.half.passes == 1 && !vp.half.hybrid;
-    bool rot = vm && rot_shape(s, nvec, c64, rp);
+    bool rot = vm && !lean && rot_shape(s, nvec, c64, rp);
     if (vm && (nvec > 1 || rot)) {
       // the system's blocks are shared by its calls: a call waits for the
       // previous one's kernels (on whatever stream it ran) before reusing them
@@ -2027,6 +2085,56 @@ constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void* g_noalloc_addr[kNoAllocMaxDevices] = {};  // device address of the array, per device
 
+// (arguments as ftlm_system_create)
+ftlm_status create_system(int n_sites, const int* two_s, const double* J, const double* d_ion, const double* e_axes,
+                          double g, const double* B, const double* pos, const ftlm_constants* k, ftlm_system** out) {
+  std::string msg;
+  auto s = std::make_unique<ftlm_system>();
+  ftlm_status st = build_host_system(n_sites, two_s, J, d_ion, e_axes, g, B, pos, k, s->hs, msg);
+  if (st != FTLM_OK) return fail(st, msg);
+  CK(cudaGetDevice(&s->device));
+  CK(cudaStreamCreateWithFlags(&s->own_stream, cudaStreamNonBlocking));
+  CK(cudaEventCreateWithFlags(&s->ev_in, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&s->ev_out, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&s->ev_apply, cudaEventDisableTiming));
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    s->id = g_next_id++;
+  }
+  const HostSystem& hs = s->hs;
+  s->rot = std::make_unique<RotDirs>();
+  if (!rot_directions(hs, *s->rot)) s->rot.reset();
+  std::vector<float> tf(hs.tab.begin(), hs.tab.end());
+  std::vector<long long> stv(hs.stride.begin(), hs.stride.end());
+  cudaError_t e = s->tab_d.ensure(hs.tab.size() * sizeof(double));
+  if (e == cudaSuccess) e = s->tab_f.ensure(tf.size() * sizeof(float));
+  if (e == cudaSuccess) e = s->stride.ensure(stv.size() * sizeof(long long));
+  if (e == cudaSuccess) e = s->q.ensure(hs.q.size() * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemcpy(s->tab_d.p, hs.tab.data(), hs.tab.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(s->tab_f.p, tf.data(), tf.size() * sizeof(float), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(s->stride.p, stv.data(), stv.size() * sizeof(long long), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(s->q.p, hs.q.data(), hs.q.size() * sizeof(int), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    s->tab_d.release();
+    s->tab_f.release();
+    s->stride.release();
+    s->q.release();
+    cudaEventDestroy(s->ev_in);
+    cudaEventDestroy(s->ev_out);
+    cudaEventDestroy(s->ev_apply);
+    cudaStreamDestroy(s->own_stream);
+    return fail(e == cudaErrorMemoryAllocation ? FTLM_ERR_OUT_OF_MEMORY : FTLM_ERR_CUDA,
+                std::string("uploading the coupling tables: ") + cudaGetErrorString(e));
+  }
+  {
+    std::lock_guard<std::mutex> lk(g_live_mu);
+    g_live.push_back(s.get());
+  }
+  *out = s.release();
+  return FTLM_OK;
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -2096,51 +2204,15 @@ ftlm_status ftlm_system_create(int n_sites, const int* two_s, const double* J, c
                                const ftlm_constants* k, ftlm_system** out) {
   if (!out) return fail(FTLM_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
-  std::string msg;
-  auto s = std::make_unique<ftlm_system>();
-  ftlm_status st = build_host_system(n_sites, two_s, J, d_ion, e_axes, g, B, pos, k, s->hs, msg);
-  if (st != FTLM_OK) return fail(st, msg);
-  CK(cudaGetDevice(&s->device));
-  CK(cudaStreamCreateWithFlags(&s->own_stream, cudaStreamNonBlocking));
-  CK(cudaEventCreateWithFlags(&s->ev_in, cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&s->ev_out, cudaEventDisableTiming));
-  CK(cudaEventCreateWithFlags(&s->ev_apply, cudaEventDisableTiming));
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    s->id = g_next_id++;
-  }
-  const HostSystem& hs = s->hs;
-  s->rot = std::make_unique<RotDirs>();
-  if (!rot_directions(hs, *s->rot)) s->rot.reset();
-  std::vector<float> tf(hs.tab.begin(), hs.tab.end());
-  std::vector<long long> stv(hs.stride.begin(), hs.stride.end());
-  cudaError_t e = s->tab_d.ensure(hs.tab.size() * sizeof(double));
-  if (e == cudaSuccess) e = s->tab_f.ensure(tf.size() * sizeof(float));
-  if (e == cudaSuccess) e = s->stride.ensure(stv.size() * sizeof(long long));
-  if (e == cudaSuccess) e = s->q.ensure(hs.q.size() * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemcpy(s->tab_d.p, hs.tab.data(), hs.tab.size() * sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(s->tab_f.p, tf.data(), tf.size() * sizeof(float), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(s->stride.p, stv.data(), stv.size() * sizeof(long long), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(s->q.p, hs.q.data(), hs.q.size() * sizeof(int), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    s->tab_d.release();
-    s->tab_f.release();
-    s->stride.release();
-    s->q.release();
-    cudaEventDestroy(s->ev_in);
-    cudaEventDestroy(s->ev_out);
-    cudaEventDestroy(s->ev_apply);
-    cudaStreamDestroy(s->own_stream);
-    return fail(e == cudaErrorMemoryAllocation ? FTLM_ERR_OUT_OF_MEMORY : FTLM_ERR_CUDA,
-                std::string("uploading the coupling tables: ") + cudaGetErrorString(e));
-  }
-  *out = s.release();
-  return FTLM_OK;
+  return with_memory({}, [&](bool) { return create_system(n_sites, two_s, J, d_ion, e_axes, g, B, pos, k, out); });
 }
 
 void ftlm_system_destroy(ftlm_system* s) {
   if (!s) return;
+  {
+    std::lock_guard<std::mutex> lk(g_live_mu);
+    g_live.erase(std::remove(g_live.begin(), g_live.end(), s), g_live.end());
+  }
   cudaDeviceSynchronize();  // the system's buffers may be in use on any stream
   purge_ctx_of(s->id);
   for (DevBuf* b : {&s->tab_f, &s->tab_d, &s->stride, &s->q, &s->A, &s->B, &s->U, &s->scal, &s->ep, &s->ecnt,
@@ -2165,7 +2237,10 @@ uint64_t ftlm_system_table_bytes(const ftlm_system* s) {
 }
 
 ftlm_status ftlm_apply_h(const ftlm_system* s, const void* x, void* y, int nvec, ftlm_dtype dtype, void* stream) {
-  return apply_h_entry(s, x, y, nvec, dtype, stream);
+  ftlm_status v = check_product(s, x, y, nvec, dtype);
+  if (v != FTLM_OK) return v;
+  return with_memory({const_cast<ftlm_system*>(s)},
+                     [&](bool lean) { return apply_h_entry(s, x, y, nvec, dtype, stream, lean); });
 }
 
 ftlm_status ftlm_apply_sdir(const ftlm_system* s, const double* u, const void* x, void* y, int nvec,
@@ -2227,18 +2302,26 @@ ftlm_status start_block_impl(const ftlm_system* cs, uint64_t seed, uint64_t vec_
   return FTLM_OK;
 }
 
+ftlm_status start_block_entry(const ftlm_system* cs, uint64_t seed, uint64_t vec_offset, void* out, int nvec,
+                              ftlm_dtype dtype, void* stream, bool pairs) {
+  ftlm_status v = check_block_args(cs, out, out, nvec, dtype);
+  if (v != FTLM_OK) return v;
+  return with_memory({const_cast<ftlm_system*>(cs)},
+                     [&](bool) { return start_block_impl(cs, seed, vec_offset, out, nvec, dtype, stream, pairs); });
+}
+
 }  // namespace
 
 extern "C" {
 
 ftlm_status ftlm_start_block(const ftlm_system* cs, uint64_t seed, uint64_t vec_offset, void* out, int nvec,
                              ftlm_dtype dtype, void* stream) {
-  return start_block_impl(cs, seed, vec_offset, out, nvec, dtype, stream, false);
+  return start_block_entry(cs, seed, vec_offset, out, nvec, dtype, stream, false);
 }
 
 ftlm_status ftlm_start_pairs(const ftlm_system* cs, uint64_t seed, uint64_t vec_offset, void* out, int nvec,
                              ftlm_dtype dtype, void* stream) {
-  return start_block_impl(cs, seed, vec_offset, out, nvec, dtype, stream, true);
+  return start_block_entry(cs, seed, vec_offset, out, nvec, dtype, stream, true);
 }
 
 ftlm_status ftlm_time_reverse(const ftlm_system* cs, const void* x, void* y, int nvec, ftlm_dtype dtype,
@@ -2260,16 +2343,16 @@ ftlm_status ftlm_run(const ftlm_system* s, const ftlm_run_params* p, ftlm_result
   ftlm_system* ms = const_cast<ftlm_system*>(s);
   ftlm_status pv = validate_params(p, {ms});  // host-only: before any lock or CUDA call
   if (pv != FTLM_OK) return pv;
-  std::lock_guard<std::mutex> lk(ms->mu);
-  if (p && p->autotune) {
-    ftlm_status vs = validate_params(p, {ms});
-    if (vs != FTLM_OK) return vs;
-    vs = check_device(ms);
-    if (vs != FTLM_OK) return vs;
-    ftlm_status a = autotune(ms, p->R, p->dtype == FTLM_C64, pick_stream(ms, p->stream));
-    if (a != FTLM_OK) return a;
-  }
-  return run_impl({ms}, p, res);
+  return with_memory({ms}, [&](bool lean) -> ftlm_status {
+    std::lock_guard<std::mutex> lk(ms->mu);
+    if (p->autotune) {
+      ftlm_status vs = check_device(ms);
+      if (vs != FTLM_OK) return vs;
+      ftlm_status a = autotune(ms, p->R, p->dtype == FTLM_C64, pick_stream(ms, p->stream), lean);
+      if (a != FTLM_OK) return a;
+    }
+    return run_impl({ms}, p, res, lean);
+  });
 }
 
 ftlm_status ftlm_run_batch(int n, const ftlm_system* const* systems, const ftlm_run_params* p,
@@ -2282,24 +2365,26 @@ ftlm_status ftlm_run_batch(int n, const ftlm_system* const* systems, const ftlm_
       if (o == systems[k]) return fail(FTLM_ERR_INVALID_ARG, "a system appears twice in the batch");
     v.push_back(const_cast<ftlm_system*>(systems[k]));
   }
-  std::vector<ftlm_system*> order = v;  // lock in address order
-  std::sort(order.begin(), order.end());
-  std::vector<std::unique_lock<std::mutex>> locks;
-  for (auto* s : order) locks.emplace_back(s->mu);
-  if (p && p->autotune) {
-    ftlm_status vs = validate_params(p, v);
-    if (vs != FTLM_OK) return vs;
-    for (auto* s : v) {
-      vs = check_device(s);
+  return with_memory(v, [&](bool lean) -> ftlm_status {
+    std::vector<ftlm_system*> order = v;  // lock in address order
+    std::sort(order.begin(), order.end());
+    std::vector<std::unique_lock<std::mutex>> locks;
+    for (auto* s : order) locks.emplace_back(s->mu);
+    if (p && p->autotune) {
+      ftlm_status vs = validate_params(p, v);
       if (vs != FTLM_OK) return vs;
+      for (auto* s : v) {
+        vs = check_device(s);
+        if (vs != FTLM_OK) return vs;
+      }
+      ftlm_system* big = v[0];
+      for (auto* s : v)
+        if (s->hs.dim > big->hs.dim) big = s;
+      ftlm_status a = autotune(big, p->R, p->dtype == FTLM_C64, pick_stream(v[0], p->stream), lean);
+      if (a != FTLM_OK) return a;
     }
-    ftlm_system* big = v[0];
-    for (auto* s : v)
-      if (s->hs.dim > big->hs.dim) big = s;
-    ftlm_status a = autotune(big, p->R, p->dtype == FTLM_C64, pick_stream(v[0], p->stream));
-    if (a != FTLM_OK) return a;
-  }
-  return run_impl(v, p, results);
+    return run_impl(v, p, results, lean);
+  });
 }
 
 ftlm_status ftlm_tune_shape(const ftlm_system* s, int nvec, ftlm_dtype dtype, int cube_bits, int group_vectors,
@@ -2373,20 +2458,11 @@ struct ftlm_csr {
   }
 };
 
-extern "C" {
-
-ftlm_status ftlm_csr_create(const ftlm_system* s, ftlm_dtype dtype, ftlm_csr** out) {
-  if (!s || !out) return fail(FTLM_ERR_INVALID_ARG, "system or out is NULL");
-  if (dtype != FTLM_C64 && dtype != FTLM_C128) return fail(FTLM_ERR_INVALID_ARG, "unknown dtype");
-  *out = nullptr;
-  const int c64 = dtype == FTLM_C64;
+namespace {
+ftlm_status create_csr(const ftlm_system* s, int c64, ftlm_csr** out) {
   const long long dim = (long long)s->hs.dim;
-  if (dim >= (1ll << 31)) return fail(FTLM_ERR_UNSUPPORTED, "the stored matrix needs dim < 2^31 (32-bit columns)");
-  int dev = 0;
-  CK(cudaGetDevice(&dev));
-  if (dev != s->device) return fail(FTLM_ERR_INVALID_ARG, "system lives on another device");
   auto m = std::make_unique<ftlm_csr>();
-  m->device = dev;
+  m->device = s->device;
   m->c64 = c64;
   m->dim = dim;
   LaunchArgs a;
@@ -2415,6 +2491,22 @@ ftlm_status ftlm_csr_create(const ftlm_system* s, ftlm_dtype dtype, ftlm_csr** o
   CK(cudaStreamSynchronize(st));
   *out = m.release();
   return FTLM_OK;
+}
+}  // namespace
+
+extern "C" {
+
+ftlm_status ftlm_csr_create(const ftlm_system* s, ftlm_dtype dtype, ftlm_csr** out) {
+  if (!s || !out) return fail(FTLM_ERR_INVALID_ARG, "system or out is NULL");
+  if (dtype != FTLM_C64 && dtype != FTLM_C128) return fail(FTLM_ERR_INVALID_ARG, "unknown dtype");
+  *out = nullptr;
+  const int c64 = dtype == FTLM_C64;
+  const long long dim = (long long)s->hs.dim;
+  if (dim >= (1ll << 31)) return fail(FTLM_ERR_UNSUPPORTED, "the stored matrix needs dim < 2^31 (32-bit columns)");
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  if (dev != s->device) return fail(FTLM_ERR_INVALID_ARG, "system lives on another device");
+  return with_memory({const_cast<ftlm_system*>(s)}, [&](bool) { return create_csr(s, c64, out); });
 }
 
 uint64_t ftlm_csr_nnz(const ftlm_csr* m) { return m ? m->nnz : 0; }

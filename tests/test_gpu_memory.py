@@ -129,3 +129,73 @@ def test_a_stored_matrix_gives_its_memory_back():
         m.close()
         assert used() == before
     s.close()
+
+
+def leave(nbytes):
+    """Takes all device memory but nbytes (to 2 MB pages); nothing of it is written."""
+    torch = torch_cuda()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    return torch.empty(max(0, free - nbytes) & ~((1 << 21) - 1), dtype=torch.uint8, device="cuda")
+
+
+def test_a_symmetric_run_that_fits_without_the_rotated_blocks():
+    """Lanczos vectors and u.S of them come before the blocks that only make the run
+    faster: 2^20 states, 64 vectors, 3 steps are 0.5 GB for each of three blocks and
+    1.5 GB for each of the two; the rotated blocks would take 1.6 GB more."""
+    s = F.System.from_dict(W.square_lattice(5, 4, seed=2))
+    kw = dict(R=64, M=3, T=T, seed=1, dtype="c64", symmetric=True)
+    hold = leave(5_400_000_000)
+    a = F.run(s, **kw)
+    del hold
+    torch_cuda().cuda.empty_cache()
+    s.close()
+    s = F.System.from_dict(W.square_lattice(5, 4, seed=2))
+    b = F.run(s, **kw)
+    assert a["shape"]["passes"] == 1 and b["shape"]["passes"] == 3
+    for k in ("alpha", "beta", "p", "M_B_sym"):         # (two gathers' roundings over three steps)
+        assert np.abs(a[k] - b[k]).max() < 2e-5 * max(np.abs(b[k]).max(), np.abs(b["beta"]).max() * (k == "alpha"))
+    s.close()
+
+
+def test_blocks_kept_for_speed_are_given_back():
+    """A run on a system whose workspace does not fit beside the rotated blocks and rows
+    that other systems keep: these give way, and are made again when they are used."""
+    torch = torch_cuda()
+    one = F.System.from_dict(W.square_lattice(5, 4, seed=2))
+    two = F.System.from_dict(W.chain(11, Bdir=(0.3, -0.2, 0.9)))
+    kw1, kw2 = dict(R=64, M=3, T=T, seed=1, dtype="c64"), dict(R=4, M=3, T=T, seed=1, dtype="c128")
+    a1, a2 = F.run(one, **kw1), F.run(two, **kw2)       # 1.6 GB of rotated blocks, 0.9 GB of rows
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = torch.view_as_complex(torch.randn(two.dim, 4, 2, device="cuda", generator=g)).to(torch.complex128)
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    F.apply_h(two, x, y, 4, "c128")                     # in flight when its rows give way
+    three = F.System.from_dict(W.square_lattice(5, 4, seed=7))
+    hold = leave(1_000_000_000)
+    a3 = F.run(three, **kw1)                            # 1.5 GB of workspace
+    del hold
+    torch.cuda.empty_cache()
+    assert np.isfinite(a3["lnZ"]).all()
+    b1, b2 = F.run(one, **kw1), F.run(two, **kw2)
+    F.apply_h(two, x, z, 4, "c128")
+    torch.cuda.synchronize()
+    assert torch.equal(y, z)
+    assert b1["shape"]["passes"] == 3
+    for k in ("alpha", "beta", "p"):
+        assert np.array_equal(a1[k], b1[k]) and np.array_equal(a2[k], b2[k])
+    for s in (one, two, three):
+        s.close()
+
+
+def test_what_does_not_fit_is_still_refused():
+    """Too little memory with nothing to give back: the same error, and the system stays usable."""
+    s = F.System.from_dict(W.square_lattice(5, 4, seed=2))
+    hold = leave(600_000_000)
+    with pytest.raises(F.FtlmError) as e:
+        F.run(s, R=64, M=3, T=T, seed=1, dtype="c64")
+    assert e.value.status == 2
+    del hold
+    torch_cuda().cuda.empty_cache()
+    assert np.isfinite(F.run(s, R=64, M=3, T=T, seed=1, dtype="c64")["lnZ"]).all()
+    s.close()
