@@ -847,6 +847,13 @@ ftlm_status with_memory(const std::vector<ftlm_system*>& sys, Body&& body) {
   return FTLM_ERR_OUT_OF_MEMORY;
 }
 
+// Whether a run over the systems takes stored rows: all of them or none.
+bool run_stores(const std::vector<ftlm_system*>& sys, int R, int M, int c64) {
+  bool all = true;
+  for (const ftlm_system* s : sys) all = all && stored_fits(s, c64, stored_limit(s, c64, (int)sys.size()), (long long)R * M);
+  return all;
+}
+
 // The system's stored rows for work on stream st: written by the first call, on
 // its st (not on the system's own stream, which another thread's run may be
 // capturing); other streams wait for them.  ok = false: the gathers run -- the
@@ -1563,9 +1570,8 @@ ftlm_status run_impl(const std::vector<ftlm_system*>& sys, const ftlm_run_params
   bool forced = lean;
   for (auto* s : sys) forced = forced || has_shape_override(s, R, c64);
   if (plan_vmaj(pl) && !pl.rot.on && !forced) {  // small systems: stored rows in the gathers' place
-    bool all = true;  // (every system's or none's: nothing is written for a batch that one system keeps on the gathers)
+    bool all = run_stores(sys, R, M, c64);  // (nothing is written for a batch that one system keeps on the gathers)
     uint64_t rows = 0;
-    for (auto* s : sys) all = all && stored_fits(s, c64, stored_limit(s, c64, n), (long long)R * M);
     for (auto* s : sys) {
       StoredRows r;
       if (all) {
@@ -1728,12 +1734,6 @@ ftlm_status autotune(ftlm_system* s, int R, int c64, cudaStream_t st, bool lean)
   {
     std::lock_guard<std::mutex> lk(g_mu);
     if (g_shapes.count(key)) return FTLM_OK;
-  }
-  {  // stored rows have no shape to choose, and every gather is slower on systems that small
-    StoredRows r;
-    bool ok = false;
-    ftlm_status rs = lean || stream_captures(st) ? FTLM_OK : ensure_stored(s, c64, stored_limit(s, c64), R, st, r, ok);
-    if (rs != FTLM_OK || ok) return rs;
   }
   std::vector<Shape> cands;
   if (s->hs.all_half && s->hs.n >= 4) {
@@ -2345,7 +2345,8 @@ ftlm_status ftlm_run(const ftlm_system* s, const ftlm_run_params* p, ftlm_result
   if (pv != FTLM_OK) return pv;
   return with_memory({ms}, [&](bool lean) -> ftlm_status {
     std::lock_guard<std::mutex> lk(ms->mu);
-    if (p->autotune) {
+    // stored rows have no shape to choose, and every gather is slower on systems that small
+    if (p->autotune && (lean || !run_stores({ms}, p->R, p->M, p->dtype == FTLM_C64))) {
       ftlm_status vs = check_device(ms);
       if (vs != FTLM_OK) return vs;
       ftlm_status a = autotune(ms, p->R, p->dtype == FTLM_C64, pick_stream(ms, p->stream), lean);
@@ -2370,9 +2371,9 @@ ftlm_status ftlm_run_batch(int n, const ftlm_system* const* systems, const ftlm_
     std::sort(order.begin(), order.end());
     std::vector<std::unique_lock<std::mutex>> locks;
     for (auto* s : order) locks.emplace_back(s->mu);
-    if (p && p->autotune) {
-      ftlm_status vs = validate_params(p, v);
-      if (vs != FTLM_OK) return vs;
+    ftlm_status vs = validate_params(p, v);
+    if (vs != FTLM_OK) return vs;
+    if (p->autotune && (lean || !run_stores(v, p->R, p->M, p->dtype == FTLM_C64))) {
       for (auto* s : v) {
         vs = check_device(s);
         if (vs != FTLM_OK) return vs;

@@ -143,3 +143,20 @@ def test_rows_beyond_l2(dtype, R):
         scale = max(np.abs(b[k]).max(), np.abs(b["beta"]).max() * (k == "alpha"))
         assert np.abs(a[k] - b[k]).max() < 10 * TOL[dtype] * scale
     s.close()
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_autotuned_runs_keep_their_stored_rows(batch):
+    """The autotuner and the run agree on which runs take stored rows (one vector, six
+    products: they do): the same bits with and without it, and no shape left behind."""
+    T = np.array([0.5, 5.0])
+    systems = [F.System.from_dict(W.chain(10, Bdir=d)) for d in ((0.3, -0.2, 0.9), (1, 0, 0.5))][:1 + batch]
+    kw = dict(R=1, M=6, T=T, seed=3, dtype="c128")
+    go = (lambda **k: F.run_batch(systems, **k)) if batch else (lambda **k: [F.run(systems[0], **k)])
+    a, b, c = go(**kw), go(autotune=True, **kw), go(**kw)
+    for x, y, z in zip(a, b, c):
+        for k in ("alpha", "beta", "p"):
+            assert np.array_equal(x[k], y[k]) and np.array_equal(x[k], z[k])
+    for s in systems:
+        F.tune_shape(s, 1, "c128", -1)
+        s.close()
