@@ -305,6 +305,39 @@ def run_ours(args):
     return line
 
 
+LINE_LIMIT = 2900  # bytes of the result line: readers that keep the end of a job's output still get all of it
+
+
+def split_line(line):
+    """The result line and what is left out of it: per-temperature lists, and, while
+    the line is still beyond LINE_LIMIT, the secondary legs, largest first.  What
+    is left out is {"detail": ...} with the same paths, for stderr."""
+    detail = {}
+
+    def drop_lists(d, out):
+        short = {}
+        for k, v in d.items():
+            if isinstance(v, dict):
+                sub = {}
+                short[k] = drop_lists(v, sub)
+                if sub:
+                    out[k] = sub
+            elif isinstance(v, list) and len(v) > 16:
+                out[k] = v
+            else:
+                short[k] = v
+        return short
+
+    short = drop_lists(line, detail)
+    for k in sorted(("other_workloads", "fp32_vs_fp64", "plain_fp64", "cpu_baseline"), key=lambda k: -len(json.dumps(short.get(k)))):
+        if len(json.dumps(short)) <= LINE_LIMIT:
+            break
+        if k in short:
+            detail[k] = line[k]
+            short[k] = None
+    return short, {"detail": detail} if detail else None
+
+
 def measured_traffic(shape):
     """DRAM bytes per launch of the dominant kernel from the committed ncu
     capture, or None when the kernel source or its launch shape has changed
@@ -811,7 +844,10 @@ def main():
         args.warmup = 3
     line = run_reference(args) if args.impl == "reference" else run_ours(args)
     if line is not None:
-        print(json.dumps(line), flush=True)
+        short, detail = split_line(line)
+        if detail:
+            print(json.dumps(detail), file=sys.stderr, flush=True)
+        print(json.dumps(short), flush=True)
 
 
 if __name__ == "__main__":

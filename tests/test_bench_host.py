@@ -55,3 +55,23 @@ def test_per_t_errors_floor_and_maxima():
     assert e["C"]["max_all_T"] == 0.0
     assert e["M_B"]["max_T_ge_0.1"] == 0.0 and e["M_B"]["max_all_T"] == pytest.approx(1.0)
     assert e["max_T_ge_0.1"] == pytest.approx(1e-2)
+
+
+def test_result_line_is_short_and_complete():
+    """The result line stays below its limit whatever the legs measured, keeps every
+    key, the headline and the end-to-end figures, and loses nothing: the rest is the
+    detail line."""
+    import json
+    per_t = {"max_T_ge_0.1": 1e-6, "per_T": [0.1234567890123] * 40, "fp64_per_T": [1.0] * 40}
+    legs = {"errors_vs_fp64": {k: dict(per_t) for k in ("lnZ", "E", "C", "M_B")}, "fp64_ms": 9.5}
+    line = {"metric": bench.METRIC, "value": 3.6e10, "unit": bench.UNIT, "config": {"workload": "x" * 300}, "e2e": {"value": 3.5e10},
+            "clocks": {"sm_mhz": 2070.0, "reasons": ["sw_power_cap"]}, "fp32_vs_fp64": {"a": legs, "b": legs, "T": [1.0] * 40},
+            "other_workloads": {f"leg{i}": {"note": "n" * 400, "value": 1.0} for i in range(20)}, "gpu_launches": 12}
+    short, detail = bench.split_line(line)
+    assert len(json.dumps(short)) <= bench.LINE_LIMIT < len(json.dumps(line))
+    assert list(short) == list(line)
+    for k in ("metric", "value", "unit", "config", "e2e", "clocks", "gpu_launches"):
+        assert short[k] == line[k]
+    assert detail["detail"]["other_workloads"] == line["other_workloads"]
+    assert detail["detail"]["fp32_vs_fp64"]["a"]["errors_vs_fp64"]["E"]["per_T"] == per_t["per_T"]
+    assert bench.split_line({"value": 1.0, "e2e": {"value": 2.0}}) == ({"value": 1.0, "e2e": {"value": 2.0}}, None)
