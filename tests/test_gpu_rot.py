@@ -258,3 +258,18 @@ def test_vectors_of_a_block_do_not_choose_for_each_other(dtype, rng):
     for k in (0, 2, 3, 4):
         assert np.array_equal(a[:, k], b[:, k]) and np.array_equal(c[:, k], b[:, 1])
     s.close()
+
+
+@pytest.mark.parametrize("dtype,shape,flat", [("c64", (5, 5), False), ("c64", (13, 2), False), ("c64", (7, 4), True),
+                                              ("c128", (12, 2), True), ("c128", (5, 5), False), ("c128", (13, 2), False)])
+def test_largest_tiles_and_five_directions(dtype, shape, flat):
+    """The large tiles with three and five directions, the largest systems of either
+    precision: the run against the gather's from the same start vector."""
+    w = W.square_lattice(*shape, seed=3, Bdir=(1, 1, 0)) if flat else buckled(*shape)
+    s = F.System.from_dict(w)
+    g = F.run(s, R=1, M=3, T=T, seed=3, dtype=dtype)
+    assert g["shape"]["passes"] == 3
+    x = empty_dev((s.dim, 1), dtype)
+    F.start_block(s, x, 1, 3, dtype=dtype)
+    close(g, F.run(s, R=1, M=3, T=T, start="user", user_start=x, dtype=dtype), 2e-5 if dtype == "c64" else 1e-12)
+    s.close()
