@@ -102,6 +102,9 @@ struct ftlm_system {
   cudaEvent_t ev_rows[2] = {nullptr, nullptr};  // recorded after they were written, on whichever stream did
   bool rows_done[2] = {false, false};           // that event has been seen complete
   bool rows_never[2] = {false, false};          // there was no room for them: the gathers run from then on
+  size_t row_bound = 0;                         // entries of a row at most
+  double row_entries = 0;                       // on average
+  int row_pairs = 0;                            // coupled pairs
   std::mutex rows_mu;
   bool apply_used = false;
   std::mutex apply_mu;   // the blocks, event and tables that products use; a run holds it only to look at them
@@ -769,7 +772,7 @@ size_t stored_limit(const ftlm_system* s, int c64, int n = 1) {
 
 // bytes of the system's stored rows; 0: too many sites for their builder
 size_t stored_bytes(const ftlm_system* s, int c64) {
-  const size_t S = (size_t)stored_row_bound(s->hs);
+  const size_t S = s->row_bound;
   return S == 0 || s->hs.dim > ((size_t)2 << 30) ? 0 : (size_t)s->hs.dim * (S * (c64 ? 12 : 20) + 4);
 }
 
@@ -777,6 +780,23 @@ size_t stored_bytes(const ftlm_system* s, int c64) {
 bool stored_fits(const ftlm_system* s, int c64, size_t limit, long long products) {
   const size_t b = stored_bytes(s, c64);
   return b != 0 && b <= (products < 4 ? kStoredL2 : limit);
+}
+
+// Whether stored rows are the faster form for so many vectors.  They cost 4.1 ps an
+// entry and vector in complex64, the gathers hardly more for many vectors than for
+// one: up to 8 vectors the rows are always ahead, then while entries x vectors take
+// less than the gathers' latency -- 31 us on spins 1/2 (the transposing route), on
+// other spins 45 us and 7.5 us a coupled pair.  Measured at 64 to 16,384 states and 1
+// to 256 vectors: 14 spins 1/2, 128 vectors 88 us (gather; 75 now, in rotated bases) against
+// 788 us from rows; 8 spins 1, 64 vectors 251 against 114, 256 vectors 257 against 404.
+// A run's gathers have no transposes but its steps' rows are cheaper too: up to 2e7
+// entries x vectors (12 spins 1/2, eight steps: 32 vectors 515 us against 477, 64: 647 against
+// 772; 7 spins 3/2: 8 vectors 576 against 502, 64: 1156 against 1827).  In complex128
+// the gathers form coefficients in FP64 and the rows win throughout.
+bool stored_pays(const ftlm_system* s, int c64, int nvec) {
+  if (!c64 || nvec <= 8) return true;
+  const double latency = s->hs.all_half ? 31.0 : 45.0 + 7.5 * s->row_pairs;
+  return 4.1e-6 * s->row_entries * (double)s->hs.dim * nvec <= latency;
 }
 
 // Rows of all live systems together, at most: a program may hold hundreds of systems
@@ -826,13 +846,15 @@ bool give_back() {
 // gives back what systems keep for speed alone and runs it once more, `lean`: without
 // taking such blocks again.  Nothing thrown crosses the C interface.
 template <typename Body>
-ftlm_status with_memory(const std::vector<ftlm_system*>& sys, Body&& body) {
+ftlm_status with_memory(ftlm_system* const* sys, int n, Body&& body) {
   try {
     for (const bool lean : {false, true}) {
       ftlm_status st;
       {
-        std::vector<std::shared_lock<std::shared_mutex>> locks;
-        for (ftlm_system* s : sys) locks.emplace_back(s->use);
+        std::shared_lock<std::shared_mutex> first;  // (one system: nothing allocated here)
+        std::vector<std::shared_lock<std::shared_mutex>> others;
+        if (n > 0) first = std::shared_lock<std::shared_mutex>(sys[0]->use);
+        for (int k = 1; k < n; ++k) others.emplace_back(sys[k]->use);
         st = body(lean);
       }
       if (st != FTLM_ERR_OUT_OF_MEMORY || lean) return st;
@@ -850,8 +872,12 @@ ftlm_status with_memory(const std::vector<ftlm_system*>& sys, Body&& body) {
 // Whether a run over the systems takes stored rows: all of them or none.
 bool run_stores(const std::vector<ftlm_system*>& sys, int R, int M, int c64) {
   bool all = true;
-  for (const ftlm_system* s : sys) all = all && stored_fits(s, c64, stored_limit(s, c64, (int)sys.size()), (long long)R * M);
-  return all;
+  double work = 0;
+  for (const ftlm_system* s : sys) {
+    all = all && stored_fits(s, c64, stored_limit(s, c64, (int)sys.size()), (long long)R * M);
+    work += s->row_entries * (double)s->hs.dim * R;
+  }
+  return all && (!c64 || R * sys.size() <= 8 || work <= 2e7);  // (see stored_pays)
 }
 
 // The system's stored rows for work on stream st: written by the first call, on
@@ -866,7 +892,7 @@ ftlm_status ensure_stored(ftlm_system* s, int c64, size_t limit, long long produ
   const int k = c64 ? 1 : 0;
   const size_t d = (size_t)s->hs.dim, esz = c64 ? 8 : 16;
   if (!stored_fits(s, c64, limit, products)) return FTLM_OK;
-  const size_t S = (size_t)stored_row_bound(s->hs);
+  const size_t S = s->row_bound;
   std::lock_guard<std::mutex> lk(s->rows_mu);
   DevBuf& b = s->rows[k];
   if (s->rows_never[k]) return FTLM_OK;
@@ -1932,7 +1958,7 @@ ftlm_status apply_h_entry(const ftlm_system* cs, const void* x, void* y, int nve
   // writing would only happen when the graph runs) nor wait for: such a call takes
   // those gathers.  So does one whose shape was set.
   const bool plain = stream_captures(st) || has_shape_override(s, nvec, c64);
-  if (!plain && !lean) {  // small systems: stored rows
+  if (!plain && !lean && stored_pays(s, c64, nvec)) {  // small systems: stored rows
     StoredArgs a;
     bool ok = false;
     ftlm_status rs = ensure_stored(s, c64, stored_limit(s, c64), nvec, st, a.rows, ok);
@@ -2102,6 +2128,8 @@ ftlm_status create_system(int n_sites, const int* two_s, const double* J, const 
     s->id = g_next_id++;
   }
   const HostSystem& hs = s->hs;
+  s->row_bound = (size_t)stored_row_bound(hs);
+  stored_row_work(hs, s->row_entries, s->row_pairs);
   s->rot = std::make_unique<RotDirs>();
   if (!rot_directions(hs, *s->rot)) s->rot.reset();
   std::vector<float> tf(hs.tab.begin(), hs.tab.end());
@@ -2204,7 +2232,7 @@ ftlm_status ftlm_system_create(int n_sites, const int* two_s, const double* J, c
                                const ftlm_constants* k, ftlm_system** out) {
   if (!out) return fail(FTLM_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
-  return with_memory({}, [&](bool) { return create_system(n_sites, two_s, J, d_ion, e_axes, g, B, pos, k, out); });
+  return with_memory(nullptr, 0, [&](bool) { return create_system(n_sites, two_s, J, d_ion, e_axes, g, B, pos, k, out); });
 }
 
 void ftlm_system_destroy(ftlm_system* s) {
@@ -2239,8 +2267,8 @@ uint64_t ftlm_system_table_bytes(const ftlm_system* s) {
 ftlm_status ftlm_apply_h(const ftlm_system* s, const void* x, void* y, int nvec, ftlm_dtype dtype, void* stream) {
   ftlm_status v = check_product(s, x, y, nvec, dtype);
   if (v != FTLM_OK) return v;
-  return with_memory({const_cast<ftlm_system*>(s)},
-                     [&](bool lean) { return apply_h_entry(s, x, y, nvec, dtype, stream, lean); });
+  ftlm_system* ms = const_cast<ftlm_system*>(s);
+  return with_memory(&ms, 1, [&](bool lean) { return apply_h_entry(s, x, y, nvec, dtype, stream, lean); });
 }
 
 ftlm_status ftlm_apply_sdir(const ftlm_system* s, const double* u, const void* x, void* y, int nvec,
@@ -2306,8 +2334,8 @@ ftlm_status start_block_entry(const ftlm_system* cs, uint64_t seed, uint64_t vec
                               ftlm_dtype dtype, void* stream, bool pairs) {
   ftlm_status v = check_block_args(cs, out, out, nvec, dtype);
   if (v != FTLM_OK) return v;
-  return with_memory({const_cast<ftlm_system*>(cs)},
-                     [&](bool) { return start_block_impl(cs, seed, vec_offset, out, nvec, dtype, stream, pairs); });
+  ftlm_system* s = const_cast<ftlm_system*>(cs);
+  return with_memory(&s, 1, [&](bool) { return start_block_impl(cs, seed, vec_offset, out, nvec, dtype, stream, pairs); });
 }
 
 }  // namespace
@@ -2343,7 +2371,7 @@ ftlm_status ftlm_run(const ftlm_system* s, const ftlm_run_params* p, ftlm_result
   ftlm_system* ms = const_cast<ftlm_system*>(s);
   ftlm_status pv = validate_params(p, {ms});  // host-only: before any lock or CUDA call
   if (pv != FTLM_OK) return pv;
-  return with_memory({ms}, [&](bool lean) -> ftlm_status {
+  return with_memory(&ms, 1, [&](bool lean) -> ftlm_status {
     std::lock_guard<std::mutex> lk(ms->mu);
     // stored rows have no shape to choose, and every gather is slower on systems that small
     if (p->autotune && (lean || !run_stores({ms}, p->R, p->M, p->dtype == FTLM_C64))) {
@@ -2366,7 +2394,7 @@ ftlm_status ftlm_run_batch(int n, const ftlm_system* const* systems, const ftlm_
       if (o == systems[k]) return fail(FTLM_ERR_INVALID_ARG, "a system appears twice in the batch");
     v.push_back(const_cast<ftlm_system*>(systems[k]));
   }
-  return with_memory(v, [&](bool lean) -> ftlm_status {
+  return with_memory(v.data(), (int)v.size(), [&](bool lean) -> ftlm_status {
     std::vector<ftlm_system*> order = v;  // lock in address order
     std::sort(order.begin(), order.end());
     std::vector<std::unique_lock<std::mutex>> locks;
@@ -2507,7 +2535,8 @@ ftlm_status ftlm_csr_create(const ftlm_system* s, ftlm_dtype dtype, ftlm_csr** o
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev != s->device) return fail(FTLM_ERR_INVALID_ARG, "system lives on another device");
-  return with_memory({const_cast<ftlm_system*>(s)}, [&](bool) { return create_csr(s, c64, out); });
+  ftlm_system* ms = const_cast<ftlm_system*>(s);
+  return with_memory(&ms, 1, [&](bool) { return create_csr(s, c64, out); });
 }
 
 uint64_t ftlm_csr_nnz(const ftlm_csr* m) { return m ? m->nnz : 0; }

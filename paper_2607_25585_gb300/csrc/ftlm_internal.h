@@ -381,6 +381,7 @@ struct SmallRunArgs {
 size_t small_run_smem(long long dim, int ctas, int c64);
 int launch_small_run(const SmallRunArgs& a, int vectors, int ctas, long long max_dim, int c64, void* stream);
 int stored_row_bound(const HostSystem& hs);
+void stored_row_work(const HostSystem& hs, double& entries, int& pairs);
 int launch_stored_build(const void* tab, const TabLayout& L, const long long* stride, const int* q, int n, int dim,
                         int S, int* col, void* val, int* cnt, int c64, void* stream);
 int launch_stored_step(const StoredArgs& a, int V, int c64, int grid, void* stream);

@@ -349,6 +349,27 @@ int stored_row_bound(const HostSystem& hs) {
   return (S + 3) & ~3;
 }
 
+// Average entries of a row, from its digits' distribution, and the coupled pairs.
+void stored_row_work(const HostSystem& hs, double& entries, int& pairs) {
+  const TabLayout& L = hs.lay;
+  const double* t = hs.tab.data();
+  auto on = [&](int at) { return t[at] != 0.0 || t[at + 1] != 0.0; };
+  entries = 1.0;
+  pairs = 0;
+  for (int i = 0; i < hs.n; ++i) {
+    const double step = 2.0 - 2.0 / hs.q[i];
+    bool field = on(L.off_hp + 2 * i) || on(L.off_bz + 2 * i);
+    for (int j = 0; j < hs.n; ++j) field = field || on(L.off_rho + 2 * (i * hs.n + j));
+    if (field) entries += step;
+    if (on(L.off_bb + 2 * i)) entries += 2.0 * std::max(0, hs.q[i] - 2) / hs.q[i];
+    for (int j = i + 1; j < hs.n; ++j) {
+      const int e = 2 * (i * hs.n + j), kinds = on(L.off_pm + e) + on(L.off_pp + e);
+      entries += kinds * 0.5 * step * (2.0 - 2.0 / hs.q[j]);
+      pairs += kinds > 0;
+    }
+  }
+}
+
 int launch_stored_build(const void* tab, const TabLayout& L, const long long* stride, const int* q, int n, int dim,
                         int S, int* col, void* val, int* cnt, int c64, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

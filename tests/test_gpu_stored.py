@@ -160,3 +160,45 @@ def test_autotuned_runs_keep_their_stored_rows(batch):
     for s in systems:
         F.tune_shape(s, 1, "c128", -1)
         s.close()
+
+
+MANY = {"halves11": (lambda: W.square_lattice(11, 1, seed=1), (8, 9, 64)),
+        "halves12": (lambda: W.square_lattice(12, 1, seed=1), (16, 23, 24, 130)),
+        "halves14": (lambda: W.square_lattice(14, 1, seed=1), (4, 8, 9, 128)),
+        "bonds14": (lambda: W.ladder(7, dipolar=False), (32, 64, 200)),
+        "ones8": (lambda: W.chain(8, Bdir=(0.3, -0.2, 0.9)), (128, 200)),
+        "threehalves6": (lambda: W.ring(N=6, two_s=3), (128, 256)),
+        "large spins": (lambda: W.ring(N=4, two_s=9), (9, 64, 128))}
+
+
+@pytest.mark.parametrize("name", MANY)
+def test_products_of_many_vectors_on_both_sides_of_the_rule(name, rng):
+    """Blocks that take stored rows and blocks that take the gathers, against the oracle."""
+    w, sizes = MANY[name][0](), MANY[name][1]
+    s = F.System.from_dict(w)
+    for R in sizes:
+        x = to_dev(rng.normal(size=(s.dim, R)) + 1j * rng.normal(size=(s.dim, R)), "c64")
+        y = empty_dev((s.dim, R), "c64")
+        F.apply_h(s, x, y, R, "c64")
+        cols = [0, R // 2, R - 1]
+        ref = oracle.apply_h(osys(w), np.ascontiguousarray(x.cpu().numpy()[:, cols]).astype(np.complex128))
+        assert rel_l2(y.cpu().numpy()[:, cols], ref) < TOL["c64"]
+    s.close()
+
+
+def test_products_of_many_vectors_are_not_left_to_the_rows():
+    """14 spins 1/2 and 128 vectors: the gathers take 0.09 ms, the stored rows 0.8 ms."""
+    torch = torch_cuda()
+    s = F.System.from_dict(W.square_lattice(14, 1, seed=1))
+    x = torch.view_as_complex(torch.randn(s.dim, 128, 2, device="cuda"))
+    y = torch.empty_like(x)
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    for _ in range(3):
+        F.apply_h(s, x, y, 128, "c64")
+    a.record()
+    for _ in range(10):
+        F.apply_h(s, x, y, 128, "c64")
+    b.record()
+    torch.cuda.synchronize()
+    assert a.elapsed_time(b) / 10 < 0.3
+    s.close()
