@@ -842,11 +842,21 @@ bool give_back() {
   return any;
 }
 
+// Allocations, event waits and copies of this thread take no part in a capture that
+// another thread has open (CUDA's default mode refuses them then, and the capture is
+// lost); in this thread's own capture they stay refused.
+struct ApartFromCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
+  ApartFromCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~ApartFromCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Runs an entry point's body for the systems; where device memory does not suffice,
 // gives back what systems keep for speed alone and runs it once more, `lean`: without
 // taking such blocks again.  Nothing thrown crosses the C interface.
 template <typename Body>
 ftlm_status with_memory(ftlm_system* const* sys, int n, Body&& body) {
+  ApartFromCaptures apart;
   try {
     for (const bool lean : {false, true}) {
       ftlm_status st;

@@ -136,3 +136,43 @@ def test_captured_product_leaves_the_system_usable(system, nvec, warm):
     b = F.run(s, R=nvec, M=3, T=T, seed=1, dtype="c64")
     assert np.array_equal(a["alpha"], b["alpha"])
     s.close()
+
+
+@pytest.mark.parametrize("system", ["halves", "ones", "small ones"])
+def test_first_products_while_another_thread_captures(system):
+    """A system's first products allocate and write what they keep; a capture that
+    another thread has open (in CUDA's default, global mode) and the products both
+    come to their end."""
+    torch = torch_cuda()
+    w = {"halves": lambda: W.square_lattice(4, 4, seed=3), "ones": lambda: W.chain(10, Bdir=(0.3, -0.2, 0.9)),
+         "small ones": lambda: W.chain(7, Bdir=(0.3, -0.2, 0.9))}[system]()
+    s = F.System.from_dict(w)
+    blocks = [dense(s, nvec, 5) for nvec in (4, 1)]
+    outs = [torch.zeros_like(x) for x in blocks]
+    a = torch.ones(1 << 10, device="cuda")
+    stream, other = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    fault = []
+
+    def products():
+        try:
+            for x, y in zip(blocks, outs):
+                F.apply_h(s, x, y, x.shape[1], "c64", stream=other)
+        except Exception as e:  # noqa: BLE001 (told to the test's thread)
+            fault.append(e)
+
+    with torch.cuda.graph(g, stream=stream):
+        a.add_(1)
+        t = threading.Thread(target=products)
+        t.start()
+        t.join()
+        a.mul_(2)
+    assert not fault
+    g.replay()
+    torch.cuda.synchronize()
+    assert float(a[0]) == 4.0
+    for x, y in zip(blocks, outs):
+        ref = oracle.apply_h(osys(w), x.cpu().numpy().astype(np.complex128))
+        assert rel_l2(y.cpu().numpy(), ref) < 1e-6
+    s.close()
