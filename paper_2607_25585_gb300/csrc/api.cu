@@ -1405,7 +1405,6 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
     d.u = U;
     d.M = M;
     d.tol = p->breakdown_tol > 0 ? p->breakdown_tol : (c64 ? 1e-6 : 1e-12);
-    observable_coefs(s->hs, p->obs_dir, d.obs);  // per instance: each system has its own field direction
     InstDesc e = d, o = d, t = d;
     e.x = A;
     e.y = B;

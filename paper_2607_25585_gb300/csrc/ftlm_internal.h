@@ -107,7 +107,6 @@ struct InstDesc {
   DevScalars sc;
   double tol = 0.0;          // breakdown tolerance
   int M = 0;
-  double obs[3] = {0, 0, 0}; // observable u.S: u_z, Re a_u, Im a_u with a_u = (u_x - i u_y)/2
   StoredRows stored;         // when the run's systems have them
 };
 
@@ -397,7 +396,7 @@ struct SdirArgs {
   long long dim = 0;
   const void* x = nullptr;
   void* y = nullptr;
-  double obs[3] = {0, 0, 0};
+  double obs[3] = {0, 0, 0};    // u_z, Re a, Im a with a = (u_x - i u_y) / 2
   const double* sigma = nullptr;
   int T = 0, n_low = 0, cols = 0;  // set by the launcher: tile rows, sites within a tile, packs of a row a CTA takes
 };

@@ -374,7 +374,7 @@ int launch_stored_build(const void* tab, const TabLayout& L, const long long* st
                         int S, int* col, void* val, int* cnt, int c64, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (n > kStoredMaxSites) return (int)cudaErrorInvalidValue;
-  const int grid = std::min((dim + kBuildWarps - 1) / kBuildWarps, 152 * 8);
+  const int grid = std::min((dim + kBuildWarps - 1) / kBuildWarps, 8 * std::max(1, device_sm_count()));
   if (c64)
     stored_build_kernel<float><<<grid, 32 * kBuildWarps, 0, st>>>((const float*)tab, L, stride, q, n, dim, S, col, (float*)val, cnt);
   else
