@@ -119,10 +119,12 @@ uint64_t ftlm_system_table_bytes(const ftlm_system* sys);
  * values, so a repeated call gives the same bits.  Which kernels run depends on
  * the system, on this call and, within a block, on each vector by itself: stored
  * rows where they take at most 32 MB (complex128 on spins other than 1/2 and
- * nvec >= 4: 2 GB), built on the first such call; for spin-1/2 blocks the
+ * nvec >= 4: 2 GB; 16 GB for all live systems), written by the first such call, and
+ * in complex64 not for more vectors than they serve well; for spin-1/2 blocks the
  * rotated-basis passes; for other spins in complex64 the tile gather; else, and
  * on a stream that is being captured, gathers that keep nothing.  Where the
- * memory for one of them cannot be had, the gathers run.
+ * memory for one of them cannot be had, the gathers run; what a system keeps for
+ * speed alone gives way when any call runs out of device memory.
  * Rounding: a gathered row's error is relative to the sum of its terms'
  * magnitudes, and rows that H does not reach are exactly zero.  The
  * rotated-basis passes' is relative to the whole vector, so they take only the

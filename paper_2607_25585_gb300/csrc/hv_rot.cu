@@ -19,7 +19,7 @@
 // Complex64 runs of five steps against complex128, 14 to 27 sites in and out of
 // the plane, five to eight seeds each, root mean square of the relative error:
 // alpha 4e-8 to 9e-8 (16e-8 at 14 sites) where the gather's is 4e-8 to 11e-8 (63e-8),
-// beta and p 3e-8 to 5e-8 in both.
+// beta and p 3e-8 to 6e-8 in both.
 //
 // The gate.  All u_k have the same polar angle theta; with t = tan(theta / 2)
 // and the azimuth's phase e^{-i phi_k} taken out per down spin,
@@ -61,10 +61,11 @@
 //
 // Bound: memory.  A step moves 8 (7 + 4 K) bytes a value in complex64 (152 for
 // K = 3), against 56 for the gather, but the gather's C(n, 2) flips take 3.5 ms
-// at n = 20 with 64 vectors, where these passes take 1.71 ms with the update
-// (3.8 ms with it before): 6.0 TB/s.  2 x 13 sites, 4 vectors: 33 -> 11.0 ms a
-// step.  In complex128 the FP64 pipe binds both: 4 x 4 sites, 50 vectors:
-// 4.0 -> 1.57 ms.  Taking one to eight vectors at a time through the three
+// at n = 20 with 64 vectors, where these passes take 1.67 ms with the update
+// (3.8 ms with it before): 6.1 TB/s.  2 x 13 sites, 4 vectors: 33 -> 11.0 ms a
+// step, 3.7 TB/s: one CTA an SM loads, exchanges and stores in turn, and the middle
+// pass (2.8 TB/s) reads rows of 32 bytes.  In complex128 the FP64 pipe binds both:
+// 4 x 4 sites, 50 vectors: 4.0 -> 1.57 ms.  Taking one to eight vectors at a time through the three
 // passes, so that W stays in L2, was slower (2.1 to 3.0 ms): each launch then
 // has too few tiles.
 #include <cuda_runtime.h>

@@ -9,7 +9,10 @@
 // written out once, on its first product (a warp a row, lanes over the terms),
 // and each product is then short sums: eight lanes a row, a group of V vectors,
 // added in a fixed order.  Zero elements are not stored, so rows that H does not
-// connect stay exactly zero, as in the gathers.
+// connect stay exactly zero, as in the gathers.  Against extended precision the rows'
+// products in complex128 have errors of 1.8 to 2.5e-16, the gathers' 3.8 to 5.0e-16.  For
+// many complex64 vectors the rows are read again for every four and the gathers win
+// (api.cu, stored_pays).
 #include <cuda_runtime.h>
 
 #include <algorithm>

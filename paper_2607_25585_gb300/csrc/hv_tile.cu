@@ -19,7 +19,7 @@
 // coefficients).  The register-cube gather loads every pair's rows through L1 and
 // waits for L2 between them.  A step of the 24 chains of 10 to 12 spins 1 with 16
 // vectors: 8.6 -> 7.0 ms; of ten 9-site molecules of spins 5/2 and 2 with 8
-// vectors: 16.1 -> 13.7 ms.  Coefficients with no imaginary part (all s+ s- ones, and s+
+// vectors: 16.1 -> 14.2 ms.  Coefficients with no imaginary part (all s+ s- ones, and s+
 // s+ ones of chains along an axis) take one packed FMA a value instead of two.
 // Tiles of 81 bases (9.3 ms) or 729 (8.4 ms, one CTA an SM) were slower.
 // Copying all the high sites' rows ahead through shared memory (8.1 ms on the chains,
