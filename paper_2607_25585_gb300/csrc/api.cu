@@ -791,8 +791,9 @@ bool stored_fits(const ftlm_system* s, int c64, size_t limit, long long products
 // 788 us from rows; 8 spins 1, 64 vectors 251 against 114, 256 vectors 257 against 404.
 // A run's gathers have no transposes but its steps' rows are cheaper too: up to 2e7
 // entries x vectors (12 spins 1/2, eight steps: 32 vectors 515 us against 477, 64: 647 against
-// 772; 7 spins 3/2: 8 vectors 576 against 502, 64: 1156 against 1827).  In complex128
-// the gathers form coefficients in FP64 and the rows win throughout.
+// 772; 7 spins 3/2: 8 vectors 576 against 502, 64: 1156 against 1827), in a batch for
+// each system by itself (24 chains of 10 spins 1/2, 48 vectors: 7.0 ms against 3.0).  In
+// complex128 the gathers form coefficients in FP64 and the rows win throughout.
 bool stored_pays(const ftlm_system* s, int c64, int nvec) {
   if (!c64 || nvec <= 8) return true;
   const double latency = s->hs.all_half ? 31.0 : 45.0 + 7.5 * s->row_pairs;
@@ -882,12 +883,11 @@ ftlm_status with_memory(ftlm_system* const* sys, int n, Body&& body) {
 // Whether a run over the systems takes stored rows: all of them or none.
 bool run_stores(const std::vector<ftlm_system*>& sys, int R, int M, int c64) {
   bool all = true;
-  double work = 0;
   for (const ftlm_system* s : sys) {
     all = all && stored_fits(s, c64, stored_limit(s, c64, (int)sys.size()), (long long)R * M);
-    work += s->row_entries * (double)s->hs.dim * R;
+    if (c64 && R > 8) all = all && s->row_entries * (double)s->hs.dim * R <= 2e7;  // (see stored_pays)
   }
-  return all && (!c64 || R * sys.size() <= 8 || work <= 2e7);  // (see stored_pays)
+  return all;
 }
 
 // The system's stored rows for work on stream st: written by the first call, on
