@@ -117,6 +117,14 @@ namespace {
 std::mutex g_live_mu;
 std::vector<ftlm_system*> g_live;  // every system that has not been destroyed
 
+// Shared: a run's capture in progress; exclusive: a wait for the whole device, which
+// CUDA refuses while any stream is being captured.
+std::shared_mutex g_capture;
+cudaError_t wait_for_device() {
+  std::unique_lock<std::shared_mutex> lk(g_capture);
+  return cudaDeviceSynchronize();
+}
+
 std::mutex g_mu;
 uint64_t g_next_id = 1;
 size_t g_prepared_smem = 0;
@@ -642,7 +650,7 @@ ftlm_status ensure_unit_tables(ftlm_system* s, int K, int c64, cudaStream_t st) 
   const int n = s->hs.n;
   const long long nunits = (long long)(s->hs.dim >> (kVmLaneBits + K));
   const size_t bytes = (size_t)nunits * vm_unit_table_stride(n, K) * (c64 ? 4 : 8);
-  if (b.p) CK(cudaDeviceSynchronize());  // a rebuild: no launch may still read the old tables
+  if (b.p) CK(wait_for_device());  // a rebuild: no launch may still read the old tables
   b.release();
   CK(b.ensure(bytes));
   CKI(launch_vm_unit_tables(reinterpret_cast<const double*>(s->tab_d.p), s->hs.lay, n, K, nunits, b.p, c64, st));
@@ -832,7 +840,7 @@ bool give_back() {
     if (!lk) continue;
     for (DevBuf* b : {&s->rW, &s->Tw, &s->rD[0], &s->rD[1], &s->Ta, &s->Tb, &s->rows[0], &s->rows[1]}) {
       if (!b->p) continue;
-      if (!any && cudaDeviceSynchronize() != cudaSuccess) return cudaGetLastError(), false;  // products may be in flight
+      if (!any && wait_for_device() != cudaSuccess) return cudaGetLastError(), false;  // products may be in flight
       any = true;
       if (b == &s->rows[0] || b == &s->rows[1]) release_stored(*b);
       else b->release();
@@ -1469,10 +1477,12 @@ ftlm_status build_ctx(RunCtx& c, const std::vector<ftlm_system*>& sys, const ftl
     c.ev.resize(4 * M + 2);
     for (auto& e : c.ev) CK(cudaEventCreate(&e));
   }
+  std::shared_lock<std::shared_mutex> capturing(g_capture);
   CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   ftlm_status es = enqueue_run(c, sys, p, pl, st);
   cudaGraph_t g = nullptr;
   cudaError_t ce = cudaStreamEndCapture(st, &g);
+  capturing.unlock();
   if (es != FTLM_OK) {
     if (g) cudaGraphDestroy(g);
     return es;
@@ -2250,7 +2260,7 @@ void ftlm_system_destroy(ftlm_system* s) {
     std::lock_guard<std::mutex> lk(g_live_mu);
     g_live.erase(std::remove(g_live.begin(), g_live.end(), s), g_live.end());
   }
-  cudaDeviceSynchronize();  // the system's buffers may be in use on any stream
+  wait_for_device();  // the system's buffers may be in use on any stream
   purge_ctx_of(s->id);
   for (DevBuf* b : {&s->tab_f, &s->tab_d, &s->stride, &s->q, &s->A, &s->B, &s->U, &s->scal, &s->ep, &s->ecnt,
                     &s->esc, &s->Hq, &s->Vs, &s->Wc, &s->Od, &s->Gre, &s->Ta, &s->Tb, &s->ut[0], &s->ut[1], &s->Ws, &s->rD[0], &s->rD[1], &s->rW, &s->rpart, &s->Tw, &s->Ts})

@@ -9,7 +9,7 @@ import pytest
 import ftlm_workloads as W
 import oracle
 import paper_2607_25585_gb300 as F
-from gpu_helpers import empty_dev, osys, rel_l2, torch_cuda
+from gpu_helpers import osys, rel_l2, torch_cuda
 
 pytestmark = pytest.mark.gpu
 T = np.array([0.5, 5.0])
@@ -22,9 +22,9 @@ def dense(s, R, seed):
 
 
 def product(s, x, stream):
-    y = empty_dev(x.shape, "c64")
-    y.zero_()
-    torch_cuda().cuda.synchronize()
+    torch = torch_cuda()
+    with torch.cuda.stream(stream):           # (nothing that waits for the whole device: a run may be capturing)
+        y = torch.zeros_like(x)
     F.apply_h(s, x, y, x.shape[1], "c64", stream=stream)
     stream.synchronize()
     return y
@@ -176,3 +176,32 @@ def test_first_products_while_another_thread_captures(system):
         ref = oracle.apply_h(osys(w), x.cpu().numpy().astype(np.complex128))
         assert rel_l2(y.cpu().numpy(), ref) < 1e-6
     s.close()
+
+
+def test_systems_come_and_go_while_others_capture():
+    """Eight threads that create a system, run it and destroy it: what waits for the
+    whole device (a destruction) waits for the captures of other threads' runs too."""
+    w = W.ring(N=6, two_s=2)
+    kw = dict(R=2, M=120, T=T, dtype="c64", reorth=True)     # (a long capture)
+    s = F.System.from_dict(w)
+    want = F.run(s, seed=1, **kw)
+    s.close()
+    faults = []
+
+    def work():
+        for _ in range(6):
+            try:
+                s = F.System.from_dict(w)
+                r = F.run(s, seed=1, **kw)
+                s.close()
+                if not np.array_equal(r["alpha"], want["alpha"]):
+                    faults.append("other numbers")
+            except Exception as e:  # noqa: BLE001 (told to the test's thread)
+                faults.append(e)
+
+    threads = [threading.Thread(target=work) for _ in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not faults, faults[:3]
