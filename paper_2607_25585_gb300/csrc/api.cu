@@ -1054,7 +1054,7 @@ struct RunCtx {
   }
 };
 
-std::vector<std::unique_ptr<RunCtx>> g_ctx;  // small cache of captured runs, newest last
+std::vector<std::shared_ptr<RunCtx>> g_ctx;  // small cache of captured runs, newest last; a run in progress keeps its own
 
 void purge_ctx_of(uint64_t id) {
   std::lock_guard<std::mutex> lk(g_mu);
@@ -1652,20 +1652,20 @@ ftlm_status run_impl(const std::vector<ftlm_system*>& sys, const ftlm_run_params
     }
   }
   const std::string key = run_key(sys, p, pl);
-  RunCtx* ctx = nullptr;
+  std::shared_ptr<RunCtx> ctx;  // (other threads' runs may drop it from the cache meanwhile)
   size_t h2d = 0;
   {
     std::lock_guard<std::mutex> lk(g_mu);
     for (auto& c : g_ctx)
-      if (c->key == key) ctx = c.get();
+      if (c->key == key) ctx = c;
   }
   if (!ctx) {
-    auto nc = std::make_unique<RunCtx>();
+    auto nc = std::make_shared<RunCtx>();
     nc->key = key;
     ftlm_status bs = build_ctx(*nc, sys, p, pl, st);
     if (bs != FTLM_OK) return bs;
     h2d = nc->h2d;
-    ctx = nc.get();
+    ctx = nc;
     std::lock_guard<std::mutex> lk(g_mu);
     g_ctx.push_back(std::move(nc));
     if (g_ctx.size() > 8) g_ctx.erase(g_ctx.begin());

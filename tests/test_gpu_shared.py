@@ -205,3 +205,29 @@ def test_systems_come_and_go_while_others_capture():
     for t in threads:
         t.join()
     assert not faults, faults[:3]
+
+
+def test_more_runs_at_once_than_captured_runs_are_kept():
+    """Eleven threads, each with a system and runs of its own: a run's captured graph
+    stays until the run has ended, however many others are captured meanwhile."""
+    w = W.ring(N=6, two_s=2)
+    T40 = np.geomspace(1, 50, 40)
+    kw = dict(R=24, M=60, T=T40, dtype="c128")
+
+    def work(k, out):
+        s = F.System.from_dict(w)
+        out[k] = [F.run(s, seed=100 * k + j, **kw) for j in range(4)]
+        s.close()
+
+    alone, at_once = {}, {}
+    for k in range(11):
+        work(k, alone)
+    threads = [threading.Thread(target=work, args=(k, at_once)) for k in range(11)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in range(11):
+        for a, b in zip(alone[k], at_once[k]):
+            for q in ("alpha", "beta", "p", "lnZ", "M_B"):
+                assert np.array_equal(a[q], b[q]), (k, q)
