@@ -1698,45 +1698,22 @@ ftlm_status run_impl(const std::vector<ftlm_system*>& sys, const ftlm_run_params
     dev_ms = ms;
   }
   const size_t per = staged_bytes(R, M);
-  struct HostPart {
-    std::vector<double> al, be, pp;  // [R][M], [R][M], [R][M][2]
-    std::vector<int> me;
-  };
-  std::vector<HostPart> host(n);
   std::vector<HostSums> sums(n);
-  for (int k = 0; k < n; ++k) {
-    HostPart& h = host[k];
+  for (int k = 0; k < n; ++k) {  // (read where the copies left them, [M][R])
     const char* src = ctx->pinned + per * k;
-    const double* alpha_d = reinterpret_cast<const double*>(src);  // [M][R]
+    const double* alpha_d = reinterpret_cast<const double*>(src);
     const double* beta_d = alpha_d + (size_t)M * R;
-    const double* p_d = beta_d + (size_t)M * R;                     // [M][R][2]
+    const double* p_d = beta_d + (size_t)M * R;
     const int* meff = reinterpret_cast<const int*>(src + sizeof(double) * staged_doubles(R, M));
-    h.al.resize((size_t)R * M);
-    h.be.resize((size_t)R * M);
-    h.pp.resize((size_t)R * M * 2);
     for (int r = 0; r < R; ++r)
-      for (int j = 0; j < M; ++j) {
-        h.al[(size_t)r * M + j] = alpha_d[(size_t)j * R + r];
-        h.be[(size_t)r * M + j] = beta_d[(size_t)j * R + r];
-        h.pp[((size_t)r * M + j) * 2] = p_d[((size_t)j * R + r) * 2];
-        h.pp[((size_t)r * M + j) * 2 + 1] = p_d[((size_t)j * R + r) * 2 + 1];
-      }
-    h.me.assign(meff, meff + R);
-    for (int r = 0; r < R; ++r)
-      if (h.me[r] < 1 || h.me[r] > M) return fail(FTLM_ERR_NUMERICAL, "start vector of zero norm");
-    sums[k] = {R, M, h.me.data(), h.al.data(), h.be.data(), h.pp.data(), (double)sys[k]->hs.dim, sys[k]->hs.g,
+      if (meff[r] < 1 || meff[r] > M) return fail(FTLM_ERR_NUMERICAL, "start vector of zero norm");
+    sums[k] = {R, M, meff, alpha_d, beta_d, p_d, 1, (size_t)R, true, (double)sys[k]->hs.dim, sys[k]->hs.g,
                p->T, p->nT, &res[k]};
   }
   host_sums_many(sums);  // eigensolves and sums of all systems
   for (int k = 0; k < n; ++k) {
-    const std::vector<double>&al = host[k].al, &be = host[k].be, &pp = host[k].pp;
-    const std::vector<int>& me = host[k].me;
     ftlm_result& out = res[k];
     if (sums[k].status != FTLM_OK) return fail(sums[k].status, sums[k].msg);
-    if (out.alpha) std::memcpy(out.alpha, al.data(), sizeof(double) * al.size());
-    if (out.beta) std::memcpy(out.beta, be.data(), sizeof(double) * be.size());
-    if (out.p) std::memcpy(out.p, pp.data(), sizeof(double) * pp.size());
-    if (out.M_eff) std::memcpy(out.M_eff, me.data(), sizeof(int) * R);
     out.device_ms = dev_ms;
     out.hv_ms = hv_ms;
     out.gap_ms = gap_ms;
@@ -1762,7 +1739,13 @@ ftlm_status run_impl(const std::vector<ftlm_system*>& sys, const ftlm_run_params
       out.sym_ms = sms;
       if (out.M_B_sym) {
         std::string m2;
-        ftlm_status hs2 = host_sums_sym(R, M, me.data(), al.data(), be.data(), Omat.data(), sys[k]->hs.g, p->T,
+        std::vector<double> al((size_t)R * M), be((size_t)R * M);  // [R][M]
+        for (int r = 0; r < R; ++r)
+          for (int j = 0; j < M; ++j) {
+            al[(size_t)r * M + j] = sums[k].alpha[(size_t)j * R + r];
+            be[(size_t)r * M + j] = sums[k].beta[(size_t)j * R + r];
+          }
+        ftlm_status hs2 = host_sums_sym(R, M, sums[k].M_eff, al.data(), be.data(), Omat.data(), sys[k]->hs.g, p->T,
                                         p->nT, out.M_B_sym, out.M_B_sym_imag, m2);
         if (hs2 != FTLM_OK) return fail(hs2, m2);
       }

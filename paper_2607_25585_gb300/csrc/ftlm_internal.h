@@ -432,7 +432,9 @@ int launch_csr_spmm(long long dim, int R, const long long* rp, const int* col, c
 struct HostSums {
   int R = 0, M = 0;
   const int* M_eff = nullptr;
-  const double *alpha = nullptr, *beta = nullptr, *p = nullptr;
+  const double *alpha = nullptr, *beta = nullptr, *p = nullptr;  // step j of run r at r * run + j * step (p: complex)
+  size_t run = 0, step = 1;
+  bool store = false;            // also write them to res, [R][M] (res->alpha, beta, p, M_eff)
   double dim = 0, g = 0;
   const double* T = nullptr;
   int nT = 0;

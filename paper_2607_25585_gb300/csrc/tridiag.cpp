@@ -123,28 +123,31 @@ bool parallel_for(int n, double total_ns, const std::function<void(int)>& fn) {
 
 // One run's eigenproblem: its Ritz values, the weights' row U_0n and the rows Re, Im
 // of sum_j conj(p_j) U_jn.
+// (In the system's one block: four vectors a run, allocated by one thread and freed by
+// another, took 0.5 ms of a batch of 24 systems of 48 vectors.)
 struct Ritz {
-  std::vector<double> eps, w0, qr, qi;
+  double *eps = nullptr, *w0 = nullptr, *qr = nullptr, *qi = nullptr;
+  int m = 0;
 };
 
 // null, or what is wrong with run r
 const char* solve_run(const HostSums& s, int r, Ritz& run) {
-  const int m = s.M_eff[r], M = s.M;
-  run.eps.assign(s.alpha + (size_t)r * M, s.alpha + (size_t)r * M + m);
+  const int m = s.M_eff[r];
+  auto at = [&](int j) { return r * s.run + j * s.step; };
+  run.m = m;
+  for (int j = 0; j < m; ++j) run.eps[j] = s.alpha[at(j)];
   std::vector<double> e(m > 1 ? m - 1 : 1, 0.0);
-  for (int j = 0; j + 1 < m; ++j) e[j] = s.beta[(size_t)r * M + j];
-  run.w0.assign(m, 0.0);
+  for (int j = 0; j + 1 < m; ++j) e[j] = s.beta[at(j)];
+  std::fill(run.w0, run.w0 + m, 0.0);
   run.w0[0] = 1.0;
-  run.qr.resize(m);
-  run.qi.resize(m);
   for (int j = 0; j < m; ++j) {  // conj(p_j)
-    run.qr[j] = s.p[((size_t)r * M + j) * 2];
-    run.qi[j] = -s.p[((size_t)r * M + j) * 2 + 1];
+    run.qr[j] = s.p[2 * at(j)];
+    run.qi[j] = -s.p[2 * at(j) + 1];
   }
   for (int j = 0; j < m; ++j)
     if (!std::isfinite(run.eps[j]) || (j + 1 < m && !std::isfinite(e[j]))) return "non-finite Lanczos coefficient in run ";
-  double* rows[3] = {run.w0.data(), run.qr.data(), run.qi.data()};
-  return ql_implicit(m, run.eps.data(), e.data(), 3, rows) ? nullptr : "tridiagonal eigensolver did not converge (run ";
+  double* rows[3] = {run.w0, run.qr, run.qi};
+  return ql_implicit(m, run.eps, e.data(), 3, rows) ? nullptr : "tridiagonal eigensolver did not converge (run ";
 }
 
 // the results at temperature t, from the solved runs in order
@@ -154,7 +157,7 @@ void sum_runs(const HostSums& s, const std::vector<Ritz>& runs, double E0, int t
   std::vector<double> ws;  // the weights, for the variance
   ws.reserve((size_t)s.R * s.M);
   for (const Ritz& run : runs)
-    for (size_t n = 0; n < run.eps.size(); ++n) {
+    for (int n = 0; n < run.m; ++n) {
       const double boltz = std::exp(-b * (run.eps[n] - E0));
       const double w = run.w0[n] * run.w0[n] * boltz;
       ws.push_back(w);
@@ -167,7 +170,7 @@ void sum_runs(const HostSums& s, const std::vector<Ritz>& runs, double E0, int t
   double var = 0.0;
   const double* w = ws.data();
   for (const Ritz& run : runs)
-    for (size_t n = 0; n < run.eps.size(); ++n) var += *w++ * (run.eps[n] - Em) * (run.eps[n] - Em);
+    for (int n = 0; n < run.m; ++n) var += *w++ * (run.eps[n] - Em) * (run.eps[n] - Em);
   ftlm_result* res = s.res;
   if (res->lnZ) res->lnZ[t] = std::log(s.dim / s.R * z) - b * E0;
   if (res->E) res->E[t] = Em;
@@ -175,15 +178,35 @@ void sum_runs(const HostSums& s, const std::vector<Ritz>& runs, double E0, int t
   if (res->M_B) res->M_B[t] = -s.g * orr / z;
   if (res->M_B_imag) res->M_B_imag[t] = -s.g * oi / z;
 }
+// the coefficients to the caller's arrays
+void store_runs(const HostSums& s) {
+  const ftlm_result& o = *s.res;
+  for (int r = 0; r < s.R; ++r) {
+    if (o.M_eff) o.M_eff[r] = s.M_eff[r];
+    for (int j = 0; j < s.M; ++j) {
+      const size_t to = (size_t)r * s.M + j, at = r * s.run + j * s.step;
+      if (o.alpha) o.alpha[to] = s.alpha[at];
+      if (o.beta) o.beta[to] = s.beta[at];
+      if (o.p) {
+        o.p[2 * to] = s.p[2 * at];
+        o.p[2 * to + 1] = s.p[2 * at + 1];
+      }
+    }
+  }
+}
+
 }  // namespace
 
 // All systems' eigenproblems, then all their temperatures, as one list of items: a
 // batch of two long runs keeps as many threads busy as a batch of many short ones
-// (2 x 64 vectors of 200 steps: a thread a system took 52 ms).  A temperature's item
-// comes after every eigenproblem's, so the one it may have to wait for is being
-// solved on another thread.
+// (2 x 64 vectors of 200 steps: a thread a system took 52 ms).  An item is as many of a
+// system's eigenproblems, or temperatures, as make 50 us: one of 8 steps takes 1 us, and
+// the threads would spend as long passing each other the counters (24 systems of 48
+// vectors: 0.7 ms more).  A temperature's item comes after every eigenproblem's, so
+// those that it may have to wait for are being solved on other threads.
 void host_sums_many(std::vector<HostSums>& sums) {
   struct Work {
+    std::vector<double> block;  // [R][4][M]
     std::vector<Ritz> runs;
     std::vector<const char*> bad;
     std::atomic<int> left{0};
@@ -192,7 +215,14 @@ void host_sums_many(std::vector<HostSums>& sums) {
   };
   const int n = (int)sums.size();
   std::vector<Work> work(n);
-  std::vector<std::pair<int, int>> solve, sum;  // (system, run), (system, temperature)
+  struct Item {
+    int k, from, to;  // system; its runs, or its temperatures
+  };
+  std::vector<Item> solve, sum;
+  auto divide = [](std::vector<Item>& items, int k, int count, double each_ns) {
+    const int step = (int)std::min<double>(count, std::max(1.0, 50e3 / each_ns));
+    for (int i = 0; i < count; i += step) items.push_back({k, i, std::min(count, i + step)});
+  };
   double ns = 0.0;
   for (int k = 0; k < n; ++k) {
     HostSums& s = sums[k];
@@ -208,36 +238,42 @@ void host_sums_many(std::vector<HostSums>& sums) {
       if (s.M_eff[r] < 1 || s.M_eff[r] > s.M) s.msg = "M_eff out of range";
     if (!s.msg.empty()) continue;
     s.status = FTLM_OK;
+    work[k].block.resize((size_t)4 * s.R * s.M);
     work[k].runs.resize(s.R);
+    for (int r = 0; r < s.R; ++r) {
+      double* b = work[k].block.data() + (size_t)4 * r * s.M;
+      work[k].runs[r] = {b, b + s.M, b + 2 * s.M, b + 3 * s.M, 0};
+    }
     work[k].bad.assign(s.R, nullptr);
     work[k].left = s.R;
-    for (int r = 0; r < s.R; ++r) solve.emplace_back(k, r);
-    for (int t = 0; t < s.nT; ++t) sum.emplace_back(k, t);
+    divide(solve, k, s.R, ql_ns(s.M, 3));
+    divide(sum, k, s.nT, kTermNs * s.M * s.R);
     ns += s.R * (ql_ns(s.M, 3) + kTermNs * s.M * s.nT);
   }
   parallel_for((int)(solve.size() + sum.size()), ns, [&](int i) {
     if (i < (int)solve.size()) {
-      const int k = solve[i].first, r = solve[i].second;
-      Work& w = work[k];
+      const Item it = solve[i];
+      Work& w = work[it.k];
       try {
-        w.bad[r] = solve_run(sums[k], r, w.runs[r]);
+        for (int r = it.from; r < it.to; ++r) w.bad[r] = solve_run(sums[it.k], r, w.runs[r]);
       } catch (...) {
         w.memory = true;
       }
-      if (w.left.fetch_sub(1) == 1) {  // the system's last: its lowest Ritz value
+      if (w.left.fetch_sub(it.to - it.from) == it.to - it.from) {  // the system's last: its lowest Ritz value
         for (const Ritz& run : w.runs)
-          for (double e : run.eps) w.E0 = std::min(w.E0, e);
+          for (int n = 0; n < run.m; ++n) w.E0 = std::min(w.E0, run.eps[n]);
         w.left.store(-1);
       }
       return;
     }
-    const auto [k, t] = sum[i - solve.size()];
-    Work& w = work[k];
+    const Item it = sum[i - solve.size()];
+    Work& w = work[it.k];
     while (w.left.load() >= 0) std::this_thread::yield();
     for (const char* b : w.bad)
       if (b || w.memory) return;
+    if (it.from == 0 && sums[it.k].store) store_runs(sums[it.k]);
     try {
-      sum_runs(sums[k], w.runs, w.E0, t);
+      for (int t = it.from; t < it.to; ++t) sum_runs(sums[it.k], w.runs, w.E0, t);
     } catch (...) {
       w.memory = true;
     }
@@ -262,7 +298,7 @@ void host_sums_many(std::vector<HostSums>& sums) {
 ftlm_status host_sums(int R, int M, const int* M_eff, const double* alpha, const double* beta, const double* p,
                       double dim, double g, const double* T, int nT, ftlm_result* res, std::string& msg) {
   std::vector<HostSums> one(1);
-  one[0] = {R, M, M_eff, alpha, beta, p, dim, g, T, nT, res};
+  one[0] = {R, M, M_eff, alpha, beta, p, (size_t)std::max(0, M), 1, false, dim, g, T, nT, res};
   host_sums_many(one);
   msg = one[0].msg;
   return one[0].status;
